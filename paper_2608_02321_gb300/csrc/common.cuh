@@ -5,7 +5,11 @@
 //            (neighbour << lbits) | edge_label, rows sorted by neighbour;
 //            vinfo u32 [V] = vertex label (low 16 bits) | (self-loop label + 1) << 16
 //            (0 in the high half = no self-loop); attrs i32 [n_attrs][V];
-//            sig u64x2 [V] = (out-, in-neighbourhood signature).
+//            sig u64x2 [V] = (out-, in-neighbourhood signature). Vertices are
+//            numbered by (degree class, label, falling degree, caller's id),
+//            class c ending at class_end[c]; orig u32 [V] =
+//            the caller's ids, and o_vinfo, o_out_off, o_in_off hold label and
+//            degrees in the caller's order (for the allocation-free filter).
 //   index:   per (GFD, level) a candidate bitmap [nwords] u32, its exclusive
 //            popcount prefix [nwords] u32 (so rank(v) is O(1)), the sorted
 //            candidate list i32, and for every level i >= 1 the index edges of
@@ -37,6 +41,12 @@ constexpr int32_t NOEDGE = -2;
 constexpr int ROW_SHIFT = 40;
 constexpr uint64_t WORK_MASK = (1ull << ROW_SHIFT) - 1;
 
+// Degree classes (edges in both directions together): class c holds the vertices
+// with more than class_degree(c) that are not in an earlier class, the last class
+// the rest.
+constexpr int N_CLASS = 4;
+__host__ __device__ constexpr uint32_t class_degree(int c) { return c == 0 ? 2048 : c == 1 ? 256 : 32; }
+
 struct DevGraph {
     int32_t n;
     int32_t n_attrs;
@@ -54,6 +64,12 @@ struct DevGraph {
     // out-neighbour w of v, sig[v].y for every in-neighbour; a clear bit proves
     // that the edge is absent
     const ulonglong2* sig;
+    uint32_t class_end[N_CLASS - 1];  // ends of the first degree classes
+    // the caller's id of each vertex, and vertex data in the caller's order
+    const uint32_t* orig;
+    const uint32_t* o_vinfo;
+    const uint32_t* o_out_off;
+    const uint32_t* o_in_off;
 };
 
 // Signature bit of a vertex id: the top 6 bits of a Fibonacci (multiplicative)

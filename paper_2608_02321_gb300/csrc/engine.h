@@ -21,15 +21,23 @@ struct gfd_graph {
     int64_t bytes = 0;
     gfd::DevGraph dg{};
     std::vector<void*> allocs;
-    std::vector<unsigned long long> label_stats;  // [65536][count, out-degree sum, in-degree sum]
-    std::vector<double> moments;                  // [65536][16], see PlanStats
+    // per vertex label below the largest one present (others: no vertices)
+    std::vector<unsigned long long> label_stats;  // [labels][count, out-degree sum, in-degree sum]
+    std::vector<double> moments;                  // [labels][16], see PlanStats
     std::vector<double> moments_all;              // [16]
     std::vector<double> elabel_frac;              // [256]
+    int32_t n_labels() const { return (int32_t)label_stats.size() / 3; }
+    // which: 0 vertices of the label (GFD_WILDCARD: all), 1 their out-degree sum, 2 their in-degree sum
+    uint64_t label_stat(int32_t L, int which) const {
+        if (L == GFD_WILDCARD) return which == 0 ? (uint64_t)n : (uint64_t)m;
+        return L < n_labels() ? label_stats[3 * (size_t)L + which] : 0;
+    }
     gfd::PlanStats plan_stats() const {
         gfd::PlanStats p;
         p.n_vertices = n;
         p.n_edges = m;
         p.moments = moments.data();
+        p.n_labels = n_labels();
         p.moments_all = moments_all.data();
         p.elabel_frac = elabel_frac.data();
         return p;
@@ -73,26 +81,30 @@ struct CompactJob {      // rank and candidate list of bm
     uint32_t* count;
     uint32_t* csum;          // per-chunk set-bit counts (scratch)
 };
+struct ScanList {        // a compacted candidate list whose vertices' adjacency is scanned
+    const int32_t* cand;
+    const uint32_t* count;
+    const uint32_t* bm;
+    const uint32_t* rank;
+};
 struct ScatterJob {      // mark vertices adjacent to the candidates of another level
-    const int32_t* qcand;
-    const uint32_t* qcount;
+    ScanList q;
     const uint32_t* filter;  // only vertices in this bitmap are marked
     uint32_t* marks;
-    int32_t scan_out;        // 1: follow out-edges of qcand, 0: in-edges
+    int32_t scan_out;        // 1: follow out-edges of q, 0: in-edges
     int32_t lab;
 };
 struct PruneJob {        // drop candidates with no neighbour in a later level
-    const int32_t* cand;
-    const uint32_t* count;
-    uint32_t* bm;
+    ScanList c;              // the candidates
+    uint32_t* out;           // their bitmap, cleared where a candidate is dropped
     int32_t ncon;
     const uint32_t* con_bm[2 * MAXK];
     int32_t con_dir[2 * MAXK];
     int32_t con_lab[2 * MAXK];
+    int32_t con_any[2 * MAXK];  // con_bm holds vertices of any label
 };
 struct CpiJob {          // index edges of one spanning-tree edge
-    const int32_t* pcand;
-    const uint32_t* pcount;
+    ScanList p;              // the parent's candidates
     const uint32_t* cbm;
     const uint32_t* crank;
     uint32_t* off;
@@ -104,35 +116,26 @@ struct CpiJob {          // index edges of one spanning-tree edge
     uint64_t* csum;          // per-chunk count sums (scratch)
 };
 
-// Adjacency lists longer than HUB_LIST entries (hubs of a skewed degree
-// distribution) are queued by the warp kernels and scanned afterwards by whole
-// blocks, so that one hub does not leave a single warp running long after the
-// rest of the launch; a full queue leaves the list to its warp.
-constexpr uint32_t HUB_LIST = 1024;
-constexpr uint32_t HUB_CAP = 1u << 19;
-struct HubQueue {
-    unsigned long long* item;  // (job << 40) | (constraint << 32) | candidate index
-    uint32_t* n;               // items queued (may exceed cap: only cap are stored)
-    uint32_t cap;
+struct ScanWork {
+    // room for the shares of a launch's jobs: scan_work_words(largest job table)
+    uint32_t* pre;
     // counting pass: [0] candidates whose adjacency was scanned, [1] adjacency
     // entries read (null: not counting)
     unsigned long long* scan;
-    // room for the exclusive prefix of a launch's per-job group counts (one
-    // more than the largest job table of the group)
-    uint32_t* jpre;
 };
+constexpr size_t scan_work_words(size_t njobs) { return (N_CLASS + 1) * (njobs + 1); }
 
 // ---- index kernels (index.cu); each launch covers all jobs given
 int launch_filter(const DevGraph& g, const FilterKey* d_keys, int nkeys, uint32_t* d_out, cudaStream_t st);
 int launch_and(const DevGraph& g, const AndJob* d_jobs, int njobs, cudaStream_t st);
 int launch_compact(const DevGraph& g, const CompactJob* d_jobs, int njobs, cudaStream_t st);
-int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const HubQueue& hq, cudaStream_t st);
-int launch_prune(const DevGraph& g, const PruneJob* d_jobs, int njobs, const HubQueue& hq, cudaStream_t st);
+int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st);
+int launch_prune(const DevGraph& g, const PruneJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st);
 // Index edges in two launches: counts, offsets and per-job totals first (the
 // caller reads the totals back and allocates exactly), then the fill.
 int launch_cpi_count(const DevGraph& g, const CpiJob* d_jobs, int njobs, uint32_t nchunks, int32_t* d_err,
-                     uint32_t* d_totals, const HubQueue& hq, cudaStream_t st);
-int launch_cpi_fill(const DevGraph& g, const CpiJob* d_jobs, int njobs, const HubQueue& hq, cudaStream_t st);
+                     uint32_t* d_totals, const ScanWork& sw, cudaStream_t st);
+int launch_cpi_fill(const DevGraph& g, const CpiJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st);
 uint32_t compact_chunks(const DevGraph& g);
 uint32_t cpi_chunks(uint64_t max_parent_candidates);
 

@@ -589,13 +589,13 @@ __device__ void expand_warps(const EnumArgs& A) {
                                 // the slot's own buffer: tuples in pattern-node order
                                 if (idx < D->viol_cap) {
                                     int32_t* out = D->viol + idx * k;
-                                    for (int q = 0; q < k; q++) out[D->order[q]] = (int32_t)m[q << 5];
+                                    for (int q = 0; q < k; q++) out[D->order[q]] = (int32_t)__ldg(g.orig + m[q << 5]);
                                 }
                             } else if (idx < A.sched->varena_cap) {
                                 // the run's arena: [slot, tuple in pattern-node order]
                                 int32_t* rec = A.sched->varena + idx * A.sched->vstride;
                                 rec[0] = s;
-                                for (int q = 0; q < k; q++) rec[1 + D->order[q]] = (int32_t)m[q << 5];
+                                for (int q = 0; q < k; q++) rec[1 + D->order[q]] = (int32_t)__ldg(g.orig + m[q << 5]);
                             }
                         }
                     }
@@ -828,12 +828,12 @@ __device__ void expand_warps(const EnumArgs& A) {
                                     if (D->viol) {
                                         if (idx < D->viol_cap) {
                                             int32_t* outp = D->viol + idx * k;
-                                            for (int q = 0; q < k; q++) outp[D->order[q]] = (int32_t)level_vertex(mo, q, L, fv);
+                                            for (int q = 0; q < k; q++) outp[D->order[q]] = (int32_t)__ldg(g.orig + level_vertex(mo, q, L, fv));
                                         }
                                     } else if (idx < A.sched->varena_cap) {
                                         int32_t* rec = A.sched->varena + idx * A.sched->vstride;
                                         rec[0] = s;
-                                        for (int q = 0; q < k; q++) rec[1 + D->order[q]] = (int32_t)level_vertex(mo, q, L, fv);
+                                        for (int q = 0; q < k; q++) rec[1 + D->order[q]] = (int32_t)__ldg(g.orig + level_vertex(mo, q, L, fv));
                                     }
                                 }
                             }

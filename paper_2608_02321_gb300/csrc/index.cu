@@ -12,13 +12,15 @@
 //   k_compact  bitmap -> exclusive popcount prefix (O(1) rank) + sorted list;
 //   k_cpi_*    step 1d: for each spanning-tree edge, the index edges from
 //              every parent candidate to the positions of its child candidates;
-//   *_hub      the same for adjacency lists over HUB_LIST entries, one block
-//              per list (queued by the warp kernels).
+// The adjacency scans (k_scatter, k_prune, k_cpi_count, k_cpi_fill) share out a
+// job's candidates by degree class: a block per hub, a warp per 1, 8 or 32
+// vertices of the other classes.
 //
 // Every launch processes a table of jobs; blocks (or warps) stride over the
 // items of each job with a per-job rotation so that small jobs spread out.
 #include <cub/cub.cuh>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 
@@ -37,10 +39,6 @@ __device__ __forceinline__ uint64_t gwarp_id() {
     return (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
 }
 __device__ __forceinline__ uint64_t nwarps_total() { return ((uint64_t)gridDim.x * blockDim.x) >> 5; }
-
-__device__ __forceinline__ bool bit_of(const uint32_t* bm, uint32_t x) {
-    return (bm[x >> 5] >> (x & 31)) & 1u;
-}
 
 __global__ void k_filter(DevGraph g, const FilterKey* __restrict__ keys, int nkeys, uint32_t* __restrict__ out) {
     extern __shared__ FilterKey sk[];
@@ -147,83 +145,203 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_compact_write(DevGraph g, c
         uint32_t excl, total;
         Scan(tmp.scan).ExclusiveSum(cnt, excl, total);
         uint32_t r = base_s + excl;
+        uint32_t first[WPT];  // list position of each word's first vertex
+#pragma unroll
         for (int q = 0; q < WPT; q++) {
-            if (w0 + q >= g.nwords) break;
-            J.rank[w0 + q] = r;
-            uint32_t x = words[q];
-            while (x) {
-                const int bpos = __ffs(x) - 1;
-                J.cand[r++] = (int32_t)((w0 + q) * 32 + bpos);
-                x &= x - 1;
-            }
+            first[q] = r;
+            if (w0 + q < g.nwords) J.rank[w0 + q] = r;
+            r += __popc(words[q]);
         }
+        // the list, by the whole warp: one word with candidates at a time, a lane
+        // per bit, so that the stores of a word are next to each other
+        int32_t* const cand = J.cand;
+        const uint32_t lane = threadIdx.x & 31;
+#pragma unroll
+        for (int q = 0; q < WPT; q++)
+            for (uint32_t some = __ballot_sync(0xffffffffu, words[q] != 0); some; some &= some - 1) {
+                const int src = __ffs(some) - 1;
+                const uint32_t x = __shfl_sync(0xffffffffu, words[q], src), at = __shfl_sync(0xffffffffu, first[q], src);
+                const uint32_t w = __shfl_sync(0xffffffffu, w0 + q, src);
+                if ((x >> lane) & 1u) cand[at + __popc(x & ((1u << lane) - 1u))] = (int32_t)(w * 32 + lane);
+            }
         if (c == nchunks - 1 && threadIdx.x == 0) *J.count = base_s + total;
         __syncthreads();
     }
 }
 
-// The adjacency kernels below give each lane of a warp one candidate and let
-// the lane scan a short list alone; lists longer than SHORT_LIST are left to
-// the whole warp, one after the other (ballot of the long ones), scanned 32
-// entries at a time without idling lanes on short lists; hub lists (over
-// HUB_LIST entries) are queued for a block each.
-constexpr uint32_t SHORT_LIST = 32;
+// The adjacency kernels below give the lanes of a warp a candidate each (32 of
+// the lowest degree class, fewer of the others); the warp then scans its lists
+// end to end as one sequence, 32 x FLAT entries at a time (scan_flat). A hub's
+// list is scanned by a block. Vertices are numbered by degree class, so a
+// candidate list holds its classes one after the other, and where they end are
+// rank lookups.
+//
+// These scans are bound by latency (a random adjacency line, then a random
+// bitmap word, from L2 or HBM) and by balance. A lane that scans its own list
+// leaves the warp waiting for its longest list with few loads in flight; a warp
+// that happens to get 32 long lists keeps the launch waiting. End to end every
+// lane has FLAT loads in flight whatever the degrees, and by classes no warp
+// gets more than 2048 entries at a time.
+constexpr int FLAT = 4;
+// candidates per warp of each class after the hubs (x the class's largest degree:
+// at most 2048 entries)
+__device__ constexpr uint32_t class_group(int c) { return c == 1 ? 1 : c == 2 ? 8 : 32; }
 
-// A lane scanning a short list alone reads UNROLL entries per round and then
-// their UNROLL bitmap words, so that each round costs two dependent loads
-// rather than two per entry.
-constexpr int UNROLL = 4;
-
-constexpr int HUB_THREADS = 512;
-
-// Queue the lanes whose list is a hub (warp-synchronous: every lane calls it);
-// true for the lanes whose item was stored.
-__device__ __forceinline__ bool hub_push(const HubQueue& q, bool want, unsigned long long item, int lane) {
-    const uint32_t b = __ballot_sync(0xffffffffu, want);
-    if (!b) return false;
-    const int leader = __ffs(b) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(q.n, (uint32_t)__popc(b));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    const uint32_t pos = base + __popc(b & ((1u << lane) - 1u));
-    if (want && pos < q.cap) {
-        q.item[pos] = item;
-        return true;
-    }
-    return false;
+// Entries of the aligned quad at b < e1 that lie in [e0, e1), as a mask.
+__device__ __forceinline__ uint32_t quad_mask(uint32_t b, uint32_t e0, uint32_t e1) {
+    uint32_t m = 15u;
+    if (b < e0) m &= m << (e0 - b);
+    if (e1 - b < 4u) m &= (1u << (e1 - b)) - 1u;
+    return m;
 }
 
-__device__ __forceinline__ uint32_t hub_count(const HubQueue& q) { return min(*q.n, q.cap); }
+// Of the entries m of the aligned quad at b, those with an allowed edge label
+// whose neighbour is in bm; x receives the neighbours, w their bitmap words.
+__device__ __forceinline__ uint32_t quad_hits(const DevGraph& g, const uint32_t* adj, uint32_t b, uint32_t m, int32_t lab,
+                                              const uint32_t* bm, uint32_t (&x)[4], uint32_t (&w)[4]) {
+    const uint4 p4 = __ldg(reinterpret_cast<const uint4*>(adj + b));
+    const uint32_t p[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+    for (int t = 0; t < 4; t++) {
+        x[t] = p[t] >> g.lbits;
+        const bool ok = ((m >> t) & 1u) && label_ok(lab, (int32_t)(p[t] & g.lmask));
+        w[t] = ok ? __ldg(bm + (x[t] >> 5)) : 0u;
+    }
+    uint32_t h = 0;
+#pragma unroll
+    for (int t = 0; t < 4; t++) h |= ((w[t] >> (x[t] & 31)) & 1u) << t;
+    return h;
+}
 
-// The adjacency kernels below take (job, group of 32 candidates) items from one
-// flat index: k_job_groups writes the exclusive prefix of the jobs' group
-// counts (total at [njobs]), and job_of finds an item's job by binary search,
-// so no warp walks the whole job table.
-__device__ __forceinline__ uint32_t job_count(const ScatterJob& J) { return *J.qcount; }
-__device__ __forceinline__ uint32_t job_count(const PruneJob& J) { return *J.count; }
-__device__ __forceinline__ uint32_t job_count(const CpiJob& J) { return *J.pcount; }
+// The adjacency a job scans.
+struct AdjRef {
+    const uint32_t* off;
+    const uint32_t* adj;
+};
+__device__ __forceinline__ AdjRef adj_ref(const DevGraph& g, bool out) {
+    return out ? AdjRef{g.out_off, g.out_adj} : AdjRef{g.in_off, g.in_adj};
+}
+
+// The warp's 32 lists, lane i holding [e0, e1) (empty for e0 = e1), scanned end
+// to end. f(hit, x, w, owner, window) is called by all lanes for every window of
+// 32 entries, in order: whether the lane's entry has allowed labels and a
+// neighbour x in bm (w: its bitmap word), and the lane whose list it is from;
+// window: position of the window in the sequence. slots: the warp's 32 int2 in
+// shared memory. ex: where the lane's list starts in the sequence (for f).
+template <typename F>
+__device__ __forceinline__ void scan_flat(const DevGraph& g, const AdjRef& A, uint32_t e0, uint32_t len, uint32_t ex,
+                                          uint32_t total, int32_t lab, const uint32_t* bm, int2* slots, int lane,
+                                          F&& f) {
+    // the non-empty lists in order: (position in adj - position in the sequence, lane)
+    const uint32_t some = __ballot_sync(0xffffffffu, len != 0);
+    if (len) slots[__popc(some & ((1u << lane) - 1u))] = make_int2((int32_t)(e0 - ex), lane);
+    __syncwarp();
+    const uint32_t upto = 0xffffffffu >> (31 - lane);
+    uint32_t begun = 0;  // lists that start before the window
+    for (uint32_t base = 0; base < total; base += 32 * FLAT) {
+        uint32_t p[FLAT], w[FLAT];
+        int owner[FLAT];
+#pragma unroll
+        for (int u = 0; u < FLAT; u++) {
+            const uint32_t wb = base + 32u * u;
+            // bit i: a list starts at the window's i-th entry
+            const uint32_t starts = __reduce_or_sync(0xffffffffu, len && ex - wb < 32u ? 1u << (ex - wb) : 0u);
+            const uint32_t o = begun + __popc(starts & upto) - 1;
+            begun += __popc(starts);
+            owner[u] = -1;
+            p[u] = 0;
+            if (wb + lane < total) {
+                const int2 s = slots[o];
+                const uint32_t e = wb + lane + (uint32_t)s.x;
+                p[u] = __ldg(A.adj + e);
+                owner[u] = s.y;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < FLAT; u++)
+            w[u] = owner[u] >= 0 && label_ok(lab, (int32_t)(p[u] & g.lmask)) ? __ldg(bm + ((p[u] >> g.lbits) >> 5)) : 0u;
+#pragma unroll
+        for (int u = 0; u < FLAT; u++) {
+            const uint32_t x = p[u] >> g.lbits;
+            f((bool)((w[u] >> (x & 31)) & 1u), x, w[u], owner[u], base + 32u * u);
+        }
+        if (total - base <= 32u * FLAT) break;  // (base + 32 FLAT could wrap)
+    }
+    __syncwarp();  // slots are written again by the next scan
+}
+
+// Exclusive warp scan of the lanes' list lengths (their sum is below 2^32: lists
+// of different vertices).
+__device__ __forceinline__ uint32_t list_starts(uint32_t len, int lane, uint32_t* total) {
+    uint32_t incl = len;
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += y;
+    }
+    *total = __shfl_sync(0xffffffffu, incl, 31);
+    return incl - len;
+}
+
+// Work of a launch over all its jobs, written by k_job_groups: ScanWork::pre
+// holds, for the J = njobs jobs, the exclusive prefix of their warp groups
+// [J + 1], that of their hubs [J + 1], and per job where its first classes end in
+// the candidate list [(N_CLASS - 1) J]. Groups and hubs are taken from one flat
+// index each; job_of finds an item's job by binary search.
+__device__ __forceinline__ const ScanList& list_of(const ScatterJob& J) { return J.q; }
+__device__ __forceinline__ const ScanList& list_of(const PruneJob& J) { return J.c; }
+__device__ __forceinline__ const ScanList& list_of(const CpiJob& J) { return J.p; }
 
 constexpr int JOB_SCAN_THREADS = 1024;
 
+// candidates of the list below vertex v (its bitmap and ranks as compacted)
+__device__ __forceinline__ uint32_t list_rank(const DevGraph& g, const ScanList& C, uint32_t v) {
+    if (v >= (uint32_t)g.n) return *C.count;
+    return C.rank[v >> 5] + __popc(C.bm[v >> 5] & ((1u << (v & 31)) - 1u));
+}
+
 template <typename Job>
-__global__ void __launch_bounds__(JOB_SCAN_THREADS) k_job_groups(const Job* __restrict__ jobs, int njobs,
+__global__ void __launch_bounds__(JOB_SCAN_THREADS) k_job_groups(DevGraph g, const Job* __restrict__ jobs, int njobs,
                                                                   uint32_t* pre) {
     using Scan = cub::BlockScan<uint32_t, JOB_SCAN_THREADS>;
     __shared__ typename Scan::TempStorage tmp;
-    __shared__ uint32_t carry;
-    if (threadIdx.x == 0) carry = 0;
+    __shared__ uint32_t carry[2];
+    uint32_t* const hpre = pre + njobs + 1;
+    uint32_t* const cls = hpre + njobs + 1;
+    if (threadIdx.x < 2) carry[threadIdx.x] = 0;
     __syncthreads();
     for (int b = 0; b < njobs; b += JOB_SCAN_THREADS) {
         const int j = b + threadIdx.x;
-        const uint32_t groups = j < njobs ? (job_count(jobs[j]) + 31) / 32 : 0;
-        uint32_t excl, total;
+        uint32_t groups = 0, hubs = 0;
+        if (j < njobs) {
+            const ScanList& C = list_of(jobs[j]);
+            uint32_t begin = hubs = list_rank(g, C, g.class_end[0]);
+            cls[(N_CLASS - 1) * j] = hubs;
+            for (int c = 1; c < N_CLASS; c++) {
+                const uint32_t end = c < N_CLASS - 1 ? list_rank(g, C, g.class_end[c]) : *C.count;
+                if (c < N_CLASS - 1) cls[(N_CLASS - 1) * j + c] = end;
+                groups += (end - begin + class_group(c) - 1) / class_group(c);
+                begin = end;
+            }
+        }
+        uint32_t excl, total, hexcl, htotal;
         Scan(tmp).ExclusiveSum(groups, excl, total);
-        if (j < njobs) pre[j] = carry + excl;
         __syncthreads();
-        if (threadIdx.x == 0) carry += total;
+        Scan(tmp).ExclusiveSum(hubs, hexcl, htotal);
+        if (j < njobs) {
+            pre[j] = carry[0] + excl;
+            hpre[j] = carry[1] + hexcl;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            carry[0] += total;
+            carry[1] += htotal;
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) pre[njobs] = carry;
+    if (threadIdx.x == 0) {
+        pre[njobs] = carry[0];
+        hpre[njobs] = carry[1];
+    }
 }
 
 // the job whose items [pre[j], pre[j+1]) hold item it (pre[njobs] > it)
@@ -237,10 +355,45 @@ __device__ __forceinline__ int job_of(const uint32_t* pre, int njobs, uint32_t i
     return lo;
 }
 
+// A launch's hubs (item = job, position in its candidate list) and warp groups.
+struct Groups {
+    const uint32_t *pre, *hpre, *cls;
+    int njobs;
+    __device__ __forceinline__ Groups(const ScanWork& w, int n)
+        : pre(w.pre), hpre(w.pre + n + 1), cls(w.pre + 2 * (n + 1)), njobs(n) {}
+    __device__ __forceinline__ uint32_t n_groups() const { return pre[njobs]; }
+    __device__ __forceinline__ uint32_t n_hubs() const { return hpre[njobs]; }
+    __device__ __forceinline__ int hub(uint32_t it, uint32_t* a) const {
+        const int j = job_of(hpre, njobs, it);
+        *a = it - hpre[j];
+        return j;
+    }
+    // job of group it; a: the lane's position in its candidate list (from the
+    // list's end on for a lane without a candidate)
+    __device__ __forceinline__ int group(uint32_t it, uint32_t lane, uint32_t* a) const {
+        const int j = job_of(pre, njobs, it);
+        const uint32_t* const end = cls + (N_CLASS - 1) * j;
+        uint32_t grp = it - pre[j], begin = end[0];
+#pragma unroll
+        for (int c = 1; c < N_CLASS - 1; c++) {
+            const uint32_t groups = (end[c] - begin + class_group(c) - 1) / class_group(c);
+            if (grp < groups) {
+                begin += grp * class_group(c) + lane;
+                *a = lane < class_group(c) && begin < end[c] ? begin : 0xffffffffu;
+                return j;
+            }
+            grp -= groups;
+            begin = end[c];
+        }
+        *a = begin + grp * 32 + lane;
+        return j;
+    }
+};
+
 // Counting pass: add this thread's scanned candidates and adjacency entries to
 // the run's counters (all lanes of the warp call it; one atomic per warp).
 template <bool COUNT>
-__device__ __forceinline__ void scan_flush(const HubQueue& q, uint64_t cands, uint64_t entries) {
+__device__ __forceinline__ void scan_flush(const ScanWork& q, uint64_t cands, uint64_t entries) {
     if (!COUNT || !q.scan) return;
     for (int d = 16; d >= 1; d >>= 1) {
         cands += __shfl_xor_sync(0xffffffffu, cands, d);
@@ -252,201 +405,210 @@ __device__ __forceinline__ void scan_flush(const HubQueue& q, uint64_t cands, ui
     }
 }
 
-__device__ __forceinline__ void load_group(const uint32_t* adj, uint32_t e, uint32_t e1, uint32_t (&p)[UNROLL]) {
+// A hub's list [e0, e1) scanned by the block: f(hits, x, w) per quad, where a
+// thread takes HUB_QUADS quads in a row per round; stop() is asked after every
+// round by all threads.
+constexpr int HUB_QUADS = 4;
+template <typename F, typename Stop>
+__device__ __forceinline__ void scan_block(const DevGraph& g, const uint32_t* adj, uint32_t e0, uint32_t e1, int32_t lab,
+                                           const uint32_t* bm, F&& f, Stop&& stop) {
+    constexpr uint32_t ROUND = 4 * HUB_QUADS * WARP_KERNEL_THREADS;
+    for (uint64_t r = e0 & ~3u; r < e1; r += ROUND) {  // block-uniform bounds
 #pragma unroll
-    for (int t = 0; t < UNROLL; t++) p[t] = e + t < e1 ? __ldg(adj + e + t) : 0u;
+        for (int q = 0; q < HUB_QUADS; q++) {
+            const uint64_t b = r + 4u * (HUB_QUADS * threadIdx.x + q);
+            uint32_t x[4], w[4], h = 0;
+            if (b < e1) h = quad_hits(g, adj, (uint32_t)b, quad_mask((uint32_t)b, e0, e1), lab, bm, x, w);
+            if (h) f(q, h, x, w);
+        }
+        if (stop()) return;
+    }
+}
+
+// Mark vertex x. Popular vertices are reached over and over, and numbered next to
+// each other, so their words would take most of the atomics: a look (possibly
+// at an old copy in L1, which only costs a needless atomic) leaves those out.
+__device__ __forceinline__ void mark(uint32_t* marks, uint32_t x) {
+    uint32_t* const w = marks + (x >> 5);
+    const uint32_t b = 1u << (x & 31);
+    if (!(__ldca(w) & b)) atomicOr(w, b);
 }
 
 template <bool COUNT>
-__global__ void k_scatter(DevGraph g, const ScatterJob* __restrict__ jobs, int njobs, HubQueue hq) {
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_scatter(DevGraph g, const ScatterJob* __restrict__ jobs,
+                                                                 int njobs, ScanWork sw) {
+    __shared__ int2 s_slots[WARP_KERNEL_THREADS];
     const int lane = threadIdx.x & 31;
-    const uint64_t gw = gwarp_id(), nw = nwarps_total();
+    int2* const slots = s_slots + (threadIdx.x & ~31);
+    const Groups G(sw, njobs);
     uint64_t sc = 0, se = 0;
-    const uint32_t ngroups = hq.jpre[njobs];
-    for (uint64_t it = gw; it < ngroups; it += nw) {
-        // the warp's group of 32 candidates: job j, group grp of that job
-        const int j = job_of(hq.jpre, njobs, (uint32_t)it);
-        const uint64_t grp = it - hq.jpre[j];
-        const ScatterJob J = jobs[j];
-        const uint32_t n = *J.qcount;
-        const uint32_t* off = J.scan_out ? g.out_off : g.in_off;
-        const uint32_t* adj = J.scan_out ? g.out_adj : g.in_adj;
-        {
-            const uint64_t a = grp * 32 + lane;
-            uint32_t e0 = 0, e1 = 0;
-            if (a < n) {
-                const uint32_t v = (uint32_t)J.qcand[a];
-                e0 = off[v];
-                e1 = off[v + 1];
-            }
-            if (hub_push(hq, e1 - e0 > HUB_LIST, ((unsigned long long)j << 40) | a, lane)) e1 = e0;
-            const bool is_long = e1 - e0 > SHORT_LIST;
-            sc += a < n && e1 > e0;
-            se += e1 - e0;
-            if (!is_long)
-                for (uint32_t e = e0; e < e1; e += UNROLL) {
-                    uint32_t p[UNROLL], f[UNROLL];
-                    load_group(adj, e, e1, p);
+    const uint32_t nhubs = G.n_hubs();
+    for (uint32_t it = blockIdx.x; it < nhubs; it += gridDim.x) {
+        uint32_t a;
+        const ScatterJob& J = jobs[G.hub(it, &a)];
+        const AdjRef A = adj_ref(g, J.scan_out);
+        const uint32_t v = (uint32_t)J.q.cand[a], e0 = A.off[v], e1 = A.off[v + 1];
+        if (threadIdx.x == 0) sc += e1 > e0, se += e1 - e0;
+        uint32_t* const marks = J.marks;
+        scan_block(g, A.adj, e0, e1, J.lab, J.filter,
+                   [&](int, uint32_t h, const uint32_t (&x)[4], const uint32_t (&)[4]) {
 #pragma unroll
-                    for (int t = 0; t < UNROLL; t++)
-                        f[t] = e + t < e1 ? __ldg(J.filter + ((p[t] >> g.lbits) >> 5)) : 0u;
-#pragma unroll
-                    for (int t = 0; t < UNROLL; t++) {
-                        const uint32_t x = p[t] >> g.lbits;
-                        if (e + t < e1 && label_ok(J.lab, (int32_t)(p[t] & g.lmask)) && ((f[t] >> (x & 31)) & 1u))
-                            atomicOr(&J.marks[x >> 5], 1u << (x & 31));
-                    }
-                }
-            for (uint32_t lm = __ballot_sync(0xffffffffu, is_long); lm; lm &= lm - 1) {
-                const int src = __ffs(lm) - 1;
-                const uint32_t b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
-                for (uint32_t e = b0 + lane; e < b1; e += 32) {
-                    const uint32_t p = adj[e];
-                    const uint32_t x = p >> g.lbits;
-                    if (label_ok(J.lab, (int32_t)(p & g.lmask)) && bit_of(J.filter, x))
-                        atomicOr(&J.marks[x >> 5], 1u << (x & 31));
-                }
-            }
+                       for (int c = 0; c < 4; c++)
+                           if ((h >> c) & 1u) mark(marks, x[c]);
+                   },
+                   [] { return false; });
+    }
+    const uint32_t ngroups = G.n_groups();
+    for (uint64_t it = gwarp_id(); it < ngroups; it += nwarps_total()) {
+        uint32_t a;
+        const ScatterJob& J = jobs[G.group((uint32_t)it, lane, &a)];
+        const AdjRef A = adj_ref(g, J.scan_out);
+        uint32_t e0 = 0, e1 = 0;
+        if (a < *J.q.count) {
+            const uint32_t v = (uint32_t)J.q.cand[a];
+            e0 = A.off[v];
+            e1 = A.off[v + 1];
         }
+        sc += e1 > e0;
+        se += e1 - e0;
+        uint32_t total;
+        const uint32_t ex = list_starts(e1 - e0, lane, &total);
+        uint32_t* const marks = J.marks;
+        scan_flat(g, A, e0, e1 - e0, ex, total, J.lab, J.filter, slots, lane,
+                  [&](bool hit, uint32_t x, uint32_t, int, uint32_t) {
+                      if (hit) mark(marks, x);
+                  });
     }
-    scan_flush<COUNT>(hq, sc, se);
+    scan_flush<COUNT>(sw, sc, se);
 }
 
-// Does the list adj[e0, e1) hold a neighbour in bm with an allowed label? One
-// lane alone (short lists) or the whole warp (cooperative).
-__device__ __forceinline__ bool any_hit_serial(const DevGraph& g, const uint32_t* adj, uint32_t e0, uint32_t e1,
-                                               int32_t lab, const uint32_t* bm, uint64_t& read) {
-    for (uint32_t e = e0; e < e1; e += UNROLL) {
-        read += min((uint32_t)UNROLL, e1 - e);
-        uint32_t p[UNROLL], w[UNROLL];
-        load_group(adj, e, e1, p);
-#pragma unroll
-        for (int t = 0; t < UNROLL; t++) w[t] = e + t < e1 ? __ldg(bm + ((p[t] >> g.lbits) >> 5)) : 0u;
-        bool hit = false;
-#pragma unroll
-        for (int t = 0; t < UNROLL; t++)
-            hit |= e + t < e1 && label_ok(lab, (int32_t)(p[t] & g.lmask)) && ((w[t] >> ((p[t] >> g.lbits) & 31)) & 1u);
-        if (hit) return true;
-    }
-    return false;
-}
-
-__device__ __forceinline__ bool any_hit_warp(const DevGraph& g, const uint32_t* adj, uint32_t e0, uint32_t e1,
-                                             int32_t lab, const uint32_t* bm, int lane, uint64_t& read) {
-    for (uint32_t b = e0; b < e1; b += 32) {
-        if (lane == 0) read += min(32u, e1 - b);
-        const uint32_t e = b + lane;
-        bool hit = false;
-        if (e < e1) {
-            const uint32_t p = adj[e];
-            hit = label_ok(lab, (int32_t)(p & g.lmask)) && bit_of(bm, p >> g.lbits);
-        }
-        if (__any_sync(0xffffffffu, hit)) return true;
-    }
-    return false;
-}
-
+// A constraint on neighbours of any vertex label hits often: each lane first
+// tries its own list's first quad, and only lists without a hit there are
+// scanned end to end.
 template <bool COUNT>
-__global__ void k_prune(DevGraph g, const PruneJob* __restrict__ jobs, int njobs, HubQueue hq) {
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_prune(DevGraph g, const PruneJob* __restrict__ jobs, int njobs,
+                                                               ScanWork sw) {
+    __shared__ int2 s_slots[WARP_KERNEL_THREADS];
+    __shared__ uint8_t s_hit[WARP_KERNEL_THREADS];
     const int lane = threadIdx.x & 31;
-    const uint64_t gw = gwarp_id(), nw = nwarps_total();
+    int2* const slots = s_slots + (threadIdx.x & ~31);
+    uint8_t* const found = s_hit + (threadIdx.x & ~31);
+    const Groups G(sw, njobs);
     uint64_t sc = 0, se = 0;
-    const uint32_t ngroups = hq.jpre[njobs];
-    for (uint64_t it = gw; it < ngroups; it += nw) {
-        // the warp's group of 32 candidates: job j, group grp of that job
-        const int j = job_of(hq.jpre, njobs, (uint32_t)it);
-        const uint64_t grp = it - hq.jpre[j];
-        const PruneJob& J = jobs[j];
-        const uint32_t n = *J.count;
+    const uint32_t nhubs = G.n_hubs();
+    for (uint32_t it = blockIdx.x; it < nhubs; it += gridDim.x) {
+        uint32_t a;
+        const PruneJob& J = jobs[G.hub(it, &a)];
+        const uint32_t v = (uint32_t)J.c.cand[a];
+        bool keep = true;
+        for (int c = 0; c < J.ncon && keep; c++) {  // block-uniform
+            const AdjRef A = adj_ref(g, J.con_dir[c]);
+            const uint32_t e0 = A.off[v], e1 = A.off[v + 1];
+            if (threadIdx.x == 0) sc++, se += e1 - e0;
+            bool hit = false;
+            keep = false;
+            scan_block(g, A.adj, e0, e1, J.con_lab[c], J.con_bm[c],
+                       [&](int, uint32_t, const uint32_t (&)[4], const uint32_t (&)[4]) { hit = true; },
+                       [&] { return keep = __syncthreads_or(hit); });
+        }
+        if (!keep && threadIdx.x == 0) atomicAnd(&J.out[v >> 5], ~(1u << (v & 31)));
+    }
+    const uint32_t ngroups = G.n_groups();
+    for (uint64_t it = gwarp_id(); it < ngroups; it += nwarps_total()) {
+        uint32_t a;
+        const PruneJob& J = jobs[G.group((uint32_t)it, lane, &a)];
         const int ncon = J.ncon;
-        {
-            const uint64_t a = grp * 32 + lane;
-            const bool valid = a < n;
-            const uint32_t v = valid ? (uint32_t)J.cand[a] : 0u;
-            bool keep = valid;
-            for (int c = 0; c < ncon; c++) {
-                const uint32_t* off = J.con_dir[c] ? g.out_off : g.in_off;
-                const uint32_t* adj = J.con_dir[c] ? g.out_adj : g.in_adj;
-                uint32_t e0 = 0, e1 = 0;
-                if (keep) {
-                    e0 = off[v];
-                    e1 = off[v + 1];
-                }
-                // a hub's constraint is decided by a block later (it clears the bit
-                // when nothing hits); the other constraints go on here
-                const bool queued = hub_push(hq, keep && e1 - e0 > HUB_LIST,
-                                             ((unsigned long long)j << 40) | ((unsigned long long)c << 32) | a, lane);
-                const bool is_long = keep && !queued && e1 - e0 > SHORT_LIST;
-                sc += keep && !queued;
-                if (keep && !queued && !is_long) keep = any_hit_serial(g, adj, e0, e1, J.con_lab[c], J.con_bm[c], se);
-                for (uint32_t lm = __ballot_sync(0xffffffffu, is_long); lm; lm &= lm - 1) {
-                    const int src = __ffs(lm) - 1;
-                    const uint32_t b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
-                    const bool hit = any_hit_warp(g, adj, b0, b1, J.con_lab[c], J.con_bm[c], lane, se);
-                    if (lane == src) keep = hit;
-                }
+        const bool valid = a < *J.c.count;
+        const uint32_t v = valid ? (uint32_t)J.c.cand[a] : 0u;
+        bool keep = valid;
+        for (int c = 0; c < ncon; c++) {
+            const AdjRef A = adj_ref(g, J.con_dir[c]);
+            const int32_t lab = J.con_lab[c];
+            const uint32_t* bm = J.con_bm[c];
+            uint32_t e0 = 0, e1 = 0;
+            if (keep) {
+                e0 = A.off[v];
+                e1 = A.off[v + 1];
             }
-            if (valid && !keep) atomicAnd(&J.bm[v >> 5], ~(1u << (v & 31)));
+            sc += keep;
+            bool hit = false;
+            if (J.con_any[c] && e0 < e1) {
+                const uint32_t b = e0 & ~3u;
+                uint32_t x[4], w[4];
+                hit = quad_hits(g, A.adj, b, quad_mask(b, e0, e1), lab, bm, x, w) != 0;
+                if (COUNT) se += min(4u - (e0 - b), e1 - e0);
+                e0 = hit || e1 - b <= 4u ? e1 : b + 4;
+            }
+            se += e1 - e0;
+            found[lane] = hit;
+            uint32_t total;
+            const uint32_t ex = list_starts(e1 - e0, lane, &total);
+            scan_flat(g, A, e0, e1 - e0, ex, total, lab, bm, slots, lane,
+                      [&](bool h, uint32_t, uint32_t, int owner, uint32_t) {
+                          if (h) found[owner] = 1;
+                      });
+            keep = keep && found[lane];
         }
+        if (valid && !keep) atomicAnd(&J.out[v >> 5], ~(1u << (v & 31)));
     }
-    scan_flush<COUNT>(hq, sc, se);
+    scan_flush<COUNT>(sw, sc, se);
 }
 
 // off[a] = number of children of parent candidate a
 template <bool COUNT>
-__global__ void k_cpi_count(DevGraph g, const CpiJob* __restrict__ jobs, int njobs, HubQueue hq) {
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_cpi_count(DevGraph g, const CpiJob* __restrict__ jobs,
+                                                                   int njobs, ScanWork sw) {
+    using Reduce = cub::BlockReduce<uint32_t, WARP_KERNEL_THREADS>;
+    __shared__ typename Reduce::TempStorage tmp;
+    __shared__ int2 s_slots[WARP_KERNEL_THREADS];
     const int lane = threadIdx.x & 31;
-    const uint64_t gw = gwarp_id(), nw = nwarps_total();
+    int2* const slots = s_slots + (threadIdx.x & ~31);
+    const Groups G(sw, njobs);
     uint64_t sc = 0, se = 0;
-    const uint32_t ngroups = hq.jpre[njobs];
-    for (uint64_t it = gw; it < ngroups; it += nw) {
-        // the warp's group of 32 candidates: job j, group grp of that job
-        const int j = job_of(hq.jpre, njobs, (uint32_t)it);
-        const uint64_t grp = it - hq.jpre[j];
-        const CpiJob J = jobs[j];
-        const uint32_t n = *J.pcount;
-        const uint32_t* off = J.out ? g.out_off : g.in_off;
-        const uint32_t* adj = J.out ? g.out_adj : g.in_adj;
-        {
-            const uint64_t a = grp * 32 + lane;
-            uint32_t e0 = 0, e1 = 0;
-            if (a < n) {
-                const uint32_t v = (uint32_t)J.pcand[a];
-                e0 = off[v];
-                e1 = off[v + 1];
-            }
-            const bool queued = hub_push(hq, e1 - e0 > HUB_LIST, ((unsigned long long)j << 40) | a, lane);
-            if (queued) e1 = e0;  // counted by a block later
-            const bool is_long = e1 - e0 > SHORT_LIST;
-            sc += a < n && e1 > e0;
-            se += e1 - e0;
-            uint32_t cnt = 0;
-            if (!is_long)
-                for (uint32_t e = e0; e < e1; e += UNROLL) {
-                    uint32_t p[UNROLL], w[UNROLL];
-                    load_group(adj, e, e1, p);
-#pragma unroll
-                    for (int t = 0; t < UNROLL; t++) w[t] = e + t < e1 ? __ldg(J.cbm + ((p[t] >> g.lbits) >> 5)) : 0u;
-#pragma unroll
-                    for (int t = 0; t < UNROLL; t++)
-                        cnt += e + t < e1 && label_ok(J.lab, (int32_t)(p[t] & g.lmask)) &&
-                               ((w[t] >> ((p[t] >> g.lbits) & 31)) & 1u);
-                }
-            for (uint32_t lm = __ballot_sync(0xffffffffu, is_long); lm; lm &= lm - 1) {
-                const int src = __ffs(lm) - 1;
-                const uint32_t b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
-                uint32_t c = 0;
-                for (uint32_t e = b0 + lane; e < b1; e += 32) {
-                    const uint32_t p = adj[e];
-                    c += label_ok(J.lab, (int32_t)(p & g.lmask)) && bit_of(J.cbm, p >> g.lbits);
-                }
-                c = __reduce_add_sync(0xffffffffu, c);
-                if (lane == src) cnt = c;
-            }
-            if (a < n && !queued) J.off[a] = cnt;
-        }
+    const uint32_t nhubs = G.n_hubs();
+    for (uint32_t it = blockIdx.x; it < nhubs; it += gridDim.x) {
+        uint32_t a;
+        const CpiJob& J = jobs[G.hub(it, &a)];
+        const AdjRef A = adj_ref(g, J.out);
+        const uint32_t v = (uint32_t)J.p.cand[a], e0 = A.off[v], e1 = A.off[v + 1];
+        if (threadIdx.x == 0) sc += e1 > e0, se += e1 - e0;
+        uint32_t cnt = 0;
+        scan_block(g, A.adj, e0, e1, J.lab, J.cbm,
+                   [&](int, uint32_t h, const uint32_t (&)[4], const uint32_t (&)[4]) { cnt += __popc(h); },
+                   [] { return false; });
+        const uint32_t total = Reduce(tmp).Sum(cnt);
+        if (threadIdx.x == 0) J.off[a] = total;
+        __syncthreads();  // tmp is reused by the next hub
     }
-    scan_flush<COUNT>(hq, sc, se);
+    const uint32_t ngroups = G.n_groups();
+    for (uint64_t it = gwarp_id(); it < ngroups; it += nwarps_total()) {
+        uint32_t a;
+        const CpiJob& J = jobs[G.group((uint32_t)it, lane, &a)];
+        const AdjRef A = adj_ref(g, J.out);
+        const bool valid = a < *J.p.count;
+        uint32_t e0 = 0, e1 = 0;
+        if (valid) {
+            const uint32_t v = (uint32_t)J.p.cand[a];
+            e0 = A.off[v];
+            e1 = A.off[v + 1];
+        }
+        sc += e1 > e0;
+        se += e1 - e0;
+        uint32_t total, cnt = 0;
+        const uint32_t len = e1 - e0, ex = list_starts(len, lane, &total);
+        scan_flat(g, A, e0, len, ex, total, J.lab, J.cbm, slots, lane,
+                  [&](bool hit, uint32_t, uint32_t, int, uint32_t window) {
+                      const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+                      // the window's entries of this lane's list: [ex, ex + len)
+                      if (hits && len && window + 32u > ex && window < ex + len) {
+                          const uint32_t lo = ex > window ? ex - window : 0u;
+                          const uint32_t hi = min(ex + len - window, 32u);
+                          cnt += __popc((hits >> lo) << (32u - hi + lo));
+                      }
+                  });
+        if (valid) J.off[a] = cnt;
+    }
+    scan_flush<COUNT>(sw, sc, se);
 }
 
 // Exclusive scan of the per-candidate counts off[0..n) in place, off[n] =
@@ -458,7 +620,7 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_cpi_sums(const CpiJob* __re
     for (uint64_t it = blockIdx.x; it < (uint64_t)njobs * nchunks; it += gridDim.x) {
         const CpiJob& J = jobs[it / nchunks];
         const uint32_t c = (uint32_t)(it % nchunks);
-        const uint32_t n = *J.pcount;
+        const uint32_t n = *J.p.count;
         if ((uint64_t)c * COMPACT_WORDS >= n && c > 0) continue;
         uint64_t cnt = 0;
         for (uint32_t a = c * COMPACT_WORDS + threadIdx.x; a < min(n, (c + 1) * COMPACT_WORDS); a += COMPACT_THREADS)
@@ -482,7 +644,7 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_cpi_scan(const CpiJob* __re
     for (uint64_t it = blockIdx.x; it < (uint64_t)njobs * nchunks; it += gridDim.x) {
         const CpiJob& J = jobs[it / nchunks];
         const uint32_t c = (uint32_t)(it % nchunks);
-        const uint32_t n = *J.pcount;
+        const uint32_t n = *J.p.count;
         const uint32_t last = n / COMPACT_WORDS;  // chunk holding off[n]
         if (c > last) continue;
         uint64_t before = 0;
@@ -519,224 +681,106 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_cpi_scan(const CpiJob* __re
     }
 }
 
+// Index edges of a group's parents are contiguous and in scan order, so the
+// warp only counts hits. A hub's edges are put in order by a block scan of the
+// threads' hits (HUB_QUADS quads in a row each) per round.
 template <bool COUNT>
-__global__ void k_cpi_fill(DevGraph g, const CpiJob* __restrict__ jobs, int njobs, HubQueue hq) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t gw = gwarp_id(), nw = nwarps_total();
-    uint64_t sc = 0, se = 0;
-    const uint32_t ngroups = hq.jpre[njobs];
-    for (uint64_t it = gw; it < ngroups; it += nw) {
-        // the warp's group of 32 candidates: job j, group grp of that job
-        const int j = job_of(hq.jpre, njobs, (uint32_t)it);
-        const uint64_t grp = it - hq.jpre[j];
-        const CpiJob J = jobs[j];
-        const uint32_t n = *J.pcount;
-        const uint32_t* off = J.out ? g.out_off : g.in_off;
-        const uint32_t* adj = J.out ? g.out_adj : g.in_adj;
-        {
-            const uint64_t a = grp * 32 + lane;
-            uint32_t e0 = 0, e1 = 0, o = 0, oend = 0;
-            if (a < n) {
-                const uint32_t v = (uint32_t)J.pcand[a];
-                o = J.off[a];
-                oend = J.off[a + 1];
-                if (oend > o) {  // a parent without index edges skips its list
-                    e0 = off[v];
-                    e1 = off[v + 1];
-                }
-            }
-            if (hub_push(hq, e1 - e0 > HUB_LIST, ((unsigned long long)j << 40) | a, lane)) e1 = e0;
-            const bool is_long = e1 - e0 > SHORT_LIST;
-            sc += a < n && e1 > e0;
-            se += e1 - e0;
-            if (!is_long)
-                for (uint32_t e = e0; e < e1; e += UNROLL) {
-                    uint32_t p[UNROLL], w[UNROLL], rk[UNROLL];
-                    load_group(adj, e, e1, p);
-#pragma unroll
-                    for (int t = 0; t < UNROLL; t++) {
-                        const uint32_t x = p[t] >> g.lbits;
-                        w[t] = e + t < e1 ? __ldg(J.cbm + (x >> 5)) : 0u;
-                        rk[t] = e + t < e1 ? __ldg(J.crank + (x >> 5)) : 0u;
-                    }
-#pragma unroll
-                    for (int t = 0; t < UNROLL; t++) {
-                        const uint32_t x = p[t] >> g.lbits;
-                        if (e + t < e1 && label_ok(J.lab, (int32_t)(p[t] & g.lmask)) && ((w[t] >> (x & 31)) & 1u)) {
-                            if (o < oend && o < J.cap)
-                                J.idx[o] = make_int2((int32_t)(rk[t] + __popc(w[t] & ((1u << (x & 31)) - 1))), (int32_t)x);
-                            o++;
-                        }
-                    }
-                }
-            for (uint32_t lm = __ballot_sync(0xffffffffu, is_long); lm; lm &= lm - 1) {
-                const int src = __ffs(lm) - 1;
-                const uint32_t b0 = __shfl_sync(0xffffffffu, e0, src), b1 = __shfl_sync(0xffffffffu, e1, src);
-                uint32_t w = __shfl_sync(0xffffffffu, o, src);
-                const uint32_t wend = __shfl_sync(0xffffffffu, oend, src);
-                for (uint32_t bb = b0; bb < b1; bb += 32) {
-                    const uint32_t e = bb + lane;
-                    bool hit = false;
-                    uint32_t x = 0;
-                    if (e < b1) {
-                        const uint32_t p = adj[e];
-                        x = p >> g.lbits;
-                        hit = label_ok(J.lab, (int32_t)(p & g.lmask)) && bit_of(J.cbm, x);
-                    }
-                    const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-                    if (hit) {
-                        const uint32_t slot = w + __popc(bal & ((1u << lane) - 1));
-                        if (slot < wend && slot < J.cap) {
-                            const uint32_t word = J.cbm[x >> 5];
-                            J.idx[slot] = make_int2((int32_t)(J.crank[x >> 5] + __popc(word & ((1u << (x & 31)) - 1))),
-                                                    (int32_t)x);
-                        }
-                    }
-                    w += __popc(bal);
-                }
-            }
-        }
-    }
-    scan_flush<COUNT>(hq, sc, se);
-}
-
-// ---- hub lists, one block per queued (job, candidate[, constraint]) item
-
-__global__ void __launch_bounds__(HUB_THREADS) k_scatter_hub(DevGraph g, const ScatterJob* __restrict__ jobs,
-                                                            HubQueue hq) {
-    const uint32_t nq = hub_count(hq);
-    for (uint32_t t = blockIdx.x; t < nq; t += gridDim.x) {
-        const unsigned long long it = hq.item[t];
-        const ScatterJob& J = jobs[it >> 40];
-        const uint32_t v = (uint32_t)J.qcand[(uint32_t)it];
-        const uint32_t* off = J.scan_out ? g.out_off : g.in_off;
-        const uint32_t* adj = J.scan_out ? g.out_adj : g.in_adj;
-        const uint32_t e1 = off[v + 1];
-        if (hq.scan && threadIdx.x == 0) {
-            atomicAdd(&hq.scan[0], 1ull);
-            atomicAdd(&hq.scan[1], (unsigned long long)(e1 - off[v]));
-        }
-        for (uint32_t e = off[v] + threadIdx.x; e < e1; e += HUB_THREADS) {
-            const uint32_t p = __ldg(adj + e);
-            const uint32_t x = p >> g.lbits;
-            if (label_ok(J.lab, (int32_t)(p & g.lmask)) && bit_of(J.filter, x))
-                atomicOr(&J.marks[x >> 5], 1u << (x & 31));
-        }
-    }
-}
-
-// A queued prune constraint: the candidate stays only if some neighbour hits.
-__global__ void __launch_bounds__(HUB_THREADS) k_prune_hub(DevGraph g, const PruneJob* __restrict__ jobs,
-                                                          HubQueue hq) {
-    const uint32_t nq = hub_count(hq);
-    for (uint32_t t = blockIdx.x; t < nq; t += gridDim.x) {
-        const unsigned long long it = hq.item[t];
-        const PruneJob& J = jobs[it >> 40];
-        const int c = (int)((it >> 32) & 0xff);
-        const uint32_t v = (uint32_t)J.cand[(uint32_t)it];
-        const uint32_t* off = J.con_dir[c] ? g.out_off : g.in_off;
-        const uint32_t* adj = J.con_dir[c] ? g.out_adj : g.in_adj;
-        const uint32_t e0 = off[v], e1 = off[v + 1];
-        bool found = false;
-        uint32_t read = 0;
-        for (uint32_t b = e0; b < e1; b += HUB_THREADS) {  // block-uniform bounds
-            const uint32_t e = b + threadIdx.x;
-            bool hit = false;
-            read += min((uint32_t)HUB_THREADS, e1 - b);
-            if (e < e1) {
-                const uint32_t p = __ldg(adj + e);
-                hit = label_ok(J.con_lab[c], (int32_t)(p & g.lmask)) && bit_of(J.con_bm[c], p >> g.lbits);
-            }
-            if (__syncthreads_or(hit)) {
-                found = true;
-                break;
-            }
-        }
-        if (hq.scan && threadIdx.x == 0) {
-            atomicAdd(&hq.scan[0], 1ull);
-            atomicAdd(&hq.scan[1], (unsigned long long)read);
-        }
-        if (!found && threadIdx.x == 0) atomicAnd(&J.bm[v >> 5], ~(1u << (v & 31)));
-    }
-}
-
-__global__ void __launch_bounds__(HUB_THREADS) k_cpi_count_hub(DevGraph g, const CpiJob* __restrict__ jobs,
-                                                              HubQueue hq) {
-    using Reduce = cub::BlockReduce<uint32_t, HUB_THREADS>;
-    __shared__ typename Reduce::TempStorage tmp;
-    const uint32_t nq = hub_count(hq);
-    for (uint32_t t = blockIdx.x; t < nq; t += gridDim.x) {
-        const unsigned long long it = hq.item[t];
-        const CpiJob& J = jobs[it >> 40];
-        const uint32_t a = (uint32_t)it;
-        const uint32_t v = (uint32_t)J.pcand[a];
-        const uint32_t* off = J.out ? g.out_off : g.in_off;
-        const uint32_t* adj = J.out ? g.out_adj : g.in_adj;
-        const uint32_t e1 = off[v + 1];
-        uint32_t cnt = 0;
-        if (hq.scan && threadIdx.x == 0) {
-            atomicAdd(&hq.scan[0], 1ull);
-            atomicAdd(&hq.scan[1], (unsigned long long)(e1 - off[v]));
-        }
-        for (uint32_t e = off[v] + threadIdx.x; e < e1; e += HUB_THREADS) {
-            const uint32_t p = __ldg(adj + e);
-            cnt += label_ok(J.lab, (int32_t)(p & g.lmask)) && bit_of(J.cbm, p >> g.lbits);
-        }
-        const uint32_t total = Reduce(tmp).Sum(cnt);
-        if (threadIdx.x == 0) J.off[a] = total;
-        __syncthreads();  // tmp is reused by the next item
-    }
-}
-
-// Ordered fill of a hub's index edges: tiles of HUB_THREADS entries, a block
-// scan gives each hit its slot after the hits of the earlier tiles.
-__global__ void __launch_bounds__(HUB_THREADS) k_cpi_fill_hub(DevGraph g, const CpiJob* __restrict__ jobs,
-                                                             HubQueue hq) {
-    using Scan = cub::BlockScan<uint32_t, HUB_THREADS>;
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_cpi_fill(DevGraph g, const CpiJob* __restrict__ jobs, int njobs,
+                                                                  ScanWork sw) {
+    using Scan = cub::BlockScan<uint32_t, WARP_KERNEL_THREADS>;
     __shared__ typename Scan::TempStorage tmp;
-    const uint32_t nq = hub_count(hq);
-    for (uint32_t t = blockIdx.x; t < nq; t += gridDim.x) {
-        const unsigned long long it = hq.item[t];
-        const CpiJob& J = jobs[it >> 40];
-        const uint32_t a = (uint32_t)it;
-        const uint32_t v = (uint32_t)J.pcand[a];
-        const uint32_t* off = J.out ? g.out_off : g.in_off;
-        const uint32_t* adj = J.out ? g.out_adj : g.in_adj;
-        const uint32_t e0 = off[v], e1 = off[v + 1];
-        const uint32_t o = J.off[a], oend = J.off[a + 1];
-        uint32_t running = 0;
-        if (hq.scan && threadIdx.x == 0) {
-            atomicAdd(&hq.scan[0], 1ull);
-            atomicAdd(&hq.scan[1], (unsigned long long)(e1 - e0));
-        }
-        for (uint32_t b = e0; b < e1; b += HUB_THREADS) {  // block-uniform bounds
-            const uint32_t e = b + threadIdx.x;
-            bool hit = false;
-            uint32_t x = 0, word = 0;
-            if (e < e1) {
-                const uint32_t p = __ldg(adj + e);
-                x = p >> g.lbits;
-                word = J.cbm[x >> 5];
-                hit = label_ok(J.lab, (int32_t)(p & g.lmask)) && ((word >> (x & 31)) & 1u);
-            }
-            uint32_t excl, total;
-            Scan(tmp).ExclusiveSum(hit ? 1u : 0u, excl, total);
-            if (hit) {
-                const uint64_t slot = (uint64_t)o + running + excl;
-                if (slot < oend && slot < J.cap)
-                    J.idx[slot] = make_int2((int32_t)(J.crank[x >> 5] + __popc(word & ((1u << (x & 31)) - 1))),
-                                            (int32_t)x);
-            }
-            running += total;
-            __syncthreads();  // tmp is reused by the next tile
-        }
+    __shared__ int2 s_slots[WARP_KERNEL_THREADS];
+    const int lane = threadIdx.x & 31;
+    int2* const slots = s_slots + (threadIdx.x & ~31);
+    const Groups G(sw, njobs);
+    uint64_t sc = 0, se = 0;
+    const uint32_t nhubs = G.n_hubs();
+    for (uint32_t it = blockIdx.x; it < nhubs; it += gridDim.x) {
+        uint32_t a;
+        const CpiJob& J = jobs[G.hub(it, &a)];
+        const AdjRef A = adj_ref(g, J.out);
+        const uint32_t v = (uint32_t)J.p.cand[a], e0 = A.off[v], e1 = A.off[v + 1];
+        uint32_t next = J.off[a];
+        const uint32_t end = J.off[a + 1];
+        if (next == end) continue;  // no index edges
+        if (threadIdx.x == 0) sc += 1, se += e1 - e0;
+        uint32_t hq[HUB_QUADS] = {}, xq[HUB_QUADS][4];
+        scan_block(g, A.adj, e0, e1, J.lab, J.cbm,
+                   [&](int q, uint32_t h, const uint32_t (&x)[4], const uint32_t (&)[4]) {
+#pragma unroll
+                       for (int i = 0; i < HUB_QUADS; i++)
+                           if (i == q) {
+                               hq[i] = h;
+#pragma unroll
+                               for (int c = 0; c < 4; c++) xq[i][c] = x[c];
+                           }
+                   },
+                   [&] {
+                       uint32_t mine = 0, excl, total;
+#pragma unroll
+                       for (int i = 0; i < HUB_QUADS; i++) mine += __popc(hq[i]);
+                       Scan(tmp).ExclusiveSum(mine, excl, total);
+                       uint32_t slot = next + excl;
+#pragma unroll
+                       for (int i = 0; i < HUB_QUADS; i++) {
+#pragma unroll
+                           for (int c = 0; c < 4; c++)
+                               if ((hq[i] >> c) & 1u) {
+                                   const uint32_t x = xq[i][c];
+                                   if (slot < J.cap)
+                                       J.idx[slot] = make_int2((int32_t)(__ldg(J.crank + (x >> 5)) +
+                                                                         __popc(__ldg(J.cbm + (x >> 5)) &
+                                                                                ((1u << (x & 31)) - 1))), (int32_t)x);
+                                   slot++;
+                               }
+                           hq[i] = 0;
+                       }
+                       next += total;
+                       __syncthreads();  // tmp is reused by the next round
+                       return next >= end;
+                   });
     }
+    const uint32_t ngroups = G.n_groups();
+    for (uint64_t it = gwarp_id(); it < ngroups; it += nwarps_total()) {
+        uint32_t a;
+        const CpiJob& J = jobs[G.group((uint32_t)it, lane, &a)];
+        const AdjRef A = adj_ref(g, J.out);
+        uint32_t e0 = 0, e1 = 0, o = 0;
+        if (a < *J.p.count) {
+            o = J.off[a];
+            if (J.off[a + 1] > o) {  // a parent without index edges skips its list
+                const uint32_t v = (uint32_t)J.p.cand[a];
+                e0 = A.off[v];
+                e1 = A.off[v + 1];
+            }
+        }
+        sc += e1 > e0;
+        se += e1 - e0;
+        uint32_t total;
+        const uint32_t ex = list_starts(e1 - e0, lane, &total);
+        uint32_t next = __shfl_sync(0xffffffffu, o, 0);
+        int2* const idx = J.idx;
+        const uint32_t* const crank = J.crank;
+        const uint64_t cap = J.cap;
+        scan_flat(g, A, e0, e1 - e0, ex, total, J.lab, J.cbm, slots, lane,
+                  [&](bool hit, uint32_t x, uint32_t w, int, uint32_t) {
+                      const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+                      if (hit) {
+                          const uint32_t slot = next + __popc(hits & ((1u << lane) - 1u));
+                          if (slot < cap)
+                              idx[slot] = make_int2((int32_t)(__ldg(crank + (x >> 5)) +
+                                                              __popc(w & ((1u << (x & 31)) - 1))), (int32_t)x);
+                      }
+                      next += __popc(hits);
+                  });
+    }
+    scan_flush<COUNT>(sw, sc, se);
 }
 
 // number of index edges of each job (read back to size the index exactly)
 __global__ void k_cpi_totals(const CpiJob* __restrict__ jobs, int njobs, uint32_t* totals) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < njobs) totals[j] = jobs[j].off[*jobs[j].pcount];
+    if (j < njobs) totals[j] = jobs[j].off[*jobs[j].p.count];
 }
 
 // Blocks of a grid-stride kernel: as many as the device holds at once. A
@@ -816,28 +860,30 @@ int launch_compact(const DevGraph& g, const CompactJob* d_jobs, int njobs, cudaS
     return check_launch("k_compact");
 }
 
-static int hub_reset(const HubQueue& hq, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(hq.n, 0, sizeof(uint32_t), st);
-    return e == cudaSuccess ? GFD_OK : cuda_fail(e, "hub queue reset");
+// the work of a launch over njobs jobs, then the kernel, one resident wave
+template <typename Job>
+static void job_groups(const DevGraph& g, const Job* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st) {
+    k_job_groups<Job><<<1, JOB_SCAN_THREADS, 0, st>>>(g, d_jobs, njobs, sw.pre);
 }
 
-int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const HubQueue& hq, cudaStream_t st) {
+#define GFD_SCAN_LAUNCH(kernel)                                                                                   \
+    do {                                                                                                          \
+        job_groups(g, d_jobs, njobs, sw, st);                                                                     \
+        if (sw.scan)                                                                                              \
+            kernel<true><<<grid_of(kernel<true>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, sw); \
+        else                                                                                                      \
+            kernel<false><<<grid_of(kernel<false>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, sw); \
+    } while (0)
+
+int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st) {
     if (njobs <= 0) return GFD_OK;
-    if (int rc = hub_reset(hq, st)) return rc;
-    k_job_groups<ScatterJob><<<1, JOB_SCAN_THREADS, 0, st>>>(d_jobs, njobs, hq.jpre);
-    if (hq.scan) k_scatter<true><<<grid_of(k_scatter<true>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, hq);
-    else k_scatter<false><<<grid_of(k_scatter<false>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, hq);
-    k_scatter_hub<<<grid_of(k_scatter_hub, HUB_THREADS), HUB_THREADS, 0, st>>>(g, d_jobs, hq);
+    GFD_SCAN_LAUNCH(k_scatter);
     return check_launch("k_scatter");
 }
 
-int launch_prune(const DevGraph& g, const PruneJob* d_jobs, int njobs, const HubQueue& hq, cudaStream_t st) {
+int launch_prune(const DevGraph& g, const PruneJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st) {
     if (njobs <= 0) return GFD_OK;
-    if (int rc = hub_reset(hq, st)) return rc;
-    k_job_groups<PruneJob><<<1, JOB_SCAN_THREADS, 0, st>>>(d_jobs, njobs, hq.jpre);
-    if (hq.scan) k_prune<true><<<grid_of(k_prune<true>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, hq);
-    else k_prune<false><<<grid_of(k_prune<false>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, hq);
-    k_prune_hub<<<grid_of(k_prune_hub, HUB_THREADS), HUB_THREADS, 0, st>>>(g, d_jobs, hq);
+    GFD_SCAN_LAUNCH(k_prune);
     return check_launch("k_prune");
 }
 
@@ -846,13 +892,9 @@ uint32_t cpi_chunks(uint64_t max_parent_candidates) {
 }
 
 int launch_cpi_count(const DevGraph& g, const CpiJob* d_jobs, int njobs, uint32_t nchunks, int32_t* d_err,
-                     uint32_t* d_totals, const HubQueue& hq, cudaStream_t st) {
+                     uint32_t* d_totals, const ScanWork& sw, cudaStream_t st) {
     if (njobs <= 0) return GFD_OK;
-    if (int rc = hub_reset(hq, st)) return rc;
-    k_job_groups<CpiJob><<<1, JOB_SCAN_THREADS, 0, st>>>(d_jobs, njobs, hq.jpre);
-    if (hq.scan) k_cpi_count<true><<<grid_of(k_cpi_count<true>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, hq);
-    else k_cpi_count<false><<<grid_of(k_cpi_count<false>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, hq);
-    k_cpi_count_hub<<<grid_of(k_cpi_count_hub, HUB_THREADS), HUB_THREADS, 0, st>>>(g, d_jobs, hq);
+    GFD_SCAN_LAUNCH(k_cpi_count);
     const int grid = (int)std::min<uint64_t>((uint64_t)njobs * nchunks, (uint64_t)device_sms() * 8);
     k_cpi_sums<<<grid, COMPACT_THREADS, 0, st>>>(d_jobs, njobs, nchunks);
     k_cpi_scan<<<grid, COMPACT_THREADS, 0, st>>>(d_jobs, njobs, nchunks, d_err);
@@ -860,13 +902,9 @@ int launch_cpi_count(const DevGraph& g, const CpiJob* d_jobs, int njobs, uint32_
     return check_launch("k_cpi_count");
 }
 
-int launch_cpi_fill(const DevGraph& g, const CpiJob* d_jobs, int njobs, const HubQueue& hq, cudaStream_t st) {
+int launch_cpi_fill(const DevGraph& g, const CpiJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st) {
     if (njobs <= 0) return GFD_OK;
-    if (int rc = hub_reset(hq, st)) return rc;
-    k_job_groups<CpiJob><<<1, JOB_SCAN_THREADS, 0, st>>>(d_jobs, njobs, hq.jpre);
-    if (hq.scan) k_cpi_fill<true><<<grid_of(k_cpi_fill<true>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, hq);
-    else k_cpi_fill<false><<<grid_of(k_cpi_fill<false>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, hq);
-    k_cpi_fill_hub<<<grid_of(k_cpi_fill_hub, HUB_THREADS), HUB_THREADS, 0, st>>>(g, d_jobs, hq);
+    GFD_SCAN_LAUNCH(k_cpi_fill);
     return check_launch("k_cpi_fill");
 }
 

@@ -109,25 +109,25 @@ k_node_candidates(DevGraph g, FilterKey key, unsigned long long* scratch, int32_
             const uint32_t v = w0 + r * 128 + lane * 4;
             uint32_t vi[4], oo[5], io[5];
             if (v + 4 <= n) {
-                const uint4 a = *reinterpret_cast<const uint4*>(g.vinfo + v);
-                const uint4 o = *reinterpret_cast<const uint4*>(g.out_off + v);
-                const uint4 i = *reinterpret_cast<const uint4*>(g.in_off + v);
+                const uint4 a = *reinterpret_cast<const uint4*>(g.o_vinfo + v);
+                const uint4 o = *reinterpret_cast<const uint4*>(g.o_out_off + v);
+                const uint4 i = *reinterpret_cast<const uint4*>(g.o_in_off + v);
                 vi[0] = a.x, vi[1] = a.y, vi[2] = a.z, vi[3] = a.w;
                 oo[0] = o.x, oo[1] = o.y, oo[2] = o.z, oo[3] = o.w;
                 io[0] = i.x, io[1] = i.y, io[2] = i.z, io[3] = i.w;
             } else {  // the graph's last vertices: offsets have n + 1 entries
 #pragma unroll
                 for (int c = 0; c < 4; c++) {
-                    vi[c] = v + c < n ? g.vinfo[v + c] : 0u;
-                    oo[c] = v + c <= n ? g.out_off[v + c] : 0u;
-                    io[c] = v + c <= n ? g.in_off[v + c] : 0u;
+                    vi[c] = v + c < n ? g.o_vinfo[v + c] : 0u;
+                    oo[c] = v + c <= n ? g.o_out_off[v + c] : 0u;
+                    io[c] = v + c <= n ? g.o_in_off[v + c] : 0u;
                 }
             }
             oo[4] = __shfl_down_sync(0xffffffffu, oo[0], 1);
             io[4] = __shfl_down_sync(0xffffffffu, io[0], 1);
             if (lane == 31) {
-                oo[4] = v + 4 <= n ? g.out_off[v + 4] : 0u;
-                io[4] = v + 4 <= n ? g.in_off[v + 4] : 0u;
+                oo[4] = v + 4 <= n ? g.o_out_off[v + 4] : 0u;
+                io[4] = v + 4 <= n ? g.o_in_off[v + 4] : 0u;
             }
 #pragma unroll
             for (int c = 0; c < 4; c++) {

@@ -143,8 +143,9 @@ int make_plan(const gfd_gfd* phi, int32_t n_attrs, const PlanStats& stats, HostP
     auto log_moment = [&](int32_t L, int a, int b) -> double {
         a = std::min(a, 3);
         b = std::min(b, 3);
-        double m = stats.moments ? (L == GFD_WILDCARD ? stats.moments_all[4 * a + b]
-                                                      : stats.moments[16 * (size_t)L + 4 * a + b])
+        double m = stats.moments ? (L == GFD_WILDCARD    ? stats.moments_all[4 * a + b]
+                                    : L < stats.n_labels ? stats.moments[16 * (size_t)L + 4 * a + b]
+                                                         : 0.0)
                                  : 1.0;
         return m > 0 ? std::log(m) : NEG;
     };

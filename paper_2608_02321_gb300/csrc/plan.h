@@ -43,7 +43,8 @@ struct HostPlan {
 struct PlanStats {
     int64_t n_vertices = 0;
     int64_t n_edges = 0;
-    const double* moments = nullptr;      // [65536][16]
+    const double* moments = nullptr;      // [n_labels][16]; labels from n_labels on have no vertices
+    int32_t n_labels = 0;
     const double* moments_all = nullptr;  // [16]
     const double* elabel_frac = nullptr;  // [256]
 };

@@ -222,8 +222,7 @@ struct Group {
     };
     std::vector<Off> offs;
     size_t o_keybm = 0, o_keys = 0, o_tmp = 0, o_cmp_sums = 0, o_cpi_sums = 0, o_cpi_tot = 0;
-    size_t o_hubq = 0, o_hubn = 0;  // hub queue of the adjacency kernels
-    size_t o_jpre = 0;               // per-launch prefix of the jobs' group counts
+    size_t o_work = 0;  // shares of the adjacency scans' jobs
     uint8_t* cpi_base = nullptr;  // index edges, sized after counting
     size_t cpi_bytes = 0;
     size_t cpi_bound = 0;  // upper bound of cpi_bytes known at planning time
@@ -248,9 +247,7 @@ namespace {
 // dir-direction adjacency of the i label class but stops at the first hit
 // (counted as half of it).
 bool td_gather_cheaper(const gfd_graph* g, int32_t label_q, int32_t label_i, int dir) {
-    auto degsum = [&](int32_t L, bool out) -> double {
-        return L == GFD_WILDCARD ? (double)g->m : (double)g->label_stats[3 * (size_t)L + (out ? 1 : 2)];
-    };
+    auto degsum = [&](int32_t L, bool out) { return (double)g->label_stat(L, out ? 1 : 2); };
     const double scatter = degsum(label_q, dir == 0);
     const double gather = 0.5 * degsum(label_i, dir == 1);
     return gather < scatter;
@@ -286,12 +283,8 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
             }
             G->slot_key[s][i] = it->second;
         }
-    auto lab_count = [&](int32_t L) -> uint64_t {
-        return L == GFD_WILDCARD ? (uint64_t)g->n : (uint64_t)g->label_stats[3 * (size_t)L];
-    };
-    auto lab_deg = [&](int32_t L, bool outdir) -> uint64_t {
-        return L == GFD_WILDCARD ? (uint64_t)g->m : (uint64_t)g->label_stats[3 * (size_t)L + (outdir ? 1 : 2)];
-    };
+    auto lab_count = [&](int32_t L) { return g->label_stat(L, 0); };
+    auto lab_deg = [&](int32_t L, bool outdir) { return g->label_stat(L, outdir ? 1 : 2); };
     Layout L;
     G->descs.assign(n, SlotDesc{});
     G->offs.resize(n);
@@ -383,9 +376,7 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
     G->o_cmp_sums = L.take(4ull * G->cmp_chunks * std::max<size_t>(1, n_compact));
     G->o_cpi_sums = L.take(8ull * G->cpi_nch * std::max<size_t>(1, n_cpi));
     G->o_cpi_tot = L.take(4ull * std::max<size_t>(1, n_cpi));
-    G->o_hubq = L.take(8ull * HUB_CAP);
-    G->o_hubn = L.take(4);
-    G->o_jpre = L.take(4ull * (std::max(n_sct, std::max(n_prn, n_cpi)) + 1));
+    G->o_work = L.take(4ull * scan_work_words(std::max(n_sct, std::max(n_prn, n_cpi))));
     // the region uploaded from the host: keys and job tables
     G->o_jobs = L.size;
     G->o_keys = L.take(sizeof(FilterKey) * std::max(1, nkeys));
@@ -427,6 +418,10 @@ int group_build(gfd_graph* g, Group* G, const Tables& T, bool refine, cudaStream
             D.wpre[l] = (uint64_t*)(base + F.wpre[l]);
         }
     }
+    auto scan_list = [&](int s, int i) {
+        const SlotDesc& D = G->descs[s];
+        return ScanList{D.cand[i], state_ncand(s, i), D.bm[i], D.rank[i]};
+    };
     auto compact_job = [&](int s, int i) {
         CompactJob J{};
         J.bm = G->descs[s].bm[i];
@@ -467,22 +462,21 @@ int group_build(gfd_graph* g, Group* G, const Tables& T, bool refine, cudaStream
                 J.bm = G->descs[s].bm[lvl];
                 J.src = keybm(G->slot_key[s][lvl]);
                 PruneJob Pj{};
-                Pj.cand = G->descs[s].cand[lvl];
-                Pj.count = state_ncand(s, lvl);
-                Pj.bm = G->descs[s].bm[lvl];
+                Pj.c = scan_list(s, lvl);
+                Pj.out = G->descs[s].bm[lvl];
                 for (const Con& c : P.td[lvl]) {
                     const int32_t lq = G->plans[s].key[c.q].label, li = G->plans[s].key[lvl].label;
                     if (td_gather_cheaper(g, lq, li, c.dir)) {
                         Pj.con_bm[Pj.ncon] = G->descs[s].bm[c.q];
                         Pj.con_dir[Pj.ncon] = c.dir;
                         Pj.con_lab[Pj.ncon] = c.lab;
+                        Pj.con_any[Pj.ncon] = lq == GFD_WILDCARD;
                         Pj.ncon++;
                         continue;
                     }
                     uint32_t* marks = (uint32_t*)(base + G->o_tmp + 4ull * nwords * tmp_used++);
                     ScatterJob S{};
-                    S.qcand = G->descs[s].cand[c.q];
-                    S.qcount = state_ncand(s, c.q);
+                    S.q = scan_list(s, c.q);
                     S.filter = J.src;
                     S.marks = marks;
                     // x needs an out-neighbour y in C(q) (x -> y): follow in-edges of y
@@ -523,22 +517,21 @@ int group_build(gfd_graph* g, Group* G, const Tables& T, bool refine, cudaStream
                 A.bm = G->descs[s].bm[lvl];
                 A.src = G->descs[s].bm[lvl];
                 PruneJob J{};
-                J.cand = G->descs[s].cand[lvl];
-                J.count = state_ncand(s, lvl);
-                J.bm = G->descs[s].bm[lvl];
+                J.c = scan_list(s, lvl);
+                J.out = G->descs[s].bm[lvl];
                 for (const Con& c : P.bu[lvl]) {
                     const int32_t lq = P.key[c.q].label, li = P.key[lvl].label;
                     if (td_gather_cheaper(g, lq, li, c.dir)) {
                         J.con_bm[J.ncon] = G->descs[s].bm[c.q];
                         J.con_dir[J.ncon] = c.dir;
                         J.con_lab[J.ncon] = c.lab;
+                        J.con_any[J.ncon] = lq == GFD_WILDCARD;
                         J.ncon++;
                         continue;
                     }
                     uint32_t* marks = (uint32_t*)(base + G->o_tmp + 4ull * nwords * tmp_used++);
                     ScatterJob S{};
-                    S.qcand = G->descs[s].cand[c.q];
-                    S.qcount = state_ncand(s, c.q);
+                    S.q = scan_list(s, c.q);
                     S.filter = G->descs[s].bm[lvl];
                     S.marks = marks;
                     S.scan_out = c.dir ? 0 : 1;
@@ -574,8 +567,7 @@ int group_build(gfd_graph* g, Group* G, const Tables& T, bool refine, cudaStream
             const int par = G->plans[s].lv[i].par;
             if (par < 0) continue;  // starts a component
             CpiJob J{};
-            J.pcand = G->descs[s].cand[par];
-            J.pcount = state_ncand(s, par);
+            J.p = scan_list(s, par);
             J.cbm = G->descs[s].bm[i];
             J.crank = G->descs[s].rank[i];
             J.off = G->descs[s].cpi_off[i];
@@ -631,9 +623,8 @@ int group_launch(gfd_graph* g, Group* G, const Tables& T, cudaMemPool_t pool, cu
                  int64_t* launches, bool count = false) {
     const DevGraph& dg = g->dg;
     uint8_t* base = G->base;
-    const HubQueue hq{(unsigned long long*)(base + G->o_hubq), (uint32_t*)(base + G->o_hubn), HUB_CAP,
-                      count ? (unsigned long long*)&T.sched->cnt[CNT_SCAN_CANDS] : nullptr,
-                      (uint32_t*)(base + G->o_jpre)};
+    const ScanWork sw{(uint32_t*)(base + G->o_work),
+                      count ? (unsigned long long*)&T.sched->cnt[CNT_SCAN_CANDS] : nullptr};
     prof.begin(PROF_FILTER, st);
     if (int rc = launch_filter(dg, (const FilterKey*)(base + G->o_keys), (int)G->keys.size(),
                                (uint32_t*)(base + G->o_keybm), st))
@@ -649,10 +640,10 @@ int group_launch(gfd_graph* g, Group* G, const Tables& T, cudaMemPool_t pool, cu
                 rc = launch_compact(dg, (const CompactJob*)(base + G->o_cmp) + ph.first, (int)ph.count, st);
                 break;
             case 2:
-                rc = launch_scatter(dg, (const ScatterJob*)(base + G->o_sct) + ph.first, (int)ph.count, hq, st);
+                rc = launch_scatter(dg, (const ScatterJob*)(base + G->o_sct) + ph.first, (int)ph.count, sw, st);
                 break;
             case 3:
-                rc = launch_prune(dg, (const PruneJob*)(base + G->o_prn) + ph.first, (int)ph.count, hq, st);
+                rc = launch_prune(dg, (const PruneJob*)(base + G->o_prn) + ph.first, (int)ph.count, sw, st);
                 break;
             case 4: {
                 cudaError_t e = cudaMemsetAsync(base + G->o_tmp, 0, 4ull * dg.nwords * ph.count, st);
@@ -661,7 +652,7 @@ int group_launch(gfd_graph* g, Group* G, const Tables& T, cudaMemPool_t pool, cu
             }
         }
         if (rc) return rc;
-        launches[PROF_REFINE] += ph.kind == 4 ? 0 : (ph.kind == 0 ? 1 : 2);  // scatter/prune: + hub kernel
+        launches[PROF_REFINE] += ph.kind == 4 ? 0 : (ph.kind == 0 ? 1 : 2);  // scatter/prune: + shares of the jobs
     }
     prof.end(PROF_REFINE, st);
     prof.begin(PROF_INDEX, st);
@@ -669,7 +660,7 @@ int group_launch(gfd_graph* g, Group* G, const Tables& T, cudaMemPool_t pool, cu
     if (ncpi) {
         CpiJob* d_cpi = (CpiJob*)(base + G->o_cpi);
         uint32_t* d_tot = (uint32_t*)(base + G->o_cpi_tot);
-        if (int rc = launch_cpi_count(dg, d_cpi, ncpi, G->cpi_nch, T.err, d_tot, hq, st)) return rc;
+        if (int rc = launch_cpi_count(dg, d_cpi, ncpi, G->cpi_nch, T.err, d_tot, sw, st)) return rc;
         // size the index edges exactly: one read-back of the per-edge totals
         std::vector<uint32_t> tot(ncpi);
         GFD_CUDA(cudaMemcpyAsync(tot.data(), d_tot, 4ull * ncpi, cudaMemcpyDeviceToHost, st));
@@ -698,7 +689,7 @@ int group_launch(gfd_graph* g, Group* G, const Tables& T, cudaMemPool_t pool, cu
         for (int s = 0; s < G->n; s++)
             GFD_CUDA(cudaMemcpyAsync(&T.desc[G->slot[s]].cpi_idx, G->descs[s].cpi_idx, sizeof(G->descs[s].cpi_idx),
                                      cudaMemcpyHostToDevice, st));
-        if (int rc = launch_cpi_fill(dg, d_cpi, ncpi, hq, st)) return rc;
+        if (int rc = launch_cpi_fill(dg, d_cpi, ncpi, sw, st)) return rc;
         launches[PROF_INDEX] += 7;
     }
     prof.end(PROF_INDEX, st);
@@ -890,7 +881,14 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
                                              cudaMemcpyDeviceToHost, st));
             }
         }
+        std::vector<uint32_t> orig((size_t)g->n);  // lists leave in the caller's ids, increasing
+        GFD_CUDA(cudaMemcpyAsync(orig.data(), g->dg.orig, 4ull * g->n, cudaMemcpyDeviceToHost, st));
         GFD_CUDA(cudaStreamSynchronize(st));
+        for (auto& lists : kept)
+            for (auto& lst : lists) {
+                for (auto& v : lst) v = (int32_t)orig[v];
+                std::sort(lst.begin(), lst.end());
+            }
     }
     for (int s = 0; s < n; s++) {
         gfd_result* r = make_result(G.plans[s], states[s], hs.steps, hs.probes, vbuf[s], st);
