@@ -133,6 +133,7 @@ struct SlotDesc {
     uint32_t* bm[MAXK];
     uint32_t* rank[MAXK];
     int32_t* cand[MAXK];
+    const uint32_t* cand_n[MAXK];  // number of candidates
     uint32_t cand_cap[MAXK];
     uint32_t* cpi_off[MAXK];  // level i >= 1
     int2* cpi_idx[MAXK];      // (position in C(i), vertex id) per index edge

@@ -1,6 +1,7 @@
 // Host-side handles and the engine interface shared by the translation units.
 #pragma once
 
+#include <array>
 #include <mutex>
 #include <string>
 #include <memory>
@@ -26,6 +27,19 @@ struct gfd_graph {
     std::vector<double> moments;                  // [labels][16], see PlanStats
     std::vector<double> moments_all;              // [16]
     std::vector<double> elabel_frac;              // [256]
+    // vertices of each label (GFD_WILDCARD: of all) in degree class c: [lo, hi)
+    std::vector<std::array<uint32_t, 2 * gfd::N_CLASS>> label_range;
+    void range_of(int32_t L, uint32_t* lo, uint32_t* hi) const {
+        for (int c = 0; c < gfd::N_CLASS; c++) {
+            if (L == GFD_WILDCARD) {
+                lo[c] = c ? dg.class_end[c - 1] : 0;
+                hi[c] = c < gfd::N_CLASS - 1 ? dg.class_end[c] : (uint32_t)n;
+            } else {
+                lo[c] = L < n_labels() ? label_range[L][2 * c] : 0;
+                hi[c] = L < n_labels() ? label_range[L][2 * c + 1] : 0;
+            }
+        }
+    }
     int32_t n_labels() const { return (int32_t)label_stats.size() / 3; }
     // which: 0 vertices of the label (GFD_WILDCARD: all), 1 their out-degree sum, 2 their in-degree sum
     uint64_t label_stat(int32_t L, int which) const {
@@ -68,43 +82,54 @@ struct gfd_result {
 namespace gfd {
 
 // ---- job descriptors of the index kernels (device memory)
-struct AndJob {          // bm = src & tmp[0] & ... & tmp[ntmp-1]
-    uint32_t* bm;
-    const uint32_t* src;
-    const uint32_t* tmp[2 * MAXK];
-    int32_t ntmp;
+
+// The candidates of a bitmap whose adjacency is scanned, shared out as work items
+// on the host: the vertices a label has in each degree class are a range [lo, hi)
+// (for the wildcard the whole class). An item is an aligned unit of 2^unit(c)
+// vertices of class c (ScanLaunch): one hub for a block in class 0, a warp's share
+// in the others. A flat range has no adjacency to scan: units of FLAT_UNIT in every
+// class, for warps.
+struct ScanRange {
+    const uint32_t* bm;
+    uint32_t lo[N_CLASS], hi[N_CLASS];
+    int32_t flat;
+};
+constexpr int FLAT_UNIT = 10;  // (log2; a lane per word)
+__host__ __device__ constexpr uint32_t scan_items(uint32_t lo, uint32_t hi, int unit) {
+    return hi <= lo ? 0u : ((hi - 1) >> unit) - (lo >> unit) + 1;
+}
+
+struct ScatterJob {      // mark vertices adjacent to the candidates of another level
+    ScanRange r;
+    const uint32_t* filter;  // only vertices in this bitmap are marked
+    uint32_t* marks;
+    int32_t scan_out;        // 1: follow out-edges of r, 0: in-edges
+    int32_t lab;
+};
+// out = the vertices of r that are in all marks and, for every constraint, have a
+// neighbour (con_dir 1: out-neighbour) in con_bm through an edge with label
+// con_lab (or any). out starts as zeros.
+struct RefineJob {
+    ScanRange r;
+    uint32_t* out;
+    int32_t nmarks, ncon;
+    const uint32_t* marks[2 * MAXK];
+    const uint32_t* con_bm[2 * MAXK];
+    int8_t con_dir[2 * MAXK];
+    int8_t con_any[2 * MAXK];   // con_bm holds vertices of any label
+    int16_t con_lab[2 * MAXK];
 };
 struct CompactJob {      // rank and candidate list of bm
     const uint32_t* bm;
     uint32_t* rank;
-    int32_t* cand;
+    int32_t* cand;           // null: no list wanted
     uint32_t* count;
     uint32_t* csum;          // per-chunk set-bit counts (scratch)
 };
-struct ScanList {        // a compacted candidate list whose vertices' adjacency is scanned
-    const int32_t* cand;
-    const uint32_t* count;
-    const uint32_t* bm;
-    const uint32_t* rank;
-};
-struct ScatterJob {      // mark vertices adjacent to the candidates of another level
-    ScanList q;
-    const uint32_t* filter;  // only vertices in this bitmap are marked
-    uint32_t* marks;
-    int32_t scan_out;        // 1: follow out-edges of q, 0: in-edges
-    int32_t lab;
-};
-struct PruneJob {        // drop candidates with no neighbour in a later level
-    ScanList c;              // the candidates
-    uint32_t* out;           // their bitmap, cleared where a candidate is dropped
-    int32_t ncon;
-    const uint32_t* con_bm[2 * MAXK];
-    int32_t con_dir[2 * MAXK];
-    int32_t con_lab[2 * MAXK];
-    int32_t con_any[2 * MAXK];  // con_bm holds vertices of any label
-};
 struct CpiJob {          // index edges of one spanning-tree edge
-    ScanList p;              // the parent's candidates
+    ScanRange r;             // the parent's candidates
+    const uint32_t* prank;   // their ranks and number
+    const uint32_t* pcount;
     const uint32_t* cbm;
     const uint32_t* crank;
     uint32_t* off;
@@ -112,32 +137,41 @@ struct CpiJob {          // index edges of one spanning-tree edge
     uint64_t cap;
     int32_t out;             // 1: children are out-neighbours of the parent candidates
     int32_t lab;
-    uint64_t* nnz_stat;
+    uint32_t chunk0;         // chunks of the earlier jobs' counts
     uint64_t* csum;          // per-chunk count sums (scratch)
+    uint32_t* total;         // number of index edges
 };
 
-struct ScanWork {
-    // room for the shares of a launch's jobs: scan_work_words(largest job table)
-    uint32_t* pre;
-    // counting pass: [0] candidates whose adjacency was scanned, [1] adjacency
-    // entries read (null: not counting)
-    unsigned long long* scan;
+// One launch of scanning jobs: warp items and block items of all jobs together,
+// the units of the classes, and (device memory, apart from the jobs so that a
+// search touches few lines) how many items of each kind the earlier jobs have.
+struct ScanLaunch {
+    uint32_t items = 0, hubs = 0;
+    int8_t unit[N_CLASS] = {};
+    const uint32_t* first = nullptr;      // [njobs]
+    const uint32_t* hub_first = nullptr;  // [njobs]
 };
-constexpr size_t scan_work_words(size_t njobs) { return (N_CLASS + 1) * (njobs + 1); }
+// counting pass: [0] candidates whose adjacency was scanned, [1] adjacency
+// entries read (null: not counting)
+using ScanCount = unsigned long long*;
 
 // ---- index kernels (index.cu); each launch covers all jobs given
 int launch_filter(const DevGraph& g, const FilterKey* d_keys, int nkeys, uint32_t* d_out, cudaStream_t st);
-int launch_and(const DevGraph& g, const AndJob* d_jobs, int njobs, cudaStream_t st);
+int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const ScanLaunch& l, ScanCount scan,
+                   cudaStream_t st);
+int launch_refine(const DevGraph& g, const RefineJob* d_jobs, int njobs, const ScanLaunch& l, ScanCount scan,
+                  cudaStream_t st);
 int launch_compact(const DevGraph& g, const CompactJob* d_jobs, int njobs, cudaStream_t st);
-int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st);
-int launch_prune(const DevGraph& g, const PruneJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st);
-// Index edges in two launches: counts, offsets and per-job totals first (the
-// caller reads the totals back and allocates exactly), then the fill.
-int launch_cpi_count(const DevGraph& g, const CpiJob* d_jobs, int njobs, uint32_t nchunks, int32_t* d_err,
-                     uint32_t* d_totals, const ScanWork& sw, cudaStream_t st);
-int launch_cpi_fill(const DevGraph& g, const CpiJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st);
+// Index edges in two steps: counts, offsets and per-job totals first, then the
+// fill (between the two the caller may read the totals back and allocate exactly).
+int launch_cpi_count(const DevGraph& g, const CpiJob* d_jobs, int njobs, const ScanLaunch& l, uint32_t chunks,
+                     int32_t* d_err, ScanCount scan, cudaStream_t st);
+int launch_cpi_fill(const DevGraph& g, const CpiJob* d_jobs, int njobs, const ScanLaunch& l, ScanCount scan,
+                    cudaStream_t st);
 uint32_t compact_chunks(const DevGraph& g);
 uint32_t cpi_chunks(uint64_t max_parent_candidates);
+// units of a launch whose bitmaps have `vertices` vertices in the last class
+void scan_units(uint64_t vertices, int most, int8_t* unit);
 
 // ---- enumeration (enumerate.cu)
 struct EnumArgs {

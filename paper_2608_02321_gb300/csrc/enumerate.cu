@@ -873,6 +873,10 @@ __device__ void slot_start(const SlotDesc* D, SlotState* S) {
     S->cur = 0;
     S->cursor[0] = 0;
     S->cb = S->ce = 0;
+    for (int i = 0; i < D->k; i++) S->ncand[i] = *D->cand_n[i];
+    S->st_cpi = 0;
+    for (int i = 1; i < D->k; i++)
+        if (D->lv[i].par >= 0) S->st_cpi += D->cpi_off[i][S->ncand[D->lv[i].par]];
     S->nrows[0] = S->ncand[0];
     S->total[0] = D->k == 1             ? (uint64_t)S->ncand[0]
                 : D->lv[1].par < 0      ? (uint64_t)S->ncand[0] * S->ncand[1]  // level 1 starts a component

@@ -469,7 +469,8 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
     std::vector<Segment> segs(flag.nsegs);
     if (!segs.empty())
         CK(cudaMemcpyAsync(segs.data(), S.at<void>(s_seg), sizeof(Segment) * segs.size(), cudaMemcpyDeviceToHost, st));
-    for (int c = 0; c < N_CLASS - 1; c++) g->dg.class_end[c] = flag.class_end[c];
+    // (0 where all classes up to one are empty: the ends never fall)
+    for (int c = 0; c < N_CLASS - 1; c++) g->dg.class_end[c] = std::max(flag.class_end[c], c ? g->dg.class_end[c - 1] : 0u);
 
     // both adjacency arrays: edges sorted by (source, destination) and by
     // (destination, source) in the inside numbering
@@ -522,6 +523,13 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
             chunks.push_back({v, v + std::min(MOMENT_CHUNK, last - v)});
             chunk_label.push_back(segs[i].label);
         }
+    }
+    g->label_range.assign(n_labels, {});
+    for (size_t i = 0; i < segs.size(); i++) {
+        int c = 0;
+        while (c < N_CLASS - 1 && segs[i].first >= g->dg.class_end[c]) c++;
+        g->label_range[segs[i].label][2 * c] = segs[i].first;
+        g->label_range[segs[i].label][2 * c + 1] = i + 1 < segs.size() ? segs[i + 1].first : (uint32_t)n;
     }
     g->moments.assign((size_t)n_labels * 16, 0.0);
     g->moments_all.assign(16, 0.0);

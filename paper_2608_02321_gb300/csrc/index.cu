@@ -4,20 +4,23 @@
 //              pushed-down constant X literals), one coalesced pass over vertex
 //              data for all filter keys;
 //   k_scatter  step 1c: mark vertices adjacent (in the direction and with the
-//   k_and      label of a pattern edge) to the candidates of another level,
-//              then intersect;
-//   k_prune    step 1c: remove candidates with no such neighbour among the
-//              candidates of another level (early exit at the first one);
-//              top-down and bottom-up use whichever of the two is cheaper;
+//              label of a pattern edge) to the candidates of another level;
+//   k_refine   step 1c: keep the candidates that are marked, and those with such
+//              a neighbour among the candidates of another level (early exit at
+//              the first one); top-down and bottom-up use whichever of marking
+//              and looking is cheaper;
 //   k_compact  bitmap -> exclusive popcount prefix (O(1) rank) + sorted list;
 //   k_cpi_*    step 1d: for each spanning-tree edge, the index edges from
-//              every parent candidate to the positions of its child candidates;
-// The adjacency scans (k_scatter, k_prune, k_cpi_count, k_cpi_fill) share out a
-// job's candidates by degree class: a block per hub, a warp per 1, 8 or 32
-// vertices of the other classes.
+//              every parent candidate to the positions of its child candidates.
 //
-// Every launch processes a table of jobs; blocks (or warps) stride over the
-// items of each job with a per-job rotation so that small jobs spread out.
+// Every launch processes a table of jobs. Candidates are read from bitmaps, so
+// refinement needs no lists: a launch per level and direction (two with marks).
+// Which vertices can be in a bitmap is known on the host (a label's range in each
+// degree class), so the jobs' shares of a launch are laid out there (ScanRange)
+// and no kernel counts or scans between two steps of the refinement. Before, with
+// a list per level and step and its compaction in between (up to seven launches
+// per level and direction), a triangle with a chain on 1M vertices took 0.50 ms
+// of refinement in 47 launches, and 16 requests on 1M vertices 7.3 ms in 690.
 #include <cub/cub.cuh>
 
 #include <algorithm>
@@ -32,7 +35,8 @@ namespace {
 
 constexpr int FILTER_THREADS = 256;
 constexpr int COMPACT_THREADS = 256;
-constexpr uint32_t COMPACT_WORDS = 1024;  // words (or counts) per chunk
+constexpr uint32_t COMPACT_WORDS = 256;   // bitmap words per chunk of the compaction
+constexpr uint32_t CPI_CHUNK = 1024;      // counts per chunk of the index offsets
 constexpr int WARP_KERNEL_THREADS = 256;
 
 __device__ __forceinline__ uint64_t gwarp_id() {
@@ -72,26 +76,6 @@ __global__ void k_filter(DevGraph g, const FilterKey* __restrict__ keys, int nke
             }
             uint32_t b = __ballot_sync(0xffffffffu, p);
             if (lane == 0) out[(uint64_t)k * g.nwords + w] = b;
-        }
-    }
-}
-
-// One block per (job, chunk of AND_WORDS words) item, so that every job's words
-// are spread over the GPU and no thread walks the job table.
-constexpr uint32_t AND_WORDS = 2048;
-constexpr int AND_THREADS = 256;
-
-__global__ void __launch_bounds__(AND_THREADS) k_and(DevGraph g, const AndJob* __restrict__ jobs, int njobs,
-                                                      uint32_t nchunks) {
-    for (uint64_t it = blockIdx.x; it < (uint64_t)njobs * nchunks; it += gridDim.x) {
-        const AndJob& J = jobs[it / nchunks];
-        const uint32_t w0 = (uint32_t)(it % nchunks) * AND_WORDS;
-        const uint32_t w1 = min(g.nwords, w0 + AND_WORDS);
-        const int ntmp = J.ntmp;
-        for (uint32_t w = w0 + threadIdx.x; w < w1; w += AND_THREADS) {
-            uint32_t x = J.src[w];
-            for (int t = 0; t < ntmp; t++) x &= J.tmp[t][w];
-            J.bm[w] = x;
         }
     }
 }
@@ -157,7 +141,7 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_compact_write(DevGraph g, c
         int32_t* const cand = J.cand;
         const uint32_t lane = threadIdx.x & 31;
 #pragma unroll
-        for (int q = 0; q < WPT; q++)
+        for (int q = 0; q < WPT && cand; q++)
             for (uint32_t some = __ballot_sync(0xffffffffu, words[q] != 0); some; some &= some - 1) {
                 const int src = __ffs(some) - 1;
                 const uint32_t x = __shfl_sync(0xffffffffu, words[q], src), at = __shfl_sync(0xffffffffu, first[q], src);
@@ -169,23 +153,24 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_compact_write(DevGraph g, c
     }
 }
 
-// The adjacency kernels below give the lanes of a warp a candidate each (32 of
-// the lowest degree class, fewer of the others); the warp then scans its lists
-// end to end as one sequence, 32 x FLAT entries at a time (scan_flat). A hub's
-// list is scanned by a block. Vertices are numbered by degree class, so a
-// candidate list holds its classes one after the other, and where they end are
-// rank lookups.
+// The adjacency kernels below give the lanes of a warp a candidate each; the warp
+// then scans its lists end to end as one sequence, 32 x FLAT entries at a time
+// (scan_flat). A hub's list is scanned by a block.
 //
 // These scans are bound by latency (a random adjacency line, then a random
 // bitmap word, from L2 or HBM) and by balance. A lane that scans its own list
 // leaves the warp waiting for its longest list with few loads in flight; a warp
 // that happens to get 32 long lists keeps the launch waiting. End to end every
-// lane has FLAT loads in flight whatever the degrees, and by classes no warp
-// gets more than 2048 entries at a time.
+// lane has FLAT loads in flight whatever the degrees, and by degree classes no
+// warp gets more than 2048 entries at a time (one vertex of up to 2048, 8 of up
+// to 256, 32 of up to 32).
 constexpr int FLAT = 4;
-// candidates per warp of each class after the hubs (x the class's largest degree:
-// at most 2048 entries)
-__device__ constexpr uint32_t class_group(int c) { return c == 1 ? 1 : c == 2 ? 8 : 32; }
+constexpr int MAX_WORDS = 32;  // most bitmap words per warp item of the last class
+// Resident blocks per SM the scanning kernels are compiled for; at 6 the
+// refinement's registers spill (a triangle with a chain on 1M vertices: 0.22 ms of
+// refinement at 5, 0.35 ms at 6).
+constexpr int SCAN_BLOCKS = 6;
+constexpr int REFINE_BLOCKS = 5;
 
 // Entries of the aligned quad at b < e1 that lie in [e0, e1), as a mask.
 __device__ __forceinline__ uint32_t quad_mask(uint32_t b, uint32_t e0, uint32_t e1) {
@@ -282,126 +267,73 @@ __device__ __forceinline__ uint32_t list_starts(uint32_t len, int lane, uint32_t
     return incl - len;
 }
 
-// Work of a launch over all its jobs, written by k_job_groups: ScanWork::pre
-// holds, for the J = njobs jobs, the exclusive prefix of their warp groups
-// [J + 1], that of their hubs [J + 1], and per job where its first classes end in
-// the candidate list [(N_CLASS - 1) J]. Groups and hubs are taken from one flat
-// index each; job_of finds an item's job by binary search.
-__device__ __forceinline__ const ScanList& list_of(const ScatterJob& J) { return J.q; }
-__device__ __forceinline__ const ScanList& list_of(const PruneJob& J) { return J.c; }
-__device__ __forceinline__ const ScanList& list_of(const CpiJob& J) { return J.p; }
-
-constexpr int JOB_SCAN_THREADS = 1024;
-
-// candidates of the list below vertex v (its bitmap and ranks as compacted)
-__device__ __forceinline__ uint32_t list_rank(const DevGraph& g, const ScanList& C, uint32_t v) {
-    if (v >= (uint32_t)g.n) return *C.count;
-    return C.rank[v >> 5] + __popc(C.bm[v >> 5] & ((1u << (v & 31)) - 1u));
-}
-
-template <typename Job>
-__global__ void __launch_bounds__(JOB_SCAN_THREADS) k_job_groups(DevGraph g, const Job* __restrict__ jobs, int njobs,
-                                                                  uint32_t* pre) {
-    using Scan = cub::BlockScan<uint32_t, JOB_SCAN_THREADS>;
-    __shared__ typename Scan::TempStorage tmp;
-    __shared__ uint32_t carry[2];
-    uint32_t* const hpre = pre + njobs + 1;
-    uint32_t* const cls = hpre + njobs + 1;
-    if (threadIdx.x < 2) carry[threadIdx.x] = 0;
-    __syncthreads();
-    for (int b = 0; b < njobs; b += JOB_SCAN_THREADS) {
-        const int j = b + threadIdx.x;
-        uint32_t groups = 0, hubs = 0;
-        if (j < njobs) {
-            const ScanList& C = list_of(jobs[j]);
-            uint32_t begin = hubs = list_rank(g, C, g.class_end[0]);
-            cls[(N_CLASS - 1) * j] = hubs;
-            for (int c = 1; c < N_CLASS; c++) {
-                const uint32_t end = c < N_CLASS - 1 ? list_rank(g, C, g.class_end[c]) : *C.count;
-                if (c < N_CLASS - 1) cls[(N_CLASS - 1) * j + c] = end;
-                groups += (end - begin + class_group(c) - 1) / class_group(c);
-                begin = end;
-            }
-        }
-        uint32_t excl, total, hexcl, htotal;
-        Scan(tmp).ExclusiveSum(groups, excl, total);
-        __syncthreads();
-        Scan(tmp).ExclusiveSum(hubs, hexcl, htotal);
-        if (j < njobs) {
-            pre[j] = carry[0] + excl;
-            hpre[j] = carry[1] + hexcl;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            carry[0] += total;
-            carry[1] += htotal;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        pre[njobs] = carry[0];
-        hpre[njobs] = carry[1];
-    }
-}
-
-// the job whose items [pre[j], pre[j+1]) hold item it (pre[njobs] > it)
-__device__ __forceinline__ int job_of(const uint32_t* pre, int njobs, uint32_t it) {
+// the job that holds item it of the launch (first: items of the earlier jobs);
+// *at: its number within the job
+__device__ __forceinline__ int job_of(const uint32_t* first, int njobs, uint32_t it, uint32_t* at) {
     int lo = 0, hi = njobs;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if (__ldg(pre + mid) <= it) lo = mid;
+        if (__ldg(first + mid) <= it) lo = mid;
         else hi = mid;
     }
+    *at = it - __ldg(first + lo);
     return lo;
 }
 
-// A launch's hubs (item = job, position in its candidate list) and warp groups.
-struct Groups {
-    const uint32_t *pre, *hpre, *cls;
-    int njobs;
-    __device__ __forceinline__ Groups(const ScanWork& w, int n)
-        : pre(w.pre), hpre(w.pre + n + 1), cls(w.pre + 2 * (n + 1)), njobs(n) {}
-    __device__ __forceinline__ uint32_t n_groups() const { return pre[njobs]; }
-    __device__ __forceinline__ uint32_t n_hubs() const { return hpre[njobs]; }
-    __device__ __forceinline__ int hub(uint32_t it, uint32_t* a) const {
-        const int j = job_of(hpre, njobs, it);
-        *a = it - hpre[j];
-        return j;
-    }
-    // job of group it; a: the lane's position in its candidate list (from the
-    // list's end on for a lane without a candidate)
-    __device__ __forceinline__ int group(uint32_t it, uint32_t lane, uint32_t* a) const {
-        const int j = job_of(pre, njobs, it);
-        const uint32_t* const end = cls + (N_CLASS - 1) * j;
-        uint32_t grp = it - pre[j], begin = end[0];
+// The vertices [a, b) of a range's warp item `it` (a = b: none).
+__device__ __forceinline__ void item_range(const ScanRange& R, uint32_t it, const ScanLaunch& l, uint32_t* a,
+                                           uint32_t* b) {
+    const bool flat = R.flat;
 #pragma unroll
-        for (int c = 1; c < N_CLASS - 1; c++) {
-            const uint32_t groups = (end[c] - begin + class_group(c) - 1) / class_group(c);
-            if (grp < groups) {
-                begin += grp * class_group(c) + lane;
-                *a = lane < class_group(c) && begin < end[c] ? begin : 0xffffffffu;
-                return j;
-            }
-            grp -= groups;
-            begin = end[c];
+    for (int c = 0; c < N_CLASS; c++) {
+        if (c == 0 && !flat) continue;
+        const int unit = flat ? FLAT_UNIT : l.unit[c];
+        const uint32_t lo = R.lo[c], hi = R.hi[c], items = scan_items(lo, hi, unit);
+        if (it < items) {
+            const uint64_t from = (uint64_t)((lo >> unit) + it) << unit;
+            *a = max(lo, (uint32_t)from);
+            *b = (uint32_t)min((unsigned long long)hi, (unsigned long long)from + (1ull << unit));
+            return;
         }
-        *a = begin + grp * 32 + lane;
-        return j;
+        it -= items;
     }
-};
+    *a = *b = 0;
+}
+
+// The word at w (lane's) of an item's vertices [a, b), bits outside cleared.
+__device__ __forceinline__ uint32_t item_mask(uint32_t w, uint32_t a, uint32_t b) {
+    uint32_t m = 0xffffffffu;
+    if (w == a >> 5) m &= m << (a & 31);
+    if (w == (b - 1) >> 5) m &= 0xffffffffu >> (31 - ((b - 1) & 31));
+    return m;
+}
+
+// The set bits of the warp's words x (lane j < nw holding word j) as a list of
+// word << 5 | bit in shared memory; returns how many.
+__device__ __forceinline__ uint32_t expand_bits(uint32_t x, uint16_t* list, int lane) {
+    uint32_t n = 0;
+    for (uint32_t some = __ballot_sync(0xffffffffu, x != 0); some; some &= some - 1) {
+        const int j = __ffs(some) - 1;
+        const uint32_t y = __shfl_sync(0xffffffffu, x, j);
+        if ((y >> lane) & 1u) list[n + __popc(y & ((1u << lane) - 1u))] = (uint16_t)(j << 5 | lane);
+        n += __popc(y);
+    }
+    __syncwarp();
+    return n;
+}
 
 // Counting pass: add this thread's scanned candidates and adjacency entries to
 // the run's counters (all lanes of the warp call it; one atomic per warp).
 template <bool COUNT>
-__device__ __forceinline__ void scan_flush(const ScanWork& q, uint64_t cands, uint64_t entries) {
-    if (!COUNT || !q.scan) return;
+__device__ __forceinline__ void scan_flush(ScanCount scan, uint64_t cands, uint64_t entries) {
+    if (!COUNT) return;
     for (int d = 16; d >= 1; d >>= 1) {
         cands += __shfl_xor_sync(0xffffffffu, cands, d);
         entries += __shfl_xor_sync(0xffffffffu, entries, d);
     }
     if ((threadIdx.x & 31) == 0) {
-        if (cands) atomicAdd(&q.scan[0], (unsigned long long)cands);
-        if (entries) atomicAdd(&q.scan[1], (unsigned long long)entries);
+        if (cands) atomicAdd(&scan[0], (unsigned long long)cands);
+        if (entries) atomicAdd(&scan[1], (unsigned long long)entries);
     }
 }
 
@@ -434,20 +366,27 @@ __device__ __forceinline__ void mark(uint32_t* marks, uint32_t x) {
     if (!(__ldca(w) & b)) atomicOr(w, b);
 }
 
+// Shared memory of a warp in the scanning kernels.
+struct ScanShared {
+    int2 slots[WARP_KERNEL_THREADS];
+    uint16_t list[WARP_KERNEL_THREADS / 32][32 * MAX_WORDS];  // an item's candidates
+};
+
 template <bool COUNT>
-__global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_scatter(DevGraph g, const ScatterJob* __restrict__ jobs,
-                                                                 int njobs, ScanWork sw) {
-    __shared__ int2 s_slots[WARP_KERNEL_THREADS];
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS, SCAN_BLOCKS) k_scatter(DevGraph g, const ScatterJob* __restrict__ jobs,
+                                                                 int njobs, ScanLaunch l, ScanCount scan) {
+    __shared__ ScanShared sh;
     const int lane = threadIdx.x & 31;
-    int2* const slots = s_slots + (threadIdx.x & ~31);
-    const Groups G(sw, njobs);
+    int2* const slots = sh.slots + (threadIdx.x & ~31);
+    uint16_t* const list = sh.list[threadIdx.x >> 5];
     uint64_t sc = 0, se = 0;
-    const uint32_t nhubs = G.n_hubs();
-    for (uint32_t it = blockIdx.x; it < nhubs; it += gridDim.x) {
-        uint32_t a;
-        const ScatterJob& J = jobs[G.hub(it, &a)];
+    for (uint32_t it = blockIdx.x; it < l.hubs; it += gridDim.x) {
+        uint32_t at;
+        const ScatterJob& J = jobs[job_of(l.hub_first, njobs, it, &at)];
+        const uint32_t v = J.r.lo[0] + at;
+        if (!((J.r.bm[v >> 5] >> (v & 31)) & 1u)) continue;
         const AdjRef A = adj_ref(g, J.scan_out);
-        const uint32_t v = (uint32_t)J.q.cand[a], e0 = A.off[v], e1 = A.off[v + 1];
+        const uint32_t e0 = A.off[v], e1 = A.off[v + 1];
         if (threadIdx.x == 0) sc += e1 > e0, se += e1 - e0;
         uint32_t* const marks = J.marks;
         scan_block(g, A.adj, e0, e1, J.lab, J.filter,
@@ -458,49 +397,59 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_scatter(DevGraph g, con
                    },
                    [] { return false; });
     }
-    const uint32_t ngroups = G.n_groups();
-    for (uint64_t it = gwarp_id(); it < ngroups; it += nwarps_total()) {
-        uint32_t a;
-        const ScatterJob& J = jobs[G.group((uint32_t)it, lane, &a)];
+    for (uint64_t it = gwarp_id(); it < l.items; it += nwarps_total()) {
+        uint32_t item, va, vb;
+        const ScatterJob& J = jobs[job_of(l.first, njobs, (uint32_t)it, &item)];
+        item_range(J.r, item, l, &va, &vb);
+        const uint32_t w0 = va >> 5, nw = (vb + 31) / 32 - w0;
+        const uint32_t x = lane < (int)nw ? J.r.bm[w0 + lane] & item_mask(w0 + lane, va, vb) : 0u;
+        if (!__any_sync(0xffffffffu, x != 0)) continue;
+        const uint32_t n = expand_bits(x, list, lane);
         const AdjRef A = adj_ref(g, J.scan_out);
-        uint32_t e0 = 0, e1 = 0;
-        if (a < *J.q.count) {
-            const uint32_t v = (uint32_t)J.q.cand[a];
-            e0 = A.off[v];
-            e1 = A.off[v + 1];
-        }
-        sc += e1 > e0;
-        se += e1 - e0;
-        uint32_t total;
-        const uint32_t ex = list_starts(e1 - e0, lane, &total);
         uint32_t* const marks = J.marks;
-        scan_flat(g, A, e0, e1 - e0, ex, total, J.lab, J.filter, slots, lane,
-                  [&](bool hit, uint32_t x, uint32_t, int, uint32_t) {
-                      if (hit) mark(marks, x);
-                  });
+        for (uint32_t i = 0; i < n; i += 32) {
+            uint32_t e0 = 0, e1 = 0;
+            if (i + lane < n) {
+                const uint32_t v = w0 * 32 + list[i + lane];
+                e0 = A.off[v];
+                e1 = A.off[v + 1];
+            }
+            sc += e1 > e0;
+            se += e1 - e0;
+            uint32_t total;
+            const uint32_t ex = list_starts(e1 - e0, lane, &total);
+            scan_flat(g, A, e0, e1 - e0, ex, total, J.lab, J.filter, slots, lane,
+                      [&](bool hit, uint32_t y, uint32_t, int, uint32_t) {
+                          if (hit) mark(marks, y);
+                      });
+        }
+        __syncwarp();  // list is written again
     }
-    scan_flush<COUNT>(sw, sc, se);
+    scan_flush<COUNT>(scan, sc, se);
 }
 
 // A constraint on neighbours of any vertex label hits often: each lane first
 // tries its own list's first quad, and only lists without a hit there are
 // scanned end to end.
 template <bool COUNT>
-__global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_prune(DevGraph g, const PruneJob* __restrict__ jobs, int njobs,
-                                                               ScanWork sw) {
-    __shared__ int2 s_slots[WARP_KERNEL_THREADS];
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS, REFINE_BLOCKS) k_refine(DevGraph g, const RefineJob* __restrict__ jobs, int njobs,
+                                                                ScanLaunch l, ScanCount scan) {
+    __shared__ ScanShared sh;
     __shared__ uint8_t s_hit[WARP_KERNEL_THREADS];
+    __shared__ uint32_t s_keep[WARP_KERNEL_THREADS / 32][MAX_WORDS];
     const int lane = threadIdx.x & 31;
-    int2* const slots = s_slots + (threadIdx.x & ~31);
+    int2* const slots = sh.slots + (threadIdx.x & ~31);
+    uint16_t* const list = sh.list[threadIdx.x >> 5];
     uint8_t* const found = s_hit + (threadIdx.x & ~31);
-    const Groups G(sw, njobs);
+    uint32_t* const kept = s_keep[threadIdx.x >> 5];
     uint64_t sc = 0, se = 0;
-    const uint32_t nhubs = G.n_hubs();
-    for (uint32_t it = blockIdx.x; it < nhubs; it += gridDim.x) {
-        uint32_t a;
-        const PruneJob& J = jobs[G.hub(it, &a)];
-        const uint32_t v = (uint32_t)J.c.cand[a];
-        bool keep = true;
+    for (uint32_t it = blockIdx.x; it < l.hubs; it += gridDim.x) {
+        uint32_t at;
+        const RefineJob& J = jobs[job_of(l.hub_first, njobs, it, &at)];
+        const uint32_t v = J.r.lo[0] + at;
+        uint32_t x = J.r.bm[v >> 5];
+        for (int m = 0; m < J.nmarks; m++) x &= J.marks[m][v >> 5];
+        bool keep = (x >> (v & 31)) & 1u;
         for (int c = 0; c < J.ncon && keep; c++) {  // block-uniform
             const AdjRef A = adj_ref(g, J.con_dir[c]);
             const uint32_t e0 = A.off[v], e1 = A.off[v + 1];
@@ -511,119 +460,164 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_prune(DevGraph g, const
                        [&](int, uint32_t, const uint32_t (&)[4], const uint32_t (&)[4]) { hit = true; },
                        [&] { return keep = __syncthreads_or(hit); });
         }
-        if (!keep && threadIdx.x == 0) atomicAnd(&J.out[v >> 5], ~(1u << (v & 31)));
+        if (keep && threadIdx.x == 0) atomicOr(&J.out[v >> 5], 1u << (v & 31));
     }
-    const uint32_t ngroups = G.n_groups();
-    for (uint64_t it = gwarp_id(); it < ngroups; it += nwarps_total()) {
-        uint32_t a;
-        const PruneJob& J = jobs[G.group((uint32_t)it, lane, &a)];
-        const int ncon = J.ncon;
-        const bool valid = a < *J.c.count;
-        const uint32_t v = valid ? (uint32_t)J.c.cand[a] : 0u;
-        bool keep = valid;
-        for (int c = 0; c < ncon; c++) {
-            const AdjRef A = adj_ref(g, J.con_dir[c]);
-            const int32_t lab = J.con_lab[c];
-            const uint32_t* bm = J.con_bm[c];
-            uint32_t e0 = 0, e1 = 0;
-            if (keep) {
-                e0 = A.off[v];
-                e1 = A.off[v + 1];
-            }
-            sc += keep;
-            bool hit = false;
-            if (J.con_any[c] && e0 < e1) {
-                const uint32_t b = e0 & ~3u;
-                uint32_t x[4], w[4];
-                hit = quad_hits(g, A.adj, b, quad_mask(b, e0, e1), lab, bm, x, w) != 0;
-                if (COUNT) se += min(4u - (e0 - b), e1 - e0);
-                e0 = hit || e1 - b <= 4u ? e1 : b + 4;
-            }
-            se += e1 - e0;
-            found[lane] = hit;
-            uint32_t total;
-            const uint32_t ex = list_starts(e1 - e0, lane, &total);
-            scan_flat(g, A, e0, e1 - e0, ex, total, lab, bm, slots, lane,
-                      [&](bool h, uint32_t, uint32_t, int owner, uint32_t) {
-                          if (h) found[owner] = 1;
-                      });
-            keep = keep && found[lane];
+    for (uint64_t it = gwarp_id(); it < l.items; it += nwarps_total()) {
+        uint32_t item, va, vb;
+        const RefineJob& J = jobs[job_of(l.first, njobs, (uint32_t)it, &item)];
+        item_range(J.r, item, l, &va, &vb);
+        const uint32_t w0 = va >> 5, nw = (vb + 31) / 32 - w0;
+        uint32_t x = 0;
+        if (lane < (int)nw) {
+            x = J.r.bm[w0 + lane] & item_mask(w0 + lane, va, vb);
+            for (int m = 0; m < J.nmarks; m++) x &= J.marks[m][w0 + lane];
         }
-        if (valid && !keep) atomicAnd(&J.out[v >> 5], ~(1u << (v & 31)));
+        const int ncon = J.ncon;
+        if (ncon == 0) {  // a flat range
+            if (x) atomicOr(&J.out[w0 + lane], x);
+            continue;
+        }
+        if (!__any_sync(0xffffffffu, x != 0)) continue;
+        kept[lane] = 0;
+        const uint32_t n = expand_bits(x, list, lane);
+        for (uint32_t i = 0; i < n; i += 32) {
+            const bool valid = i + lane < n;
+            const uint32_t at = valid ? list[i + lane] : 0u, v = w0 * 32 + at;
+            bool keep = valid;
+            for (int c = 0; c < ncon; c++) {
+                const AdjRef A = adj_ref(g, J.con_dir[c]);
+                const int32_t lab = J.con_lab[c];
+                const uint32_t* bm = J.con_bm[c];
+                uint32_t e0 = 0, e1 = 0;
+                if (keep) {
+                    e0 = A.off[v];
+                    e1 = A.off[v + 1];
+                }
+                sc += keep;
+                bool hit = false;
+                if (J.con_any[c] && e0 < e1) {
+                    const uint32_t b = e0 & ~3u;
+                    uint32_t y[4], w[4];
+                    hit = quad_hits(g, A.adj, b, quad_mask(b, e0, e1), lab, bm, y, w) != 0;
+                    if (COUNT) se += min(4u - (e0 - b), e1 - e0);
+                    e0 = hit || e1 - b <= 4u ? e1 : b + 4;
+                }
+                se += e1 - e0;
+                found[lane] = hit;
+                uint32_t total;
+                const uint32_t ex = list_starts(e1 - e0, lane, &total);
+                scan_flat(g, A, e0, e1 - e0, ex, total, lab, bm, slots, lane,
+                          [&](bool h, uint32_t, uint32_t, int owner, uint32_t) {
+                              if (h) found[owner] = 1;
+                          });
+                keep = keep && found[lane];
+            }
+            if (keep) atomicOr(&kept[at >> 5], 1u << (at & 31));
+        }
+        __syncwarp();
+        if (lane < (int)nw && kept[lane]) atomicOr(&J.out[w0 + lane], kept[lane]);
+        __syncwarp();  // list and kept are written again
     }
-    scan_flush<COUNT>(sw, sc, se);
+    scan_flush<COUNT>(scan, sc, se);
+}
+
+// Position in the parent's candidate list of the first candidate at or after
+// vertex a.
+__device__ __forceinline__ uint32_t parent_rank(const CpiJob& J, uint32_t a) {
+    return J.prank[a >> 5] + __popc(J.r.bm[a >> 5] & ((1u << (a & 31)) - 1u));
 }
 
 // off[a] = number of children of parent candidate a
 template <bool COUNT>
-__global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_cpi_count(DevGraph g, const CpiJob* __restrict__ jobs,
-                                                                   int njobs, ScanWork sw) {
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS, SCAN_BLOCKS) k_cpi_count(DevGraph g, const CpiJob* __restrict__ jobs,
+                                                                   int njobs, ScanLaunch l, ScanCount scan) {
     using Reduce = cub::BlockReduce<uint32_t, WARP_KERNEL_THREADS>;
     __shared__ typename Reduce::TempStorage tmp;
-    __shared__ int2 s_slots[WARP_KERNEL_THREADS];
+    __shared__ ScanShared sh;
     const int lane = threadIdx.x & 31;
-    int2* const slots = s_slots + (threadIdx.x & ~31);
-    const Groups G(sw, njobs);
+    int2* const slots = sh.slots + (threadIdx.x & ~31);
+    uint16_t* const list = sh.list[threadIdx.x >> 5];
     uint64_t sc = 0, se = 0;
-    const uint32_t nhubs = G.n_hubs();
-    for (uint32_t it = blockIdx.x; it < nhubs; it += gridDim.x) {
-        uint32_t a;
-        const CpiJob& J = jobs[G.hub(it, &a)];
+    for (uint32_t it = blockIdx.x; it < l.hubs; it += gridDim.x) {
+        uint32_t at;
+        const CpiJob& J = jobs[job_of(l.hub_first, njobs, it, &at)];
+        const uint32_t v = J.r.lo[0] + at;
+        if (!((J.r.bm[v >> 5] >> (v & 31)) & 1u)) continue;
         const AdjRef A = adj_ref(g, J.out);
-        const uint32_t v = (uint32_t)J.p.cand[a], e0 = A.off[v], e1 = A.off[v + 1];
+        const uint32_t e0 = A.off[v], e1 = A.off[v + 1];
         if (threadIdx.x == 0) sc += e1 > e0, se += e1 - e0;
         uint32_t cnt = 0;
         scan_block(g, A.adj, e0, e1, J.lab, J.cbm,
                    [&](int, uint32_t h, const uint32_t (&)[4], const uint32_t (&)[4]) { cnt += __popc(h); },
                    [] { return false; });
         const uint32_t total = Reduce(tmp).Sum(cnt);
-        if (threadIdx.x == 0) J.off[a] = total;
+        if (threadIdx.x == 0) J.off[parent_rank(J, v)] = total;
         __syncthreads();  // tmp is reused by the next hub
     }
-    const uint32_t ngroups = G.n_groups();
-    for (uint64_t it = gwarp_id(); it < ngroups; it += nwarps_total()) {
-        uint32_t a;
-        const CpiJob& J = jobs[G.group((uint32_t)it, lane, &a)];
+    for (uint64_t it = gwarp_id(); it < l.items; it += nwarps_total()) {
+        uint32_t item, va, vb;
+        const CpiJob& J = jobs[job_of(l.first, njobs, (uint32_t)it, &item)];
+        item_range(J.r, item, l, &va, &vb);
+        const uint32_t w0 = va >> 5, nw = (vb + 31) / 32 - w0;
+        const uint32_t x = lane < (int)nw ? J.r.bm[w0 + lane] & item_mask(w0 + lane, va, vb) : 0u;
+        if (!__any_sync(0xffffffffu, x != 0)) continue;
+        const uint32_t n = expand_bits(x, list, lane);
         const AdjRef A = adj_ref(g, J.out);
-        const bool valid = a < *J.p.count;
-        uint32_t e0 = 0, e1 = 0;
-        if (valid) {
-            const uint32_t v = (uint32_t)J.p.cand[a];
-            e0 = A.off[v];
-            e1 = A.off[v + 1];
+        uint32_t* const off = J.off + parent_rank(J, va);
+        for (uint32_t i = 0; i < n; i += 32) {
+            const bool valid = i + lane < n;
+            uint32_t e0 = 0, e1 = 0;
+            if (valid) {
+                const uint32_t v = w0 * 32 + list[i + lane];
+                e0 = A.off[v];
+                e1 = A.off[v + 1];
+            }
+            sc += e1 > e0;
+            se += e1 - e0;
+            uint32_t total, cnt = 0;
+            const uint32_t len = e1 - e0, ex = list_starts(len, lane, &total);
+            scan_flat(g, A, e0, len, ex, total, J.lab, J.cbm, slots, lane,
+                      [&](bool hit, uint32_t, uint32_t, int, uint32_t window) {
+                          const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+                          // the window's entries of this lane's list: [ex, ex + len)
+                          if (hits && len && window + 32u > ex && window < ex + len) {
+                              const uint32_t lo = ex > window ? ex - window : 0u;
+                              const uint32_t hi = min(ex + len - window, 32u);
+                              cnt += __popc((hits >> lo) << (32u - hi + lo));
+                          }
+                      });
+            if (valid) off[i + lane] = cnt;
         }
-        sc += e1 > e0;
-        se += e1 - e0;
-        uint32_t total, cnt = 0;
-        const uint32_t len = e1 - e0, ex = list_starts(len, lane, &total);
-        scan_flat(g, A, e0, len, ex, total, J.lab, J.cbm, slots, lane,
-                  [&](bool hit, uint32_t, uint32_t, int, uint32_t window) {
-                      const uint32_t hits = __ballot_sync(0xffffffffu, hit);
-                      // the window's entries of this lane's list: [ex, ex + len)
-                      if (hits && len && window + 32u > ex && window < ex + len) {
-                          const uint32_t lo = ex > window ? ex - window : 0u;
-                          const uint32_t hi = min(ex + len - window, 32u);
-                          cnt += __popc((hits >> lo) << (32u - hi + lo));
-                      }
-                  });
-        if (valid) J.off[a] = cnt;
+        __syncwarp();  // list is written again
     }
-    scan_flush<COUNT>(sw, sc, se);
+    scan_flush<COUNT>(scan, sc, se);
 }
 
 // Exclusive scan of the per-candidate counts off[0..n) in place, off[n] =
-// total, in two passes over (job, chunk) items like the compaction above.
+// total, in two passes over the jobs' chunks of CPI_CHUNK counts (as many as the
+// parent's label has vertices for) like the compaction above.
+__device__ __forceinline__ const CpiJob& chunk_job(const CpiJob* jobs, int njobs, uint32_t it, uint32_t* c) {
+    int lo = 0, hi = njobs;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (jobs[mid].chunk0 <= it) lo = mid;
+        else hi = mid;
+    }
+    *c = it - jobs[lo].chunk0;
+    return jobs[lo];
+}
+
 __global__ void __launch_bounds__(COMPACT_THREADS) k_cpi_sums(const CpiJob* __restrict__ jobs, int njobs,
-                                                              uint32_t nchunks) {
+                                                              uint32_t chunks) {
     using Reduce = cub::BlockReduce<uint64_t, COMPACT_THREADS>;
     __shared__ typename Reduce::TempStorage tmp;
-    for (uint64_t it = blockIdx.x; it < (uint64_t)njobs * nchunks; it += gridDim.x) {
-        const CpiJob& J = jobs[it / nchunks];
-        const uint32_t c = (uint32_t)(it % nchunks);
-        const uint32_t n = *J.p.count;
-        if ((uint64_t)c * COMPACT_WORDS >= n && c > 0) continue;
+    for (uint32_t it = blockIdx.x; it < chunks; it += gridDim.x) {
+        uint32_t c;
+        const CpiJob& J = chunk_job(jobs, njobs, it, &c);
+        const uint32_t n = *J.pcount;
+        if ((uint64_t)c * CPI_CHUNK >= n && c > 0) continue;
         uint64_t cnt = 0;
-        for (uint32_t a = c * COMPACT_WORDS + threadIdx.x; a < min(n, (c + 1) * COMPACT_WORDS); a += COMPACT_THREADS)
+        for (uint32_t a = c * CPI_CHUNK + threadIdx.x; a < min(n, (c + 1) * CPI_CHUNK); a += COMPACT_THREADS)
             cnt += J.off[a];
         cnt = Reduce(tmp).Sum(cnt);
         if (threadIdx.x == 0) J.csum[c] = cnt;
@@ -632,7 +626,7 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_cpi_sums(const CpiJob* __re
 }
 
 __global__ void __launch_bounds__(COMPACT_THREADS) k_cpi_scan(const CpiJob* __restrict__ jobs, int njobs,
-                                                              uint32_t nchunks, int32_t* err) {
+                                                              uint32_t chunks, int32_t* err) {
     using Scan = cub::BlockScan<uint64_t, COMPACT_THREADS>;
     using Reduce = cub::BlockReduce<uint64_t, COMPACT_THREADS>;
     __shared__ union {
@@ -640,19 +634,19 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_cpi_scan(const CpiJob* __re
         typename Reduce::TempStorage reduce;
     } tmp;
     __shared__ uint64_t base_s;
-    constexpr int EPT = COMPACT_WORDS / COMPACT_THREADS;
-    for (uint64_t it = blockIdx.x; it < (uint64_t)njobs * nchunks; it += gridDim.x) {
-        const CpiJob& J = jobs[it / nchunks];
-        const uint32_t c = (uint32_t)(it % nchunks);
-        const uint32_t n = *J.p.count;
-        const uint32_t last = n / COMPACT_WORDS;  // chunk holding off[n]
+    constexpr int EPT = CPI_CHUNK / COMPACT_THREADS;
+    for (uint32_t it = blockIdx.x; it < chunks; it += gridDim.x) {
+        uint32_t c;
+        const CpiJob& J = chunk_job(jobs, njobs, it, &c);
+        const uint32_t n = *J.pcount;
+        const uint32_t last = n / CPI_CHUNK;  // chunk holding off[n]
         if (c > last) continue;
         uint64_t before = 0;
         for (uint32_t q = threadIdx.x; q < c; q += COMPACT_THREADS) before += J.csum[q];
         before = Reduce(tmp.reduce).Sum(before);
         if (threadIdx.x == 0) base_s = before;
         __syncthreads();
-        const uint32_t a0 = c * COMPACT_WORDS + threadIdx.x * EPT;
+        const uint32_t a0 = c * CPI_CHUNK + threadIdx.x * EPT;
         uint32_t vals[EPT];
         uint64_t cnt = 0;
         for (int q = 0; q < EPT; q++) {
@@ -675,34 +669,36 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_cpi_scan(const CpiJob* __re
                 tot = 0;  // leave an empty index
             }
             J.off[n] = (uint32_t)tot;
-            if (J.nnz_stat) atomicAdd((unsigned long long*)J.nnz_stat, (unsigned long long)tot);
+            *J.total = (uint32_t)tot;
         }
         __syncthreads();
     }
 }
 
-// Index edges of a group's parents are contiguous and in scan order, so the
+// Index edges of an item's parents are contiguous and in scan order, so the
 // warp only counts hits. A hub's edges are put in order by a block scan of the
 // threads' hits (HUB_QUADS quads in a row each) per round.
 template <bool COUNT>
-__global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_cpi_fill(DevGraph g, const CpiJob* __restrict__ jobs, int njobs,
-                                                                  ScanWork sw) {
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS, SCAN_BLOCKS) k_cpi_fill(DevGraph g, const CpiJob* __restrict__ jobs, int njobs,
+                                                                  ScanLaunch l, ScanCount scan) {
     using Scan = cub::BlockScan<uint32_t, WARP_KERNEL_THREADS>;
     __shared__ typename Scan::TempStorage tmp;
-    __shared__ int2 s_slots[WARP_KERNEL_THREADS];
+    __shared__ ScanShared sh;
     const int lane = threadIdx.x & 31;
-    int2* const slots = s_slots + (threadIdx.x & ~31);
-    const Groups G(sw, njobs);
+    int2* const slots = sh.slots + (threadIdx.x & ~31);
+    uint16_t* const list = sh.list[threadIdx.x >> 5];
     uint64_t sc = 0, se = 0;
-    const uint32_t nhubs = G.n_hubs();
-    for (uint32_t it = blockIdx.x; it < nhubs; it += gridDim.x) {
-        uint32_t a;
-        const CpiJob& J = jobs[G.hub(it, &a)];
-        const AdjRef A = adj_ref(g, J.out);
-        const uint32_t v = (uint32_t)J.p.cand[a], e0 = A.off[v], e1 = A.off[v + 1];
+    for (uint32_t it = blockIdx.x; it < l.hubs; it += gridDim.x) {
+        uint32_t at;
+        const CpiJob& J = jobs[job_of(l.hub_first, njobs, it, &at)];
+        const uint32_t v = J.r.lo[0] + at;
+        if (!((J.r.bm[v >> 5] >> (v & 31)) & 1u)) continue;
+        const uint32_t a = parent_rank(J, v);
         uint32_t next = J.off[a];
         const uint32_t end = J.off[a + 1];
         if (next == end) continue;  // no index edges
+        const AdjRef A = adj_ref(g, J.out);
+        const uint32_t e0 = A.off[v], e1 = A.off[v + 1];
         if (threadIdx.x == 0) sc += 1, se += e1 - e0;
         uint32_t hq[HUB_QUADS] = {}, xq[HUB_QUADS][4];
         scan_block(g, A.adj, e0, e1, J.lab, J.cbm,
@@ -740,47 +736,49 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS) k_cpi_fill(DevGraph g, co
                        return next >= end;
                    });
     }
-    const uint32_t ngroups = G.n_groups();
-    for (uint64_t it = gwarp_id(); it < ngroups; it += nwarps_total()) {
-        uint32_t a;
-        const CpiJob& J = jobs[G.group((uint32_t)it, lane, &a)];
+    for (uint64_t it = gwarp_id(); it < l.items; it += nwarps_total()) {
+        uint32_t item, va, vb;
+        const CpiJob& J = jobs[job_of(l.first, njobs, (uint32_t)it, &item)];
+        item_range(J.r, item, l, &va, &vb);
+        const uint32_t w0 = va >> 5, nw = (vb + 31) / 32 - w0;
+        const uint32_t x = lane < (int)nw ? J.r.bm[w0 + lane] & item_mask(w0 + lane, va, vb) : 0u;
+        if (!__any_sync(0xffffffffu, x != 0)) continue;
+        const uint32_t n = expand_bits(x, list, lane);
         const AdjRef A = adj_ref(g, J.out);
-        uint32_t e0 = 0, e1 = 0, o = 0;
-        if (a < *J.p.count) {
-            o = J.off[a];
-            if (J.off[a + 1] > o) {  // a parent without index edges skips its list
-                const uint32_t v = (uint32_t)J.p.cand[a];
-                e0 = A.off[v];
-                e1 = A.off[v + 1];
-            }
-        }
-        sc += e1 > e0;
-        se += e1 - e0;
-        uint32_t total;
-        const uint32_t ex = list_starts(e1 - e0, lane, &total);
-        uint32_t next = __shfl_sync(0xffffffffu, o, 0);
+        const uint32_t* const off = J.off + parent_rank(J, va);
         int2* const idx = J.idx;
         const uint32_t* const crank = J.crank;
         const uint64_t cap = J.cap;
-        scan_flat(g, A, e0, e1 - e0, ex, total, J.lab, J.cbm, slots, lane,
-                  [&](bool hit, uint32_t x, uint32_t w, int, uint32_t) {
-                      const uint32_t hits = __ballot_sync(0xffffffffu, hit);
-                      if (hit) {
-                          const uint32_t slot = next + __popc(hits & ((1u << lane) - 1u));
-                          if (slot < cap)
-                              idx[slot] = make_int2((int32_t)(__ldg(crank + (x >> 5)) +
-                                                              __popc(w & ((1u << (x & 31)) - 1))), (int32_t)x);
-                      }
-                      next += __popc(hits);
-                  });
+        for (uint32_t i = 0; i < n; i += 32) {
+            uint32_t e0 = 0, e1 = 0, o = 0;
+            if (i + lane < n) {
+                o = off[i + lane];
+                if (off[i + lane + 1] > o) {  // a parent without index edges skips its list
+                    const uint32_t v = w0 * 32 + list[i + lane];
+                    e0 = A.off[v];
+                    e1 = A.off[v + 1];
+                }
+            }
+            sc += e1 > e0;
+            se += e1 - e0;
+            uint32_t total;
+            const uint32_t ex = list_starts(e1 - e0, lane, &total);
+            uint32_t next = __shfl_sync(0xffffffffu, o, 0);
+            scan_flat(g, A, e0, e1 - e0, ex, total, J.lab, J.cbm, slots, lane,
+                      [&](bool hit, uint32_t y, uint32_t w, int, uint32_t) {
+                          const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+                          if (hit) {
+                              const uint32_t slot = next + __popc(hits & ((1u << lane) - 1u));
+                              if (slot < cap)
+                                  idx[slot] = make_int2((int32_t)(__ldg(crank + (y >> 5)) +
+                                                                  __popc(w & ((1u << (y & 31)) - 1))), (int32_t)y);
+                          }
+                          next += __popc(hits);
+                      });
+        }
+        __syncwarp();  // list is written again
     }
-    scan_flush<COUNT>(sw, sc, se);
-}
-
-// number of index edges of each job (read back to size the index exactly)
-__global__ void k_cpi_totals(const CpiJob* __restrict__ jobs, int njobs, uint32_t* totals) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < njobs) totals[j] = jobs[j].off[*jobs[j].p.count];
+    scan_flush<COUNT>(scan, sc, se);
 }
 
 // Blocks of a grid-stride kernel: as many as the device holds at once. A
@@ -839,14 +837,6 @@ int launch_filter(const DevGraph& g, const FilterKey* d_keys, int nkeys, uint32_
     return GFD_OK;
 }
 
-int launch_and(const DevGraph& g, const AndJob* d_jobs, int njobs, cudaStream_t st) {
-    if (njobs <= 0 || g.nwords == 0) return GFD_OK;
-    const uint32_t nch = (g.nwords + AND_WORDS - 1) / AND_WORDS;
-    const int grid = (int)std::min<uint64_t>((uint64_t)njobs * nch, (uint64_t)device_sms() * 16);
-    k_and<<<grid, AND_THREADS, 0, st>>>(g, d_jobs, njobs, nch);
-    return check_launch("k_and");
-}
-
 uint32_t compact_chunks(const DevGraph& g) {
     return std::max<uint32_t>(1, (g.nwords + COMPACT_WORDS - 1) / COMPACT_WORDS);
 }
@@ -860,52 +850,67 @@ int launch_compact(const DevGraph& g, const CompactJob* d_jobs, int njobs, cudaS
     return check_launch("k_compact");
 }
 
-// the work of a launch over njobs jobs, then the kernel, one resident wave
+uint32_t cpi_chunks(uint64_t max_parent_candidates) { return (uint32_t)(max_parent_candidates / CPI_CHUNK + 1); }
+
+// A large launch takes larger units, so that its warps' lanes fill up although the
+// bitmaps are sparse and an item's fixed cost (finding its job, its words) is
+// spread; a small one smaller units, so that its few candidates reach all SMs and
+// no warp gets more than 2048 entries. In between, the last class's unit leaves
+// every resident warp about four items, up to 2^most vertices: 8 for refinement,
+// whose bitmaps are dense at first (batch of 256 GFDs on 4M vertices: 55 / 48 / 44 /
+// 38 / 38.5 ms at 5 .. 9, with units of 4 to 8 vertices in class 1 and 32 to 64 in
+// class 2 from 8 on; 45 ms with 32 in class 1, whose warps then get 64k entries),
+// 10 for the index edges, whose parents are sparse (23.9 / 21.9 / 21.7 ms at 8 ..
+// 10; 43.6 ms with units of 128 vertices in the last class and 8 in class 2).
+void scan_units(uint64_t vertices, int most, int8_t* unit) {
+    const uint64_t per_warp = vertices / ((uint64_t)device_sms() * 48 * 4);
+    int u = 5;
+    while (u < most && (2ull << u) <= per_warp) u++;
+    unit[0] = 0;
+    unit[1] = u >= 8 ? 2 : 0;
+    unit[2] = u >= 8 ? 6 : 3;
+    unit[3] = (int8_t)u;
+}
+
+namespace {
+
+// At most one resident wave, at least a warp per item and a block per hub.
 template <typename Job>
-static void job_groups(const DevGraph& g, const Job* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st) {
-    k_job_groups<Job><<<1, JOB_SCAN_THREADS, 0, st>>>(g, d_jobs, njobs, sw.pre);
+int launch_scan(void (*kernel)(DevGraph, const Job*, int, ScanLaunch, ScanCount), const DevGraph& g, const Job* d_jobs,
+                int njobs, const ScanLaunch& l, ScanCount scan, cudaStream_t st, const char* what) {
+    const uint64_t want = std::max<uint64_t>(((uint64_t)l.items + WARP_KERNEL_THREADS / 32 - 1) / (WARP_KERNEL_THREADS / 32), l.hubs);
+    if (njobs <= 0 || want == 0) return GFD_OK;
+    const int grid = (int)std::min<uint64_t>(want, (uint64_t)grid_of(kernel, WARP_KERNEL_THREADS));
+    kernel<<<grid, WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, l, scan);
+    return check_launch(what);
 }
 
-#define GFD_SCAN_LAUNCH(kernel)                                                                                   \
-    do {                                                                                                          \
-        job_groups(g, d_jobs, njobs, sw, st);                                                                     \
-        if (sw.scan)                                                                                              \
-            kernel<true><<<grid_of(kernel<true>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, sw); \
-        else                                                                                                      \
-            kernel<false><<<grid_of(kernel<false>, WARP_KERNEL_THREADS), WARP_KERNEL_THREADS, 0, st>>>(g, d_jobs, njobs, sw); \
-    } while (0)
+}  // namespace
 
-int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st) {
+int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const ScanLaunch& l, ScanCount scan,
+                   cudaStream_t st) {
+    return launch_scan(scan ? k_scatter<true> : k_scatter<false>, g, d_jobs, njobs, l, scan, st, "k_scatter");
+}
+
+int launch_refine(const DevGraph& g, const RefineJob* d_jobs, int njobs, const ScanLaunch& l, ScanCount scan,
+                  cudaStream_t st) {
+    return launch_scan(scan ? k_refine<true> : k_refine<false>, g, d_jobs, njobs, l, scan, st, "k_refine");
+}
+
+int launch_cpi_count(const DevGraph& g, const CpiJob* d_jobs, int njobs, const ScanLaunch& l, uint32_t chunks,
+                     int32_t* d_err, ScanCount scan, cudaStream_t st) {
     if (njobs <= 0) return GFD_OK;
-    GFD_SCAN_LAUNCH(k_scatter);
-    return check_launch("k_scatter");
+    if (int rc = launch_scan(scan ? k_cpi_count<true> : k_cpi_count<false>, g, d_jobs, njobs, l, scan, st, "k_cpi_count"))
+        return rc;
+    const int grid = (int)std::min<uint64_t>(chunks, (uint64_t)device_sms() * 8);
+    k_cpi_sums<<<grid, COMPACT_THREADS, 0, st>>>(d_jobs, njobs, chunks);
+    k_cpi_scan<<<grid, COMPACT_THREADS, 0, st>>>(d_jobs, njobs, chunks, d_err);
+    return check_launch("k_cpi_scan");
 }
 
-int launch_prune(const DevGraph& g, const PruneJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st) {
-    if (njobs <= 0) return GFD_OK;
-    GFD_SCAN_LAUNCH(k_prune);
-    return check_launch("k_prune");
-}
-
-uint32_t cpi_chunks(uint64_t max_parent_candidates) {
-    return (uint32_t)(max_parent_candidates / COMPACT_WORDS + 1);
-}
-
-int launch_cpi_count(const DevGraph& g, const CpiJob* d_jobs, int njobs, uint32_t nchunks, int32_t* d_err,
-                     uint32_t* d_totals, const ScanWork& sw, cudaStream_t st) {
-    if (njobs <= 0) return GFD_OK;
-    GFD_SCAN_LAUNCH(k_cpi_count);
-    const int grid = (int)std::min<uint64_t>((uint64_t)njobs * nchunks, (uint64_t)device_sms() * 8);
-    k_cpi_sums<<<grid, COMPACT_THREADS, 0, st>>>(d_jobs, njobs, nchunks);
-    k_cpi_scan<<<grid, COMPACT_THREADS, 0, st>>>(d_jobs, njobs, nchunks, d_err);
-    k_cpi_totals<<<(njobs + 255) / 256, 256, 0, st>>>(d_jobs, njobs, d_totals);
-    return check_launch("k_cpi_count");
-}
-
-int launch_cpi_fill(const DevGraph& g, const CpiJob* d_jobs, int njobs, const ScanWork& sw, cudaStream_t st) {
-    if (njobs <= 0) return GFD_OK;
-    GFD_SCAN_LAUNCH(k_cpi_fill);
-    return check_launch("k_cpi_fill");
+int launch_cpi_fill(const DevGraph& g, const CpiJob* d_jobs, int njobs, const ScanLaunch& l, ScanCount scan,
+                    cudaStream_t st) {
+    return launch_scan(scan ? k_cpi_fill<true> : k_cpi_fill<false>, g, d_jobs, njobs, l, scan, st, "k_cpi_fill");
 }
 
 }  // namespace gfd

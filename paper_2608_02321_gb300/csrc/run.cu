@@ -27,9 +27,8 @@
 #include <cstdlib>
 #include <cstring>
 #include <deque>
-#include <map>
 #include <memory>
-#include <tuple>
+#include <unordered_map>
 #include <vector>
 
 #include "engine.h"
@@ -202,9 +201,40 @@ EnumArgs enum_args(const gfd_graph* g, const Tables& T) {
 
 // ------------------------------------------------------------------ groups
 struct Phase {
-    int kind;  // 0 and, 1 compact, 2 scatter, 3 prune, 4 clear marks
+    int kind;  // 0 scatter, 1 refine
     size_t first, count;
+    ScanLaunch launch;
 };
+
+// The refinement of a group, planned before any pointer is known. Bitmaps are
+// written once and known by number: [0, keys) the candidate filters', then the
+// refinements' results. A result is determined by its source, its constraints and
+// the bitmaps they look at, so GFDs of the group that refine the same candidates
+// in the same way (and nodes of one GFD that look alike) share it, and everything
+// built from it: rank, candidate list and index edges.
+struct ConSpec {
+    int bm;       // neighbours wanted in this bitmap
+    int dir;      // 1: out-neighbours
+    int lab;
+    bool gather;  // looked up from the candidates; else marked from bm's vertices
+};
+struct RefineSpec {
+    int src, dst;
+    std::vector<ConSpec> cons;
+};
+struct IndexSpec {
+    int parent, child;  // final bitmaps (Group::finals)
+    int dir, lab;
+    uint64_t bound;     // most index edges there can be
+};
+struct VecHash {
+    size_t operator()(const std::vector<int32_t>& v) const {
+        uint64_t h = 1469598103934665603ull;
+        for (int32_t x : v) h = (h ^ (uint32_t)x) * 1099511628211ull;
+        return (size_t)(h ^ (h >> 32));
+    }
+};
+using VecMap = std::unordered_map<std::vector<int32_t>, int, VecHash>;
 
 }  // namespace
 
@@ -213,33 +243,52 @@ struct Group {
     std::vector<int> slot;
     std::vector<HostPlan> plans;
     std::vector<SlotDesc> descs;
-    std::vector<std::array<int, MAXK>> slot_key;
     std::vector<FilterKey> keys;
+    std::vector<int> bm_key;                 // the filter key (so the label) of each bitmap
+    std::vector<RefineSpec> refines;         // in launch order
+    std::vector<size_t> phase_end;           // refines of each phase end here
+    size_t n_marks = 0;
+    std::vector<int> finals;                 // bitmaps that are some level's candidates
+    std::vector<char> final_list;            // a candidate list is wanted
+    std::vector<std::array<int, MAXK>> level_final, level_index;  // per (GFD, level)
+    std::vector<IndexSpec> index;
     uint8_t* base = nullptr;
     size_t bytes = 0;
     struct Off {
-        size_t bm[MAXK], rank[MAXK], cand[MAXK], cpi_off[MAXK], cpi_idx[MAXK], rows[MAXK], wpre[MAXK];
+        size_t rows[MAXK], wpre[MAXK];
     };
     std::vector<Off> offs;
-    size_t o_keybm = 0, o_keys = 0, o_tmp = 0, o_cmp_sums = 0, o_cpi_sums = 0, o_cpi_tot = 0;
-    size_t o_work = 0;  // shares of the adjacency scans' jobs
-    uint8_t* cpi_base = nullptr;  // index edges, sized after counting
+    std::vector<size_t> o_rank, o_cand;      // per final
+    std::vector<size_t> o_off, o_idx;        // per index (o_idx only when in the workspace)
+    size_t o_keybm = 0, o_zero = 0, o_zero_end = 0, o_counts = 0, o_bm = 0, o_marks = 0;
+    size_t o_cmp_sums = 0, o_cpi_sums = 0, o_cpi_tot = 0;
+    bool idx_inside = false;      // index edges in the workspace, at their bound
+    uint8_t* cpi_base = nullptr;  // else: allocated exactly after counting
     size_t cpi_bytes = 0;
     size_t cpi_bound = 0;  // upper bound of cpi_bytes known at planning time
-    size_t o_jobs = 0, o_and = 0, o_cmp = 0, o_sct = 0, o_prn = 0, o_cpi = 0, jobs_end = 0;
-    uint32_t cmp_chunks = 1, cpi_nch = 1;
-    size_t td_need = 0;
-    std::vector<AndJob> and_jobs;
+    size_t o_jobs = 0, o_keys = 0, o_first = 0, o_cmp = 0, o_sct = 0, o_ref = 0, o_cpi = 0, jobs_end = 0;
+    uint32_t cmp_chunks = 1, cpi_nch = 0;
     std::vector<CompactJob> compact_jobs;
     std::vector<ScatterJob> scatter_jobs;
-    std::vector<PruneJob> prune_jobs;
+    std::vector<RefineJob> refine_jobs;
     std::vector<CpiJob> cpi_jobs;
+    std::vector<uint32_t> first;  // ScanLaunch::first and hub_first of all launches
     std::vector<Phase> phases;
+    ScanLaunch cpi_launch;
     std::vector<SlotState> state_img;  // host image of the cleared states (kept until copied)
     int live = 0;  // slots of this group still running (sessions)
 };
 
 namespace {
+
+// Index edges up to this many bytes (their bound, from degree sums) are part of
+// the workspace: no read-back of the counts, no second allocation. Beyond, the
+// counts are read back (one synchronisation) and exactly as much is allocated.
+constexpr size_t IDX_INSIDE = (size_t)1 << 30;
+
+// Largest units (log2 of vertices) of the adjacency scans, see scan_units.
+constexpr int REFINE_UNIT = 8;
+constexpr int INDEX_UNIT = 10;
 
 // Top-down constraint "x in C(i) needs a neighbour in C(q) through an edge
 // leaving x (dir 1) or entering x (dir 0)": scattering from C(q) scans the
@@ -266,37 +315,102 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
         if (int rc = make_plan(phis[s], g->n_attrs, g->plan_stats(), &G->plans[s],
                                !(o && (o->flags & GFD_FLAG_NON_INDUCED)), o && (o->flags & GFD_FLAG_PUSH_X)))
             return rc;
-    std::map<std::vector<int64_t>, int> key_id;
-    G->slot_key.resize(n);
+    VecMap key_id;
+    std::vector<std::array<int, MAXK>> cur(n);  // per (GFD, level): the bitmap that holds its candidates so far
     for (int s = 0; s < n; s++)
         for (int i = 0; i < G->plans[s].k; i++) {
             const FilterKey& K = G->plans[s].key[i];
-            std::vector<int64_t> t = {K.label, K.dout_min, K.din_min, K.self_exp, K.n_attr};
+            std::vector<int32_t> t = {K.label, (int32_t)K.dout_min, (int32_t)K.din_min, K.self_exp, K.n_attr};
             for (int a = 0; a < K.n_attr; a++) {
                 t.push_back(K.attr_a[a]);
                 t.push_back(K.attr_c[a]);
             }
-            auto it = key_id.find(t);
-            if (it == key_id.end()) {
-                it = key_id.emplace(t, (int)G->keys.size()).first;
+            const auto it = key_id.emplace(std::move(t), (int)G->keys.size());
+            if (it.second) {
+                G->bm_key.push_back((int)G->keys.size());
                 G->keys.push_back(K);
             }
-            G->slot_key[s][i] = it->second;
+            cur[s][i] = it.first->second;
         }
+    const int nkeys = (int)G->keys.size();
     auto lab_count = [&](int32_t L) { return g->label_stat(L, 0); };
     auto lab_deg = [&](int32_t L, bool outdir) { return g->label_stat(L, outdir ? 1 : 2); };
+    // refinement: top-down level by level, then bottom-up. Each constraint is
+    // applied in the cheaper direction: marks from the other level's candidates
+    // (cost ~ their degree sum), or a look from the level's own candidates that
+    // stops at the first hit.
+    VecMap done;
+    auto refine_level = [&](int s, int lvl, const std::vector<Con>& cons) {
+        if (cons.empty()) return;
+        const HostPlan& P = G->plans[s];
+        RefineSpec R;
+        R.src = cur[s][lvl];
+        std::vector<int32_t> t = {R.src};
+        for (const Con& c : cons) {
+            const bool gather = td_gather_cheaper(g, P.key[c.q].label, P.key[lvl].label, c.dir);
+            R.cons.push_back({cur[s][c.q], c.dir, c.lab, gather});
+            t.insert(t.end(), {cur[s][c.q], c.dir, c.lab, gather});
+        }
+        const auto it = done.emplace(std::move(t), (int)G->bm_key.size());
+        if (it.second) {
+            R.dst = (int)G->bm_key.size();
+            G->bm_key.push_back(G->bm_key[R.src]);
+            for (const ConSpec& c : R.cons) G->n_marks += !c.gather;
+            G->refines.push_back(std::move(R));
+        }
+        cur[s][lvl] = it.first->second;
+    };
+    int maxk = 0;
+    for (auto& P : G->plans) maxk = std::max(maxk, P.k);
+    auto end_phase = [&] {
+        if (G->refines.size() > (G->phase_end.empty() ? 0 : G->phase_end.back())) G->phase_end.push_back(G->refines.size());
+    };
+    if (!(o && (o->flags & GFD_FLAG_NO_REFINE))) {
+        for (int lvl = 0; lvl < maxk; lvl++) {
+            for (int s = 0; s < n; s++)
+                if (lvl < G->plans[s].k) refine_level(s, lvl, G->plans[s].td[lvl]);
+            end_phase();
+        }
+        for (int lvl = maxk - 1; lvl >= 0; lvl--) {
+            for (int s = 0; s < n; s++)
+                if (lvl < G->plans[s].k) refine_level(s, lvl, G->plans[s].bu[lvl]);
+            end_phase();
+        }
+    }
+    // the levels' final bitmaps, and the index edges of the spanning trees
+    std::vector<int> final_of(G->bm_key.size(), -1);
+    G->level_final.resize(n);
+    G->level_index.resize(n);
+    VecMap index_id;
+    for (int s = 0; s < n; s++) {
+        const HostPlan& P = G->plans[s];
+        for (int i = 0; i < P.k; i++) {
+            int& f = final_of[cur[s][i]];
+            if (f < 0) {
+                f = (int)G->finals.size();
+                G->finals.push_back(cur[s][i]);
+                G->final_list.push_back(0);
+            }
+            G->level_final[s][i] = f;
+            // lists are read for roots, levels that start a component, and by request
+            if (i == 0 || P.lv[i].par < 0 || (o && (o->flags & GFD_FLAG_KEEP_CANDIDATES))) G->final_list[f] = 1;
+        }
+        for (int i = 1; i < P.k; i++) {
+            const int par = P.lv[i].par;
+            if (par < 0) continue;  // starts a component: no index edges
+            const int pf = G->level_final[s][par], cf = G->level_final[s][i];
+            const auto it = index_id.emplace(std::vector<int32_t>{pf, cf, P.lv[i].tdir, P.lv[i].tlab}, (int)G->index.size());
+            if (it.second) {
+                const int32_t plab = P.key[par].label;
+                G->index.push_back({pf, cf, P.lv[i].tdir, P.lv[i].tlab,
+                                    std::min<uint64_t>(lab_deg(plab, P.lv[i].tdir == 1), (uint64_t)g->m)});
+            }
+            G->level_index[s][i] = it.first->second;
+        }
+    }
     Layout L;
     G->descs.assign(n, SlotDesc{});
     G->offs.resize(n);
-    for (int lvl = 0; lvl < MAXK; lvl++) {
-        size_t c = 0, b = 0;
-        for (int s = 0; s < n; s++)
-            if (lvl < G->plans[s].k) {
-                c += G->plans[s].td[lvl].size();
-                b += G->plans[s].bu[lvl].size();
-            }
-        G->td_need = std::max(G->td_need, std::max(c, b));
-    }
     for (int s = 0; s < n; s++) {
         const HostPlan& P = G->plans[s];
         SlotDesc& D = G->descs[s];
@@ -327,64 +441,48 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
         D.chunk = chunk;
         Group::Off& F = G->offs[s];
         for (int i = 0; i < P.k; i++) {
-            const int32_t lab = phis[s]->node_label[P.order[i]];
-            D.cand_cap[i] = (uint32_t)std::min<uint64_t>(lab_count(lab), (uint64_t)g->n);
-            F.bm[i] = L.take(4ull * nwords);
-            F.rank[i] = L.take(4ull * nwords);
-            F.cand[i] = L.take(4ull * std::max<uint32_t>(1, D.cand_cap[i]));
-        }
-        for (int i = 1; i < P.k; i++) {
-            const int par = P.lv[i].par;
-            if (par < 0) continue;  // starts a component: no index edges
-            const int32_t plab = phis[s]->node_label[P.order[par]];
-            D.cpi_cap[i] = std::min<uint64_t>(lab_deg(plab, P.lv[i].tdir == 1), (uint64_t)g->m);
-            F.cpi_off[i] = L.take(4ull * (D.cand_cap[par] + 1ull));
-            G->cpi_bound += 8ull * std::max<uint64_t>(1, D.cpi_cap[i]) + 256;
+            D.cand_cap[i] = (uint32_t)lab_count(P.key[i].label);
+            if (i > 0 && P.lv[i].par >= 0) D.cpi_cap[i] = G->index[G->level_index[s][i]].bound;
         }
         for (int l = 1; l <= P.k - 2; l++) {
             F.rows[l] = L.take(4ull * row_width(l) * chunk);
             F.wpre[l] = L.take(8ull * chunk);
         }
     }
-    const int nkeys = (int)G->keys.size();
-    G->o_keybm = L.take(4ull * nwords * std::max(1, nkeys));
-    G->o_tmp = L.take(4ull * nwords * std::max<size_t>(1, G->td_need));
-    // job counts, known before any pointer is
-    const bool refine = !(o && (o->flags & GFD_FLAG_NO_REFINE));
-    size_t n_compact = 0, n_cpi = 0, n_and = 0, n_sct = 0, n_prn = 0;
-    for (int s = 0; s < n; s++) {
-        const HostPlan& P = G->plans[s];
-        for (int i = 1; i < P.k; i++) n_cpi += P.lv[i].par >= 0;
-        n_and += P.k;
-        n_compact += P.k;
-        for (int i = 0; i < P.k; i++) {
-            n_sct += refine ? P.td[i].size() + P.bu[i].size() : 0;
-            const bool pr = refine && !P.bu[i].empty();   // bottom-up: an AND and a gather at most
-            const bool tdg = refine && !P.td[i].empty();  // at most one top-down gather per level
-            n_prn += pr + tdg;
-            n_and += pr;
-            n_compact += 2 * pr + tdg;
-        }
+    const size_t bm_bytes = 4ull * nwords;
+    auto label_of = [&](int bm) { return G->keys[G->bm_key[bm]].label; };
+    G->o_keybm = L.take(bm_bytes * std::max(1, nkeys));
+    // zeroed by one call: the finals' counts, the refinements' results and marks
+    G->o_zero = L.size;
+    G->o_counts = L.take(4ull * G->finals.size());
+    G->o_bm = L.take(bm_bytes * (G->bm_key.size() - nkeys));
+    G->o_marks = L.take(bm_bytes * G->n_marks);
+    G->o_zero_end = L.size;
+    for (size_t f = 0; f < G->finals.size(); f++) {
+        G->o_rank.push_back(L.take(bm_bytes));
+        G->o_cand.push_back(G->final_list[f] ? L.take(4ull * std::max<uint64_t>(1, lab_count(label_of(G->finals[f])))) : 0);
+    }
+    for (const IndexSpec& X : G->index) {
+        const uint64_t cap = lab_count(label_of(G->finals[X.parent]));
+        G->o_off.push_back(L.take(4ull * (cap + 1)));
+        G->cpi_nch += cpi_chunks(cap);
+        G->cpi_bound += 8ull * std::max<uint64_t>(1, X.bound) + 256;
     }
     G->cmp_chunks = compact_chunks(g->dg);
-    uint64_t max_pcand = 0;
-    for (int s = 0; s < n; s++)
-        for (int i = 1; i < G->plans[s].k; i++)
-            if (G->plans[s].lv[i].par >= 0)
-                max_pcand = std::max<uint64_t>(max_pcand, G->descs[s].cand_cap[G->plans[s].lv[i].par]);
-    G->cpi_nch = cpi_chunks(max_pcand);
-    G->o_cmp_sums = L.take(4ull * G->cmp_chunks * std::max<size_t>(1, n_compact));
-    G->o_cpi_sums = L.take(8ull * G->cpi_nch * std::max<size_t>(1, n_cpi));
-    G->o_cpi_tot = L.take(4ull * std::max<size_t>(1, n_cpi));
-    G->o_work = L.take(4ull * scan_work_words(std::max(n_sct, std::max(n_prn, n_cpi))));
+    G->o_cmp_sums = L.take(4ull * G->cmp_chunks * G->finals.size());
+    G->o_cpi_sums = L.take(8ull * std::max<uint32_t>(1, G->cpi_nch));
+    G->o_cpi_tot = L.take(4ull * std::max<size_t>(1, G->index.size()));
+    G->idx_inside = G->cpi_bound <= IDX_INSIDE;
+    if (G->idx_inside)
+        for (const IndexSpec& X : G->index) G->o_idx.push_back(L.take(8ull * std::max<uint64_t>(1, X.bound)));
     // the region uploaded from the host: keys and job tables
     G->o_jobs = L.size;
     G->o_keys = L.take(sizeof(FilterKey) * std::max(1, nkeys));
-    G->o_and = L.take(sizeof(AndJob) * std::max<size_t>(1, n_and));
-    G->o_cmp = L.take(sizeof(CompactJob) * std::max<size_t>(1, n_compact));
-    G->o_sct = L.take(sizeof(ScatterJob) * std::max<size_t>(1, n_sct));
-    G->o_prn = L.take(sizeof(PruneJob) * std::max<size_t>(1, n_prn));
-    G->o_cpi = L.take(sizeof(CpiJob) * std::max<size_t>(1, n_cpi));
+    G->o_cmp = L.take(sizeof(CompactJob) * std::max<size_t>(1, G->finals.size()));
+    G->o_sct = L.take(sizeof(ScatterJob) * std::max<size_t>(1, G->n_marks));
+    G->o_ref = L.take(sizeof(RefineJob) * std::max<size_t>(1, G->refines.size()));
+    G->o_cpi = L.take(sizeof(CpiJob) * std::max<size_t>(1, G->index.size()));
+    G->o_first = L.take(8ull * (G->n_marks + G->refines.size() + G->index.size()));
     G->jobs_end = L.size;
     G->bytes = L.size;
     return GFD_OK;
@@ -392,25 +490,135 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
 
 // Absolute pointers, job tables and their upload; the descriptors go to the
 // slot tables at the group's slots, whose states are cleared.
-int group_build(gfd_graph* g, Group* G, const Tables& T, bool refine, cudaStream_t st) {
-    const uint32_t nwords = g->dg.nwords;
+int group_build(gfd_graph* g, Group* G, const Tables& T, cudaStream_t st) {
+    const size_t bm_bytes = 4ull * g->dg.nwords;
+    const int nkeys = (int)G->keys.size();
     uint8_t* base = G->base;
     const int n = G->n;
-    auto state_ncand = [&](int s, int i) { return &T.state[G->slot[s]].ncand[i]; };
-    auto keybm = [&](int key) { return (uint32_t*)(base + G->o_keybm + 4ull * nwords * key); };
-    int maxk = 0;
-    for (auto& P : G->plans) maxk = std::max(maxk, P.k);
+    auto bitmap = [&](int id) {
+        return (uint32_t*)(base + (id < nkeys ? G->o_keybm + bm_bytes * id : G->o_bm + bm_bytes * (id - nkeys)));
+    };
+    auto label_of = [&](int bm) { return G->keys[G->bm_key[bm]].label; };
+    // a job's share of a launch: its items come after those of the jobs before it
+    auto range_of = [&](int bm, bool flat) {
+        ScanRange r{};
+        r.bm = bitmap(bm);
+        r.flat = flat;
+        g->range_of(label_of(bm), r.lo, r.hi);
+        return r;
+    };
+    // (64-bit sums: a launch of more than 2^32 items is refused)
+    auto lay_out = [&](auto* jobs, size_t count, int most, ScanLaunch* l) -> int {
+        uint64_t vertices = 0, items = 0, hubs = 0;
+        for (size_t j = 0; j < count; j++)
+            if (!jobs[j].r.flat) vertices += jobs[j].r.hi[N_CLASS - 1] - jobs[j].r.lo[N_CLASS - 1];
+        scan_units(vertices, most, l->unit);
+        const size_t at = G->first.size();
+        G->first.resize(at + 2 * count);
+        l->first = (const uint32_t*)(base + G->o_first) + at;
+        l->hub_first = l->first + count;
+        for (size_t j = 0; j < count; j++) {
+            const ScanRange& r = jobs[j].r;
+            G->first[at + j] = (uint32_t)items;
+            G->first[at + count + j] = (uint32_t)hubs;
+            for (int c = 0; c < N_CLASS; c++) {
+                const uint32_t k = scan_items(r.lo[c], r.hi[c], r.flat ? FLAT_UNIT : l->unit[c]);
+                if (c == 0 && !r.flat) hubs += k;
+                else items += k;
+            }
+        }
+        if (items > 0xffffffffull || hubs > 0xffffffffull) {
+            set_error(GFD_ERR_UNSUPPORTED, "index build of %d GFDs has more than 2^32 work items (split the batch)", n);
+            return GFD_ERR_UNSUPPORTED;
+        }
+        l->items = (uint32_t)items;
+        l->hubs = (uint32_t)hubs;
+        return GFD_OK;
+    };
+    size_t from = 0;
+    uint32_t* next_marks = (uint32_t*)(base + G->o_marks);
+    for (size_t end : G->phase_end) {
+        Phase sc{0, G->scatter_jobs.size(), 0, {}}, rf{1, G->refine_jobs.size(), 0, {}};
+        for (size_t i = from; i < end; i++) {
+            const RefineSpec& R = G->refines[i];
+            RefineJob J{};
+            J.out = bitmap(R.dst);
+            for (const ConSpec& c : R.cons) {
+                if (c.gather) {
+                    J.con_bm[J.ncon] = bitmap(c.bm);
+                    J.con_dir[J.ncon] = (int8_t)c.dir;
+                    J.con_lab[J.ncon] = (int16_t)c.lab;
+                    J.con_any[J.ncon] = label_of(c.bm) == GFD_WILDCARD;
+                    J.ncon++;
+                    continue;
+                }
+                ScatterJob S{};
+                S.r = range_of(c.bm, false);
+                S.filter = bitmap(R.src);
+                S.marks = next_marks;
+                // x needs an out-neighbour y in C(q) (x -> y): follow in-edges of y
+                S.scan_out = c.dir ? 0 : 1;
+                S.lab = c.lab;
+                G->scatter_jobs.push_back(S);
+                J.marks[J.nmarks++] = next_marks;
+                next_marks += g->dg.nwords;
+            }
+            J.r = range_of(R.src, J.ncon == 0);
+            G->refine_jobs.push_back(J);
+        }
+        from = end;
+        sc.count = G->scatter_jobs.size() - sc.first;
+        rf.count = G->refine_jobs.size() - rf.first;
+        if (int rc = lay_out(G->scatter_jobs.data() + sc.first, sc.count, REFINE_UNIT, &sc.launch)) return rc;
+        if (int rc = lay_out(G->refine_jobs.data() + rf.first, rf.count, REFINE_UNIT, &rf.launch)) return rc;
+        if (sc.count) G->phases.push_back(sc);
+        G->phases.push_back(rf);
+    }
+    auto rank_of = [&](int f) { return (uint32_t*)(base + G->o_rank[f]); };
+    auto count_of = [&](int f) { return (uint32_t*)(base + G->o_counts) + f; };
+    for (size_t f = 0; f < G->finals.size(); f++) {
+        CompactJob J{};
+        J.bm = bitmap(G->finals[f]);
+        J.rank = rank_of((int)f);
+        J.cand = G->final_list[f] ? (int32_t*)(base + G->o_cand[f]) : nullptr;
+        J.count = count_of((int)f);
+        J.csum = (uint32_t*)(base + G->o_cmp_sums + 4ull * G->cmp_chunks * f);
+        G->compact_jobs.push_back(J);
+    }
+    uint32_t chunk = 0;
+    for (size_t x = 0; x < G->index.size(); x++) {
+        const IndexSpec& X = G->index[x];
+        CpiJob J{};
+        J.r = range_of(G->finals[X.parent], false);
+        J.prank = rank_of(X.parent);
+        J.pcount = count_of(X.parent);
+        J.cbm = bitmap(G->finals[X.child]);
+        J.crank = rank_of(X.child);
+        J.off = (uint32_t*)(base + G->o_off[x]);
+        J.idx = G->idx_inside ? (int2*)(base + G->o_idx[x]) : nullptr;
+        J.cap = X.bound;
+        J.out = X.dir;
+        J.lab = X.lab;
+        J.chunk0 = chunk;
+        J.csum = (uint64_t*)(base + G->o_cpi_sums) + chunk;
+        J.total = (uint32_t*)(base + G->o_cpi_tot) + x;
+        chunk += cpi_chunks(g->label_stat(label_of(G->finals[X.parent]), 0));
+        G->cpi_jobs.push_back(J);
+    }
+    if (int rc = lay_out(G->cpi_jobs.data(), G->cpi_jobs.size(), INDEX_UNIT, &G->cpi_launch)) return rc;
     for (int s = 0; s < n; s++) {
         const HostPlan& P = G->plans[s];
         SlotDesc& D = G->descs[s];
         const Group::Off& F = G->offs[s];
         for (int i = 0; i < P.k; i++) {
-            D.bm[i] = (uint32_t*)(base + F.bm[i]);
-            D.rank[i] = (uint32_t*)(base + F.rank[i]);
-            D.cand[i] = (int32_t*)(base + F.cand[i]);
-            if (i >= 1) {
-                D.cpi_off[i] = P.lv[i].par >= 0 ? (uint32_t*)(base + F.cpi_off[i]) : nullptr;
-                D.cpi_idx[i] = nullptr;  // allocated once the index edges are counted
+            const int f = G->level_final[s][i];
+            D.bm[i] = bitmap(G->finals[f]);
+            D.rank[i] = rank_of(f);
+            D.cand[i] = G->final_list[f] ? (int32_t*)(base + G->o_cand[f]) : nullptr;
+            D.cand_n[i] = count_of(f);
+            if (i >= 1 && P.lv[i].par >= 0) {
+                D.cpi_off[i] = G->cpi_jobs[G->level_index[s][i]].off;
+                D.cpi_idx[i] = G->cpi_jobs[G->level_index[s][i]].idx;  // null until the index edges are counted
             }
         }
         for (int l = 1; l <= P.k - 2; l++) {
@@ -418,172 +626,11 @@ int group_build(gfd_graph* g, Group* G, const Tables& T, bool refine, cudaStream
             D.wpre[l] = (uint64_t*)(base + F.wpre[l]);
         }
     }
-    auto scan_list = [&](int s, int i) {
-        const SlotDesc& D = G->descs[s];
-        return ScanList{D.cand[i], state_ncand(s, i), D.bm[i], D.rank[i]};
-    };
-    auto compact_job = [&](int s, int i) {
-        CompactJob J{};
-        J.bm = G->descs[s].bm[i];
-        J.rank = G->descs[s].rank[i];
-        J.cand = G->descs[s].cand[i];
-        J.count = state_ncand(s, i);
-        J.csum = (uint32_t*)(base + G->o_cmp_sums + 4ull * G->cmp_chunks * G->compact_jobs.size());
-        return J;
-    };
-    G->phases.clear();
-    if (!refine) {
-        size_t a0 = G->and_jobs.size(), c0 = G->compact_jobs.size();
-        for (int s = 0; s < n; s++)
-            for (int i = 0; i < G->plans[s].k; i++) {
-                AndJob J{};
-                J.bm = G->descs[s].bm[i];
-                J.src = keybm(G->slot_key[s][i]);
-                G->and_jobs.push_back(J);
-                G->compact_jobs.push_back(compact_job(s, i));
-            }
-        G->phases.push_back({0, a0, G->and_jobs.size() - a0});
-        G->phases.push_back({1, c0, G->compact_jobs.size() - c0});
-    } else {
-        // top-down, level by level. Each constraint from an earlier level is
-        // applied in the cheaper direction: scatter marks from the earlier
-        // level's candidates (cost ~ their degree sum), or, after compaction,
-        // keep the level's own candidates that have a neighbour there
-        // (a gather that stops at the first hit).
-        for (int lvl = 0; lvl < maxk; lvl++) {
-            size_t a0 = G->and_jobs.size(), c0 = G->compact_jobs.size(), s0 = G->scatter_jobs.size();
-            size_t p0 = G->prune_jobs.size();
-            size_t tmp_used = 0;
-            std::vector<int> gathered;
-            for (int s = 0; s < n; s++) {
-                const HostPlan& P = G->plans[s];
-                if (lvl >= P.k) continue;
-                AndJob J{};
-                J.bm = G->descs[s].bm[lvl];
-                J.src = keybm(G->slot_key[s][lvl]);
-                PruneJob Pj{};
-                Pj.c = scan_list(s, lvl);
-                Pj.out = G->descs[s].bm[lvl];
-                for (const Con& c : P.td[lvl]) {
-                    const int32_t lq = G->plans[s].key[c.q].label, li = G->plans[s].key[lvl].label;
-                    if (td_gather_cheaper(g, lq, li, c.dir)) {
-                        Pj.con_bm[Pj.ncon] = G->descs[s].bm[c.q];
-                        Pj.con_dir[Pj.ncon] = c.dir;
-                        Pj.con_lab[Pj.ncon] = c.lab;
-                        Pj.con_any[Pj.ncon] = lq == GFD_WILDCARD;
-                        Pj.ncon++;
-                        continue;
-                    }
-                    uint32_t* marks = (uint32_t*)(base + G->o_tmp + 4ull * nwords * tmp_used++);
-                    ScatterJob S{};
-                    S.q = scan_list(s, c.q);
-                    S.filter = J.src;
-                    S.marks = marks;
-                    // x needs an out-neighbour y in C(q) (x -> y): follow in-edges of y
-                    S.scan_out = c.dir ? 0 : 1;
-                    S.lab = c.lab;
-                    G->scatter_jobs.push_back(S);
-                    J.tmp[J.ntmp++] = marks;
-                }
-                G->and_jobs.push_back(J);
-                G->compact_jobs.push_back(compact_job(s, lvl));
-                if (Pj.ncon) {
-                    G->prune_jobs.push_back(Pj);
-                    gathered.push_back(s);
-                }
-            }
-            if (tmp_used) G->phases.push_back({4, 0, tmp_used});
-            if (G->scatter_jobs.size() > s0) G->phases.push_back({2, s0, G->scatter_jobs.size() - s0});
-            G->phases.push_back({0, a0, G->and_jobs.size() - a0});
-            G->phases.push_back({1, c0, G->compact_jobs.size() - c0});
-            if (!gathered.empty()) {
-                const size_t c1 = G->compact_jobs.size();
-                for (int s : gathered) G->compact_jobs.push_back(compact_job(s, lvl));
-                G->phases.push_back({3, p0, G->prune_jobs.size() - p0});
-                G->phases.push_back({1, c1, G->compact_jobs.size() - c1});
-            }
-        }
-        // bottom-up, reverse level order; each constraint from a later level
-        // is applied in the cheaper direction, as top-down
-        for (int lvl = maxk - 1; lvl >= 0; lvl--) {
-            size_t a0 = G->and_jobs.size(), c0 = G->compact_jobs.size(), s0 = G->scatter_jobs.size();
-            size_t p0 = G->prune_jobs.size();
-            size_t tmp_used = 0;
-            std::vector<int> gathered;
-            for (int s = 0; s < n; s++) {
-                const HostPlan& P = G->plans[s];
-                if (lvl >= P.k || P.bu[lvl].empty()) continue;
-                AndJob A{};
-                A.bm = G->descs[s].bm[lvl];
-                A.src = G->descs[s].bm[lvl];
-                PruneJob J{};
-                J.c = scan_list(s, lvl);
-                J.out = G->descs[s].bm[lvl];
-                for (const Con& c : P.bu[lvl]) {
-                    const int32_t lq = P.key[c.q].label, li = P.key[lvl].label;
-                    if (td_gather_cheaper(g, lq, li, c.dir)) {
-                        J.con_bm[J.ncon] = G->descs[s].bm[c.q];
-                        J.con_dir[J.ncon] = c.dir;
-                        J.con_lab[J.ncon] = c.lab;
-                        J.con_any[J.ncon] = lq == GFD_WILDCARD;
-                        J.ncon++;
-                        continue;
-                    }
-                    uint32_t* marks = (uint32_t*)(base + G->o_tmp + 4ull * nwords * tmp_used++);
-                    ScatterJob S{};
-                    S.q = scan_list(s, c.q);
-                    S.filter = G->descs[s].bm[lvl];
-                    S.marks = marks;
-                    S.scan_out = c.dir ? 0 : 1;
-                    S.lab = c.lab;
-                    G->scatter_jobs.push_back(S);
-                    A.tmp[A.ntmp++] = marks;
-                }
-                if (A.ntmp) {
-                    G->and_jobs.push_back(A);
-                    G->compact_jobs.push_back(compact_job(s, lvl));
-                }
-                if (J.ncon) {
-                    G->prune_jobs.push_back(J);
-                    gathered.push_back(s);
-                }
-            }
-            if (tmp_used) G->phases.push_back({4, 0, tmp_used});
-            if (G->scatter_jobs.size() > s0) G->phases.push_back({2, s0, G->scatter_jobs.size() - s0});
-            if (G->and_jobs.size() > a0) {
-                G->phases.push_back({0, a0, G->and_jobs.size() - a0});
-                G->phases.push_back({1, c0, G->compact_jobs.size() - c0});
-            }
-            if (!gathered.empty()) {
-                const size_t c1 = G->compact_jobs.size();
-                for (int s : gathered) G->compact_jobs.push_back(compact_job(s, lvl));
-                G->phases.push_back({3, p0, G->prune_jobs.size() - p0});
-                G->phases.push_back({1, c1, G->compact_jobs.size() - c1});
-            }
-        }
-    }
-    for (int s = 0; s < n; s++)
-        for (int i = 1; i < G->plans[s].k; i++) {
-            const int par = G->plans[s].lv[i].par;
-            if (par < 0) continue;  // starts a component
-            CpiJob J{};
-            J.p = scan_list(s, par);
-            J.cbm = G->descs[s].bm[i];
-            J.crank = G->descs[s].rank[i];
-            J.off = G->descs[s].cpi_off[i];
-            J.idx = G->descs[s].cpi_idx[i];
-            J.cap = G->descs[s].cpi_cap[i];
-            J.out = G->plans[s].lv[i].tdir;
-            J.lab = G->plans[s].lv[i].tlab;
-            J.nnz_stat = &T.state[G->slot[s]].st_cpi;
-            J.csum = (uint64_t*)(base + G->o_cpi_sums + 8ull * G->cpi_nch * G->cpi_jobs.size());
-            G->cpi_jobs.push_back(J);
-        }
     // one host image of keys and job tables (each table within its region)
-    const size_t need[6] = {sizeof(FilterKey) * G->keys.size(), sizeof(AndJob) * G->and_jobs.size(),
-                            sizeof(CompactJob) * G->compact_jobs.size(), sizeof(ScatterJob) * G->scatter_jobs.size(),
-                            sizeof(PruneJob) * G->prune_jobs.size(), sizeof(CpiJob) * G->cpi_jobs.size()};
-    const size_t at[7] = {G->o_keys, G->o_and, G->o_cmp, G->o_sct, G->o_prn, G->o_cpi, G->jobs_end};
+    const size_t need[6] = {sizeof(FilterKey) * G->keys.size(), sizeof(CompactJob) * G->compact_jobs.size(),
+                            sizeof(ScatterJob) * G->scatter_jobs.size(), sizeof(RefineJob) * G->refine_jobs.size(),
+                            sizeof(CpiJob) * G->cpi_jobs.size(), 4 * G->first.size()};
+    const size_t at[7] = {G->o_keys, G->o_cmp, G->o_sct, G->o_ref, G->o_cpi, G->o_first, G->jobs_end};
     for (int t = 0; t < 6; t++)
         if (at[t] + need[t] > at[t + 1]) {
             set_error(GFD_ERR_CUDA, "internal: job table %d needs %zu bytes, region holds %zu", t, need[t],
@@ -595,11 +642,11 @@ int group_build(gfd_graph* g, Group* G, const Tables& T, bool refine, cudaStream
         if (bytes) memcpy(img.data() + (off - G->o_jobs), p, bytes);
     };
     put(G->o_keys, G->keys.data(), sizeof(FilterKey) * G->keys.size());
-    put(G->o_and, G->and_jobs.data(), sizeof(AndJob) * G->and_jobs.size());
     put(G->o_cmp, G->compact_jobs.data(), sizeof(CompactJob) * G->compact_jobs.size());
     put(G->o_sct, G->scatter_jobs.data(), sizeof(ScatterJob) * G->scatter_jobs.size());
-    put(G->o_prn, G->prune_jobs.data(), sizeof(PruneJob) * G->prune_jobs.size());
+    put(G->o_ref, G->refine_jobs.data(), sizeof(RefineJob) * G->refine_jobs.size());
     put(G->o_cpi, G->cpi_jobs.data(), sizeof(CpiJob) * G->cpi_jobs.size());
+    put(G->o_first, G->first.data(), 4 * G->first.size());
     GFD_CUDA(cudaMemcpyAsync(base + G->o_jobs, img.data(), img.size(), cudaMemcpyHostToDevice, st));
     // descriptors into the slot tables (contiguous runs in one copy) and states
     // cleared, idle (cur = -1): a serving session's running enumeration may
@@ -623,74 +670,65 @@ int group_launch(gfd_graph* g, Group* G, const Tables& T, cudaMemPool_t pool, cu
                  int64_t* launches, bool count = false) {
     const DevGraph& dg = g->dg;
     uint8_t* base = G->base;
-    const ScanWork sw{(uint32_t*)(base + G->o_work),
-                      count ? (unsigned long long*)&T.sched->cnt[CNT_SCAN_CANDS] : nullptr};
+    const ScanCount scan = count ? (ScanCount)&T.sched->cnt[CNT_SCAN_CANDS] : nullptr;
     prof.begin(PROF_FILTER, st);
     if (int rc = launch_filter(dg, (const FilterKey*)(base + G->o_keys), (int)G->keys.size(),
                                (uint32_t*)(base + G->o_keybm), st))
         return rc;
     launches[PROF_FILTER]++;
+    GFD_CUDA(cudaMemsetAsync(base + G->o_zero, 0, G->o_zero_end - G->o_zero, st));
     prof.end(PROF_FILTER, st);
     prof.begin(PROF_REFINE, st);
     for (const Phase& ph : G->phases) {
-        int rc = GFD_OK;
-        switch (ph.kind) {
-            case 0: rc = launch_and(dg, (const AndJob*)(base + G->o_and) + ph.first, (int)ph.count, st); break;
-            case 1:
-                rc = launch_compact(dg, (const CompactJob*)(base + G->o_cmp) + ph.first, (int)ph.count, st);
-                break;
-            case 2:
-                rc = launch_scatter(dg, (const ScatterJob*)(base + G->o_sct) + ph.first, (int)ph.count, sw, st);
-                break;
-            case 3:
-                rc = launch_prune(dg, (const PruneJob*)(base + G->o_prn) + ph.first, (int)ph.count, sw, st);
-                break;
-            case 4: {
-                cudaError_t e = cudaMemsetAsync(base + G->o_tmp, 0, 4ull * dg.nwords * ph.count, st);
-                rc = e == cudaSuccess ? GFD_OK : cuda_fail(e, "cudaMemsetAsync");
-                break;
-            }
-        }
+        const int rc = ph.kind == 0 ? launch_scatter(dg, (const ScatterJob*)(base + G->o_sct) + ph.first, (int)ph.count,
+                                                     ph.launch, scan, st)
+                                    : launch_refine(dg, (const RefineJob*)(base + G->o_ref) + ph.first, (int)ph.count,
+                                                    ph.launch, scan, st);
         if (rc) return rc;
-        launches[PROF_REFINE] += ph.kind == 4 ? 0 : (ph.kind == 0 ? 1 : 2);  // scatter/prune: + shares of the jobs
+        launches[PROF_REFINE]++;
     }
+    if (int rc = launch_compact(dg, (const CompactJob*)(base + G->o_cmp), (int)G->compact_jobs.size(), st)) return rc;
+    launches[PROF_REFINE] += 2;
     prof.end(PROF_REFINE, st);
     prof.begin(PROF_INDEX, st);
     const int ncpi = (int)G->cpi_jobs.size();
     if (ncpi) {
         CpiJob* d_cpi = (CpiJob*)(base + G->o_cpi);
-        uint32_t* d_tot = (uint32_t*)(base + G->o_cpi_tot);
-        if (int rc = launch_cpi_count(dg, d_cpi, ncpi, G->cpi_nch, T.err, d_tot, sw, st)) return rc;
-        // size the index edges exactly: one read-back of the per-edge totals
-        std::vector<uint32_t> tot(ncpi);
-        GFD_CUDA(cudaMemcpyAsync(tot.data(), d_tot, 4ull * ncpi, cudaMemcpyDeviceToHost, st));
-        GFD_CUDA(cudaStreamSynchronize(st));
-        std::vector<size_t> at(ncpi);
-        size_t bytes = 256;
-        for (int j = 0; j < ncpi; j++) {
-            at[j] = bytes;
-            bytes = (bytes + 8ull * std::max<uint32_t>(1, tot[j]) + 255) & ~(size_t)255;
-        }
-        void* p = nullptr;
-        if (int rc = pool_alloc(pool, bytes, st, &p, "index edges")) return rc;
-        G->cpi_base = (uint8_t*)p;
-        G->cpi_bytes = bytes;
-        int j = 0;
-        for (int s = 0; s < G->n; s++)
-            for (int i = 1; i < G->plans[s].k; i++) {
-                if (G->plans[s].lv[i].par < 0) continue;  // same jobs, same order as built
-                int2* idx = (int2*)(G->cpi_base + at[j]);
-                G->cpi_jobs[j].idx = idx;
-                G->cpi_jobs[j].cap = tot[j];
-                G->descs[s].cpi_idx[i] = idx;
-                j++;
+        if (int rc = launch_cpi_count(dg, d_cpi, ncpi, G->cpi_launch, G->cpi_nch, T.err, scan, st)) return rc;
+        if (!G->idx_inside) {
+            // size the index edges exactly: one read-back of the per-edge totals
+            std::vector<uint32_t> tot(ncpi);
+            GFD_CUDA(cudaMemcpyAsync(tot.data(), base + G->o_cpi_tot, 4ull * ncpi, cudaMemcpyDeviceToHost, st));
+            GFD_CUDA(cudaStreamSynchronize(st));
+            std::vector<size_t> at(ncpi);
+            size_t bytes = 256;
+            for (int j = 0; j < ncpi; j++) {
+                at[j] = bytes;
+                bytes = (bytes + 8ull * std::max<uint32_t>(1, tot[j]) + 255) & ~(size_t)255;
             }
-        GFD_CUDA(cudaMemcpyAsync(d_cpi, G->cpi_jobs.data(), sizeof(CpiJob) * ncpi, cudaMemcpyHostToDevice, st));
-        for (int s = 0; s < G->n; s++)
-            GFD_CUDA(cudaMemcpyAsync(&T.desc[G->slot[s]].cpi_idx, G->descs[s].cpi_idx, sizeof(G->descs[s].cpi_idx),
-                                     cudaMemcpyHostToDevice, st));
-        if (int rc = launch_cpi_fill(dg, d_cpi, ncpi, sw, st)) return rc;
-        launches[PROF_INDEX] += 7;
+            void* p = nullptr;
+            if (int rc = pool_alloc(pool, bytes, st, &p, "index edges")) return rc;
+            G->cpi_base = (uint8_t*)p;
+            G->cpi_bytes = bytes;
+            for (int j = 0; j < ncpi; j++) {
+                G->cpi_jobs[j].idx = (int2*)(G->cpi_base + at[j]);
+                G->cpi_jobs[j].cap = tot[j];
+            }
+            for (int s = 0; s < G->n; s++)
+                for (int i = 1; i < G->plans[s].k; i++)
+                    if (G->plans[s].lv[i].par >= 0) G->descs[s].cpi_idx[i] = G->cpi_jobs[G->level_index[s][i]].idx;
+            GFD_CUDA(cudaMemcpyAsync(d_cpi, G->cpi_jobs.data(), sizeof(CpiJob) * ncpi, cudaMemcpyHostToDevice, st));
+            // (descriptors of neighbouring slots in one copy)
+            for (int s = 0; s < G->n;) {
+                int e = s + 1;
+                while (e < G->n && G->slot[e] == G->slot[e - 1] + 1) e++;
+                GFD_CUDA(cudaMemcpyAsync(&T.desc[G->slot[s]], &G->descs[s], sizeof(SlotDesc) * (e - s),
+                                         cudaMemcpyHostToDevice, st));
+                s = e;
+            }
+        }
+        if (int rc = launch_cpi_fill(dg, d_cpi, ncpi, G->cpi_launch, scan, st)) return rc;
+        launches[PROF_INDEX] += 4;
     }
     prof.end(PROF_INDEX, st);
     return GFD_OK;
@@ -765,7 +803,6 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
         return GFD_ERR_UNSUPPORTED;
     }
     const int32_t flags = o ? o->flags : 0;
-    const bool refine = !(flags & GFD_FLAG_NO_REFINE);
     const bool persistent = !(flags & GFD_FLAG_HOST_LOOP);
     const bool use_graph = !(flags & GFD_FLAG_NO_GRAPH);
     const int variant = pick_variant(g, o);
@@ -797,7 +834,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     G.base = (uint8_t*)wb;
     G.slot.resize(n);
     for (int s = 0; s < n; s++) G.slot[s] = s;
-    if (int rc = group_build(g, &G, T, refine, st)) return rc;
+    if (int rc = group_build(g, &G, T, st)) return rc;
     ProfEvents prof;
     if (int rc = prof.init((flags & GFD_FLAG_PROFILE) != 0)) return rc;
     int64_t launches[5] = {0, 0, 0, 0, 0};
@@ -1090,7 +1127,7 @@ int session_admit(gfd_session* S) {
         const gfd_gfd* one[1] = {&R->phi};
         if (int rc = group_plan(S->g, one, 1, &S->opts, per_slot, &trial)) return rc;
         const int64_t req_bytes =
-            (int64_t)(trial.bytes + trial.cpi_bound) + (int64_t)(4ull * trial.plans[0].k * S->viol_cap);
+            (int64_t)(trial.bytes + (trial.idx_inside ? 0 : trial.cpi_bound)) + (int64_t)(4ull * trial.plans[0].k * S->viol_cap);
         const bool idle = S->used == 0 && take.empty();  // always admit into an idle device
         if (!idle && S->used + need + req_bytes > S->budget) break;
         need += req_bytes;
@@ -1128,8 +1165,7 @@ int session_admit(gfd_session* S) {
         sl.req = std::move(take[i]);
     }
     G->live = n;
-    const bool refine = !(S->opts.flags & GFD_FLAG_NO_REFINE);
-    if (int rc = group_build(S->g, G.get(), S->T, refine, sa)) return rc;
+    if (int rc = group_build(S->g, G.get(), S->T, sa)) return rc;
     ProfEvents prof;
     int64_t launches[5] = {0, 0, 0, 0, 0};
     const int lrc = group_launch(S->g, G.get(), S->T, S->pool, sa, prof, launches);
