@@ -153,9 +153,6 @@ int gfd_result_candidates(const gfd_result* r, int32_t node, const int32_t** lis
 }
 
 void gfd_result_free(gfd_result* r) {
-    if (!r) return;
-    if (r->d_viol) cudaFree(r->d_viol);
-    cudaGetLastError();  // a failure here must not surface in a later, unrelated call
     delete r;
 }
 

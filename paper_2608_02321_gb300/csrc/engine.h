@@ -12,6 +12,29 @@
 
 namespace gfd {
 struct Engine;
+
+// The graph's stream-ordered memory pool: destroyed with the last graph or
+// result that refers to it (a freed graph gives back what is unused).
+struct Pool {
+    cudaMemPool_t p = nullptr;
+    ~Pool() {
+        if (p) cudaMemPoolDestroy(p);
+        cudaGetLastError();
+    }
+};
+
+// Device memory of the pool shared by results (the short lists of one call) or
+// owned by one. Freed without naming a stream: the call's may be gone by then.
+struct DevBlock {
+    void* p = nullptr;
+    std::shared_ptr<Pool> pool;
+    DevBlock(void* q, std::shared_ptr<Pool> from) : p(q), pool(std::move(from)) {}
+    DevBlock(const DevBlock&) = delete;
+    ~DevBlock() {
+        if (p) cudaFree(p);
+        cudaGetLastError();  // a failure here must not surface in a later, unrelated call
+    }
+};
 }
 
 struct gfd_graph {
@@ -68,7 +91,9 @@ struct gfd_result {
     int32_t k = 0;
     uint64_t n_matches = 0;
     uint64_t n_viol = 0;
-    int32_t* d_viol = nullptr;  // device, unsorted, owned by the result
+    int32_t* d_viol = nullptr;  // device, unsorted, in mem
+    std::shared_ptr<gfd::DevBlock> mem;
+    int32_t vbits = 32;         // bits of a vertex id
     bool fetched = false;
     std::unique_ptr<int32_t[]> tuples;  // host copy made by gfd_result_tuples
     double prof_ms[5] = {0, 0, 0, 0, 0};

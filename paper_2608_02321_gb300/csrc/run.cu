@@ -36,12 +36,13 @@
 namespace gfd {
 
 struct Engine {
-    cudaMemPool_t pool = nullptr;
+    std::shared_ptr<Pool> pool;
 };
 
 void engine_free(Engine* e) {
     if (!e) return;
-    if (e->pool) cudaMemPoolDestroy(e->pool);
+    if (e->pool) cudaMemPoolTrimTo(e->pool->p, 0);  // (results may keep the pool itself)
+    cudaGetLastError();
     delete e;
 }
 
@@ -58,7 +59,7 @@ struct Layout {
     }
 };
 
-int get_pool(gfd_graph* g, cudaMemPool_t* out) {
+int get_pool(gfd_graph* g, std::shared_ptr<Pool>* out) {
     if (!g->eng) g->eng = new Engine();
     if (!g->eng->pool) {
         int dev = 0;
@@ -67,9 +68,11 @@ int get_pool(gfd_graph* g, cudaMemPool_t* out) {
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
-        GFD_CUDA(cudaMemPoolCreate(&g->eng->pool, &props));
+        auto pool = std::make_shared<Pool>();
+        GFD_CUDA(cudaMemPoolCreate(&pool->p, &props));
         uint64_t thr = UINT64_MAX;
-        GFD_CUDA(cudaMemPoolSetAttribute(g->eng->pool, cudaMemPoolAttrReleaseThreshold, &thr));
+        GFD_CUDA(cudaMemPoolSetAttribute(pool->p, cudaMemPoolAttrReleaseThreshold, &thr));
+        g->eng->pool = std::move(pool);
     }
     *out = g->eng->pool;
     return GFD_OK;
@@ -289,6 +292,10 @@ constexpr size_t IDX_INSIDE = (size_t)1 << 30;
 // Largest units (log2 of vertices) of the adjacency scans, see scan_units.
 constexpr int REFINE_UNIT = 8;
 constexpr int INDEX_UNIT = 10;
+
+// Violation lists up to this many bytes share one allocation per call (which
+// lives until the last of their results is freed); larger ones have their own.
+constexpr size_t SHARED_LIST = 64 << 10;
 
 // Top-down constraint "x in C(i) needs a neighbour in C(q) through an edge
 // leaving x (dir 1) or entering x (dir 0)": scattering from C(q) scans the
@@ -757,8 +764,8 @@ int64_t default_budget(const gfd_graph* g, const gfd_opts* o) {
     // free for this one too (the pool keeps what it has allocated)
     if (g && g->eng && g->eng->pool) {
         uint64_t reserved = 0, used = 0;
-        if (cudaMemPoolGetAttribute(g->eng->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
-            cudaMemPoolGetAttribute(g->eng->pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+        if (cudaMemPoolGetAttribute(g->eng->pool->p, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+            cudaMemPoolGetAttribute(g->eng->pool->p, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
             reserved > used)
             fr += (size_t)(reserved - used);
         cudaGetLastError();
@@ -769,13 +776,16 @@ int64_t default_budget(const gfd_graph* g, const gfd_opts* o) {
     return (int64_t)std::min<size_t>((size_t)128 << 30, fr / 2);
 }
 
-gfd_result* make_result(const HostPlan& P, const SlotState& S, uint64_t steps, uint64_t probes, int32_t* d_viol,
-                        cudaStream_t st) {
+gfd_result* make_result(const gfd_graph* g, const HostPlan& P, const SlotState& S, uint64_t steps, uint64_t probes,
+                        int32_t* d_viol, std::shared_ptr<DevBlock> mem, cudaStream_t st) {
     gfd_result* r = new gfd_result();
     r->k = P.k;
     r->n_matches = S.n_matches;
     r->n_viol = S.n_viol;
     r->d_viol = d_viol;
+    r->mem = std::move(mem);
+    r->vbits = 1;
+    while (r->vbits < 32 && (1ll << r->vbits) < (int64_t)g->n) r->vbits++;
     r->stream = st;
     r->stat[0] = steps;
     r->stat[1] = S.st_work;
@@ -816,8 +826,9 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     if (int rc = group_plan(g, phis, n, o, budget / n, &G, o && o->frontier_budget_bytes > 0)) return rc;
     int kmax = 1;
     for (auto& P : G.plans) kmax = std::max(kmax, P.k);
-    cudaMemPool_t pool;
-    if (int rc = get_pool(g, &pool)) return rc;
+    std::shared_ptr<Pool> shared_pool;
+    if (int rc = get_pool(g, &shared_pool)) return rc;
+    const cudaMemPool_t pool = shared_pool->p;
     Tables T;
     if (int rc = tables_alloc(pool, n, block_threads, pick_tile_iters(g, o), kmax, vcap, true, st, &T)) return rc;
     struct Free {
@@ -885,19 +896,29 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     // split the arena into one violation list per GFD (order within a list is
     // arbitrary; gfd_result_tuples sorts)
     std::vector<int32_t*> vbuf(n, nullptr);
-    struct VFree {
-        std::vector<int32_t*>* v;
-        cudaStream_t st;
-        ~VFree() {
-            for (auto p : *v)
-                if (p) cudaFreeAsync(p, st);
-        }
-    } vfree{&vbuf, st};
-    for (int s = 0; s < n; s++) {
-        if (!states[s].n_viol) continue;
+    std::vector<std::shared_ptr<DevBlock>> vmem(n);
+    size_t small = 0;
+    auto list_bytes = [&](int s) { return 4ull * states[s].n_viol * G.plans[s].k; };
+    for (int s = 0; s < n; s++)
+        if (list_bytes(s) <= SHARED_LIST) small += list_bytes(s);
+    if (small) {
         void* p = nullptr;
-        if (int rc = pool_alloc(pool, 4ull * states[s].n_viol * G.plans[s].k, st, &p, "violation list")) return rc;
+        if (int rc = pool_alloc(pool, small, st, &p, "violation lists")) return rc;
+        auto block = std::make_shared<DevBlock>(p, shared_pool);
+        int32_t* at = (int32_t*)p;
+        for (int s = 0; s < n; s++)
+            if (states[s].n_viol && list_bytes(s) <= SHARED_LIST) {
+                vbuf[s] = at;
+                vmem[s] = block;
+                at += list_bytes(s) / 4;
+            }
+    }
+    for (int s = 0; s < n; s++) {
+        if (list_bytes(s) <= SHARED_LIST) continue;
+        void* p = nullptr;
+        if (int rc = pool_alloc(pool, list_bytes(s), st, &p, "violation list")) return rc;
         vbuf[s] = (int32_t*)p;
+        vmem[s] = std::make_shared<DevBlock>(p, shared_pool);
     }
     if (hs.varena_used) {
         GFD_CUDA(cudaMemcpyAsync(T.vptr, vbuf.data(), sizeof(int32_t*) * n, cudaMemcpyHostToDevice, st));
@@ -928,8 +949,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
             }
     }
     for (int s = 0; s < n; s++) {
-        gfd_result* r = make_result(G.plans[s], states[s], hs.steps, hs.probes, vbuf[s], st);
-        vbuf[s] = nullptr;
+        gfd_result* r = make_result(g, G.plans[s], states[s], hs.steps, hs.probes, vbuf[s], std::move(vmem[s]), st);
         if (count) {
             for (int c = 0; c < N_CNT; c++) r->stat[7 + c] = hs.cnt[c];
             // the host's figures: distinct filter keys and candidate bitmaps
@@ -993,6 +1013,7 @@ struct gfd_session {
     gfd::SlotState* h_states = nullptr;  // pinned snapshot after a round
     gfd::Sched* h_sched = nullptr;
     int32_t* h_err = nullptr;
+    std::shared_ptr<gfd::Pool> shared_pool;
     cudaMemPool_t pool = nullptr;
     gfd::Tables T;
     int variant = 0;
@@ -1039,7 +1060,8 @@ int session_create(gfd_graph* g, int32_t max_slots, const gfd_opts* o, gfd_sessi
     GFD_CUDA(cudaMallocHost((void**)&S->h_states, sizeof(SlotState) * max_slots));
     GFD_CUDA(cudaMallocHost((void**)&S->h_sched, sizeof(Sched)));
     GFD_CUDA(cudaMallocHost((void**)&S->h_err, sizeof(int32_t)));
-    if (int rc = get_pool(g, &S->pool)) return rc;
+    if (int rc = get_pool(g, &S->shared_pool)) return rc;
+    S->pool = S->shared_pool->p;
     if (int rc = tables_alloc(S->pool, max_slots, S->block_threads, pick_tile_iters(g, o), 0, 0, false, S->st, &S->T))
         return rc;
     if (int rc = mark_idle(S->T.state, max_slots, S->st)) return rc;  // every slot starts idle
@@ -1300,7 +1322,8 @@ int session_step(gfd_session* S, int32_t* n_advanced, int32_t* n_running, int32_
                 r->stat[6] += 1;
                 cudaFreeAsync(sl.viol, S->st);
             } else {
-                r = make_result(sl.group->plans[sl.index], states[i], hs.steps, hs.probes, sl.viol, S->st);
+                r = make_result(S->g, sl.group->plans[sl.index], states[i], hs.steps, hs.probes, sl.viol,
+                                std::make_shared<DevBlock>(sl.viol, S->shared_pool), S->st);
             }
             sl.viol = nullptr;  // now owned by the result (or freed above)
             S->done.emplace_back(sl.id, r);
@@ -1421,17 +1444,88 @@ int autotune(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opts
 // ------------------------------------------------------------------ result sort
 namespace {
 
+// Where a result's tuples are and go.
+struct PackSrc {
+    const int32_t* p;   // the result's unsorted tuples
+    int32_t k;
+    int32_t pad;
+    uint64_t row_off;   // first row of the result (in the rows of all results, and in sorted order)
+    uint64_t int_off;   // first int of the result in the packed output
+};
+
+// the result whose rows hold row g (src[nres].row_off = all rows)
+__device__ __forceinline__ int src_of(const PackSrc* src, int nres, uint64_t g) {
+    int lo = 0, hi = nres;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (src[mid].row_off <= g) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// Short lists: a warp per tuple counts the tuples of its result that come before
+// it (tuples of a result differ, so the count is its place) and writes it there.
+// One launch instead of the 20 or more of a radix sort: 400 tuples of 3 take 5 us
+// (the whole fetch on 20k vertices: 250 -> 32 us, with scratch from the graph's pool).
+__global__ void __launch_bounds__(256) k_rank_rows(const PackSrc* src, PackSrc one, int nres, uint64_t total,
+                                                   int32_t* out) {
+    const int lane = threadIdx.x & 31;
+    for (uint64_t g = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; g < total;
+         g += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
+        PackSrc s = one;
+        uint64_t end = total;
+        if (src) {
+            const int i = src_of(src, nres, g);
+            s = src[i];
+            end = src[i + 1].row_off;
+        }
+        const int k = s.k;
+        const int32_t* const mine = s.p + (g - s.row_off) * k;
+        const int32_t first = mine[0];
+        const uint32_t rows = (uint32_t)(end - s.row_off);
+        uint32_t before = 0;
+        for (uint32_t j = lane; j < rows; j += 32) {
+            const int32_t* const row = s.p + (uint64_t)j * k;
+            const int32_t a = row[0];
+            if (a != first) {
+                before += a < first;
+            } else {
+                int c = 1;
+                while (c < k && row[c] == mine[c]) c++;
+                before += c < k && row[c] < mine[c];
+            }
+        }
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (lane < k) out[s.int_off + (uint64_t)before * k + lane] = mine[lane];
+    }
+}
+// Pairs of tuples compared at most (the sum of the results' squared counts):
+// 2^26 pairs take 60 us, about what a radix sort takes at its smallest.
+constexpr uint64_t RANK_PAIRS = 1ull << 26;
+
 __global__ void k_iota(uint32_t* p, uint64_t n) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
         p[i] = (uint32_t)i;
 }
 
-// key[i] = (t[perm[i]][c0] << 32) | t[perm[i]][c1]  (c0 < 0: high half zero)
-__global__ void k_gather_key(const int32_t* t, int k, const uint32_t* perm, uint64_t n, int c0, int c1, uint64_t* key) {
+// Long lists: least-significant-first stable radix sorts of a carried permutation.
+// The sort key of a row is the bit string of its columns, most significant first:
+// the result's number (rbits), then k ids of vbits each; a pass sorts bits
+// [b0, b0 + 64) of it, so that no pass is spent on bits that no id has.
+__global__ void k_gather_key(const int32_t* t, int W, int rbits, int vbits, const uint32_t* perm, uint64_t n, int b0,
+                             uint64_t* key) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const int32_t* row = t + (uint64_t)perm[i] * k;
-        const uint64_t hi = c0 >= 0 ? (uint64_t)(uint32_t)row[c0] : 0;
-        key[i] = (hi << 32) | (uint64_t)(uint32_t)row[c1];
+        const int32_t* row = t + (uint64_t)perm[i] * W;
+        uint64_t x = 0;
+        int at = -b0;  // position of the column's lowest bit in the key
+        for (int c = W - 1; c >= 0 && at < 64; c--) {
+            const int bits = c == 0 && rbits >= 0 ? rbits : vbits;
+            const uint64_t v = (uint32_t)row[c];
+            if (at + bits > 0) x |= at >= 0 ? v << at : v >> -at;
+            at += bits;
+        }
+        key[i] = x;
     }
 }
 
@@ -1446,26 +1540,13 @@ __global__ void k_gather_rows(const int32_t* t, int k, const uint32_t* perm, uin
 // width W = 1 + max k, column 0 the result's index (most significant), the
 // tuple after it (zero-padded; only rows of the same result are ever compared
 // past column 0).
-struct PackSrc {
-    const int32_t* p;   // the result's unsorted tuples
-    int32_t k;
-    int32_t pad;
-    uint64_t row_off;   // first row of the result in the matrix (and in sorted order)
-    uint64_t int_off;   // first int of the result in the packed output
-};
-
 __global__ void k_pack_multi(const PackSrc* src, int nres, uint64_t total, int W, int32_t* M) {
     for (uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; g < total; g += (uint64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = nres;  // src[lo].row_off <= g < src[hi].row_off (src[nres] = total)
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (src[mid].row_off <= g) lo = mid;
-            else hi = mid;
-        }
-        const PackSrc s = src[lo];
+        const int i = src_of(src, nres, g);
+        const PackSrc s = src[i];
         const uint64_t local = g - s.row_off;
         int32_t* row = M + g * W;
-        row[0] = lo;
+        row[0] = i;
         for (int c = 0; c < W - 1; c++) row[1 + c] = c < s.k ? s.p[local * s.k + c] : 0;
     }
 }
@@ -1480,6 +1561,56 @@ __global__ void k_unpack_multi(const PackSrc* src, const int32_t* M, int W, cons
     }
 }
 
+// Scratch of a sort: one allocation of the result's pool.
+struct SortScratch {
+    Layout L;
+    uint8_t* base = nullptr;
+    cudaStream_t st;
+    explicit SortScratch(cudaStream_t s) : st(s) { L.size = 0; }
+    int alloc(const gfd_result* r) {
+        void* p = nullptr;
+        if (int rc = pool_alloc(r->mem->pool->p, L.size, st, &p, "violation sort")) return rc;
+        base = (uint8_t*)p;
+        return GFD_OK;
+    }
+    ~SortScratch() {
+        if (base) cudaFreeAsync(base, st);
+    }
+};
+
+// Permutation that sorts the n rows of t (width W, `bits` key bits in all, rbits
+// of column 0 or -1 when it is an id like the others).
+struct RadixRows {
+    size_t o_p0, o_p1, o_k0, o_k1, o_tmp, tmp_bytes = 0;
+    int plan(uint64_t n, SortScratch* S) {
+        cub::DoubleBuffer<uint64_t> kb(nullptr, nullptr);
+        cub::DoubleBuffer<uint32_t> pb(nullptr, nullptr);
+        GFD_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, kb, pb, (int64_t)n, 0, 64, S->st));
+        o_p0 = S->L.take(4 * n);
+        o_p1 = S->L.take(4 * n);
+        o_k0 = S->L.take(8 * n);
+        o_k1 = S->L.take(8 * n);
+        o_tmp = S->L.take(tmp_bytes);
+        return GFD_OK;
+    }
+    int sort(const int32_t* t, int W, int rbits, int vbits, uint64_t n, int grid, const SortScratch& S, uint32_t** perm) {
+        cub::DoubleBuffer<uint64_t> kb((uint64_t*)(S.base + o_k0), (uint64_t*)(S.base + o_k1));
+        cub::DoubleBuffer<uint32_t> pb((uint32_t*)(S.base + o_p0), (uint32_t*)(S.base + o_p1));
+        k_iota<<<grid, 256, 0, S.st>>>(pb.Current(), n);
+        const int bits = rbits >= 0 ? rbits + (W - 1) * vbits : W * vbits;
+        for (int b0 = 0; b0 < bits; b0 += 64) {
+            k_gather_key<<<grid, 256, 0, S.st>>>(t, W, rbits, vbits, pb.Current(), n, b0, kb.Current());
+            GFD_CUDA(cub::DeviceRadixSort::SortPairs(S.base + o_tmp, tmp_bytes, kb, pb, (int64_t)n, 0,
+                                                     std::min(64, bits - b0), S.st));
+        }
+        *perm = pb.Current();
+        return GFD_OK;
+    }
+};
+
+int rows_grid(uint64_t n) { return (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)device_sms() * 16); }
+int rank_grid(uint64_t n) { return (int)std::min<uint64_t>((n + 7) / 8, (uint64_t)device_sms() * 8); }
+
 }  // namespace
 
 // Device-to-host copy of results into caller memory, synchronous. (A staged
@@ -1493,8 +1624,7 @@ int copy_to_host(void* dst, const void* src, size_t bytes, cudaStream_t st) {
 }
 
 // Lexicographic order of the violation tuples (Vio is a set; this fixes a
-// canonical order): least-significant-first stable radix sorts over pairs of
-// columns, carrying a permutation.
+// canonical order).
 int result_fetch(gfd_result* r) {
     if (r->fetched) return GFD_OK;
     const uint64_t n = r->n_viol;
@@ -1518,56 +1648,40 @@ int result_sort_copy(gfd_result* r, int32_t* dst) {
     const int k = r->k;
     if (n == 0) return GFD_OK;
     cudaStream_t st = r->stream;
-    uint32_t *p0, *p1;
-    uint64_t *k0, *k1;
-    int32_t* sorted;
-    GFD_CUDA(cudaMallocAsync((void**)&p0, 4 * n, st));
-    GFD_CUDA(cudaMallocAsync((void**)&p1, 4 * n, st));
-    GFD_CUDA(cudaMallocAsync((void**)&k0, 8 * n, st));
-    GFD_CUDA(cudaMallocAsync((void**)&k1, 8 * n, st));
-    GFD_CUDA(cudaMallocAsync((void**)&sorted, 4 * n * k, st));
-    const int grid = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)device_sms() * 16);
-    k_iota<<<grid, 256, 0, st>>>(p0, n);
-    size_t tb = 0;
-    cub::DoubleBuffer<uint64_t> kb(k0, k1);
-    cub::DoubleBuffer<uint32_t> pb(p0, p1);
-    GFD_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, kb, pb, (int64_t)n, 0, 64, st));
-    void* tmp;
-    GFD_CUDA(cudaMallocAsync(&tmp, tb, st));
-    int rc = GFD_OK;
-    for (int c1 = k - 1; c1 >= 0; c1 -= 2) {
-        const int c0 = c1 - 1;
-        k_gather_key<<<grid, 256, 0, st>>>(r->d_viol, k, pb.Current(), n, c0, c1, kb.Current());
-        cudaError_t e = cub::DeviceRadixSort::SortPairs(tmp, tb, kb, pb, (int64_t)n, 0, c0 >= 0 ? 64 : 32, st);
-        if (e != cudaSuccess) {
-            rc = cuda_fail(e, "cub::DeviceRadixSort::SortPairs");
-            break;
-        }
+    SortScratch S(st);
+    const bool rank = n <= RANK_PAIRS / n;
+    RadixRows R;
+    if (!rank)
+        if (int rc = R.plan(n, &S)) return rc;
+    const size_t o_out = S.L.take(4 * n * k);
+    if (int rc = S.alloc(r)) return rc;
+    int32_t* sorted = (int32_t*)(S.base + o_out);
+    if (rank) {
+        k_rank_rows<<<rank_grid(n), 256, 0, st>>>(nullptr, PackSrc{r->d_viol, k, 0, 0, 0}, 1, n, sorted);
+    } else {
+        uint32_t* perm = nullptr;
+        if (int rc = R.sort(r->d_viol, k, -1, r->vbits, n, rows_grid(n), S, &perm)) return rc;
+        k_gather_rows<<<rows_grid(n), 256, 0, st>>>(r->d_viol, k, perm, n, sorted);
     }
-    if (rc == GFD_OK) {
-        k_gather_rows<<<grid, 256, 0, st>>>(r->d_viol, k, pb.Current(), n, sorted);
-        rc = copy_to_host(dst, sorted, 4 * n * k, st);
-    }
-    cudaFreeAsync(tmp, st);
-    cudaFreeAsync(p0, st);
-    cudaFreeAsync(p1, st);
-    cudaFreeAsync(k0, st);
-    cudaFreeAsync(k1, st);
-    cudaFreeAsync(sorted, st);
-    return rc;
+    GFD_CUDA(cudaGetLastError());
+    return copy_to_host(dst, sorted, 4 * n * k, st);
 }
 
 int results_sort_copy(gfd_result* const* rs, int n, int32_t* out, uint64_t capacity) {
     std::vector<PackSrc> src((size_t)n + 1);
-    uint64_t total = 0, ints = 0;
-    int kmax = 1;
+    uint64_t total = 0, ints = 0, pairs = 0;
+    int kmax = 1, vbits = 1;
     cudaStream_t st = nullptr;
+    const gfd_result* any = nullptr;
     for (int r = 0; r < n; r++) {
         src[r] = PackSrc{rs[r]->d_viol, rs[r]->k, 0, total, ints};
         total += rs[r]->n_viol;
         ints += rs[r]->n_viol * (uint64_t)rs[r]->k;
         kmax = std::max(kmax, rs[r]->k);
-        if (rs[r]->n_viol && !st) st = rs[r]->stream;
+        vbits = std::max(vbits, rs[r]->vbits);
+        pairs += rs[r]->n_viol < RANK_PAIRS ? rs[r]->n_viol * rs[r]->n_viol : RANK_PAIRS + 1;
+        pairs = std::min(pairs, RANK_PAIRS + 1);
+        if (rs[r]->n_viol && !any) any = rs[r];
     }
     src[n] = PackSrc{nullptr, 1, 0, total, ints};
     if (capacity < ints) {
@@ -1576,6 +1690,7 @@ int results_sort_copy(gfd_result* const* rs, int n, int32_t* out, uint64_t capac
         return GFD_ERR_INVALID_ARG;
     }
     if (total == 0) return GFD_OK;
+    st = any->stream;
     // Each result's violation list is written on the stream of the call that
     // made it (the split runs after that call returns). The sort runs on the
     // first such stream, so it first waits for every other one.
@@ -1597,51 +1712,34 @@ int results_sort_copy(gfd_result* const* rs, int n, int32_t* out, uint64_t capac
             if (int rc = result_sort_copy(rs[r], out + src[r].int_off)) return rc;
         return GFD_OK;
     }
+    SortScratch S(st);
+    const size_t o_src = S.L.take(sizeof(PackSrc) * ((size_t)n + 1)), o_out = S.L.take(4 * ints);
+    const bool rank = pairs <= RANK_PAIRS;
     const int W = kmax + 1;
-    PackSrc* d_src;
-    uint32_t *p0, *p1;
-    uint64_t *k0, *k1;
-    int32_t *M, *dout;
-    GFD_CUDA(cudaMallocAsync((void**)&d_src, sizeof(PackSrc) * ((size_t)n + 1), st));
-    GFD_CUDA(cudaMallocAsync((void**)&M, 4ull * total * W, st));
-    GFD_CUDA(cudaMallocAsync((void**)&p0, 4 * total, st));
-    GFD_CUDA(cudaMallocAsync((void**)&p1, 4 * total, st));
-    GFD_CUDA(cudaMallocAsync((void**)&k0, 8 * total, st));
-    GFD_CUDA(cudaMallocAsync((void**)&k1, 8 * total, st));
-    GFD_CUDA(cudaMallocAsync((void**)&dout, 4 * ints, st));
+    RadixRows R;
+    size_t o_M = 0;
+    if (!rank) {
+        if (int rc = R.plan(total, &S)) return rc;
+        o_M = S.L.take(4ull * total * W);
+    }
+    if (int rc = S.alloc(any)) return rc;
+    PackSrc* d_src = (PackSrc*)(S.base + o_src);
+    int32_t* dout = (int32_t*)(S.base + o_out);
     GFD_CUDA(cudaMemcpyAsync(d_src, src.data(), sizeof(PackSrc) * ((size_t)n + 1), cudaMemcpyHostToDevice, st));
-    const int grid = (int)std::min<uint64_t>((total + 255) / 256, (uint64_t)device_sms() * 16);
-    k_pack_multi<<<grid, 256, 0, st>>>(d_src, n, total, W, M);
-    k_iota<<<grid, 256, 0, st>>>(p0, total);
-    size_t tb = 0;
-    cub::DoubleBuffer<uint64_t> kb(k0, k1);
-    cub::DoubleBuffer<uint32_t> pb(p0, p1);
-    GFD_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, kb, pb, (int64_t)total, 0, 64, st));
-    void* tmp;
-    GFD_CUDA(cudaMallocAsync(&tmp, tb, st));
-    int rc = GFD_OK;
-    for (int c1 = W - 1; c1 >= 0; c1 -= 2) {  // least significant pair of columns first
-        const int c0 = c1 - 1;
-        k_gather_key<<<grid, 256, 0, st>>>(M, W, pb.Current(), total, c0, c1, kb.Current());
-        cudaError_t e = cub::DeviceRadixSort::SortPairs(tmp, tb, kb, pb, (int64_t)total, 0, c0 >= 0 ? 64 : 32, st);
-        if (e != cudaSuccess) {
-            rc = cuda_fail(e, "cub::DeviceRadixSort::SortPairs");
-            break;
-        }
+    if (rank) {
+        k_rank_rows<<<rank_grid(total), 256, 0, st>>>(d_src, PackSrc{}, n, total, dout);
+    } else {
+        int32_t* M = (int32_t*)(S.base + o_M);
+        const int grid = rows_grid(total);
+        int rbits = 0;
+        while ((1ll << rbits) < n) rbits++;
+        k_pack_multi<<<grid, 256, 0, st>>>(d_src, n, total, W, M);
+        uint32_t* perm = nullptr;
+        if (int rc = R.sort(M, W, rbits, vbits, total, grid, S, &perm)) return rc;
+        k_unpack_multi<<<grid, 256, 0, st>>>(d_src, M, W, perm, total, dout);
     }
-    if (rc == GFD_OK) {
-        k_unpack_multi<<<grid, 256, 0, st>>>(d_src, M, W, pb.Current(), total, dout);
-        rc = copy_to_host(out, dout, 4 * ints, st);
-    }
-    cudaFreeAsync(tmp, st);
-    cudaFreeAsync(d_src, st);
-    cudaFreeAsync(M, st);
-    cudaFreeAsync(p0, st);
-    cudaFreeAsync(p1, st);
-    cudaFreeAsync(k0, st);
-    cudaFreeAsync(k1, st);
-    cudaFreeAsync(dout, st);
-    return rc;
+    GFD_CUDA(cudaGetLastError());
+    return copy_to_host(out, dout, 4 * ints, st);
 }
 
 }  // namespace gfd
