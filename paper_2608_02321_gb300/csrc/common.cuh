@@ -14,7 +14,7 @@
 //            popcount prefix [nwords] u32 (so rank(v) is O(1)), the sorted
 //            candidate list i32, and for every level i >= 1 the index edges of
 //            the spanning-tree edge (parent(i), i): off u32 [|C(parent)|+1],
-//            idx int2 [nnz] = (position in C(i), vertex id).
+//            idx int2 [nnz] = (position in C(i), vertex id), u32 ids at the last level.
 //   frontier: per (GFD, level l >= 1) a buffer of partial matches, row-major
 //            [chunk][2(l+1)+2] i32 = l+1 vertex ids, l+1 candidate positions, the
 //            generator chosen for level l+1 and the start of the parent's index
@@ -64,6 +64,12 @@ struct DevGraph {
     // out-neighbour w of v, sig[v].y for every in-neighbour; a clear bit proves
     // that the edge is absent
     const ulonglong2* sig;
+    // row filters: 8 bits per adjacency entry; the bits [8 off[x], 8 off[x + 1]) are
+    // a one-hash Bloom filter of x's list (filter_bit), so about 12 % of the vertices
+    // that are not in a list have their bit set, however long it is (a 64-bit
+    // signature is full from a hundred neighbours on)
+    const uint8_t* out_filter;
+    const uint8_t* in_filter;
     uint32_t class_end[N_CLASS - 1];  // ends of the first degree classes
     // the caller's id of each vertex, and vertex data in the caller's order
     const uint32_t* orig;
@@ -75,6 +81,12 @@ struct DevGraph {
 // Signature bit of a vertex id: the top 6 bits of a Fibonacci (multiplicative)
 // hash.
 __host__ __device__ __forceinline__ uint32_t sig_bit(uint32_t v) { return (v * 0x9E3779B1u) >> 26; }
+
+// Bit of vertex v in the filter of a row with d entries.
+__host__ __device__ __forceinline__ uint32_t filter_bit(uint32_t v, uint32_t d) {
+    const uint32_t bits = 8u * (d < (1u << 28) ? d : 1u << 28);
+    return (uint32_t)(((uint64_t)(v * 0x9E3779B1u) * bits) >> 32);
+}
 
 // Candidate filter key (Section III.B step 1a-1b): label, degree lower bounds
 // (self-loops excluded on both sides) and the self-loop expectation.
@@ -136,16 +148,22 @@ struct SlotDesc {
     const uint32_t* cand_n[MAXK];  // number of candidates
     uint32_t cand_cap[MAXK];
     uint32_t* cpi_off[MAXK];  // level i >= 1
-    int2* cpi_idx[MAXK];      // (position in C(i), vertex id) per index edge
+    int2* cpi_idx[MAXK];      // (position in C(i), vertex id) per index edge; at the last level,
+                              // where no position is needed, the vertex ids alone (u32)
     uint64_t cpi_cap[MAXK];
     // frontier
     int32_t* rows[MAXK];      // level l >= 1
     uint64_t* wpre[MAXK];     // level l >= 1
-    uint64_t chunk;           // max work items per step (= row capacity)
+    uint64_t chunk;           // row capacity of each (= work items per step that may each give a row)
+    // the same in one of the run's large buffers (byte offsets), see Sched::big_owner
+    uint64_t big_rows[MAXK], big_wpre[MAXK];
+    uint64_t big_chunk;
     // violation output of this slot (serving); null: the run's shared arena
     int32_t* viol;
     uint64_t viol_cap;
 };
+
+constexpr int N_BIG = 4;
 
 // Mutable per-slot state (device).
 struct SlotState {
@@ -156,11 +174,17 @@ struct SlotState {
     uint64_t total[MAXK];     // work items at level l
     uint64_t cursor[MAXK];    // work items of level l already expanded
     uint64_t ctr[MAXK];       // packed rows/work counter of level l (filled by l-1)
+    uint64_t row_limit;       // counter value of the first rows of the step that found no room (~0: none)
     uint64_t cb, ce;          // current step's work range at level `cur`
     uint64_t n_matches;
     uint64_t n_viol;
     uint64_t st_work, st_rows, st_probes, st_steps, st_cpi;
     uint32_t tile;            // work items per tile in the current step
+    uint32_t big;             // large buffer the slot holds + 1, 0 none
+    // partial matches of level l: where they are, and how many fit
+    int32_t* rows[MAXK];
+    uint64_t* wpre[MAXK];
+    uint64_t cap[MAXK];
 };
 
 // Counters of the counting pass (GFD_FLAG_COUNT): what one run's kernels
@@ -216,6 +240,10 @@ struct Sched {
     uint64_t varena_used;
     int32_t vstride;
     int32_t pad2;
+    // Large frontier buffers of a batch: slots that are still running when no
+    // more than N_BIG are take one each (its holder + 1, 0 free), since their own
+    // share of the budget is a small part of it.
+    uint32_t big_owner[N_BIG];
     uint64_t cnt[N_CNT];      // counting pass only
     // next tile of the current step handed out to a warp that finished its
     // first one (tiles below the warp count go to warps by index); on its own

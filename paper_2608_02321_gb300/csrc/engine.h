@@ -158,7 +158,8 @@ struct CpiJob {          // index edges of one spanning-tree edge
     const uint32_t* cbm;
     const uint32_t* crank;
     uint32_t* off;
-    int2* idx;               // (position in C(child), vertex id)
+    int2* idx;               // (position in C(child), vertex id); ids: only the vertex ids (u32)
+    int32_t ids;
     uint64_t cap;
     int32_t out;             // 1: children are out-neighbours of the parent candidates
     int32_t lab;
@@ -208,6 +209,10 @@ struct EnumArgs {
     int32_t n_slots;
     int32_t tile;         // largest number of work items per tile
     int32_t n_warps;      // warps of the expansion grid (0: unknown, tiles of `tile`)
+    int32_t kmax;         // nodes of the largest pattern a slot may hold
+    uint8_t* big;         // N_BIG large frontier buffers of big_bytes each (null: none)
+    uint64_t big_bytes;
+    uint32_t columns;     // words of a warp's columns in shared memory (set at launch)
 };
 int enum_init(const EnumArgs& a, cudaStream_t st);
 // Mark slots [0, n) idle; start the listed slots (host ids) after their index is built.

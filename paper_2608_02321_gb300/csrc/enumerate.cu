@@ -39,7 +39,7 @@ namespace gfd {
 namespace {
 
 constexpr int CTRL_THREADS = 1024;
-constexpr uint64_t LAST_LEVEL_CHUNK = 1ull << 25;  // work items per step at the last level
+constexpr uint64_t LAST_LEVEL_CHUNK = 1ull << 25;  // work items per step at the last two levels
 // generator stored in a row for a next level that starts a pattern component:
 // its candidates are the level's candidate list (fan-out |C| for every row)
 constexpr int GEN_LIST = 4;
@@ -133,21 +133,9 @@ __device__ __forceinline__ int32_t edge_label(const DevGraph& g, uint32_t a, uin
     return NOEDGE;
 }
 
-// m: the partial match in shared memory, level q at m[32 q] (one column per lane)
-__device__ __forceinline__ bool lit_holds(const DevGraph& g, const DevLit& L, const uint32_t* m,
-                                          uint32_t* reads = nullptr) {
-    if (reads) ++*reads;
-    const int32_t va = __ldg(g.attrs + (uint64_t)L.a * g.n + m[L.xl << 5]);
-    if (va == GFD_ATTR_ABSENT) return false;
-    if (L.kind == 0) return va == L.c;
-    if (reads) ++*reads;
-    const int32_t vb = __ldg(g.attrs + (uint64_t)L.b * g.n + m[L.yl << 5]);
-    return vb != GFD_ATTR_ABSENT && va == vb;
-}
-
-// The same with the vertex of level lv given in a register (v) instead of the
-// shared-memory column (used when another lane's column holds the earlier
-// levels).
+// A partial match is a column in shared memory: level q at m[32 q]. Vertex of
+// level q when that of level lv is given in a register (v) and the column holds
+// the earlier ones.
 __device__ __forceinline__ uint32_t level_vertex(const uint32_t* m, int q, int lv, uint32_t v) {
     return q == lv ? v : m[q << 5];
 }
@@ -167,32 +155,10 @@ __device__ __forceinline__ bool lit_holds_at(const DevGraph& g, const DevLit& L,
 // without being stored.
 constexpr uint32_t FUSE_FANOUT = 64;
 // Tiles of a step that fuses the last level are this many times smaller.
-constexpr uint64_t FUSED_TILE_DIV = 2;
+constexpr uint64_t FUSED_TILE_DIV = 4;
 // Number the last level's tiles after the other intermediate levels' (else
 // both are numbered together, in slot order).
 constexpr bool LAST_LEVEL_TILES_LAST = true;
-
-// Largest r in [0, n) with S[r] <= w (S non-decreasing, S[0] <= w). The index
-// offsets are read-only during enumeration; the frontier prefix is rewritten
-// between steps, so it is read through L2 only (ld.global.cg).
-__device__ __forceinline__ uint32_t find_row(const uint32_t* S, uint64_t n, uint64_t w) {
-    uint64_t lo = 0, hi = n;  // invariant: S[lo] <= w, answer in [lo, hi)
-    while (hi - lo > 1) {
-        const uint64_t mid = (lo + hi) >> 1;
-        if ((uint64_t)__ldg(S + mid) <= w) lo = mid;
-        else hi = mid;
-    }
-    return (uint32_t)lo;
-}
-__device__ __forceinline__ uint32_t find_row(const uint64_t* S, uint64_t n, uint64_t w) {
-    uint64_t lo = 0, hi = n;
-    while (hi - lo > 1) {
-        const uint64_t mid = (lo + hi) >> 1;
-        if (__ldcg((const unsigned long long*)S + mid) <= w) lo = mid;
-        else hi = mid;
-    }
-    return (uint32_t)lo;
-}
 
 // Loads of data rewritten between steps (frontier rows and prefixes, the
 // per-step tile prefix): plain weak loads, which may be served from L1. In the
@@ -228,6 +194,12 @@ __device__ __forceinline__ uint32_t find_row_in(const uint64_t* S, uint32_t lo, 
 // a's bit in b's in-signature, so either clear bit proves it absent.
 __device__ __forceinline__ uint64_t sig_half(const DevGraph& g, uint32_t x, int half) {
     return __ldg(reinterpret_cast<const unsigned long long*>(g.sig) + 2 * (uint64_t)x + half);
+}
+
+// May v be in the adjacency row [e0, e0 + d) of x (in: its in-neighbours)?
+__device__ __forceinline__ bool row_filter(const DevGraph& g, bool in, uint32_t e0, uint32_t d, uint32_t v) {
+    const uint32_t bit = filter_bit(v, d);
+    return (__ldg((in ? g.in_filter : g.out_filter) + e0 + (bit >> 3)) >> (bit & 7)) & 1u;
 }
 
 // position of v in the sorted candidate list of a level: O(1) from the bitmap
@@ -266,6 +238,140 @@ __device__ __forceinline__ uint64_t warp_excl_scan(uint64_t x, int lane, uint64_
     return incl - x;
 }
 
+// The adjacency row of the first required edge (besides the generator's) at its
+// image; d = 0: there is none.
+struct NeededRow {
+    uint32_t e0, d;
+};
+
+// Per warp in (dynamic) shared memory.
+struct WarpShared {
+    uint32_t chk[2 * MAXK];   // the current tile's pair checks, packed
+    uint32_t chk2[2 * MAXK];  // the last level's, for fused expansion
+    int2 list[32];            // fused expansion: a partial match's candidates (see below)
+    uint64_t need[32];        // signature bits a candidate of the lane's partial match needs
+    NeededRow row[32];        // and the row it must be in
+    int32_t* rows;            // where the tile's new partial matches go
+    uint64_t* wpre;
+    uint64_t cap;
+    uint64_t unused;
+    uint32_t qv[64];          // candidates that have them, waiting for their other checks,
+    uint8_t qo[64];           // and whose they are: lane | generator << 5
+    __device__ uint32_t* m(int col) { return reinterpret_cast<uint32_t*>(this + 1) + col; }  // [32 q + col]: the columns
+};
+// columns for patterns of up to kmax nodes (rows are loaded in groups of four)
+__host__ __device__ constexpr int column_words(int kmax) { return ((kmax + 3) & ~3) * 32; }
+constexpr size_t warp_shared_bytes(int kmax) { return sizeof(WarpShared) + 4 * (size_t)column_words(kmax); }
+
+// Every pattern pair of v, the candidate of a level, with the earlier images in
+// the column m, but check `skip`: the n packed checks cw, the first nreq of them
+// required edges. v's signature comes first (one load for all pairs): a clear bit
+// settles an absent edge and refutes a required one. Only the pairs it leaves
+// open look into the other end's row filter, and only those that leaves open
+// search the shorter adjacency list.
+template <bool COUNT>
+__device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m, const uint32_t* cw, int n, int nreq,
+                                            int skip, uint32_t v, uint32_t& probes, Counters<COUNT>& cn) {
+    if (n == 0) return true;
+    const ulonglong2 sv = __ldg(g.sig + v);  // out-, in-neighbours
+    cn.add(CNT_SIG_LOADS, 1);
+    uint32_t open = 0;
+    for (int c = 0; c < n; c++) {
+        const uint32_t wd = cw[c];
+        const uint32_t x = m[(wd & 15u) << 5];
+        const uint64_t half = (wd >> 4) & 1u ? sv.x : sv.y;  // edge v -> x, else x -> v
+        open |= (uint32_t)((half >> sig_bit(x)) & 1ull) << c;
+        if (COUNT && c != skip) {
+            cn.add(CNT_CHECKS, 1);
+            if (c >= nreq) {
+                const bool out = (wd >> 4) & 1u;
+                const uint32_t dv = out ? g.out_off[v + 1] - g.out_off[v] : g.in_off[v + 1] - g.in_off[v];
+                const uint32_t dx = out ? g.in_off[x + 1] - g.in_off[x] : g.out_off[x + 1] - g.out_off[x];
+                cn.add(CNT_NEG_CHECKS, 1);
+                cn.add(CNT_NEG_LOGD, ceil_log2_1(min(dv, dx)));
+            }
+        }
+    }
+    uint32_t required = (1u << nreq) - 1u;  // (at most 2 (MAXK - 1) = 30 checks)
+    if (skip >= 0) {
+        open &= ~(1u << skip);
+        required &= ~(1u << skip);
+    }
+    probes += n - (skip >= 0);
+    if (COUNT) cn.add(CNT_SIG_SETTLED, n - (skip >= 0) - __popc(open));
+    if ((open & required) != required) return false;
+    for (; open; open &= open - 1) {
+        const int c = __ffs(open) - 1;
+        const uint32_t wd = cw[c];
+        const uint32_t x = m[(wd & 15u) << 5];
+        const bool out = (wd >> 4) & 1u;
+        const int32_t ex = (int32_t)(int16_t)(wd >> 16);
+        int32_t gl = NOEDGE;
+        cn.add(CNT_SIG_LOADS, 1);
+        const uint32_t* const off = out ? g.in_off : g.out_off;
+        const uint32_t e0 = __ldg(off + x), e1 = __ldg(off + x + 1);
+        if (e0 < e1 && row_filter(g, out, e0, e1 - e0, v)) {
+            cn.add(CNT_SEARCHES, 1);
+            gl = out ? edge_label(g, v, g.out_off[v], g.out_off[v + 1], x, e0, e1, cn.loads())
+                     : edge_label(g, x, e0, e1, v, g.in_off[v], g.in_off[v + 1], cn.loads());
+        } else {
+            cn.add(CNT_SIG_SETTLED, 1);
+        }
+        if (!exp_ok(ex, gl)) return false;
+    }
+    return true;
+}
+
+// Does the spanning-tree edge between v and its parent's image xp agree? (v comes
+// from another generator than the parent's index edges.)
+template <bool COUNT>
+__device__ __forceinline__ bool tree_edge_agrees(const DevGraph& g, const LevelPlan& P, uint32_t xp, uint32_t v,
+                                                 uint32_t& probes, Counters<COUNT>& cn) {
+    // the parent's signature first, then v's
+    bool maybe = (sig_half(g, xp, P.tdir ? 0 : 1) >> sig_bit(v)) & 1ull;
+    cn.add(CNT_SIG_LOADS, 1);
+    if (maybe) {
+        maybe = (sig_half(g, v, P.tdir ? 1 : 0) >> sig_bit(xp)) & 1ull;
+        cn.add(CNT_SIG_LOADS, 1);
+    }
+    int32_t gl = NOEDGE;
+    cn.add(CNT_CHECKS, 1);
+    if (maybe) {
+        cn.add(CNT_SEARCHES, 1);
+        gl = P.tdir ? edge_label(g, xp, g.out_off[xp], g.out_off[xp + 1], v, g.in_off[v], g.in_off[v + 1], cn.loads())
+                    : edge_label(g, v, g.out_off[v], g.out_off[v + 1], xp, g.in_off[xp], g.in_off[xp + 1], cn.loads());
+    } else {
+        cn.add(CNT_SIG_SETTLED, 1);
+    }
+    probes++;
+    return exp_ok(P.tlab, gl);
+}
+
+// Signature bits that a candidate of level P needs for its required edges to the
+// images in column m, when its candidates come from generator gen (whose own
+// check, or for gen 0 the tree edge, holds already).
+// row: where the first of these edges is looked up in the row filter, which tells
+// more than a long list's signature.
+__device__ __forceinline__ uint64_t needed_bits(const DevGraph& g, const LevelPlan& P, const uint32_t* m,
+                                                const uint32_t* cw, int gen, NeededRow* row) {
+    uint64_t need = ~0ull;
+    *row = NeededRow{0, 0};
+    const int skip = gen >= 1 && gen != GEN_LIST ? P.gen[gen - 1] : -1;
+    if (skip >= 0) need = sig_half(g, m[P.par << 5], P.tdir ? 0 : 1);
+    for (int c = P.nreq - 1; c >= 0; c--) {
+        if (c == skip) continue;
+        const uint32_t x = m[(cw[c] & 15u) << 5];
+        const bool in = (cw[c] >> 4) & 1u;  // edge v -> x: v among x's in-neighbours
+        need &= sig_half(g, x, in);
+        if (c == (skip == 0)) {
+            const uint32_t* const off = in ? g.in_off : g.out_off;
+            row->e0 = __ldg(off + x);
+            row->d = __ldg(off + x + 1) - row->e0;
+        }
+    }
+    return need;
+}
+
 // The expansion step, warp-synchronous: every warp takes its own tiles of
 // work items (no block-wide barrier in the loop). A tile belongs to one slot
 // and one level; the warp finds them (and the rows the tile covers) with
@@ -273,20 +379,24 @@ __device__ __forceinline__ uint64_t warp_excl_scan(uint64_t x, int lane, uint64_
 // GEN = false: the common case (connected patterns, X checked at the last
 // level only), compiled without the general paths so that it keeps its
 // registers; GEN = true adds component starts and X pushed down.
+//
+// The last level has most of the work items, and most fail their first required
+// edge. So its candidates pass two stages: every lane fetches one and tests the
+// signature bits that the partial match's required edges need together (one
+// 64-bit mask per partial match, `need`), some 40 instructions per 32 candidates;
+// those that pass wait in a queue until 32 are together for the other checks,
+// the literals and the output, which then run with full warps.
 template <int NT, bool GEN, bool COUNT>
 __device__ void expand_warps(const EnumArgs& A) {
-    // Per warp in shared memory: the lanes' partial matches (level q of lane t
-    // at [32 q + t], so the lanes' dynamically indexed reads hit distinct
-    // banks) and the current tile's pair checks, packed.
-    __shared__ uint32_t s_m[NT / 32][MAXK * 32];
-    __shared__ uint32_t s_chk[NT / 32][2 * MAXK];
-    __shared__ uint32_t s_chk2[NT / 32][2 * MAXK];  // the last level's, for fused expansion
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    WarpShared& W = *reinterpret_cast<WarpShared*>(s_dyn + (threadIdx.x >> 5) * (sizeof(WarpShared) + 4u * A.columns));
     Counters<COUNT> cn;
     uint32_t attr_reads = 0;
     const int lane = threadIdx.x & 31;
-    uint32_t* const m = &s_m[threadIdx.x >> 5][lane];
-    uint32_t* const cw = s_chk[threadIdx.x >> 5];
-    uint32_t* const cw2 = s_chk2[threadIdx.x >> 5];
+    const uint32_t below = (1u << lane) - 1u;
+    uint32_t* const m = W.m(lane);
+    uint32_t* const cw = W.chk;
+    uint32_t* const cw2 = W.chk2;
     const uint64_t gwarp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const DevGraph& g = A.g;
@@ -314,10 +424,15 @@ __device__ void expand_warps(const EnumArgs& A) {
         const int nchk = LP.nchk;
         __syncwarp();  // the previous tile's checks are no longer read
         if (lane < nchk) cw[lane] = LP.chk_w[lane];
+        if (lane == 0 && !last) {
+            W.rows = (int32_t*)__ldcg((const unsigned long long*)&S->rows[i]);
+            W.wpre = (uint64_t*)__ldcg((const unsigned long long*)&S->wpre[i]);
+            W.cap = __ldcg((const unsigned long long*)&S->cap[i]);
+        }
         __syncwarp();
         const uint32_t* S0 = i > 0 ? D->cpi_off[i] : nullptr;
-        const uint64_t* Sl = l >= 1 ? D->wpre[l] : nullptr;
-        const int32_t* rows_l = l >= 1 ? D->rows[l] : nullptr;
+        const uint64_t* Sl = l >= 1 ? (const uint64_t*)__ldcg((const unsigned long long*)&S->wpre[l]) : nullptr;
+        const int32_t* rows_l = l >= 1 ? (const int32_t*)__ldcg((const unsigned long long*)&S->rows[l]) : nullptr;
         const uint64_t nrows = k == 1 ? 0 : (l == 0 ? (uint64_t)S->ncand[0]
                                                     : (uint64_t)__ldcg((const unsigned long long*)&S->nrows[l]));
         const int rw = row_width(l);  // ints per row at level l: ids, positions, generator, index base
@@ -337,15 +452,163 @@ __device__ void expand_warps(const EnumArgs& A) {
                 rhi1 = (uint32_t)nrows;
             }
         }
-        // The tile's items, compiled for the last level (literal check,
-        // violations) and for the others (fan-out, new partial matches), each
-        // for the roots (level 0: candidate list, 32-bit index offsets) and for
-        // stored partial matches (rows, 64-bit prefixes), so that no path
-        // carries another's registers.
+        uint32_t tile_matches = 0;
+        // Complete matches (ok lanes: v at the last level L, the earlier levels in
+        // column c): check the X literals of this level, count (with X pushed down
+        // only if they hold), check Y, emit violations.
+        auto finish = [&](bool ok, int L, uint32_t v, const uint32_t* c) {
+            bool viol = false;
+            if (ok) {
+                bool x_ok = true;
+                for (int q = 0; q < D->nx && x_ok; q++)
+                    if (!GEN || D->lit[q].lvl == L)
+                        x_ok = lit_holds_at(g, D->lit[q], c, L, v, COUNT ? &attr_reads : nullptr);
+                if (GEN) tile_matches += x_ok || !D->push_x;
+                else tile_matches++;
+                if (x_ok) {
+                    bool y_ok = !D->y_false;
+                    for (int q = 0; q < D->ny && y_ok; q++)
+                        y_ok = lit_holds_at(g, D->lit[D->nx + q], c, L, v, COUNT ? &attr_reads : nullptr);
+                    viol = !y_ok;
+                }
+            }
+            const uint32_t vb = __ballot_sync(0xffffffffu, viol);
+            if (!vb) return;
+            unsigned long long base = 0;
+            if (lane == 0) {
+                const unsigned long long nv = __popc(vb);
+                const unsigned long long old = atomicAdd((unsigned long long*)&S->n_viol, nv);
+                base = D->viol ? old : atomicAdd((unsigned long long*)&A.sched->varena_used, nv);
+            }
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (viol) {
+                const uint64_t idx = base + __popc(vb & below);
+                if (D->viol) {
+                    // the slot's own buffer: tuples in pattern-node order
+                    if (idx < D->viol_cap) {
+                        int32_t* out = D->viol + idx * k;
+                        for (int q = 0; q < k; q++) out[D->order[q]] = (int32_t)__ldg(g.orig + level_vertex(c, q, L, v));
+                    }
+                } else if (idx < A.sched->varena_cap) {
+                    // the run's arena: [slot, tuple in pattern-node order]
+                    int32_t* rec = A.sched->varena + idx * A.sched->vstride;
+                    rec[0] = s;
+                    for (int q = 0; q < k; q++) rec[1 + D->order[q]] = (int32_t)__ldg(g.orig + level_vertex(c, q, L, v));
+                }
+            }
+        };
+        // First stage of the last level (plan P, level L): one candidate per lane
+        // (ok lanes: position e in the source of generator gen, needed bits), the
+        // ones that pass appended to the queue.
+        auto first_stage = [&](const LevelPlan& P, int L, uint32_t queued, bool ok, uint32_t e, int gen, int owner,
+                               const uint64_t need, const NeededRow row) -> uint32_t {
+            uint32_t v = 0;
+            if (ok) {
+                cn.add(CNT_ITEMS, 1);
+                cn.add(CNT_ITEMS_LAST, 1);
+                if (gen == 0) {
+                    v = __ldg(reinterpret_cast<const uint32_t*>(D->cpi_idx[L]) + e);  // ids only at the last level
+                } else if (GEN && gen == GEN_LIST) {
+                    v = (uint32_t)__ldg(D->cand[L] + e);
+                } else {
+                    // from the adjacency of the other end of a required back edge
+                    const int cg = P.gen[gen - 1];
+                    const uint32_t p = P.chk_dir[cg] ? __ldg(g.in_adj + e) : __ldg(g.out_adj + e);
+                    v = p >> g.lbits;
+                    ok = exp_ok(P.chk_exp[cg], (int32_t)(p & g.lmask));
+                }
+                ok = ok && ((need >> sig_bit(v)) & 1ull);
+                if (ok && row.d) {
+                    // the row's check: the first required one that is not the generator's
+                    const int c = gen >= 1 && gen != GEN_LIST && P.gen[gen - 1] == 0 ? 1 : 0;
+                    ok = row_filter(g, P.chk_dir[c], row.e0, row.d, v);
+                }
+                if (ok && gen != 0 && !(GEN && gen == GEN_LIST)) ok = (__ldg(D->bm[L] + (v >> 5)) >> (v & 31)) & 1u;
+            }
+            const uint32_t pass = __ballot_sync(0xffffffffu, ok);
+            if (ok) {
+                const uint32_t at = queued + __popc(pass & below);
+                W.qv[at] = v;
+                W.qo[at] = (uint8_t)(owner | gen << 5);
+            }
+            __syncwarp();
+            return queued + __popc(pass);
+        };
+        // Second stage: the other checks of queue entry `at` (ok lanes), finish.
+        auto second_stage = [&](const LevelPlan& P, int L, const uint32_t* checks, bool ok, uint32_t at) {
+            uint32_t v = 0;
+            const uint32_t* c = m;
+            if (ok) {
+                v = W.qv[at];
+                const int gen = W.qo[at] >> 5;
+                c = W.m(W.qo[at] & 31);
+                for (int q = 0; q < L && ok; q++)  // injectivity
+                    if (((P.inj >> q) & 1u) && c[q << 5] == v) ok = false;
+                const int skip = gen >= 1 && gen != GEN_LIST ? P.gen[gen - 1] : -1;
+                if (ok && skip >= 0) ok = tree_edge_agrees<COUNT>(g, P, c[P.par << 5], v, probes, cn);
+                ok = ok && pairs_agree<COUNT>(g, c, checks, P.nchk, P.nreq, skip, v, probes, cn);
+            }
+            finish(ok, L, v, c);
+        };
+        auto count_partial = [&](const LevelPlan& P, const uint32_t* c) {
+            // counting pass: the partial match is expanded once; a merge-based
+            // intersection would scan the adjacency of each backward non-tree
+            // neighbour's image
+            cn.add(CNT_PARTIALS, 1);
+            uint64_t bd = 0;
+            for (int q = 0; q < P.nreq; q++) {
+                const uint32_t x = c[P.chk_q[q] << 5];
+                bd += P.chk_dir[q] ? g.in_off[x + 1] - g.in_off[x] : g.out_off[x + 1] - g.out_off[x];
+            }
+            cn.add(CNT_BACK_DEG, bd);
+        };
+        // The last level of stored partial matches (more than FUSE_FANOUT
+        // candidates each), one row after the other: its vertices in column 0, so
+        // that every lane reads the same ones.
+        auto run_last_rows = [&] {
+            cn.cycles(CNT_CYC_TILE);
+            uint64_t w = wb;
+            for (uint32_t r = rlo; w < we; r++) {
+                const uint64_t start = ld_front(Sl + r);
+                const uint64_t end = r + 1 < rhi1 ? min(we, ld_front(Sl + r + 1)) : we;
+                const int32_t* const rowp = rows_l + (uint64_t)r * rw;
+                __syncwarp();  // the previous row is no longer read
+                if (lane <= l) *W.m(lane << 5) = (uint32_t)rowp[lane];
+                __syncwarp();
+                const int gen = rowp[2 * (l + 1)];
+                uint32_t base = (uint32_t)rowp[2 * (l + 1) + 1];
+                const uint32_t* const c0 = W.m(0);
+                if (gen >= 1 && !(GEN && gen == GEN_LIST)) {
+                    const int cg = LP.gen[gen - 1];
+                    const uint32_t x = c0[LP.chk_q[cg] << 5];
+                    base = LP.chk_dir[cg] ? __ldg(g.in_off + x) : __ldg(g.out_off + x);
+                }
+                if (COUNT && lane == 0 && w == start) count_partial(LP, c0);
+                NeededRow nrow;
+                const uint64_t need = needed_bits(g, LP, c0, cw, gen, &nrow);
+                uint32_t queued = 0;
+                while (w < end || queued) {
+                    if (w < end) {
+                        queued = first_stage(LP, i, queued, w + lane < end, base + (uint32_t)(w - start) + lane, gen, 0, need, nrow);
+                        w += 32;
+                        if (queued < 32 && w < end) continue;
+                    }
+                    const uint32_t take = min(queued, 32u);
+                    second_stage(LP, i, cw, lane < (int)take, queued - take + lane);
+                    queued -= take;
+                    __syncwarp();
+                    cn.iteration(true);
+                }
+                w = end;
+            }
+        };
+        // The tile's items at an intermediate level (or, with LAST, of the roots
+        // of a pattern of one or two nodes), compiled for the roots (level 0:
+        // candidate list, 32-bit index offsets) and for stored partial matches
+        // (rows, 64-bit prefixes), so that no path carries another's registers.
         auto run_tile = [&](auto last_tag, auto root_tag) {
             constexpr bool LAST = decltype(last_tag)::value;
             constexpr bool ROOT = decltype(root_tag)::value;  // expanding the roots (ROOT)
-            uint32_t tile_matches = 0;
             uint32_t cur = rlo;  // row of the first work item of the iteration
             // a tile that makes partial matches of the second-to-last level
             // expands the last level of those with small fan-outs at once
@@ -371,7 +634,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                 // back to a binary search (root candidates may have no fan-out).
                 uint64_t sr = 0;
                 if (list1) {
-                    r = ok ? (uint32_t)(w / c1) : 0u;
+                    r = GEN && ok ? (uint32_t)(w / max(c1, (uint64_t)1)) : 0u;
                     sr = (uint64_t)r * c1;
                 } else if (k > 1) {
                     const uint64_t widx = (uint64_t)cur + lane;
@@ -414,8 +677,8 @@ __device__ void expand_warps(const EnumArgs& A) {
                             m[0] = (uint32_t)D->cand[0][r];
                         } else {
                             // the row's ids in 16-byte loads (rows are padded to 16 B;
-                            // m has room for the LAST group), generator and index base
-                            // in one 8-byte load
+                            // the columns have room for the last group), generator and
+                            // index base in one 8-byte load
                             rowp = rows_l + (uint64_t)r * rw;
                             const int4* r4 = reinterpret_cast<const int4*>(rowp);
                             for (int q = 0; q <= l; q += 4) {
@@ -430,32 +693,16 @@ __device__ void expand_warps(const EnumArgs& A) {
                             ent = (uint32_t)gb.y + o;
                         }
                         int skip = -1;
-                        // the first pair check's earlier image is the same for all the
-                        // row's candidates: its signature half (the one that holds v
-                        // if the edge exists) is loaded while the candidate is fetched
-                        uint64_t sx0 = 0;
-                        if (nchk > 0) {
-                            const uint32_t w0c = cw[0];
-                            sx0 = sig_half(g, m[(w0c & 15u) << 5], (w0c >> 4) & 1u);
-                        }
-                        if (COUNT && o == 0) {
-                            // the row's first item: the partial match is expanded once;
-                            // a merge-based intersection would scan the adjacency of
-                            // each backward non-tree neighbour's image
-                            cn.add(CNT_PARTIALS, 1);
-                            uint64_t bd = 0;
-                            for (int c = 0; c < nchk; c++) {
-                                if (LP.chk_exp[c] == EXP_NONE) continue;
-                                const uint32_t x = m[LP.chk_q[c] << 5];
-                                bd += LP.chk_dir[c] ? g.in_off[x + 1] - g.in_off[x] : g.out_off[x + 1] - g.out_off[x];
-                            }
-                            cn.add(CNT_BACK_DEG, bd);
-                        }
+                        if (COUNT && o == 0) count_partial(LP, m);
                         if (choice == 0) {
                             // candidates from the index edges of the spanning-tree parent
-                            const int2 e = __ldg(D->cpi_idx[i] + ent);
-                            j = e.x;
-                            v = (uint32_t)e.y;
+                            if (LAST) {
+                                v = __ldg(reinterpret_cast<const uint32_t*>(D->cpi_idx[i]) + ent);
+                            } else {
+                                const int2 e = __ldg(D->cpi_idx[i] + ent);
+                                j = e.x;
+                                v = (uint32_t)e.y;
+                            }
                         } else if (GEN && choice == GEN_LIST) {
                             // the level starts a component: its candidate list
                             j = (int32_t)ent;
@@ -474,140 +721,32 @@ __device__ void expand_warps(const EnumArgs& A) {
                                  ((__ldg(D->bm[i] + (v >> 5)) >> (v & 31)) & 1u);
                             if (ok) {
                                 j = cand_rank(D->bm[i], D->rank[i], v);
-                                const uint32_t xp = m[LP.par << 5];
-                                // tree edge xp -> v (tdir 1) or v -> xp: the parent's
-                                // signature first, then v's
-                                bool maybe = (sig_half(g, xp, LP.tdir ? 0 : 1) >> sig_bit(v)) & 1ull;
-                                cn.add(CNT_SIG_LOADS, 1);
-                                if (maybe) {
-                                    maybe = (sig_half(g, v, LP.tdir ? 1 : 0) >> sig_bit(xp)) & 1ull;
-                                    cn.add(CNT_SIG_LOADS, 1);
-                                }
-                                int32_t gl = NOEDGE;
-                                cn.add(CNT_CHECKS, 1);
-                                if (maybe) {
-                                    cn.add(CNT_SEARCHES, 1);
-                                    gl = LP.tdir ? edge_label(g, xp, g.out_off[xp], g.out_off[xp + 1], v, g.in_off[v], g.in_off[v + 1], cn.loads())
-                                                 : edge_label(g, v, g.out_off[v], g.out_off[v + 1], xp, g.in_off[xp], g.in_off[xp + 1], cn.loads());
-                                } else {
-                                    cn.add(CNT_SIG_SETTLED, 1);
-                                }
-                                probes++;
-                                ok = exp_ok(LP.tlab, gl);
+                                ok = tree_edge_agrees<COUNT>(g, LP, m[LP.par << 5], v, probes, cn);
                             }
                         }
-                        // injectivity
+                        // injectivity, then every other pattern pair, both directions
                         for (int q = 0; q <= l && ok; q++)
                             if (((LP.inj >> q) & 1u) && m[q << 5] == v) ok = false;
-                        // every other pattern pair, both directions (required edges
-                        // first): v's neighbourhood signatures settle most pairs (a
-                        // clear bit proves the edge absent); the rest search the
-                        // shorter adjacency list
-                        if (ok && nchk > 0) {
-                            const uint32_t bv = sig_bit(v);
-                            uint64_t svo = 0, svi = 0;  // v's signature, loaded when needed
-                            bool have_sv = false;
-                            for (int c = 0; c < nchk && ok; c++) {
-                                if (c == skip) continue;
-                                const uint32_t wd = cw[c];
-                                const uint32_t x = m[(wd & 15u) << 5];
-                                const bool out = (wd >> 4) & 1u;  // edge v -> x, else x -> v
-                                const int32_t ex = (int32_t)(int16_t)(wd >> 16);
-                                int32_t gl = NOEDGE;
-                                cn.add(CNT_CHECKS, 1);
-                                // v's bit in x's signature (x's in-neighbours for v -> x),
-                                // then x's bit in v's: a clear bit proves the edge absent
-                                const uint64_t sx = c == 0 ? sx0 : sig_half(g, x, out ? 1 : 0);
-                                if (c != 0) cn.add(CNT_SIG_LOADS, 1);
-                                bool maybe = (sx >> bv) & 1ull;
-                                if (maybe) {
-                                    if (!have_sv) {
-                                        const ulonglong2 sg = __ldg(g.sig + v);
-                                        svo = sg.x;
-                                        svi = sg.y;
-                                        have_sv = true;
-                                        cn.add(CNT_SIG_LOADS, 1);
-                                    }
-                                    maybe = ((out ? svo : svi) >> sig_bit(x)) & 1ull;
-                                }
-                                if (COUNT && ex == EXP_NONE) {
-                                    const uint32_t dv = out ? g.out_off[v + 1] - g.out_off[v] : g.in_off[v + 1] - g.in_off[v];
-                                    const uint32_t dx = out ? g.in_off[x + 1] - g.in_off[x] : g.out_off[x + 1] - g.out_off[x];
-                                    cn.add(CNT_NEG_CHECKS, 1);
-                                    cn.add(CNT_NEG_LOGD, ceil_log2_1(min(dv, dx)));
-                                }
-                                if (maybe) {
-                                    cn.add(CNT_SEARCHES, 1);
-                                    gl = out ? edge_label(g, v, g.out_off[v], g.out_off[v + 1], x, g.in_off[x], g.in_off[x + 1],
-                                                          cn.loads())
-                                             : edge_label(g, x, g.out_off[x], g.out_off[x + 1], v, g.in_off[v], g.in_off[v + 1],
-                                                          cn.loads());
-                                } else {
-                                    cn.add(CNT_SIG_SETTLED, 1);
-                                }
-                                probes++;
-                                ok = exp_ok(ex, gl);
-                            }
-                        }
+                        ok = ok && pairs_agree<COUNT>(g, m, cw, nchk, LP.nreq, skip, v, probes, cn);
                     }
                     m[i << 5] = v;
                     // X pushed down: the X literals whose ends are matched at this
-                    // level (before the LAST one; the LAST level checks its own below)
+                    // level (before the last one; the last level checks its own)
                     if (GEN && ok && D->push_x && !LAST)
                         for (int q = 0; q < D->nx && ok; q++)
-                            if (D->lit[q].lvl == i) ok = lit_holds(g, D->lit[q], m, COUNT ? &attr_reads : nullptr);
+                            if (D->lit[q].lvl == i) ok = lit_holds_at(g, D->lit[q], m, i, v, COUNT ? &attr_reads : nullptr);
                 }
                 if (LAST) {
-                    // complete match: check the X literals of this level, count it
-                    // (with X pushed down only if they hold), check Y, emit a violation
-                    bool viol = false;
-                    if (ok) {
-                        bool x_ok = true;
-                        for (int q = 0; q < D->nx && x_ok; q++)
-                            if (!GEN || D->lit[q].lvl == i) x_ok = lit_holds(g, D->lit[q], m, COUNT ? &attr_reads : nullptr);
-                        if (GEN) tile_matches += x_ok || !D->push_x;
-                        else tile_matches++;
-                        if (x_ok) {
-                            bool y_ok = !D->y_false;
-                            for (int q = 0; q < D->ny && y_ok; q++)
-                                y_ok = lit_holds(g, D->lit[D->nx + q], m, COUNT ? &attr_reads : nullptr);
-                            viol = !y_ok;
-                        }
-                    }
-                    const uint32_t vb = __ballot_sync(0xffffffffu, viol);
-                    if (vb) {
-                        unsigned long long base = 0;
-                        if (lane == 0) {
-                            const unsigned long long nv = __popc(vb);
-                            const unsigned long long old = atomicAdd((unsigned long long*)&S->n_viol, nv);
-                            base = D->viol ? old : atomicAdd((unsigned long long*)&A.sched->varena_used, nv);
-                        }
-                        base = __shfl_sync(0xffffffffu, base, 0);
-                        if (viol) {
-                            const uint64_t idx = base + __popc(vb & ((1u << lane) - 1u));
-                            if (D->viol) {
-                                // the slot's own buffer: tuples in pattern-node order
-                                if (idx < D->viol_cap) {
-                                    int32_t* out = D->viol + idx * k;
-                                    for (int q = 0; q < k; q++) out[D->order[q]] = (int32_t)__ldg(g.orig + m[q << 5]);
-                                }
-                            } else if (idx < A.sched->varena_cap) {
-                                // the run's arena: [slot, tuple in pattern-node order]
-                                int32_t* rec = A.sched->varena + idx * A.sched->vstride;
-                                rec[0] = s;
-                                for (int q = 0; q < k; q++) rec[1 + D->order[q]] = (int32_t)__ldg(g.orig + m[q << 5]);
-                            }
-                        }
-                    }
+                    finish(ok, i, v, m);
                 } else {
                     // partial match of level i: append it with its fan-out for level
                     // i+1, taken from the shortest candidate generator (dead ends,
                     // with no fan-out, are dropped)
                     uint64_t fo = 0;
-                    uint32_t nbase = 0;
+                    uint32_t nbase = 0;  // where its candidates start in the generator's source
                     int gen = 0;
+                    const LevelPlan& L2 = D->lv[i + 1];
                     if (ok) {
-                        const LevelPlan& L2 = D->lv[i + 1];
                         const int pn = L2.par;
                         if (GEN && pn < 0) {
                             // level i+1 starts a component: its whole candidate list
@@ -622,39 +761,56 @@ __device__ void expand_warps(const EnumArgs& A) {
                         for (int q = 0; q < L2.ngen; q++) {
                             const int cg = L2.gen[q];
                             const uint32_t x = m[L2.chk_q[cg] << 5];
-                            const uint32_t d = L2.chk_dir[cg] ? __ldg(g.in_off + x + 1) - __ldg(g.in_off + x)
-                                                              : __ldg(g.out_off + x + 1) - __ldg(g.out_off + x);
+                            const uint32_t* const off = L2.chk_dir[cg] ? g.in_off : g.out_off;
+                            const uint32_t e0 = __ldg(off + x), d = __ldg(off + x + 1) - e0;
                             if (d < fo) {
                                 fo = d;
                                 gen = q + 1;
+                                if (fuse) nbase = e0;
                             }
                         }
                     }
                     ok = ok && fo > 0;
-                    const bool fuse_me = fuse && ok && fo <= FUSE_FANOUT;  // expanded below, not stored
-                    const bool row_me = ok && !fuse_me;
+                    bool fuse_me = fuse && ok && fo <= FUSE_FANOUT;  // expanded below, not stored
+                    bool row_me = ok && !fuse_me;
                     const uint64_t packed = row_me ? ((1ull << ROW_SHIFT) | fo) : 0ull;
-                    uint64_t total;
-                    const uint64_t excl = warp_excl_scan(packed, lane, &total);
+                    uint64_t total = 0, excl = 0;
+                    if (__any_sync(0xffffffffu, row_me)) excl = warp_excl_scan(packed, lane, &total);
                     if (total) {
                         unsigned long long old = 0;
+                        bool over = false;
                         if (lane == 0) {
-                            old = atomicAdd((unsigned long long*)&S->ctr[i], (unsigned long long)total);
-                            if ((old & WORK_MASK) + (total & WORK_MASK) > WORK_MASK ||
-                                (old >> ROW_SHIFT) + (total >> ROW_SHIFT) > D->chunk)
-                                atomicExch(&S->err, DERR_COUNTER_OVERFLOW);
+                            auto no_room = [&](unsigned long long c) {
+                                return (c & WORK_MASK) + (total & WORK_MASK) > WORK_MASK ||
+                                       (c >> ROW_SHIFT) + (total >> ROW_SHIFT) > W.cap;
+                            };
+                            // a full level is not counted up any further (the few warps
+                            // that still do stay below the counter's 2^24 rows)
+                            over = fuse && no_room(__ldcg((const unsigned long long*)&S->ctr[i]));
+                            if (!over) {
+                                old = atomicAdd((unsigned long long*)&S->ctr[i], (unsigned long long)total);
+                                over = no_room(old);
+                                if (over && fuse) atomicMin((unsigned long long*)&S->row_limit, old);
+                                else if (over) atomicExch(&S->err, DERR_COUNTER_OVERFLOW);
+                            }
                         }
                         old = __shfl_sync(0xffffffffu, old, 0);
+                        // a step that fuses takes more items than the level has rows
+                        // for: partial matches without a row are expanded here too
+                        if (fuse && __shfl_sync(0xffffffffu, (int)over, 0)) {
+                            row_me = false;
+                            fuse_me = ok;
+                        }
                         // the warp's new partial matches take rows [row0, row0 + its
                         // count) of the level's buffer, in lane order
                         if (row_me) {
                             const uint64_t row = (old >> ROW_SHIFT) + (excl >> ROW_SHIFT);
-                            if (row < D->chunk) {
+                            if (row < W.cap) {
                                 cn.add(CNT_ROWS, 1);
                                 // the row (ids, positions, generator, index base,
                                 // padding) in 16-byte stores, four ints at a time
                                 const int nw = row_width(i);
-                                int32_t* dst = D->rows[i] + row * nw;
+                                int32_t* dst = W.rows + row * nw;
                                 for (int t = 0; t < nw; t += 4) {
                                     int32_t e4[4];
     #pragma unroll
@@ -675,184 +831,76 @@ __device__ void expand_warps(const EnumArgs& A) {
                                     }
                                     *reinterpret_cast<int4*>(dst + t) = make_int4(e4[0], e4[1], e4[2], e4[3]);
                                 }
-                                D->wpre[i][row] = (old & WORK_MASK) + (excl & WORK_MASK);
+                                W.wpre[row] = (old & WORK_MASK) + (excl & WORK_MASK);
                             }
                         }
                     }
                     if (fuse) {
                         // The last level of the lanes' new partial matches with small
-                        // fan-outs, by the whole warp, 32 items at a time: item t
-                        // belongs to the lane whose [fex, fex + ffo) holds t; that
-                        // lane's shared-memory column holds the partial match.
-                        const uint32_t ffo = fuse_me ? (uint32_t)fo : 0u;
-                        uint32_t fin = ffo;
-                        for (int d = 1; d < 32; d <<= 1) {
-                            const uint32_t y = __shfl_up_sync(0xffffffffu, fin, d);
-                            if (lane >= d) fin += y;
-                        }
-                        const uint32_t fex = fin - ffo;
-                        const uint32_t ftot = __shfl_sync(0xffffffffu, fin, 31);
-                        if (lane == 0 && ftot) atomicAdd((unsigned long long*)&S->st_work, (unsigned long long)ftot);
-                        __syncwarp();  // the lanes' columns, written above, are read by other lanes
+                        // fan-outs, by the whole warp, end to end: W.list holds the
+                        // non-empty ones in order (start in the generator's source -
+                        // start in the sequence, lane | generator << 8); which of them
+                        // an item belongs to follows from the bits of the sequence's
+                        // window at which lists start. No candidate can have an empty
+                        // set of needed bits.
                         const int L = k - 1;
-                        const LevelPlan& LQ = D->lv[L];
-                        const int nchk2 = LQ.nchk;
-                        for (uint32_t fb = 0; fb < ftot; fb += 32) {
-                            const uint32_t it = fb + lane;
-                            int own = 0;
-                            for (int st = 16; st >= 1; st >>= 1) {
-                                const uint32_t x = __shfl_sync(0xffffffffu, fex, own + st);
-                                if (x <= it) own += st;
-                            }
-                            const uint32_t fo2 = it - __shfl_sync(0xffffffffu, fex, own);
-                            const uint32_t onb = __shfl_sync(0xffffffffu, nbase, own);
-                            const int och = __shfl_sync(0xffffffffu, gen, own);
-                            const uint32_t* mo = &s_m[threadIdx.x >> 5][own];
-                            bool iok = it < ftot;
-                            uint32_t fv = 0;
-                            int fskip = -1;
-                            if (iok) {
-                                cn.add(CNT_ITEMS, 1);
-                                cn.add(CNT_ITEMS_LAST, 1);
-                                if (COUNT && fo2 == 0) {
-                                    cn.add(CNT_PARTIALS, 1);
-                                    uint64_t bd = 0;
-                                    for (int c = 0; c < nchk2; c++) {
-                                        if (LQ.chk_exp[c] == EXP_NONE) continue;
-                                        const uint32_t x = mo[LQ.chk_q[c] << 5];
-                                        bd += LQ.chk_dir[c] ? g.in_off[x + 1] - g.in_off[x] : g.out_off[x + 1] - g.out_off[x];
-                                    }
-                                    cn.add(CNT_BACK_DEG, bd);
-                                }
-                                if (och == 0) {
-                                    fv = (uint32_t)__ldg(D->cpi_idx[L] + onb + fo2).y;
-                                } else if (GEN && och == GEN_LIST) {
-                                    fv = (uint32_t)__ldg(D->cand[L] + fo2);
-                                } else {
-                                    // from the adjacency of the other end of a required back
-                                    // edge: keep those in C(u) and probe the tree edge
-                                    const int cg = LQ.gen[och - 1];
-                                    fskip = cg;
-                                    const uint32_t x = mo[LQ.chk_q[cg] << 5];
-                                    const uint32_t pe = LQ.chk_dir[cg] ? __ldg(g.in_adj + __ldg(g.in_off + x) + fo2)
-                                                                       : __ldg(g.out_adj + __ldg(g.out_off + x) + fo2);
-                                    fv = pe >> g.lbits;
-                                    iok = exp_ok(LQ.chk_exp[cg], (int32_t)(pe & g.lmask)) &&
-                                          ((__ldg(D->bm[L] + (fv >> 5)) >> (fv & 31)) & 1u);
-                                    if (iok) {
-                                        const uint32_t xp = mo[LQ.par << 5];
-                                        bool maybe = (sig_half(g, xp, LQ.tdir ? 0 : 1) >> sig_bit(fv)) & 1ull;
-                                        if (maybe) maybe = (sig_half(g, fv, LQ.tdir ? 1 : 0) >> sig_bit(xp)) & 1ull;
-                                        int32_t gl = NOEDGE;
-                                        cn.add(CNT_CHECKS, 1);
-                                        if (maybe) {
-                                            cn.add(CNT_SEARCHES, 1);
-                                            gl = LQ.tdir ? edge_label(g, xp, g.out_off[xp], g.out_off[xp + 1], fv, g.in_off[fv],
-                                                                      g.in_off[fv + 1], cn.loads())
-                                                         : edge_label(g, fv, g.out_off[fv], g.out_off[fv + 1], xp, g.in_off[xp],
-                                                                      g.in_off[xp + 1], cn.loads());
-                                        } else {
-                                            cn.add(CNT_SIG_SETTLED, 1);
-                                        }
-                                        probes++;
-                                        iok = exp_ok(LQ.tlab, gl);
-                                    }
-                                }
-                                // injectivity, then the other pattern pairs
-                                for (int q = 0; q < L && iok; q++)
-                                    if (((LQ.inj >> q) & 1u) && mo[q << 5] == fv) iok = false;
-                                if (iok && nchk2 > 0) {
-                                    const uint32_t bv = sig_bit(fv);
-                                    uint64_t svo = 0, svi = 0;
-                                    bool have_sv = false;
-                                    for (int c = 0; c < nchk2 && iok; c++) {
-                                        if (c == fskip) continue;
-                                        const uint32_t wd = cw2[c];
-                                        const uint32_t x = mo[(wd & 15u) << 5];
-                                        const bool out = (wd >> 4) & 1u;
-                                        const int32_t ex = (int32_t)(int16_t)(wd >> 16);
-                                        cn.add(CNT_CHECKS, 1);
-                                        cn.add(CNT_SIG_LOADS, 1);
-                                        bool maybe = (sig_half(g, x, out ? 1 : 0) >> bv) & 1ull;
-                                        if (maybe) {
-                                            if (!have_sv) {
-                                                const ulonglong2 sg = __ldg(g.sig + fv);
-                                                svo = sg.x;
-                                                svi = sg.y;
-                                                have_sv = true;
-                                            }
-                                            maybe = ((out ? svo : svi) >> sig_bit(x)) & 1ull;
-                                        }
-                                        int32_t gl = NOEDGE;
-                                        if (maybe) {
-                                            cn.add(CNT_SEARCHES, 1);
-                                            gl = out ? edge_label(g, fv, g.out_off[fv], g.out_off[fv + 1], x, g.in_off[x],
-                                                                  g.in_off[x + 1], cn.loads())
-                                                     : edge_label(g, x, g.out_off[x], g.out_off[x + 1], fv, g.in_off[fv],
-                                                                  g.in_off[fv + 1], cn.loads());
-                                        } else {
-                                            cn.add(CNT_SIG_SETTLED, 1);
-                                        }
-                                        probes++;
-                                        iok = exp_ok(ex, gl);
-                                    }
-                                }
-                            }
-                            // complete match: X, count, Y, emit (as at the last level)
-                            bool fviol = false;
-                            if (iok) {
-                                bool x_ok = true;
-                                for (int q = 0; q < D->nx && x_ok; q++)
-                                    if (!GEN || D->lit[q].lvl == L)
-                                        x_ok = lit_holds_at(g, D->lit[q], mo, L, fv, COUNT ? &attr_reads : nullptr);
-                                if (GEN) tile_matches += x_ok || !D->push_x;
-                                else tile_matches++;
-                                if (x_ok) {
-                                    bool y_ok = !D->y_false;
-                                    for (int q = 0; q < D->ny && y_ok; q++)
-                                        y_ok = lit_holds_at(g, D->lit[D->nx + q], mo, L, fv, COUNT ? &attr_reads : nullptr);
-                                    fviol = !y_ok;
-                                }
-                            }
-                            const uint32_t vb = __ballot_sync(0xffffffffu, fviol);
-                            if (vb) {
-                                unsigned long long base = 0;
-                                if (lane == 0) {
-                                    const unsigned long long nv = __popc(vb);
-                                    const unsigned long long oldv = atomicAdd((unsigned long long*)&S->n_viol, nv);
-                                    base = D->viol ? oldv : atomicAdd((unsigned long long*)&A.sched->varena_used, nv);
-                                }
-                                base = __shfl_sync(0xffffffffu, base, 0);
-                                if (fviol) {
-                                    const uint64_t idx = base + __popc(vb & ((1u << lane) - 1u));
-                                    if (D->viol) {
-                                        if (idx < D->viol_cap) {
-                                            int32_t* outp = D->viol + idx * k;
-                                            for (int q = 0; q < k; q++) outp[D->order[q]] = (int32_t)__ldg(g.orig + level_vertex(mo, q, L, fv));
-                                        }
-                                    } else if (idx < A.sched->varena_cap) {
-                                        int32_t* rec = A.sched->varena + idx * A.sched->vstride;
-                                        rec[0] = s;
-                                        for (int q = 0; q < k; q++) rec[1 + D->order[q]] = (int32_t)__ldg(g.orig + level_vertex(mo, q, L, fv));
-                                    }
-                                }
-                            }
+                        uint32_t left = fuse_me ? (uint32_t)fo : 0u;
+                        if (left) {
+                            const uint64_t need = needed_bits(g, L2, m, cw2, gen, &W.row[lane]);
+                            W.need[lane] = need;
+                            if (need == 0) left = 0;
+                            if (COUNT) count_partial(L2, m);
                         }
+                        // (a sequence of at most 32 x 2^26 items at a time)
+                        do {
+                            const uint32_t ffo = min(left, 1u << 26);
+                            uint32_t fin = ffo;
+                            for (int d = 1; d < 32; d <<= 1) {
+                                const uint32_t y = __shfl_up_sync(0xffffffffu, fin, d);
+                                if (lane >= d) fin += y;
+                            }
+                            const uint32_t fex = fin - ffo;
+                            const uint32_t ftot = __shfl_sync(0xffffffffu, fin, 31);
+                            if (lane == 0 && ftot) atomicAdd((unsigned long long*)&S->st_work, (unsigned long long)ftot);
+                            const uint32_t some = __ballot_sync(0xffffffffu, ffo != 0);
+                            if (ffo) W.list[__popc(some & below)] = make_int2((int32_t)(nbase - fex), lane | gen << 8);
+                            __syncwarp();  // columns, needed bits and lists are read by other lanes
+                            uint32_t begun = 0, queued = 0;
+                            for (uint32_t fb = 0; fb < ftot || queued; fb += 32) {
+                                if (fb < ftot) {
+                                    const uint32_t starts =
+                                        __reduce_or_sync(0xffffffffu, ffo && fex - fb < 32u ? 1u << (fex - fb) : 0u);
+                                    const uint32_t own = begun + __popc(starts & (below << 1 | 1u)) - 1;
+                                    begun += __popc(starts);
+                                    const bool it = fb + lane < ftot;
+                                    const int2 e = W.list[it ? own : 0];
+                                    queued = first_stage(L2, L, queued, it, fb + lane + (uint32_t)e.x, e.y >> 8, e.y & 31,
+                                                         W.need[e.y & 31], W.row[e.y & 31]);
+                                    if (queued < 32 && fb + 32 < ftot) continue;
+                                }
+                                const uint32_t take = min(queued, 32u);
+                                second_stage(L2, L, cw2, lane < (int)take, queued - take + lane);
+                                queued -= take;
+                                __syncwarp();  // the queue is written again
+                            }
+                            left -= ffo;
+                            nbase += ffo;
+                        } while (__any_sync(0xffffffffu, left != 0));
                     }
                 }
                 cn.iteration(LAST);
             }
-            if (LAST || fuse) {
-                const unsigned long long tm = __reduce_add_sync(0xffffffffu, tile_matches);
-                if (lane == 0 && tm) atomicAdd((unsigned long long*)&S->n_matches, tm);
-            }
         };
         if (last) {
             if (l == 0) run_tile(std::true_type{}, std::true_type{});
-            else run_tile(std::true_type{}, std::false_type{});
+            else run_last_rows();
         } else {
             if (l == 0) run_tile(std::false_type{}, std::true_type{});
             else run_tile(std::false_type{}, std::false_type{});
+        }
+        if (last || i == k - 2) {
+            const unsigned long long tm = __reduce_add_sync(0xffffffffu, tile_matches);
+            if (lane == 0 && tm) atomicAdd((unsigned long long*)&S->n_matches, tm);
         }
         uint32_t nt = 0;
         if (lane == 0) nt = atomicAdd(&A.sched->tile_next, 1u);
@@ -878,6 +926,12 @@ __device__ void slot_start(const SlotDesc* D, SlotState* S) {
     for (int i = 1; i < D->k; i++)
         if (D->lv[i].par >= 0) S->st_cpi += D->cpi_off[i][S->ncand[D->lv[i].par]];
     S->nrows[0] = S->ncand[0];
+    S->big = 0;
+    for (int l = 1; l <= D->k - 2; l++) {
+        S->rows[l] = D->rows[l];
+        S->wpre[l] = D->wpre[l];
+        S->cap[l] = D->chunk;
+    }
     S->total[0] = D->k == 1             ? (uint64_t)S->ncand[0]
                 : D->lv[1].par < 0      ? (uint64_t)S->ncand[0] * S->ncand[1]  // level 1 starts a component
                                         : (uint64_t)D->cpi_off[1][S->ncand[0]];
@@ -906,6 +960,8 @@ __device__ void control_step(const EnumArgs& A, bool first) {
         expired_s = now - A.sched->t_start > A.sched->run_limit_ns;
         if (expired_s) A.sched->err = DERR_TIMEOUT;
     }
+    // few slots left after the last step: each takes a large buffer
+    const bool few = A.big && !first && A.sched->active <= N_BIG;
     __syncthreads();
     for (int base = 0; base < A.n_slots; base += CT) {
         const int s = base + threadIdx.x;
@@ -920,7 +976,9 @@ __device__ void control_step(const EnumArgs& A, bool first) {
                 S->cursor[l] = S->ce;
                 S->st_steps++;
                 if (k > 1 && l + 1 <= k - 2) {
-                    const uint64_t c = __ldcg((const unsigned long long*)&S->ctr[l + 1]);
+                    // rows from row_limit on found no room (and were not written)
+                    const uint64_t c = min(__ldcg((const unsigned long long*)&S->ctr[l + 1]),
+                                           __ldcg((const unsigned long long*)&S->row_limit));
                     const uint64_t rows = c >> ROW_SHIFT;
                     if (rows > 0) {
                         S->nrows[l + 1] = rows;
@@ -933,15 +991,30 @@ __device__ void control_step(const EnumArgs& A, bool first) {
             }
             while (S->cur >= 0 && S->cursor[S->cur] >= S->total[S->cur]) S->cur--;
             if (__ldcg(&S->err) || expired_s) S->cur = -1;
+            if (S->cur < 0 && S->big) {
+                atomicExch(&A.sched->big_owner[S->big - 1], 0u);
+                S->big = 0;
+            }
             if (S->cur >= 0) {
                 const int l = S->cur;
+                for (uint32_t b = 0; few && !S->big && b < N_BIG; b++)
+                    if (atomicCAS(&A.sched->big_owner[b], 0u, (uint32_t)s + 1) == 0) S->big = b + 1;
+                if (S->big && l + 1 <= k - 2) {  // the level to fill is empty: it moves there
+                    uint8_t* const buf = A.big + (S->big - 1) * A.big_bytes;
+                    S->rows[l + 1] = (int32_t*)(buf + D->big_rows[l + 1]);
+                    S->wpre[l + 1] = (uint64_t*)(buf + D->big_wpre[l + 1]);
+                    S->cap[l + 1] = D->big_chunk;
+                }
                 S->cb = S->cursor[l];
-                // the last level writes no partial matches, so its steps are not
-                // bounded by the row buffers
-                const bool to_last = k == 1 || l + 1 == k - 1;
-                const uint64_t step = to_last ? max(D->chunk, (uint64_t)LAST_LEVEL_CHUNK) : D->chunk;
+                // the last level writes no partial matches, and the one before (fused)
+                // expands those without a row at once, so their steps are not bounded
+                // by the row buffers; a chunk of them per step left the last few large
+                // GFDs of a batch with hundreds of steps of a few iterations per warp
+                const bool wide = k == 1 || l + 1 >= k - 2;
+                const uint64_t step = wide ? max(D->chunk, (uint64_t)LAST_LEVEL_CHUNK) : S->cap[l + 1];
                 S->ce = min(S->cb + step, S->total[l]);
                 if (k > 1 && l + 1 <= k - 2) S->ctr[l + 1] = 0;
+                S->row_limit = ~0ull;
                 S->st_work += S->ce - S->cb;
                 atomicAdd(&active_s, 1);
                 atomicAdd(&work_s, (unsigned long long)(S->ce - S->cb));
@@ -1085,7 +1158,11 @@ int launch_persistent(const EnumArgs& a, cudaStream_t st, int64_t* launches) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persistent<NT, MINB, GEN, COUNT>, NT, 0);
+    const size_t smem = warp_shared_bytes(a.kmax) * (NT / 32);
+    cudaError_t e = cudaFuncSetAttribute(k_persistent<NT, MINB, GEN, COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(warp_shared_bytes(MAXK) * (NT / 32)));
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_persistent<NT, MINB, GEN, COUNT>, NT, smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
     if (per_sm < 1) {
         set_error(GFD_ERR_CUDA, "persistent enumeration kernel cannot be resident");
@@ -1094,8 +1171,9 @@ int launch_persistent(const EnumArgs& a, cudaStream_t st, int64_t* launches) {
     const int grid = sms * per_sm;
     EnumArgs args = a;
     args.n_warps = grid * (NT / 32);
+    args.columns = (uint32_t)column_words(a.kmax);
     void* params[] = {&args};
-    e = cudaLaunchCooperativeKernel((const void*)k_persistent<NT, MINB, GEN, COUNT>, dim3(grid), dim3(NT), params, 0,
+    e = cudaLaunchCooperativeKernel((const void*)k_persistent<NT, MINB, GEN, COUNT>, dim3(grid), dim3(NT), params, smem,
                                     st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel");
     if (launches) *launches += 1;
@@ -1103,19 +1181,23 @@ int launch_persistent(const EnumArgs& a, cudaStream_t st, int64_t* launches) {
 }
 
 template <int NT, int MINB, bool GEN>
-int expand_grid() {
+int expand_grid(size_t smem) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_expand<NT, MINB, GEN>, NT, 0);
+    cudaFuncSetAttribute(k_expand<NT, MINB, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(warp_shared_bytes(MAXK) * (NT / 32)));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_expand<NT, MINB, GEN>, NT, smem);
     return sms * std::max(per_sm, 1);
 }
 
 template <int NT, int MINB, bool GEN>
 int host_loop(const EnumArgs& a0, bool use_graph, cudaStream_t st, int64_t* launches) {
-    const int grid = expand_grid<NT, MINB, GEN>();
+    const size_t smem = warp_shared_bytes(a0.kmax) * (NT / 32);
+    const int grid = expand_grid<NT, MINB, GEN>(smem);
     EnumArgs a = a0;
     a.n_warps = grid * (NT / 32);
+    a.columns = (uint32_t)column_words(a0.kmax);
     int32_t* h_active = nullptr;
     cudaError_t e = cudaMallocHost(&h_active, sizeof(int32_t));
     if (e != cudaSuccess) return cuda_fail(e, "cudaMallocHost");
@@ -1127,7 +1209,7 @@ int host_loop(const EnumArgs& a0, bool use_graph, cudaStream_t st, int64_t* laun
         e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             for (int it = 0; it < per_check; it++) {
-                k_expand<NT, MINB, GEN><<<grid, NT, 0, st>>>(a);
+                k_expand<NT, MINB, GEN><<<grid, NT, smem, st>>>(a);
                 k_control<<<1, CTRL_THREADS, 0, st>>>(a, 0);
             }
             e = cudaStreamEndCapture(st, &graph);
@@ -1145,7 +1227,7 @@ int host_loop(const EnumArgs& a0, bool use_graph, cudaStream_t st, int64_t* laun
             if (launches) *launches += 2 * per_check;
         } else {
             for (int it = 0; it < per_check; it++) {
-                k_expand<NT, MINB, GEN><<<grid, NT, 0, st>>>(a);
+                k_expand<NT, MINB, GEN><<<grid, NT, smem, st>>>(a);
                 k_control<<<1, CTRL_THREADS, 0, st>>>(a, 0);
             }
             e = cudaGetLastError();
@@ -1238,13 +1320,15 @@ namespace {
 
 template <int NT, int MINB, bool GEN>
 int capture_steps_t(const EnumArgs& a0, int steps, cudaStream_t st, cudaGraph_t* graph, cudaGraphExec_t* exec) {
-    const int grid = expand_grid<NT, MINB, GEN>();
+    const size_t smem = warp_shared_bytes(a0.kmax) * (NT / 32);
+    const int grid = expand_grid<NT, MINB, GEN>(smem);
     EnumArgs a = a0;
     a.n_warps = grid * (NT / 32);
+    a.columns = (uint32_t)column_words(a0.kmax);
     cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         for (int it = 0; it < steps; it++) {
-            k_expand<NT, MINB, GEN><<<grid, NT, 0, st>>>(a);
+            k_expand<NT, MINB, GEN><<<grid, NT, smem, st>>>(a);
             k_control<<<1, CTRL_THREADS, 0, st>>>(a, 0);
         }
         e = cudaStreamEndCapture(st, graph);

@@ -196,6 +196,20 @@ __global__ void k_signature(const uint32_t* off, const uint32_t* adj, int32_t n,
     }
 }
 
+// One warp per vertex: the row filter of its list (words zeroed before).
+__global__ void k_row_filter(const uint32_t* off, const uint32_t* adj, int32_t n, int32_t lbits, uint32_t* filter) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t v = warp; v < n; v += nwarps) {
+        const uint32_t a = off[v], b = off[v + 1];
+        for (uint32_t e = a + lane; e < b; e += 32) {
+            const uint64_t bit = 8ull * a + filter_bit(adj[e] >> lbits, b - a);
+            atomicOr(&filter[bit >> 5], 1u << (bit & 31));
+        }
+    }
+}
+
 // Degree moments of one label's vertices, one block per chunk [first, last) of
 // its range: out[16 c + 4 a + b] = sum of dout^a din^b (a, b in 0..3), added up in
 // a fixed order (the host adds the chunks), so that plans do not vary.
@@ -352,7 +366,7 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
     const size_t N = (size_t)n, M = (size_t)m, NA = N * std::max(1, d->n_attrs);
     Block R;  // resident
     const size_t r_out_off = R.take(4 * (N + 1)), r_in_off = R.take(4 * (N + 1)), r_out_adj = R.take(4 * M + 16),
-                 r_in_adj = R.take(4 * M + 16), r_vinfo = R.take(4 * N), r_attrs = R.take(4 * NA), r_sig = R.take(16 * N),
+                 r_in_adj = R.take(4 * M + 16), r_vinfo = R.take(4 * N), r_attrs = R.take(4 * NA), r_sig = R.take(16 * N), r_filter = R.take(2 * (M + 256)),
                  r_orig = R.take(4 * N), r_ovinfo = R.take(4 * N), r_oout = R.take(4 * (N + 1)),
                  r_oin = R.take(4 * (N + 1));
     int rc;
@@ -491,6 +505,10 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
     }
     k_signature<<<grid_for((int64_t)n * 32), 256, 0, st>>>(out_off, out_adj, n, lbits, 0, sig);
     k_signature<<<grid_for((int64_t)n * 32), 256, 0, st>>>(in_off, in_adj, n, lbits, 1, sig);
+    uint8_t *out_filter = R.at<uint8_t>(r_filter), *in_filter = out_filter + ((M + 255) & ~(size_t)255);
+    CK(cudaMemsetAsync(out_filter, 0, 2 * (M + 256), st));
+    k_row_filter<<<grid_for((int64_t)n * 32), 256, 0, st>>>(out_off, out_adj, n, lbits, (uint32_t*)out_filter);
+    k_row_filter<<<grid_for((int64_t)n * 32), 256, 0, st>>>(in_off, in_adj, n, lbits, (uint32_t*)in_filter);
     CK(cudaGetLastError());
     if (have_in) {
         // the caller's reverse CSR must be exactly the transpose
@@ -576,6 +594,8 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
     dg.vinfo = vinfo;
     dg.attrs = attrs;
     dg.sig = (const ulonglong2*)sig;
+    dg.out_filter = out_filter;
+    dg.in_filter = in_filter;
     dg.orig = orig;
     dg.o_vinfo = o_vinfo;
     dg.o_out_off = o_out;

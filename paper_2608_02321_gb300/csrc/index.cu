@@ -723,7 +723,9 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, SCAN_BLOCKS) k_cpi_fill(D
                            for (int c = 0; c < 4; c++)
                                if ((hq[i] >> c) & 1u) {
                                    const uint32_t x = xq[i][c];
-                                   if (slot < J.cap)
+                                   if (slot < J.cap && J.ids)
+                                       reinterpret_cast<uint32_t*>(J.idx)[slot] = x;
+                                   else if (slot < J.cap)
                                        J.idx[slot] = make_int2((int32_t)(__ldg(J.crank + (x >> 5)) +
                                                                          __popc(__ldg(J.cbm + (x >> 5)) &
                                                                                 ((1u << (x & 31)) - 1))), (int32_t)x);
@@ -747,6 +749,7 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, SCAN_BLOCKS) k_cpi_fill(D
         const AdjRef A = adj_ref(g, J.out);
         const uint32_t* const off = J.off + parent_rank(J, va);
         int2* const idx = J.idx;
+        const bool ids = J.ids;
         const uint32_t* const crank = J.crank;
         const uint64_t cap = J.cap;
         for (uint32_t i = 0; i < n; i += 32) {
@@ -769,7 +772,9 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, SCAN_BLOCKS) k_cpi_fill(D
                           const uint32_t hits = __ballot_sync(0xffffffffu, hit);
                           if (hit) {
                               const uint32_t slot = next + __popc(hits & ((1u << lane) - 1u));
-                              if (slot < cap)
+                              if (slot < cap && ids)
+                                  reinterpret_cast<uint32_t*>(idx)[slot] = y;
+                              else if (slot < cap)
                                   idx[slot] = make_int2((int32_t)(__ldg(crank + (y >> 5)) +
                                                                   __popc(w & ((1u << (y & 31)) - 1))), (int32_t)y);
                           }

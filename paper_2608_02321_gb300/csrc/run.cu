@@ -189,7 +189,7 @@ int tables_alloc(cudaMemPool_t pool, int max_slots, int block_threads, int tile_
     return GFD_OK;
 }
 
-EnumArgs enum_args(const gfd_graph* g, const Tables& T) {
+EnumArgs enum_args(const gfd_graph* g, const Tables& T, int kmax) {
     EnumArgs A;
     A.g = g->dg;
     A.slots = T.desc;
@@ -199,6 +199,10 @@ EnumArgs enum_args(const gfd_graph* g, const Tables& T) {
     A.n_slots = T.max_slots;
     A.tile = T.tile;
     A.n_warps = 0;
+    A.kmax = kmax;
+    A.big = nullptr;
+    A.big_bytes = 0;
+    A.columns = 0;
     return A;
 }
 
@@ -228,7 +232,9 @@ struct RefineSpec {
 struct IndexSpec {
     int parent, child;  // final bitmaps (Group::finals)
     int dir, lab;
+    bool ids;           // for a last level: vertex ids alone
     uint64_t bound;     // most index edges there can be
+    size_t entry() const { return ids ? 4 : 8; }
 };
 struct VecHash {
     size_t operator()(const std::vector<int32_t>& v) const {
@@ -265,6 +271,8 @@ struct Group {
     std::vector<size_t> o_off, o_idx;        // per index (o_idx only when in the workspace)
     size_t o_keybm = 0, o_zero = 0, o_zero_end = 0, o_counts = 0, o_bm = 0, o_marks = 0;
     size_t o_cmp_sums = 0, o_cpi_sums = 0, o_cpi_tot = 0;
+    uint64_t big_bytes = 0;       // each large frontier buffer (0: none)
+    size_t o_big = 0;
     bool idx_inside = false;      // index edges in the workspace, at their bound
     uint8_t* cpi_base = nullptr;  // else: allocated exactly after counting
     size_t cpi_bytes = 0;
@@ -312,9 +320,13 @@ bool td_gather_cheaper(const gfd_graph* g, int32_t label_q, int32_t label_i, int
 // Plans, capacities and the workspace layout of a group (host only). With
 // strict_budget, a frontier_per_slot that cannot hold MIN_CHUNK partial matches
 // at every level of some GFD is an error instead of being raised to that.
+constexpr uint64_t BIG_MIN_CHUNK = 1 << 16;
 constexpr uint64_t MIN_CHUNK = 1024;
+// rows are counted in 24 bits; warps that find no room may still add theirs (at
+// most 32 each)
+constexpr uint64_t MAX_CHUNK = (1ull << 24) - (1ull << 20);
 int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* o, int64_t frontier_per_slot,
-               Group* G, bool strict_budget = false) {
+               Group* G, bool strict_budget = false, bool with_big = false) {
     const uint32_t nwords = g->dg.nwords;
     G->n = n;
     G->plans.resize(n);
@@ -406,10 +418,11 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
             const int par = P.lv[i].par;
             if (par < 0) continue;  // starts a component: no index edges
             const int pf = G->level_final[s][par], cf = G->level_final[s][i];
-            const auto it = index_id.emplace(std::vector<int32_t>{pf, cf, P.lv[i].tdir, P.lv[i].tlab}, (int)G->index.size());
+            const auto it = index_id.emplace(std::vector<int32_t>{pf, cf, P.lv[i].tdir, P.lv[i].tlab, i == P.k - 1},
+                                             (int)G->index.size());
             if (it.second) {
                 const int32_t plab = P.key[par].label;
-                G->index.push_back({pf, cf, P.lv[i].tdir, P.lv[i].tlab,
+                G->index.push_back({pf, cf, P.lv[i].tdir, P.lv[i].tlab, i == P.k - 1,
                                     std::min<uint64_t>(lab_deg(plab, P.lv[i].tdir == 1), (uint64_t)g->m)});
             }
             G->level_index[s][i] = it.first->second;
@@ -418,6 +431,23 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
     Layout L;
     G->descs.assign(n, SlotDesc{});
     G->offs.resize(n);
+    // A quarter of a batch's frontier budget goes to the N_BIG large buffers when
+    // the GFDs are many and their own shares stay large without it. Batch of 256
+    // GFDs on 4M vertices with 48 GiB: 443 steps -> 49, enumeration 172 -> 147 ms
+    // (its last slots, with 1/256 of the budget each, took 435 of the steps).
+    size_t big_need = 0;
+    uint64_t widest = 0;
+    for (auto& P : G->plans) {
+        uint64_t b = 0;
+        for (int l = 1; l <= P.k - 2; l++) b += 4ull * row_width(l) + 8;
+        widest = std::max(widest, b);
+    }
+    const bool big = with_big && n > 2 * N_BIG && !(o && o->chunk_rows > 0) && widest &&
+                     (uint64_t)frontier_per_slot / 4 * 3 / widest >= BIG_MIN_CHUNK;
+    if (big) {
+        G->big_bytes = (uint64_t)frontier_per_slot * n / (4 * N_BIG) & ~(uint64_t)255;
+        frontier_per_slot = frontier_per_slot / 4 * 3;
+    }
     for (int s = 0; s < n; s++) {
         const HostPlan& P = G->plans[s];
         SlotDesc& D = G->descs[s];
@@ -435,7 +465,7 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
         uint64_t row_bytes = 0;
         for (int l = 1; l <= P.k - 2; l++) row_bytes += 4ull * row_width(l) + 8;
         uint64_t chunk = o && o->chunk_rows > 0 ? (uint64_t)o->chunk_rows
-                                                : (row_bytes ? (uint64_t)frontier_per_slot / row_bytes : (1ull << 24) - 1);
+                                                : (row_bytes ? (uint64_t)frontier_per_slot / row_bytes : MAX_CHUNK);
         if (strict_budget && !(o && o->chunk_rows > 0) && chunk < MIN_CHUNK) {
             set_error(GFD_ERR_OUT_OF_MEMORY,
                       "frontier budget of %lld bytes per GFD holds fewer than %llu partial matches per level of GFD "
@@ -444,9 +474,19 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
                       (unsigned long long)(MIN_CHUNK * row_bytes));
             return GFD_ERR_OUT_OF_MEMORY;
         }
-        chunk = std::max<uint64_t>(MIN_CHUNK, std::min<uint64_t>(chunk, (1ull << 24) - 1));
+        chunk = std::max<uint64_t>(MIN_CHUNK, std::min<uint64_t>(chunk, MAX_CHUNK));
         D.chunk = chunk;
         Group::Off& F = G->offs[s];
+        if (big && row_bytes) {
+            Layout B;
+            B.size = 0;
+            D.big_chunk = std::max(chunk, std::min<uint64_t>(MAX_CHUNK, (G->big_bytes - 256 * 2 * MAXK) / row_bytes));
+            for (int l = 1; l <= P.k - 2; l++) {
+                D.big_rows[l] = B.take(4ull * row_width(l) * D.big_chunk);
+                D.big_wpre[l] = B.take(8ull * D.big_chunk);
+            }
+            big_need = std::max(big_need, B.size);
+        }
         for (int i = 0; i < P.k; i++) {
             D.cand_cap[i] = (uint32_t)lab_count(P.key[i].label);
             if (i > 0 && P.lv[i].par >= 0) D.cpi_cap[i] = G->index[G->level_index[s][i]].bound;
@@ -455,6 +495,10 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
             F.rows[l] = L.take(4ull * row_width(l) * chunk);
             F.wpre[l] = L.take(8ull * chunk);
         }
+    }
+    if (big) {
+        G->big_bytes = big_need;
+        G->o_big = L.take(G->big_bytes * N_BIG);
     }
     const size_t bm_bytes = 4ull * nwords;
     auto label_of = [&](int bm) { return G->keys[G->bm_key[bm]].label; };
@@ -473,7 +517,7 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
         const uint64_t cap = lab_count(label_of(G->finals[X.parent]));
         G->o_off.push_back(L.take(4ull * (cap + 1)));
         G->cpi_nch += cpi_chunks(cap);
-        G->cpi_bound += 8ull * std::max<uint64_t>(1, X.bound) + 256;
+        G->cpi_bound += X.entry() * std::max<uint64_t>(1, X.bound) + 256;
     }
     G->cmp_chunks = compact_chunks(g->dg);
     G->o_cmp_sums = L.take(4ull * G->cmp_chunks * G->finals.size());
@@ -481,7 +525,7 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
     G->o_cpi_tot = L.take(4ull * std::max<size_t>(1, G->index.size()));
     G->idx_inside = G->cpi_bound <= IDX_INSIDE;
     if (G->idx_inside)
-        for (const IndexSpec& X : G->index) G->o_idx.push_back(L.take(8ull * std::max<uint64_t>(1, X.bound)));
+        for (const IndexSpec& X : G->index) G->o_idx.push_back(L.take(X.entry() * std::max<uint64_t>(1, X.bound)));
     // the region uploaded from the host: keys and job tables
     G->o_jobs = L.size;
     G->o_keys = L.take(sizeof(FilterKey) * std::max(1, nkeys));
@@ -603,6 +647,7 @@ int group_build(gfd_graph* g, Group* G, const Tables& T, cudaStream_t st) {
         J.crank = rank_of(X.child);
         J.off = (uint32_t*)(base + G->o_off[x]);
         J.idx = G->idx_inside ? (int2*)(base + G->o_idx[x]) : nullptr;
+        J.ids = X.ids;
         J.cap = X.bound;
         J.out = X.dir;
         J.lab = X.lab;
@@ -711,7 +756,7 @@ int group_launch(gfd_graph* g, Group* G, const Tables& T, cudaMemPool_t pool, cu
             size_t bytes = 256;
             for (int j = 0; j < ncpi; j++) {
                 at[j] = bytes;
-                bytes = (bytes + 8ull * std::max<uint32_t>(1, tot[j]) + 255) & ~(size_t)255;
+                bytes = (bytes + G->index[j].entry() * std::max<uint32_t>(1, tot[j]) + 255) & ~(size_t)255;
             }
             void* p = nullptr;
             if (int rc = pool_alloc(pool, bytes, st, &p, "index edges")) return rc;
@@ -823,7 +868,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     Group G;
     const int64_t budget = (!o || o->frontier_budget_bytes <= 0) && g->tuned_budget > 0 ? g->tuned_budget
                                                                                         : default_budget(g, o);
-    if (int rc = group_plan(g, phis, n, o, budget / n, &G, o && o->frontier_budget_bytes > 0)) return rc;
+    if (int rc = group_plan(g, phis, n, o, budget / n, &G, o && o->frontier_budget_bytes > 0, true)) return rc;
     int kmax = 1;
     for (auto& P : G.plans) kmax = std::max(kmax, P.k);
     std::shared_ptr<Pool> shared_pool;
@@ -853,7 +898,11 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     const int lrc = group_launch(g, &G, T, pool, st, prof, launches, count);
     fr.p.push_back(G.cpi_base);
     if (lrc) return lrc;
-    const EnumArgs A = enum_args(g, T);
+    EnumArgs A = enum_args(g, T, kmax);
+    if (G.big_bytes) {
+        A.big = G.base + G.o_big;
+        A.big_bytes = G.big_bytes;
+    }
     if (int rc = enum_init(A, st)) return rc;
     bool general = false;  // any slot needing the general expansion
     for (int s = 0; s < n; s++) general |= G.plans[s].push_x || G.plans[s].n_components > 1;
@@ -1066,7 +1115,7 @@ int session_create(gfd_graph* g, int32_t max_slots, const gfd_opts* o, gfd_sessi
         return rc;
     if (int rc = mark_idle(S->T.state, max_slots, S->st)) return rc;  // every slot starts idle
     // the enumeration steps of one round, captured once (the tables never move)
-    const EnumArgs A = enum_args(g, S->T);
+    const EnumArgs A = enum_args(g, S->T, MAXK);  // any request
     if (int rc = capture_steps(A, S->variant, S->steps_per_round, S->st, &S->graph, &S->exec)) return rc;
     GFD_CUDA(cudaStreamSynchronize(S->st));
     *out = S.release();
@@ -1197,7 +1246,7 @@ int session_admit(gfd_session* S) {
     // whatever round it is running)
     GFD_CUDA(cudaEventRecord(S->ev_admit, sa));
     GFD_CUDA(cudaStreamWaitEvent(S->st, S->ev_admit, 0));
-    if (int rc = init_slots(enum_args(S->g, S->T), G->slot.data(), n, S->st)) return rc;
+    if (int rc = init_slots(enum_args(S->g, S->T, MAXK), G->slot.data(), n, S->st)) return rc;
     for (int i = 0; i < n; i++) S->slots[G->slot[i]].started = true;
     return GFD_OK;
 }
