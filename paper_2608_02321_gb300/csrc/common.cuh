@@ -82,11 +82,12 @@ struct DevGraph {
 // hash.
 __host__ __device__ __forceinline__ uint32_t sig_bit(uint32_t v) { return (v * 0x9E3779B1u) >> 26; }
 
-// Bit of vertex v in the filter of a row with d entries.
-__host__ __device__ __forceinline__ uint32_t filter_bit(uint32_t v, uint32_t d) {
-    const uint32_t bits = 8u * (d < (1u << 28) ? d : 1u << 28);
+// Bits of the filter of a row with d entries, and the bit of vertex v in it.
+__host__ __device__ __forceinline__ uint32_t filter_bits(uint32_t d) { return 8u * (d < (1u << 28) ? d : 1u << 28); }
+__host__ __device__ __forceinline__ uint32_t filter_bit_of(uint32_t v, uint32_t bits) {
     return (uint32_t)(((uint64_t)(v * 0x9E3779B1u) * bits) >> 32);
 }
+__host__ __device__ __forceinline__ uint32_t filter_bit(uint32_t v, uint32_t d) { return filter_bit_of(v, filter_bits(d)); }
 
 // Candidate filter key (Section III.B step 1a-1b): label, degree lower bounds
 // (self-loops excluded on both sides) and the self-loop expectation.

@@ -119,6 +119,7 @@ __device__ __forceinline__ int32_t edge_label(const DevGraph& g, uint32_t a, uin
     }
     const uint32_t end = hi;
     const uint32_t kk = key << g.lbits;
+    #pragma unroll 1
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
         if (loads) ++*loads;
@@ -173,6 +174,7 @@ __device__ __forceinline__ uint64_t ld_front(const uint64_t* p) { return *p; }
 
 // r in [lo, hi) with S[r] <= w < S[r+1]: the search limited to the rows of a tile.
 __device__ __forceinline__ uint32_t find_row_in(const uint32_t* S, uint32_t lo, uint32_t hi, uint64_t w) {
+    #pragma unroll 1
     while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) >> 1;
         if ((uint64_t)__ldg(S + mid) <= w) lo = mid;
@@ -181,6 +183,7 @@ __device__ __forceinline__ uint32_t find_row_in(const uint32_t* S, uint32_t lo, 
     return lo;
 }
 __device__ __forceinline__ uint32_t find_row_in(const uint64_t* S, uint32_t lo, uint32_t hi, uint64_t w) {
+    #pragma unroll 1
     while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) >> 1;
         if (__ldcg((const unsigned long long*)S + mid) <= w) lo = mid;
@@ -212,6 +215,7 @@ __device__ __forceinline__ int32_t cand_rank(const uint32_t* bm, const uint32_t*
 // Each round probes 32 evenly spaced entries and keeps the last one <= w.
 template <typename T>
 __device__ __forceinline__ uint32_t warp_find(const T* S, uint64_t lo, uint64_t hi, uint64_t w, int lane) {
+    #pragma unroll 1
     while (hi - lo > 32) {
         const uint64_t step = (hi - lo + 31) / 32;
         const uint64_t idx = lo + (uint64_t)lane * step;
@@ -230,6 +234,7 @@ __device__ __forceinline__ uint32_t warp_find(const T* S, uint64_t lo, uint64_t 
 // Exclusive warp scan of 64-bit values; *total receives the warp's sum.
 __device__ __forceinline__ uint64_t warp_excl_scan(uint64_t x, int lane, uint64_t* total) {
     uint64_t incl = x;
+    #pragma unroll 1
     for (int d = 1; d < 32; d <<= 1) {
         const uint64_t y = __shfl_up_sync(0xffffffffu, incl, d);
         if (lane >= d) incl += y;
@@ -238,25 +243,39 @@ __device__ __forceinline__ uint64_t warp_excl_scan(uint64_t x, int lane, uint64_
     return incl - x;
 }
 
-// The adjacency row of the first required edge (besides the generator's) at its
-// image; d = 0: there is none.
-struct NeededRow {
-    uint32_t e0, d;
+// A row filter: bits of it from base on (0: no filter to pass).
+struct FilterRow {
+    const uint8_t* base;
+    uint32_t bits;
+    __device__ __forceinline__ bool may_hold(uint32_t v) const {
+        const uint32_t b = filter_bit_of(v, bits);
+        return (__ldg(base + (b >> 3)) >> (b & 7)) & 1u;
+    }
 };
+
+// Fused expansion: the last-level candidates of one partial match in the warp's
+// sequence. src: where they start in their generator's source - where they start
+// in the sequence; who: lane | generator << 5.
+struct LastList {
+    const uint8_t* base;
+    uint32_t bits;
+    uint32_t src;
+};
+
+constexpr int LAST_WINDOWS = 2;  // windows of 32 candidates in flight at the last level
 
 // Per warp in (dynamic) shared memory.
 struct WarpShared {
     uint32_t chk[2 * MAXK];   // the current tile's pair checks, packed
     uint32_t chk2[2 * MAXK];  // the last level's, for fused expansion
-    int2 list[32];            // fused expansion: a partial match's candidates (see below)
-    uint64_t need[32];        // signature bits a candidate of the lane's partial match needs
-    NeededRow row[32];        // and the row it must be in
+    LastList list[32];        // fused expansion: the partial matches' candidates, in order
+    uint8_t who[32];          // whose each is: lane | generator << 5
     int32_t* rows;            // where the tile's new partial matches go
     uint64_t* wpre;
     uint64_t cap;
     uint64_t unused;
-    uint32_t qv[64];          // candidates that have them, waiting for their other checks,
-    uint8_t qo[64];           // and whose they are: lane | generator << 5
+    uint32_t qv[32 + 32 * LAST_WINDOWS];  // last-level candidates waiting for their other checks,
+    uint8_t qo[32 + 32 * LAST_WINDOWS];   // and whose they are: lane | generator << 5
     __device__ uint32_t* m(int col) { return reinterpret_cast<uint32_t*>(this + 1) + col; }  // [32 q + col]: the columns
 };
 // columns for patterns of up to kmax nodes (rows are loaded in groups of four)
@@ -276,6 +295,7 @@ __device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m
     const ulonglong2 sv = __ldg(g.sig + v);  // out-, in-neighbours
     cn.add(CNT_SIG_LOADS, 1);
     uint32_t open = 0;
+    #pragma unroll 1
     for (int c = 0; c < n; c++) {
         const uint32_t wd = cw[c];
         const uint32_t x = m[(wd & 15u) << 5];
@@ -300,6 +320,7 @@ __device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m
     probes += n - (skip >= 0);
     if (COUNT) cn.add(CNT_SIG_SETTLED, n - (skip >= 0) - __popc(open));
     if ((open & required) != required) return false;
+    #pragma unroll 1
     for (; open; open &= open - 1) {
         const int c = __ffs(open) - 1;
         const uint32_t wd = cw[c];
@@ -347,31 +368,31 @@ __device__ __forceinline__ bool tree_edge_agrees(const DevGraph& g, const LevelP
     return exp_ok(P.tlab, gl);
 }
 
-// Signature bits that a candidate of level P needs for its required edges to the
-// images in column m, when its candidates come from generator gen (whose own
-// check, or for gen 0 the tree edge, holds already).
-// row: where the first of these edges is looked up in the row filter, which tells
-// more than a long list's signature.
-__device__ __forceinline__ uint64_t needed_bits(const DevGraph& g, const LevelPlan& P, const uint32_t* m,
-                                                const uint32_t* cw, int gen, NeededRow* row) {
-    uint64_t need = ~0ull;
-    *row = NeededRow{0, 0};
-    const int skip = gen >= 1 && gen != GEN_LIST ? P.gen[gen - 1] : -1;
-    if (skip >= 0) need = sig_half(g, m[P.par << 5], P.tdir ? 0 : 1);
-    for (int c = P.nreq - 1; c >= 0; c--) {
-        if (c == skip) continue;
+// Where a last-level candidate (plan P, checks cw, from generator gen) of the
+// partial match in column m must be found first: the row filter of the first
+// required edge that is not the generator's, at its image. bits 0: none.
+__device__ __forceinline__ FilterRow first_row(const DevGraph& g, const LevelPlan& P, const uint32_t* m,
+                                               const uint32_t* cw, int gen) {
+    FilterRow f{nullptr, 0};
+    const int c = gen >= 1 && gen != GEN_LIST && P.gen[gen - 1] == 0 ? 1 : 0;
+    if (c < P.nreq) {
         const uint32_t x = m[(cw[c] & 15u) << 5];
         const bool in = (cw[c] >> 4) & 1u;  // edge v -> x: v among x's in-neighbours
-        need &= sig_half(g, x, in);
-        if (c == (skip == 0)) {
-            const uint32_t* const off = in ? g.in_off : g.out_off;
-            row->e0 = __ldg(off + x);
-            row->d = __ldg(off + x + 1) - row->e0;
-        }
+        const uint32_t* const off = in ? g.in_off : g.out_off;
+        const uint32_t e0 = __ldg(off + x);
+        f.base = (in ? g.in_filter : g.out_filter) + e0;
+        f.bits = filter_bits(__ldg(off + x + 1) - e0);
+        // (a generator's list is no longer than this one, so it is not empty)
     }
-    return need;
+    return f;
 }
 
+// The loops below have few rounds and are not unrolled (left to itself the
+// compiler unrolls most of them by four): the expansion's code, 150 KB unrolled and
+// 119 KB like this, does not fit the instruction caches, and its warps are each in
+// another part of it. Batch of 256 GFDs on 4M vertices: 144 -> 135 ms, a session of
+// 48 requests 39 -> 36 ms of rounds.
+//
 // The expansion step, warp-synchronous: every warp takes its own tiles of
 // work items (no block-wide barrier in the loop). A tile belongs to one slot
 // and one level; the warp finds them (and the rows the tile covers) with
@@ -381,11 +402,10 @@ __device__ __forceinline__ uint64_t needed_bits(const DevGraph& g, const LevelPl
 // registers; GEN = true adds component starts and X pushed down.
 //
 // The last level has most of the work items, and most fail their first required
-// edge. So its candidates pass two stages: every lane fetches one and tests the
-// signature bits that the partial match's required edges need together (one
-// 64-bit mask per partial match, `need`), some 40 instructions per 32 candidates;
-// those that pass wait in a queue until 32 are together for the other checks,
-// the literals and the output, which then run with full warps.
+// edge. So its candidates pass two stages: every lane fetches two and looks them up
+// in the row filter of that edge's other end (FilterRow, set up once per partial
+// match); those that pass wait in a queue until 32 are together for the other
+// checks, the literals and the output, which then run with full warps.
 template <int NT, bool GEN, bool COUNT>
 __device__ void expand_warps(const EnumArgs& A) {
     extern __shared__ __align__(16) uint8_t s_dyn[];
@@ -402,6 +422,7 @@ __device__ void expand_warps(const EnumArgs& A) {
     const DevGraph& g = A.g;
     const uint32_t total_tiles = *(volatile uint32_t*)&A.sched->total_tiles;
     uint32_t probes = 0;  // a statistic (saturates per warp)
+    #pragma unroll 1
     for (uint64_t t = gwarp; t < total_tiles;) {
         cn.mark();
         // the step's tiles: those of fusing slots first, then those of the other
@@ -460,6 +481,7 @@ __device__ void expand_warps(const EnumArgs& A) {
             bool viol = false;
             if (ok) {
                 bool x_ok = true;
+                #pragma unroll 1
                 for (int q = 0; q < D->nx && x_ok; q++)
                     if (!GEN || D->lit[q].lvl == L)
                         x_ok = lit_holds_at(g, D->lit[q], c, L, v, COUNT ? &attr_reads : nullptr);
@@ -467,6 +489,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                 else tile_matches++;
                 if (x_ok) {
                     bool y_ok = !D->y_false;
+                    #pragma unroll 1
                     for (int q = 0; q < D->ny && y_ok; q++)
                         y_ok = lit_holds_at(g, D->lit[D->nx + q], c, L, v, COUNT ? &attr_reads : nullptr);
                     viol = !y_ok;
@@ -487,52 +510,50 @@ __device__ void expand_warps(const EnumArgs& A) {
                     // the slot's own buffer: tuples in pattern-node order
                     if (idx < D->viol_cap) {
                         int32_t* out = D->viol + idx * k;
+                        #pragma unroll 1
                         for (int q = 0; q < k; q++) out[D->order[q]] = (int32_t)__ldg(g.orig + level_vertex(c, q, L, v));
                     }
                 } else if (idx < A.sched->varena_cap) {
                     // the run's arena: [slot, tuple in pattern-node order]
                     int32_t* rec = A.sched->varena + idx * A.sched->vstride;
                     rec[0] = s;
+                    #pragma unroll 1
                     for (int q = 0; q < k; q++) rec[1 + D->order[q]] = (int32_t)__ldg(g.orig + level_vertex(c, q, L, v));
                 }
             }
         };
-        // First stage of the last level (plan P, level L): one candidate per lane
-        // (ok lanes: position e in the source of generator gen, needed bits), the
-        // ones that pass appended to the queue.
-        auto first_stage = [&](const LevelPlan& P, int L, uint32_t queued, bool ok, uint32_t e, int gen, int owner,
-                               const uint64_t need, const NeededRow row) -> uint32_t {
-            uint32_t v = 0;
+        // First stage of the last level (plan P, level L): an item's candidate from
+        // the source of its generator,
+        auto last_raw = [&](const LevelPlan& P, const uint32_t* ids, uint32_t e, int gen) -> uint32_t {
+            if (gen == 0) return __ldg(ids + e);  // (index edges of the last level: ids alone)
+            if (GEN && gen == GEN_LIST) return (uint32_t)__ldg(ids + e);
+            return P.chk_dir[P.gen[gen - 1]] ? __ldg(g.in_adj + e) : __ldg(g.out_adj + e);
+        };
+        // and appending it to the queue if its row filter lets it pass.
+        auto first_stage = [&](const LevelPlan& P, int L, uint32_t queued, bool ok, uint32_t raw, int who,
+                               const FilterRow f) -> uint32_t {
+            uint32_t v = raw;
             if (ok) {
                 cn.add(CNT_ITEMS, 1);
                 cn.add(CNT_ITEMS_LAST, 1);
-                if (gen == 0) {
-                    v = __ldg(reinterpret_cast<const uint32_t*>(D->cpi_idx[L]) + e);  // ids only at the last level
-                } else if (GEN && gen == GEN_LIST) {
-                    v = (uint32_t)__ldg(D->cand[L] + e);
-                } else {
-                    // from the adjacency of the other end of a required back edge
-                    const int cg = P.gen[gen - 1];
-                    const uint32_t p = P.chk_dir[cg] ? __ldg(g.in_adj + e) : __ldg(g.out_adj + e);
-                    v = p >> g.lbits;
-                    ok = exp_ok(P.chk_exp[cg], (int32_t)(p & g.lmask));
-                }
-                ok = ok && ((need >> sig_bit(v)) & 1ull);
-                if (ok && row.d) {
-                    // the row's check: the first required one that is not the generator's
-                    const int c = gen >= 1 && gen != GEN_LIST && P.gen[gen - 1] == 0 ? 1 : 0;
-                    ok = row_filter(g, P.chk_dir[c], row.e0, row.d, v);
-                }
-                if (ok && gen != 0 && !(GEN && gen == GEN_LIST)) ok = (__ldg(D->bm[L] + (v >> 5)) >> (v & 31)) & 1u;
+                const int gen = who >> 5;
+                const bool adjacent = gen != 0 && !(GEN && gen == GEN_LIST);
+                if (adjacent) v = raw >> g.lbits;
+                if (f.bits) ok = f.may_hold(v);
+                if (adjacent && ok)  // from the adjacency of the other end of a required back edge
+                    ok = exp_ok(P.chk_exp[P.gen[gen - 1]], (int32_t)(raw & g.lmask)) &&
+                         ((__ldg(D->bm[L] + (v >> 5)) >> (v & 31)) & 1u);
             }
             const uint32_t pass = __ballot_sync(0xffffffffu, ok);
             if (ok) {
                 const uint32_t at = queued + __popc(pass & below);
                 W.qv[at] = v;
-                W.qo[at] = (uint8_t)(owner | gen << 5);
+                W.qo[at] = (uint8_t)who;
             }
-            __syncwarp();
             return queued + __popc(pass);
+        };
+        auto last_source = [&](int L, int gen) {
+            return GEN && gen == GEN_LIST ? (const uint32_t*)D->cand[L] : (const uint32_t*)D->cpi_idx[L];
         };
         // Second stage: the other checks of queue entry `at` (ok lanes), finish.
         auto second_stage = [&](const LevelPlan& P, int L, const uint32_t* checks, bool ok, uint32_t at) {
@@ -542,6 +563,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                 v = W.qv[at];
                 const int gen = W.qo[at] >> 5;
                 c = W.m(W.qo[at] & 31);
+                #pragma unroll 1
                 for (int q = 0; q < L && ok; q++)  // injectivity
                     if (((P.inj >> q) & 1u) && c[q << 5] == v) ok = false;
                 const int skip = gen >= 1 && gen != GEN_LIST ? P.gen[gen - 1] : -1;
@@ -556,6 +578,7 @@ __device__ void expand_warps(const EnumArgs& A) {
             // neighbour's image
             cn.add(CNT_PARTIALS, 1);
             uint64_t bd = 0;
+            #pragma unroll 1
             for (int q = 0; q < P.nreq; q++) {
                 const uint32_t x = c[P.chk_q[q] << 5];
                 bd += P.chk_dir[q] ? g.in_off[x + 1] - g.in_off[x] : g.out_off[x + 1] - g.out_off[x];
@@ -568,6 +591,7 @@ __device__ void expand_warps(const EnumArgs& A) {
         auto run_last_rows = [&] {
             cn.cycles(CNT_CYC_TILE);
             uint64_t w = wb;
+            #pragma unroll 1
             for (uint32_t r = rlo; w < we; r++) {
                 const uint64_t start = ld_front(Sl + r);
                 const uint64_t end = r + 1 < rhi1 ? min(we, ld_front(Sl + r + 1)) : we;
@@ -584,20 +608,32 @@ __device__ void expand_warps(const EnumArgs& A) {
                     base = LP.chk_dir[cg] ? __ldg(g.in_off + x) : __ldg(g.out_off + x);
                 }
                 if (COUNT && lane == 0 && w == start) count_partial(LP, c0);
-                NeededRow nrow;
-                const uint64_t need = needed_bits(g, LP, c0, cw, gen, &nrow);
+                const FilterRow f = first_row(g, LP, c0, cw, gen);
+                const uint32_t* const ids = last_source(i, gen);
                 uint32_t queued = 0;
+                #pragma unroll 1
                 while (w < end || queued) {
                     if (w < end) {
-                        queued = first_stage(LP, i, queued, w + lane < end, base + (uint32_t)(w - start) + lane, gen, 0, need, nrow);
-                        w += 32;
-                        if (queued < 32 && w < end) continue;
+                        uint32_t raw[LAST_WINDOWS];
+#pragma unroll
+                        for (int u = 0; u < LAST_WINDOWS; u++) {
+                            raw[u] = 0;
+                            if (w + 32 * u + lane < end) raw[u] = last_raw(LP, ids, base + (uint32_t)(w - start) + 32 * u + lane, gen);
+                        }
+#pragma unroll
+                        for (int u = 0; u < LAST_WINDOWS; u++)
+                            queued = first_stage(LP, i, queued, w + 32 * u + lane < end, raw[u], gen << 5, f);
+                        __syncwarp();
+                        w += 32 * LAST_WINDOWS;
                     }
-                    const uint32_t take = min(queued, 32u);
-                    second_stage(LP, i, cw, lane < (int)take, queued - take + lane);
-                    queued -= take;
-                    __syncwarp();
-                    cn.iteration(true);
+                    #pragma unroll 1
+                    while (queued >= 32 || (w >= end && queued)) {
+                        const uint32_t take = min(queued, 32u);
+                        second_stage(LP, i, cw, lane < (int)take, queued - take + lane);
+                        queued -= take;
+                        __syncwarp();
+                        cn.iteration(true);
+                    }
                 }
                 w = end;
             }
@@ -620,6 +656,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                 __syncwarp();
             }
             cn.cycles(CNT_CYC_TILE);
+            #pragma unroll 1
             for (uint64_t w0 = wb; w0 < we; w0 += 32) {
                 const uint64_t w = w0 + lane;
                 bool ok = w < we;
@@ -641,6 +678,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                     const uint64_t sv = widx < rhi1 ? (ROOT ? (uint64_t)__ldg(S0 + widx) : ld_front(Sl + widx))
                                                     : ~0ull;
                     int pos = 0;
+                    #pragma unroll 1
                     for (int step = 16; step >= 1; step >>= 1) {
                         const uint64_t x = __shfl_sync(0xffffffffu, sv, pos + step);
                         if (x <= w) pos += step;
@@ -681,6 +719,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                             // index base in one 8-byte load
                             rowp = rows_l + (uint64_t)r * rw;
                             const int4* r4 = reinterpret_cast<const int4*>(rowp);
+                            #pragma unroll 1
                             for (int q = 0; q <= l; q += 4) {
                                 const int4 t4 = r4[q >> 2];
                                 m[q << 5] = (uint32_t)t4.x;
@@ -725,6 +764,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                             }
                         }
                         // injectivity, then every other pattern pair, both directions
+                        #pragma unroll 1
                         for (int q = 0; q <= l && ok; q++)
                             if (((LP.inj >> q) & 1u) && m[q << 5] == v) ok = false;
                         ok = ok && pairs_agree<COUNT>(g, m, cw, nchk, LP.nreq, skip, v, probes, cn);
@@ -733,6 +773,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                     // X pushed down: the X literals whose ends are matched at this
                     // level (before the last one; the last level checks its own)
                     if (GEN && ok && D->push_x && !LAST)
+                        #pragma unroll 1
                         for (int q = 0; q < D->nx && ok; q++)
                             if (D->lit[q].lvl == i) ok = lit_holds_at(g, D->lit[q], m, i, v, COUNT ? &attr_reads : nullptr);
                 }
@@ -758,6 +799,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                             nbase = __ldg(co + ppn);
                             fo = __ldg(co + ppn + 1) - nbase;
                         }
+                        #pragma unroll 1
                         for (int q = 0; q < L2.ngen; q++) {
                             const int cg = L2.gen[q];
                             const uint32_t x = m[L2.chk_q[cg] << 5];
@@ -811,6 +853,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                                 // padding) in 16-byte stores, four ints at a time
                                 const int nw = row_width(i);
                                 int32_t* dst = W.rows + row * nw;
+                                #pragma unroll 1
                                 for (int t = 0; t < nw; t += 4) {
                                     int32_t e4[4];
     #pragma unroll
@@ -838,23 +881,23 @@ __device__ void expand_warps(const EnumArgs& A) {
                     if (fuse) {
                         // The last level of the lanes' new partial matches with small
                         // fan-outs, by the whole warp, end to end: W.list holds the
-                        // non-empty ones in order (start in the generator's source -
-                        // start in the sequence, lane | generator << 8); which of them
-                        // an item belongs to follows from the bits of the sequence's
-                        // window at which lists start. No candidate can have an empty
-                        // set of needed bits.
+                        // non-empty ones in order; which of them an item belongs to
+                        // follows from the bits of the sequence's window at which lists
+                        // start.
                         const int L = k - 1;
                         uint32_t left = fuse_me ? (uint32_t)fo : 0u;
+                        FilterRow f{nullptr, 0};
                         if (left) {
-                            const uint64_t need = needed_bits(g, L2, m, cw2, gen, &W.row[lane]);
-                            W.need[lane] = need;
-                            if (need == 0) left = 0;
+                            f = first_row(g, L2, m, cw2, gen);
                             if (COUNT) count_partial(L2, m);
                         }
+                        const uint32_t* const ids = last_source(L, GEN && L2.par < 0 ? GEN_LIST : 0);
                         // (a sequence of at most 32 x 2^26 items at a time)
+                        #pragma unroll 1
                         do {
                             const uint32_t ffo = min(left, 1u << 26);
                             uint32_t fin = ffo;
+                            #pragma unroll 1
                             for (int d = 1; d < 32; d <<= 1) {
                                 const uint32_t y = __shfl_up_sync(0xffffffffu, fin, d);
                                 if (lane >= d) fin += y;
@@ -863,25 +906,45 @@ __device__ void expand_warps(const EnumArgs& A) {
                             const uint32_t ftot = __shfl_sync(0xffffffffu, fin, 31);
                             if (lane == 0 && ftot) atomicAdd((unsigned long long*)&S->st_work, (unsigned long long)ftot);
                             const uint32_t some = __ballot_sync(0xffffffffu, ffo != 0);
-                            if (ffo) W.list[__popc(some & below)] = make_int2((int32_t)(nbase - fex), lane | gen << 8);
-                            __syncwarp();  // columns, needed bits and lists are read by other lanes
+                            if (ffo) {
+                                W.list[__popc(some & below)] = LastList{f.base, f.bits, nbase - fex};
+                                W.who[__popc(some & below)] = (uint8_t)(lane | gen << 5);
+                            }
+                            __syncwarp();  // columns and lists are read by other lanes
                             uint32_t begun = 0, queued = 0;
-                            for (uint32_t fb = 0; fb < ftot || queued; fb += 32) {
+                            #pragma unroll 1
+                            for (uint32_t fb = 0; fb < ftot || queued;) {
                                 if (fb < ftot) {
-                                    const uint32_t starts =
-                                        __reduce_or_sync(0xffffffffu, ffo && fex - fb < 32u ? 1u << (fex - fb) : 0u);
-                                    const uint32_t own = begun + __popc(starts & (below << 1 | 1u)) - 1;
-                                    begun += __popc(starts);
-                                    const bool it = fb + lane < ftot;
-                                    const int2 e = W.list[it ? own : 0];
-                                    queued = first_stage(L2, L, queued, it, fb + lane + (uint32_t)e.x, e.y >> 8, e.y & 31,
-                                                         W.need[e.y & 31], W.row[e.y & 31]);
-                                    if (queued < 32 && fb + 32 < ftot) continue;
+                                    // which list an item is of: the lists that start up to it
+                                    // (bit j of starts: one starts at the window's entry j)
+                                    uint32_t raw[LAST_WINDOWS], own[LAST_WINDOWS];
+#pragma unroll
+                                    for (int u = 0; u < LAST_WINDOWS; u++) {
+                                        const uint32_t at = fb + 32 * u;
+                                        const uint32_t starts =
+                                            __reduce_or_sync(0xffffffffu, ffo && fex - at < 32u ? 1u << (fex - at) : 0u);
+                                        own[u] = begun + __popc(starts & (below << 1 | 1u)) - 1;
+                                        begun += __popc(starts);
+                                        raw[u] = 0;
+                                        if (at + lane < ftot) raw[u] = last_raw(L2, ids, at + lane + W.list[own[u]].src, W.who[own[u]] >> 5);
+                                        else own[u] = 0;
+                                    }
+#pragma unroll
+                                    for (int u = 0; u < LAST_WINDOWS; u++) {
+                                        const LastList e = W.list[own[u]];
+                                        queued = first_stage(L2, L, queued, fb + 32 * u + lane < ftot, raw[u], W.who[own[u]],
+                                                             FilterRow{e.base, e.bits});
+                                    }
+                                    __syncwarp();
+                                    fb += 32 * LAST_WINDOWS;
                                 }
-                                const uint32_t take = min(queued, 32u);
-                                second_stage(L2, L, cw2, lane < (int)take, queued - take + lane);
-                                queued -= take;
-                                __syncwarp();  // the queue is written again
+                                #pragma unroll 1
+                                while (queued >= 32 || (fb >= ftot && queued)) {
+                                    const uint32_t take = min(queued, 32u);
+                                    second_stage(L2, L, cw2, lane < (int)take, queued - take + lane);
+                                    queued -= take;
+                                    __syncwarp();  // the queue is written again
+                                }
                             }
                             left -= ffo;
                             nbase += ffo;
