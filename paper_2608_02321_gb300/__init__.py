@@ -10,6 +10,7 @@ from __future__ import annotations
 import ctypes as C
 import os
 import threading
+from array import array
 
 import numpy as np
 
@@ -181,25 +182,54 @@ class _GfdBuf:
     """ctypes image of one GFD (keeps its arrays alive)."""
 
     def __init__(self, gfd):
+        try:
+            self._pack(gfd)
+        except (TypeError, ValueError, OverflowError, AttributeError):
+            self._convert(gfd)
+
+    def _pack(self, gfd):
+        """Plain sequences of whole numbers, as nearly all GFDs hold them: packed
+        without numpy or a ctypes object per literal (5 us a GFD against 14, which
+        a batch of 64 on a small graph took a quarter of its time for). Anything
+        else raises and is left to _convert."""
+        nl = array("i", gfd.node_label)
+        es, ed, el = array("i"), array("i"), array("i")
+        for a, b, c in gfd.edges:
+            es.append(a)
+            ed.append(b)
+            el.append(c)
+
+        def lits(ls):
+            flat = array("i")
+            for q in ls:
+                flat.extend((q.kind, q.x, q.a, q.y, q.b, q.c))
+            return flat
+        X, Y = lits(gfd.X), lits(gfd.Y)
+        self.keep = (nl, es, ed, el, X, Y)
+        p = [v.buffer_info()[0] if v else None for v in self.keep]
+        self.s = gfd_gfd(len(nl), p[0], len(es), p[1], p[2], p[3], len(X) // 6, p[4], len(Y) // 6, p[5],
+                         1 if gfd.y_false else 0)
+
+    def _convert(self, gfd):
         k = len(gfd.node_label)
-        self.nl = _i32(gfd.node_label)
+        nl = _i32(gfd.node_label)
         e = np.asarray(gfd.edges, dtype=np.int32).reshape(-1, 3)
-        self.es, self.ed, self.el = _i32(e[:, 0]), _i32(e[:, 1]), _i32(e[:, 2])
+        es, ed, el = _i32(e[:, 0]), _i32(e[:, 1]), _i32(e[:, 2])
 
         def lits(ls):
             arr = (gfd_literal * max(1, len(ls)))()
             for i, l in enumerate(ls):
                 arr[i] = gfd_literal(l.kind, l.x, l.a, l.y, l.b, l.c)
             return arr
-        self.X = lits(gfd.X)
-        self.Y = lits(gfd.Y)
+        X, Y = lits(gfd.X), lits(gfd.Y)
+        self.keep = (nl, es, ed, el, X, Y)
         s = gfd_gfd()
         s.k = k
-        s.node_label = _ptr(self.nl)
+        s.node_label = _ptr(nl)
         s.m = e.shape[0]
-        s.esrc, s.edst, s.elabel = _ptr(self.es), _ptr(self.ed), _ptr(self.el)
-        s.nx, s.X = len(gfd.X), C.cast(self.X, C.c_void_p)
-        s.ny, s.Y = len(gfd.Y), C.cast(self.Y, C.c_void_p)
+        s.esrc, s.edst, s.elabel = _ptr(es), _ptr(ed), _ptr(el)
+        s.nx, s.X = len(gfd.X), C.cast(X, C.c_void_p)
+        s.ny, s.Y = len(gfd.Y), C.cast(Y, C.c_void_p)
         s.y_false = 1 if gfd.y_false else 0
         self.s = s
 
