@@ -175,6 +175,8 @@ struct SlotState {
     uint64_t total[MAXK];     // work items at level l
     uint64_t cursor[MAXK];    // work items of level l already expanded
     uint64_t ctr[MAXK];       // packed rows/work counter of level l (filled by l-1)
+    uint64_t wide;            // work items of the next step that fuses the last level
+    uint64_t work0;           // st_work when the step was planned
     uint64_t row_limit;       // counter value of the first rows of the step that found no room (~0: none)
     uint64_t cb, ce;          // current step's work range at level `cur`
     uint64_t n_matches;

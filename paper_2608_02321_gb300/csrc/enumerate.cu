@@ -39,7 +39,10 @@ namespace gfd {
 namespace {
 
 constexpr int CTRL_THREADS = 1024;
-constexpr uint64_t LAST_LEVEL_CHUNK = 1ull << 25;  // work items per step at the last two levels
+constexpr uint64_t LAST_LEVEL_CHUNK = 1ull << 25;  // most work items per step at the last two levels
+// last-level items that a step of the level before should lead to at most (some
+// tenths of a second, far below the limit of a wait at the grid barrier)
+constexpr uint64_t FUSED_STEP_WORK = 1ull << 33;
 // generator stored in a row for a next level that starts a pattern component:
 // its candidates are the level's candidate list (fan-out |C| for every row)
 constexpr int GEN_LIST = 4;
@@ -990,6 +993,7 @@ __device__ void slot_start(const SlotDesc* D, SlotState* S) {
         if (D->lv[i].par >= 0) S->st_cpi += D->cpi_off[i][S->ncand[D->lv[i].par]];
     S->nrows[0] = S->ncand[0];
     S->big = 0;
+    S->wide = 0;
     for (int l = 1; l <= D->k - 2; l++) {
         S->rows[l] = D->rows[l];
         S->wpre[l] = D->wpre[l];
@@ -1043,6 +1047,19 @@ __device__ void control_step(const EnumArgs& A, bool first) {
                     const uint64_t c = min(__ldcg((const unsigned long long*)&S->ctr[l + 1]),
                                            __ldcg((const unsigned long long*)&S->row_limit));
                     const uint64_t rows = c >> ROW_SHIFT;
+                    if (l + 1 == k - 2 && S->ce > S->cb) {
+                        // The next such step: as many items as would, like this step's,
+                        // fill four fifths of the rows and lead to FUSED_STEP_WORK
+                        // last-level items, and at most eight times as many. Items that
+                        // find no row are expanded in place by the warp that has them,
+                        // so that must stay the exception.
+                        const uint64_t items = S->ce - S->cb, cap = S->cap[l + 1];
+                        const uint64_t work = (c & WORK_MASK) + (__ldcg((const unsigned long long*)&S->st_work) - S->work0);
+                        uint64_t fit = min((uint64_t)LAST_LEVEL_CHUNK, 8 * max(items, cap));
+                        if (rows) fit = min(fit, cap * 4 / 5 * items / rows);
+                        if (work) fit = min(fit, FUSED_STEP_WORK / work * items + FUSED_STEP_WORK % work * items / work);
+                        S->wide = fit;
+                    }
                     if (rows > 0) {
                         S->nrows[l + 1] = rows;
                         S->total[l + 1] = c & WORK_MASK;
@@ -1070,15 +1087,17 @@ __device__ void control_step(const EnumArgs& A, bool first) {
                 }
                 S->cb = S->cursor[l];
                 // the last level writes no partial matches, and the one before (fused)
-                // expands those without a row at once, so their steps are not bounded
-                // by the row buffers; a chunk of them per step left the last few large
-                // GFDs of a batch with hundreds of steps of a few iterations per warp
-                const bool wide = k == 1 || l + 1 >= k - 2;
-                const uint64_t step = wide ? max(D->chunk, (uint64_t)LAST_LEVEL_CHUNK) : S->cap[l + 1];
+                // few, and expands those without a row at once, so their steps are not
+                // bounded by the row buffers; a chunk of them per step left the last few
+                // large GFDs of a batch with hundreds of steps of a few iterations per warp
+                const uint64_t step = k == 1 || l + 1 == k - 1 ? max(D->chunk, (uint64_t)LAST_LEVEL_CHUNK)
+                                      : l + 1 == k - 2         ? max(S->cap[l + 1], S->wide)
+                                                               : S->cap[l + 1];
                 S->ce = min(S->cb + step, S->total[l]);
                 if (k > 1 && l + 1 <= k - 2) S->ctr[l + 1] = 0;
                 S->row_limit = ~0ull;
                 S->st_work += S->ce - S->cb;
+                S->work0 = S->st_work;
                 atomicAdd(&active_s, 1);
                 atomicAdd(&work_s, (unsigned long long)(S->ce - S->cb));
             }
