@@ -379,10 +379,11 @@ def main():
     b_enum = (model["enum_index_reads"] + model["enum_back_scans"] + model["enum_negative_probes"]
               + model["literal_reads"] + model["output"])
     b_step = sum(model.values())
-    # what the kernel itself loads: 8 B per index entry (position, id), 16 B
-    # per signature, one sector per search step actually taken and per
-    # attribute, the partial matches written, the output
-    b_kernel = (8 * cnt["items"] + 16 * cnt["sig_loads"] + 32 * cnt["search_loads"] + 32 * cnt["attr_reads"]
+    # what the kernel itself loads: 8 B per index entry (position, id; 4 B at the
+    # last level, ids alone), 16 B per signature or row filter lookup, one sector
+    # per search step actually taken and per attribute, the partial matches
+    # written, the output
+    b_kernel = (8 * cnt["items"] - 4 * cnt["items_last"] + 16 * cnt["sig_loads"] + 32 * cnt["search_loads"] + 32 * cnt["attr_reads"]
                 + 8 * cnt["rows"] + out_bytes)
     t_enum = float(np.mean(enum_ms)) / 1000.0
     peaks = {}

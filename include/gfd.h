@@ -174,7 +174,8 @@ typedef struct {
                                       GFD_ERR_OUT_OF_MEMORY (calls with
                                       chunk_rows set, and sessions, use at
                                       least 1024 instead) */
-    int32_t chunk_rows;            /* partial matches expanded per step and GFD */
+    int32_t chunk_rows;            /* partial matches held per level and GFD (0: from
+                                      the budget) */
     int32_t kernel_variant;        /* enumeration kernel: 0 = the graph's tuned
                                       choice (gfd_autotune) or the default;
                                       1..6 = a fixed variant (threads per block
@@ -274,10 +275,10 @@ double gfd_result_profile(const gfd_result *r, int32_t which, int64_t *launches)
  * candidate list), 8 of them at the last level, 9 partial matches expanded,
  * 10 sum over expanded partial matches of the adjacency lengths of their
  * backward non-tree neighbours' images, 11 pair checks, 12 of them settled by
- * the neighbourhood signature, 13 adjacency binary searches, 14 adjacency
+ * a neighbourhood signature or row filter, 13 adjacency binary searches, 14 adjacency
  * entries those searches read, 15 absent-edge checks, 16 sum over absent-edge
  * checks of ceil(log2(d + 1)) (d the shorter adjacency list), 17 signature
- * loads, 18 attribute loads of literal checks, 19 partial matches written,
+ * and row filter loads, 18 attribute loads of literal checks, 19 partial matches written,
  * 20 candidates whose adjacency the refinement and index build scanned, 21
  * adjacency entries they read, 22 warp iterations of the expansion, 23 sum over
  * them of the largest number of search loads one lane made, 24..26 SM cycles

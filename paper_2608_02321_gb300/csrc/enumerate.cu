@@ -9,8 +9,9 @@
 // edge of r's tree parent), found by binary search in the exclusive prefix of
 // the rows' fan-outs, so hub vertices are split evenly over threads. Each work
 // item yields at most one partial match of level l+1, so a level-l chunk of
-// `chunk` items always fits the next buffer; when a level is exhausted the slot
-// pops back to the previous level (depth-first), bounding memory.
+// `cap` items always fits the next buffer (steps that make the second-to-last
+// level take more, since they store few of theirs); when a level is exhausted the
+// slot pops back to the previous level (depth-first), bounding memory.
 //
 // A candidate v for pattern node u = order[i] extending partial match m passes
 // when: v != m[q] for earlier label-compatible levels q (injectivity), and for
@@ -20,7 +21,7 @@
 // Section II; the CFL-Match index alone would allow them, Section III). The
 // spanning-tree edge to the parent is guaranteed by the index and skipped.
 //
-// Survivors are appended with one atomic per block on a packed 64-bit counter
+// Survivors are appended with one atomic per warp on a packed 64-bit counter
 // (rows << 40 | fan-out sum), which gives each row both its index and the
 // exclusive prefix of fan-outs needed by the next step's search, consistently.
 //
@@ -304,17 +305,21 @@ __device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m
         const uint32_t x = m[(wd & 15u) << 5];
         const uint64_t half = (wd >> 4) & 1u ? sv.x : sv.y;  // edge v -> x, else x -> v
         open |= (uint32_t)((half >> sig_bit(x)) & 1ull) << c;
-        if (COUNT && c != skip) {
-            cn.add(CNT_CHECKS, 1);
-            if (c >= nreq) {
-                const bool out = (wd >> 4) & 1u;
-                const uint32_t dv = out ? g.out_off[v + 1] - g.out_off[v] : g.in_off[v + 1] - g.in_off[v];
-                const uint32_t dx = out ? g.in_off[x + 1] - g.in_off[x] : g.out_off[x + 1] - g.out_off[x];
-                cn.add(CNT_NEG_CHECKS, 1);
-                cn.add(CNT_NEG_LOGD, ceil_log2_1(min(dv, dx)));
-            }
-        }
+        if (COUNT && c != skip) cn.add(CNT_CHECKS, 1);
     }
+    // counting pass: the absent edges, of candidates whose required edges agree
+    bool counted = !COUNT;
+    auto count_absent = [&] {
+        counted = true;
+        for (int c = nreq; c < n; c++) {
+            const uint32_t x = m[(cw[c] & 15u) << 5];
+            const bool out = (cw[c] >> 4) & 1u;
+            const uint32_t dv = out ? g.out_off[v + 1] - g.out_off[v] : g.in_off[v + 1] - g.in_off[v];
+            const uint32_t dx = out ? g.in_off[x + 1] - g.in_off[x] : g.out_off[x + 1] - g.out_off[x];
+            cn.add(CNT_NEG_CHECKS, 1);
+            cn.add(CNT_NEG_LOGD, ceil_log2_1(min(dv, dx)));
+        }
+    };
     uint32_t required = (1u << nreq) - 1u;  // (at most 2 (MAXK - 1) = 30 checks)
     if (skip >= 0) {
         open &= ~(1u << skip);
@@ -326,6 +331,7 @@ __device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m
     #pragma unroll 1
     for (; open; open &= open - 1) {
         const int c = __ffs(open) - 1;
+        if (COUNT && c >= nreq && !counted) count_absent();
         const uint32_t wd = cw[c];
         const uint32_t x = m[(wd & 15u) << 5];
         const bool out = (wd >> 4) & 1u;
@@ -343,6 +349,7 @@ __device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m
         }
         if (!exp_ok(ex, gl)) return false;
     }
+    if (COUNT && !counted) count_absent();
     return true;
 }
 
