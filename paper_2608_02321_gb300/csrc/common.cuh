@@ -41,6 +41,16 @@ constexpr int32_t NOEDGE = -2;
 constexpr int ROW_SHIFT = 40;
 constexpr uint64_t WORK_MASK = (1ull << ROW_SHIFT) - 1;
 
+// What adding a warp's partial matches (add, packed alike) to a counter that reads
+// c comes to, with room for cap rows. A sum of fan-outs past WORK_MASK carries into
+// the rows and starts again near 0, so adders after it may see room again: it must
+// end the slot. Rows only grow: once they are out they stay out.
+enum : int { ROWS_FIT = 0, ROWS_OUT = 1, WORK_OUT = 2 };
+__host__ __device__ inline int counter_add(uint64_t c, uint64_t add, uint64_t cap) {
+    if ((c >> ROW_SHIFT) + (add >> ROW_SHIFT) > cap) return ROWS_OUT;
+    return (c & WORK_MASK) + (add & WORK_MASK) > WORK_MASK ? WORK_OUT : ROWS_FIT;
+}
+
 // Degree classes (edges in both directions together): class c holds the vertices
 // with more than class_degree(c) that are not in an earlier class, the last class
 // the rest. Limits of 512, 128 and 32 shorten the longest work items of small

@@ -830,28 +830,26 @@ __device__ void expand_warps(const EnumArgs& A) {
                     if (__any_sync(0xffffffffu, row_me)) excl = warp_excl_scan(packed, lane, &total);
                     if (total) {
                         unsigned long long old = 0;
-                        bool over = false;
+                        int full = ROWS_FIT;
                         if (lane == 0) {
-                            auto no_room = [&](unsigned long long c) {
-                                return (c & WORK_MASK) + (total & WORK_MASK) > WORK_MASK ||
-                                       (c >> ROW_SHIFT) + (total >> ROW_SHIFT) > W.cap;
-                            };
                             // a full level is not counted up any further (the few warps
                             // that still do stay below the counter's 2^24 rows)
-                            over = fuse && no_room(__ldcg((const unsigned long long*)&S->ctr[i]));
-                            if (!over) {
+                            if (fuse) full = counter_add(__ldcg((const unsigned long long*)&S->ctr[i]), total, W.cap);
+                            if (full == ROWS_FIT) {
                                 old = atomicAdd((unsigned long long*)&S->ctr[i], (unsigned long long)total);
-                                over = no_room(old);
-                                if (over && fuse) atomicMin((unsigned long long*)&S->row_limit, old);
-                                else if (over) atomicExch(&S->err, DERR_COUNTER_OVERFLOW);
+                                full = counter_add(old, total, W.cap);
+                                if (full == ROWS_OUT && fuse) atomicMin((unsigned long long*)&S->row_limit, old);
                             }
+                            if (full == WORK_OUT || (full && !fuse)) atomicExch(&S->err, DERR_COUNTER_OVERFLOW);
                         }
                         old = __shfl_sync(0xffffffffu, old, 0);
                         // a step that fuses takes more items than the level has rows
                         // for: partial matches without a row are expanded here too
-                        if (fuse && __shfl_sync(0xffffffffu, (int)over, 0)) {
+                        // (not those of a sum that is out: the slot has ended)
+                        full = fuse ? __shfl_sync(0xffffffffu, full, 0) : ROWS_FIT;
+                        if (full) {
                             row_me = false;
-                            fuse_me = ok;
+                            fuse_me = ok && full == ROWS_OUT;
                         }
                         // the warp's new partial matches take rows [row0, row0 + its
                         // count) of the level's buffer, in lane order
