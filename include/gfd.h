@@ -161,7 +161,7 @@ typedef struct {
 
 #define GFD_FLAG_COUNT         0x80 /* counting pass: run the enumeration with an
                                        instrumented kernel that counts what the
-                                       run reads (gfd_result_stat 7..28); the
+                                       run reads (gfd_result_stat 7..29); the
                                        results are unchanged, the run is slower */
 
 /* Tuning options; a NULL gfd_opts* or zero fields select the defaults. */
@@ -269,8 +269,8 @@ double gfd_result_profile(const gfd_result *r, int32_t which, int64_t *launches)
 /* Statistics of the run: 0 supersteps, 1 work items expanded, 2 partial
  * matches written, 3 edge-lookup probes (whole run), 4 candidate-list entries
  * (sum over pattern nodes), 5 index entries, 6 number of extra runs made
- * because the violations of the call outgrew max_violations_hint. With
- * GFD_FLAG_COUNT, 7..28 are the whole call's counters of what its kernels read:
+ * because the violations of the call outgrew max_violations_hint, or because the
+ * size of a step was misjudged. With GFD_FLAG_COUNT, 7..29 are the whole call's counters of what its kernels read:
  * 7 work items (entries of the index lists N_u, Section III.B, or of another
  * candidate list), 8 of them at the last level, 9 partial matches expanded,
  * 10 sum over expanded partial matches of the adjacency lengths of their
@@ -285,7 +285,8 @@ double gfd_result_profile(const gfd_result *r, int32_t which, int64_t *launches)
  * warps spent setting up tiles, in iterations at intermediate levels and at the
  * last level, 27 warp iterations at intermediate levels, 28 the number of
  * distinct filter keys (high 32 bits) and of candidate bitmaps compacted (low
- * 32 bits). */
+ * 32 bits), 29 partial matches that found no row in their step and were expanded
+ * where they were made. */
 uint64_t gfd_result_stat(const gfd_result *r, int32_t which);
 /* The refined candidate list C(u) of pattern node `node` (Section III.B step
  * 1c: label and degree filter, then top-down and bottom-up refinement), kept by

@@ -230,7 +230,8 @@ enum : int {
     CNT_CYC_LAST,      // SM cycles of warp iterations at the last level
     CNT_ITERS_MID,     // warp iterations at intermediate levels
     CNT_HOST,          // filled by the host: distinct filter keys << 32 | bitmaps
-    N_CNT = 22
+    CNT_NO_ROW,        // partial matches expanded where they were made for want of a row
+    N_CNT = 23
 };
 
 // Scheduler state shared by all slots of a run (device).
@@ -248,6 +249,7 @@ struct Sched {
     uint64_t probes;
     uint64_t t_start;         // globaltimer at the first step
     uint64_t run_limit_ns;    // limit of the whole enumeration
+    uint64_t spilled;         // last-level candidates expanded in this step for want of a row
     // violations of all slots: records [slot, h(x_0), ..., h(x_{k-1})] of
     // vstride ints appended at varena_used; records past varena_cap are counted
     // but not stored
@@ -273,6 +275,8 @@ enum : int32_t {
     DERR_COUNTER_OVERFLOW = 1,
     DERR_TIMEOUT = 2,
     DERR_CAPACITY = 3,
+    DERR_WIDE = 4,  // a step grown beyond its level's rows, or in a large buffer, did not come out:
+                    // again with steps of as many items as there are rows, without large buffers
 };
 
 __host__ __device__ inline bool label_ok(int32_t want, int32_t have) {

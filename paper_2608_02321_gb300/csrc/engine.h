@@ -210,6 +210,7 @@ struct EnumArgs {
     int32_t tile;         // largest number of work items per tile
     int32_t n_warps;      // warps of the expansion grid (0: unknown, tiles of `tile`)
     int32_t kmax;         // nodes of the largest pattern a slot may hold
+    int32_t narrow;       // steps take no more items than the level to fill has rows
     uint8_t* big;         // N_BIG large frontier buffers of big_bytes each (null: none)
     uint64_t big_bytes;
     uint32_t columns;     // words of a warp's columns in shared memory (set at launch)
@@ -245,7 +246,10 @@ int device_sms();
 int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out);
 void graph_free(gfd_graph* g);
 void engine_free(Engine* e);
-int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opts* o, gfd_result** out);
+// narrow: no step takes more items than the level that it fills has rows, and no
+// large buffers (the second run of a call in which such a step did not come out).
+int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opts* o, gfd_result** out,
+              bool narrow = false);
 int session_create(gfd_graph* g, int32_t max_slots, const gfd_opts* o, gfd_session** out);
 void session_free(gfd_session* s);
 int session_submit(gfd_session* s, const gfd_gfd* phi, int64_t* id);

@@ -41,9 +41,13 @@ namespace {
 
 constexpr int CTRL_THREADS = 1024;
 constexpr uint64_t LAST_LEVEL_CHUNK = 1ull << 25;  // most work items per step at the last two levels
-// last-level items that a step of the level before should lead to at most (some
-// tenths of a second, far below the limit of a wait at the grid barrier)
+// Last-level items that a step of the level before should lead to at most, all its
+// slots together, and that it may expand in place for want of a row (0.3 s for lists
+// of 200,000, far below the limit of a wait at the grid barrier).
 constexpr uint64_t FUSED_STEP_WORK = 1ull << 33;
+// Longest candidate list expanded in place for want of a row: one warp's work, up to
+// a tile of them (2^27 items, about a second) before it looks for the next.
+constexpr uint32_t SPILL_FANOUT = 1u << 18;
 // generator stored in a row for a next level that starts a pattern component:
 // its candidates are the level's candidate list (fan-out |C| for every row)
 constexpr int GEN_LIST = 4;
@@ -840,13 +844,27 @@ __device__ void expand_warps(const EnumArgs& A) {
                                 full = counter_add(old, total, W.cap);
                                 if (full == ROWS_OUT && fuse) atomicMin((unsigned long long*)&S->row_limit, old);
                             }
-                            if (full == WORK_OUT || (full && !fuse)) atomicExch(&S->err, DERR_COUNTER_OVERFLOW);
+                            if (full == WORK_OUT || (full && !fuse)) {
+                                const uint64_t items = __ldcg((const unsigned long long*)&S->ce) - __ldcg((const unsigned long long*)&S->cb);
+                                atomicExch(&S->err, __ldcg(&S->big) || items > W.cap ? DERR_WIDE : DERR_COUNTER_OVERFLOW);
+                            }
                         }
                         old = __shfl_sync(0xffffffffu, old, 0);
                         // a step that fuses takes more items than the level has rows
                         // for: partial matches without a row are expanded here too
-                        // (not those of a sum that is out: the slot has ended)
+                        // (not those of a slot that has ended)
                         full = fuse ? __shfl_sync(0xffffffffu, full, 0) : ROWS_FIT;
+                        if (full == ROWS_OUT) {
+                            // within bounds: the step's size is a guess from the one before
+                            const uint64_t work = total & WORK_MASK;
+                            bool stop = __reduce_max_sync(0xffffffffu, row_me ? (uint32_t)fo : 0u) > SPILL_FANOUT;
+                            if (lane == 0) {
+                                stop = stop || atomicAdd((unsigned long long*)&A.sched->spilled, (unsigned long long)work) + work > FUSED_STEP_WORK;
+                                if (stop) atomicExch(&S->err, DERR_WIDE);
+                            }
+                            if (__shfl_sync(0xffffffffu, (int)stop, 0)) full = WORK_OUT;
+                            else cn.add(CNT_NO_ROW, row_me);
+                        }
                         if (full) {
                             row_me = false;
                             fuse_me = ok && full == ROWS_OUT;
@@ -893,70 +911,64 @@ __device__ void expand_warps(const EnumArgs& A) {
                         // follows from the bits of the sequence's window at which lists
                         // start.
                         const int L = k - 1;
-                        uint32_t left = fuse_me ? (uint32_t)fo : 0u;
+                        // (at most 32 x SPILL_FANOUT items)
+                        const uint32_t ffo = fuse_me ? (uint32_t)fo : 0u;
                         FilterRow f{nullptr, 0};
-                        if (left) {
+                        if (ffo) {
                             f = first_row(g, L2, m, cw2, gen);
                             if (COUNT) count_partial(L2, m);
                         }
                         const uint32_t* const ids = last_source(L, GEN && L2.par < 0 ? GEN_LIST : 0);
-                        // (a sequence of at most 32 x 2^26 items at a time)
+                        uint32_t fin = ffo;
                         #pragma unroll 1
-                        do {
-                            const uint32_t ffo = min(left, 1u << 26);
-                            uint32_t fin = ffo;
-                            #pragma unroll 1
-                            for (int d = 1; d < 32; d <<= 1) {
-                                const uint32_t y = __shfl_up_sync(0xffffffffu, fin, d);
-                                if (lane >= d) fin += y;
-                            }
-                            const uint32_t fex = fin - ffo;
-                            const uint32_t ftot = __shfl_sync(0xffffffffu, fin, 31);
-                            if (lane == 0 && ftot) atomicAdd((unsigned long long*)&S->st_work, (unsigned long long)ftot);
-                            const uint32_t some = __ballot_sync(0xffffffffu, ffo != 0);
-                            if (ffo) {
-                                W.list[__popc(some & below)] = LastList{f.base, f.bits, nbase - fex};
-                                W.who[__popc(some & below)] = (uint8_t)(lane | gen << 5);
-                            }
-                            __syncwarp();  // columns and lists are read by other lanes
-                            uint32_t begun = 0, queued = 0;
-                            #pragma unroll 1
-                            for (uint32_t fb = 0; fb < ftot || queued;) {
-                                if (fb < ftot) {
-                                    // which list an item is of: the lists that start up to it
-                                    // (bit j of starts: one starts at the window's entry j)
-                                    uint32_t raw[LAST_WINDOWS], own[LAST_WINDOWS];
+                        for (int d = 1; d < 32; d <<= 1) {
+                            const uint32_t y = __shfl_up_sync(0xffffffffu, fin, d);
+                            if (lane >= d) fin += y;
+                        }
+                        const uint32_t fex = fin - ffo;
+                        const uint32_t ftot = __shfl_sync(0xffffffffu, fin, 31);
+                        if (lane == 0 && ftot) atomicAdd((unsigned long long*)&S->st_work, (unsigned long long)ftot);
+                        const uint32_t some = __ballot_sync(0xffffffffu, ffo != 0);
+                        if (ffo) {
+                            W.list[__popc(some & below)] = LastList{f.base, f.bits, nbase - fex};
+                            W.who[__popc(some & below)] = (uint8_t)(lane | gen << 5);
+                        }
+                        __syncwarp();  // columns and lists are read by other lanes
+                        uint32_t begun = 0, queued = 0;
+                        #pragma unroll 1
+                        for (uint32_t fb = 0; fb < ftot || queued;) {
+                            if (fb < ftot) {
+                                // which list an item is of: the lists that start up to it
+                                // (bit j of starts: one starts at the window's entry j)
+                                uint32_t raw[LAST_WINDOWS], own[LAST_WINDOWS];
 #pragma unroll
-                                    for (int u = 0; u < LAST_WINDOWS; u++) {
-                                        const uint32_t at = fb + 32 * u;
-                                        const uint32_t starts =
-                                            __reduce_or_sync(0xffffffffu, ffo && fex - at < 32u ? 1u << (fex - at) : 0u);
-                                        own[u] = begun + __popc(starts & (below << 1 | 1u)) - 1;
-                                        begun += __popc(starts);
-                                        raw[u] = 0;
-                                        if (at + lane < ftot) raw[u] = last_raw(L2, ids, at + lane + W.list[own[u]].src, W.who[own[u]] >> 5);
-                                        else own[u] = 0;
-                                    }
+                                for (int u = 0; u < LAST_WINDOWS; u++) {
+                                    const uint32_t at = fb + 32 * u;
+                                    const uint32_t starts =
+                                        __reduce_or_sync(0xffffffffu, ffo && fex - at < 32u ? 1u << (fex - at) : 0u);
+                                    own[u] = begun + __popc(starts & (below << 1 | 1u)) - 1;
+                                    begun += __popc(starts);
+                                    raw[u] = 0;
+                                    if (at + lane < ftot) raw[u] = last_raw(L2, ids, at + lane + W.list[own[u]].src, W.who[own[u]] >> 5);
+                                    else own[u] = 0;
+                                }
 #pragma unroll
-                                    for (int u = 0; u < LAST_WINDOWS; u++) {
-                                        const LastList e = W.list[own[u]];
-                                        queued = first_stage(L2, L, queued, fb + 32 * u + lane < ftot, raw[u], W.who[own[u]],
-                                                             FilterRow{e.base, e.bits});
-                                    }
-                                    __syncwarp();
-                                    fb += 32 * LAST_WINDOWS;
+                                for (int u = 0; u < LAST_WINDOWS; u++) {
+                                    const LastList e = W.list[own[u]];
+                                    queued = first_stage(L2, L, queued, fb + 32 * u + lane < ftot, raw[u], W.who[own[u]],
+                                                         FilterRow{e.base, e.bits});
                                 }
-                                #pragma unroll 1
-                                while (queued >= 32 || (fb >= ftot && queued)) {
-                                    const uint32_t take = min(queued, 32u);
-                                    second_stage(L2, L, cw2, lane < (int)take, queued - take + lane);
-                                    queued -= take;
-                                    __syncwarp();  // the queue is written again
-                                }
+                                __syncwarp();
+                                fb += 32 * LAST_WINDOWS;
                             }
-                            left -= ffo;
-                            nbase += ffo;
-                        } while (__any_sync(0xffffffffu, left != 0));
+                            #pragma unroll 1
+                            while (queued >= 32 || (fb >= ftot && queued)) {
+                                const uint32_t take = min(queued, 32u);
+                                second_stage(L2, L, cw2, lane < (int)take, queued - take + lane);
+                                queued -= take;
+                                __syncwarp();  // the queue is written again
+                            }
+                        }
                     }
                 }
                 cn.iteration(LAST);
@@ -1031,9 +1043,12 @@ __device__ void control_step(const EnumArgs& A, bool first) {
         if (first || A.sched->t_start == 0) A.sched->t_start = now;
         expired_s = now - A.sched->t_start > A.sched->run_limit_ns;
         if (expired_s) A.sched->err = DERR_TIMEOUT;
+        A.sched->spilled = 0;
     }
     // few slots left after the last step: each takes a large buffer
-    const bool few = A.big && !first && A.sched->active <= N_BIG;
+    const int32_t active = first ? 0 : A.sched->active;
+    const bool few = A.big && !first && active <= N_BIG;
+    const uint64_t share = FUSED_STEP_WORK / (uint64_t)max(active, 1);
     __syncthreads();
     for (int base = 0; base < A.n_slots; base += CT) {
         const int s = base + threadIdx.x;
@@ -1054,16 +1069,17 @@ __device__ void control_step(const EnumArgs& A, bool first) {
                     const uint64_t rows = c >> ROW_SHIFT;
                     if (l + 1 == k - 2 && S->ce > S->cb) {
                         // The next such step: as many items as would, like this step's,
-                        // fill four fifths of the rows and lead to FUSED_STEP_WORK
-                        // last-level items, and at most eight times as many. Items that
-                        // find no row are expanded in place by the warp that has them,
-                        // so that must stay the exception.
+                        // fill four fifths of the rows and lead to the slot's share of
+                        // FUSED_STEP_WORK last-level items, and at most eight times as
+                        // many. Items that find no row are expanded in place by the warp
+                        // that has them, so that must stay the exception (and short).
                         const uint64_t items = S->ce - S->cb, cap = S->cap[l + 1];
                         const uint64_t work = (c & WORK_MASK) + (__ldcg((const unsigned long long*)&S->st_work) - S->work0);
                         uint64_t fit = min((uint64_t)LAST_LEVEL_CHUNK, 8 * max(items, cap));
                         if (rows) fit = min(fit, cap * 4 / 5 * items / rows);
-                        if (work) fit = min(fit, FUSED_STEP_WORK / work * items + FUSED_STEP_WORK % work * items / work);
-                        S->wide = fit;
+                        if (work) fit = min(fit, share / work * items + share % work * items / work);
+                        const bool long_lists = D->lv[k - 1].par < 0 && S->ncand[k - 1] > SPILL_FANOUT;
+                        S->wide = A.narrow || long_lists ? 0 : fit;
                     }
                     if (rows > 0) {
                         S->nrows[l + 1] = rows;

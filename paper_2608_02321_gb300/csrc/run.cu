@@ -200,6 +200,7 @@ EnumArgs enum_args(const gfd_graph* g, const Tables& T, int kmax) {
     A.tile = T.tile;
     A.n_warps = 0;
     A.kmax = kmax;
+    A.narrow = 0;
     A.big = nullptr;
     A.big_bytes = 0;
     A.columns = 0;
@@ -846,7 +847,7 @@ gfd_result* make_result(const gfd_graph* g, const HostPlan& P, const SlotState& 
 }  // namespace
 
 // ------------------------------------------------------------------ batch runs
-int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opts* o, gfd_result** out) {
+int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opts* o, gfd_result** out, bool narrow) {
     if (!g || (!phis && n > 0) || !out || n < 0) {
         set_error(GFD_ERR_INVALID_ARG, "validate: NULL argument");
         return GFD_ERR_INVALID_ARG;
@@ -868,7 +869,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     Group G;
     const int64_t budget = (!o || o->frontier_budget_bytes <= 0) && g->tuned_budget > 0 ? g->tuned_budget
                                                                                         : default_budget(g, o);
-    if (int rc = group_plan(g, phis, n, o, budget / n, &G, o && o->frontier_budget_bytes > 0, true)) return rc;
+    if (int rc = group_plan(g, phis, n, o, budget / n, &G, o && o->frontier_budget_bytes > 0, !narrow)) return rc;
     int kmax = 1;
     for (auto& P : G.plans) kmax = std::max(kmax, P.k);
     std::shared_ptr<Pool> shared_pool;
@@ -879,10 +880,12 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     struct Free {
         std::vector<void*> p;
         cudaStream_t st;
-        ~Free() {
+        void now() {
             for (void* q : p)
                 if (q) cudaFreeAsync(q, st);
+            p.clear();
         }
+        ~Free() { now(); }
     } fr{{T.base}, st};
     void* wb = nullptr;
     if (int rc = pool_alloc(pool, G.bytes, st, &wb, "device workspace")) return rc;
@@ -899,6 +902,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     fr.p.push_back(G.cpi_base);
     if (lrc) return lrc;
     EnumArgs A = enum_args(g, T, kmax);
+    A.narrow = narrow;
     if (G.big_bytes) {
         A.big = G.base + G.o_big;
         A.big_bytes = G.big_bytes;
@@ -927,17 +931,33 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
         set_error(GFD_ERR_OVERFLOW, "index capacity exceeded");
         return GFD_ERR_OVERFLOW;
     }
-    for (int s = 0; s < n; s++)
-        if (states[s].err) {
+    bool again = false;
+    for (int s = 0; s < n; s++) {
+        if (states[s].err == DERR_WIDE) {
+            again = true;
+        } else if (states[s].err) {
             set_error(GFD_ERR_OVERFLOW, "GFD %d: partial-match counter overflow (lower chunk_rows)", s);
             return GFD_ERR_OVERFLOW;
         }
+    }
+    if (again) {
+        // a step's partial matches without a row were more, or longer, than may be
+        // expanded in place: once more with steps that always have their rows
+        fr.now();
+        GFD_CUDA(cudaStreamSynchronize(st));
+        gfd_opts o2 = o ? *o : gfd_opts{};
+        o2.cuda_stream = st;
+        const int rc = run_batch(g, phis, n, &o2, out, true);
+        if (rc == GFD_OK)
+            for (int s = 0; s < n; s++) out[s]->stat[6] += 1;
+        return rc;
+    }
     if (hs.varena_used > vcap) {
         // the violations did not fit: run again with room for exactly all of them
         gfd_opts o2 = o ? *o : gfd_opts{};
         o2.max_violations_hint = (int64_t)hs.varena_used;
         o2.cuda_stream = st;
-        const int rc = run_batch(g, phis, n, &o2, out);
+        const int rc = run_batch(g, phis, n, &o2, out, narrow);
         if (rc == GFD_OK)
             for (int s = 0; s < n; s++) out[s]->stat[6] += 1;
         return rc;
@@ -1355,19 +1375,20 @@ int session_step(gfd_session* S, int32_t* n_advanced, int32_t* n_running, int32_
             SlotHost& sl = S->slots[i];
             // slots started after the round's snapshot are not in it
             if (!in_round[i] || !sl.busy || states[i].cur >= 0) continue;
-            if (states[i].err) {
+            if (states[i].err && states[i].err != DERR_WIDE) {
                 set_error(GFD_ERR_OVERFLOW, "request %lld: partial-match counter overflow", (long long)sl.id);
                 return GFD_ERR_OVERFLOW;
             }
             gfd_result* r = nullptr;
-            if (states[i].n_viol > sl.viol_cap) {
-                // more violations than the request's buffer holds: validate it again alone
+            if (states[i].err == DERR_WIDE || states[i].n_viol > sl.viol_cap) {
+                // a wide step did not come out, or there are more violations than the
+                // request's buffer holds: validate it again alone
                 gfd_opts o2 = S->opts;
                 o2.cuda_stream = S->st;
                 o2.flags &= ~GFD_FLAG_HOST_LOOP;
-                o2.max_violations_hint = (int64_t)states[i].n_viol;
+                o2.max_violations_hint = (int64_t)std::max(states[i].n_viol, sl.viol_cap);
                 const gfd_gfd* one[1] = {&sl.req->phi};
-                if (int rc = run_batch(S->g, one, 1, &o2, &r)) return rc;
+                if (int rc = run_batch(S->g, one, 1, &o2, &r, states[i].err == DERR_WIDE)) return rc;
                 r->stat[6] += 1;
                 cudaFreeAsync(sl.viol, S->st);
             } else {
