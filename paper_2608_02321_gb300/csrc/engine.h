@@ -200,6 +200,7 @@ uint32_t cpi_chunks(uint64_t max_parent_candidates);
 void scan_units(uint64_t vertices, int most, int8_t* unit);
 
 // ---- enumeration (enumerate.cu)
+constexpr int MAX_TILE_ITERS = 64;  // gfd_opts::tile_iters at most: 32 times as many work items per tile
 struct EnumArgs {
     DevGraph g;
     const SlotDesc* slots;

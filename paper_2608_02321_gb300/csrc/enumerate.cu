@@ -48,6 +48,8 @@ constexpr uint64_t FUSED_STEP_WORK = 1ull << 33;
 // Longest candidate list expanded in place for want of a row: one warp's work, up to
 // a tile of them (2^27 items, about a second) before it looks for the next.
 constexpr uint32_t SPILL_FANOUT = 1u << 18;
+// A warp counts a tile's matches, at most SPILL_FANOUT of each item, in 32 bits.
+static_assert(32ull * MAX_TILE_ITERS * SPILL_FANOUT < 1ull << 32, "matches of a tile");
 // generator stored in a row for a next level that starts a pattern component:
 // its candidates are the level's candidate list (fan-out |C| for every row)
 constexpr int GEN_LIST = 4;
@@ -163,6 +165,7 @@ __device__ __forceinline__ bool lit_holds_at(const DevGraph& g, const DevLit& L,
 // candidates at the last level are expanded by the warp that makes them,
 // without being stored.
 constexpr uint32_t FUSE_FANOUT = 64;
+static_assert(FUSE_FANOUT <= SPILL_FANOUT);
 // Tiles of a step that fuses the last level are this many times smaller.
 constexpr uint64_t FUSED_TILE_DIV = 4;
 // Number the last level's tiles after the other intermediate levels' (else
@@ -487,7 +490,7 @@ __device__ void expand_warps(const EnumArgs& A) {
                 rhi1 = (uint32_t)nrows;
             }
         }
-        uint32_t tile_matches = 0;
+        uint32_t tile_matches = 0;  // (of the whole tile: below 2^32, see SPILL_FANOUT)
         // Complete matches (ok lanes: v at the last level L, the earlier levels in
         // column c): check the X literals of this level, count (with X pushed down
         // only if they hold), check Y, emit violations.

@@ -793,9 +793,9 @@ int pick_variant(const gfd_graph* g, const gfd_opts* o) {
     return g->tuned_variant >= 0 ? g->tuned_variant : 0;
 }
 
-// work items per block visit in units of the block size (1..64)
+// work items per block visit in units of the block size (1..MAX_TILE_ITERS)
 int pick_tile_iters(const gfd_graph* g, const gfd_opts* o) {
-    if (o && o->tile_iters >= 1) return std::min(o->tile_iters, 64);
+    if (o && o->tile_iters >= 1) return std::min(o->tile_iters, MAX_TILE_ITERS);
     return g->tuned_tile_iters > 0 ? g->tuned_tile_iters : 8;
 }
 
