@@ -435,7 +435,9 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
     // A quarter of a batch's frontier budget goes to the N_BIG large buffers when
     // the GFDs are many and their own shares stay large without it. Batch of 256
     // GFDs on 4M vertices with 48 GiB: 443 steps -> 49, enumeration 172 -> 147 ms
-    // (its last slots, with 1/256 of the budget each, took 435 of the steps).
+    // (its last slots, with 1/256 of the budget each, took 435 of the steps). Below 13
+    // GFDs a large buffer, 1/16 of the budget, is no larger than their own shares of
+    // the other three quarters (and would have to exceed the budget to be).
     size_t big_need = 0;
     uint64_t widest = 0;
     for (auto& P : G->plans) {
@@ -443,7 +445,7 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
         for (int l = 1; l <= P.k - 2; l++) b += 4ull * row_width(l) + 8;
         widest = std::max(widest, b);
     }
-    const bool big = with_big && n > 2 * N_BIG && !(o && o->chunk_rows > 0) && widest &&
+    const bool big = with_big && n > 3 * N_BIG && !(o && o->chunk_rows > 0) && widest &&
                      (uint64_t)frontier_per_slot / 4 * 3 / widest >= BIG_MIN_CHUNK;
     if (big) {
         G->big_bytes = (uint64_t)frontier_per_slot * n / (4 * N_BIG) & ~(uint64_t)255;
