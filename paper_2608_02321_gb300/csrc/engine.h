@@ -23,14 +23,28 @@ struct Pool {
     }
 };
 
+// The end of a call's last kernel, which may still be running when the call returns.
+struct Done {
+    cudaEvent_t ev = nullptr;
+    ~Done() {
+        if (ev) cudaEventDestroy(ev);
+        cudaGetLastError();
+    }
+};
+
 // Device memory of the pool shared by results (the short lists of one call) or
-// owned by one. Freed without naming a stream: the call's may be gone by then.
+// owned by one. Freed without naming a stream, since the call's may be gone by then:
+// such a free waits for nothing, so the kernel that writes the memory is waited for
+// (else the pool could hand it to another stream, or unmap it, under that kernel).
 struct DevBlock {
     void* p = nullptr;
     std::shared_ptr<Pool> pool;
-    DevBlock(void* q, std::shared_ptr<Pool> from) : p(q), pool(std::move(from)) {}
+    std::shared_ptr<Done> written;  // null: written before the call returned
+    DevBlock(void* q, std::shared_ptr<Pool> from, std::shared_ptr<Done> by = nullptr)
+        : p(q), pool(std::move(from)), written(std::move(by)) {}
     DevBlock(const DevBlock&) = delete;
     ~DevBlock() {
+        if (written && written->ev) cudaEventSynchronize(written->ev);
         if (p) cudaFree(p);
         cudaGetLastError();  // a failure here must not surface in a later, unrelated call
     }

@@ -968,6 +968,8 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     // arbitrary; gfd_result_tuples sorts)
     std::vector<int32_t*> vbuf(n, nullptr);
     std::vector<std::shared_ptr<DevBlock>> vmem(n);
+    auto split = std::make_shared<Done>();
+    if (hs.varena_used) GFD_CUDA(cudaEventCreateWithFlags(&split->ev, cudaEventDisableTiming));
     size_t small = 0;
     auto list_bytes = [&](int s) { return 4ull * states[s].n_viol * G.plans[s].k; };
     for (int s = 0; s < n; s++)
@@ -975,7 +977,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     if (small) {
         void* p = nullptr;
         if (int rc = pool_alloc(pool, small, st, &p, "violation lists")) return rc;
-        auto block = std::make_shared<DevBlock>(p, shared_pool);
+        auto block = std::make_shared<DevBlock>(p, shared_pool, split);
         int32_t* at = (int32_t*)p;
         for (int s = 0; s < n; s++)
             if (states[s].n_viol && list_bytes(s) <= SHARED_LIST) {
@@ -989,12 +991,13 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
         void* p = nullptr;
         if (int rc = pool_alloc(pool, list_bytes(s), st, &p, "violation list")) return rc;
         vbuf[s] = (int32_t*)p;
-        vmem[s] = std::make_shared<DevBlock>(p, shared_pool);
+        vmem[s] = std::make_shared<DevBlock>(p, shared_pool, split);
     }
     if (hs.varena_used) {
         GFD_CUDA(cudaMemcpyAsync(T.vptr, vbuf.data(), sizeof(int32_t*) * n, cudaMemcpyHostToDevice, st));
         GFD_CUDA(cudaMemsetAsync(T.vcur, 0, 8ull * n, st));
         if (int rc = launch_split(T.desc, T.varena, hs.varena_used, T.vstride, T.vptr, T.vcur, st)) return rc;
+        GFD_CUDA(cudaEventRecord(split->ev, st));
         launches[PROF_ENUM] += 1;  // the split belongs to the enumeration's output
     }
     // the refined candidate lists, kept for inspection when asked for
