@@ -1636,20 +1636,38 @@ __global__ void k_unpack_multi(const PackSrc* src, const int32_t* M, int W, cons
     }
 }
 
-// Scratch of a sort: one allocation of the result's pool.
+// Scratch of a sort: one allocation of the result's pool, which takes it from what it
+// holds unused. If the pool had to grow by more than SORT_KEEP for it, it shrinks again
+// afterwards (by itself it gives nothing back before the graph is freed).
+constexpr size_t SORT_KEEP = (size_t)64 << 20;
 struct SortScratch {
     Layout L;
     uint8_t* base = nullptr;
     cudaStream_t st;
+    std::shared_ptr<Pool> pool;
+    uint64_t reserved = 0;  // what the pool held before
     explicit SortScratch(cudaStream_t s) : st(s) { L.size = 0; }
+    static uint64_t held(cudaMemPool_t p) {
+        uint64_t x = 0;
+        if (cudaMemPoolGetAttribute(p, cudaMemPoolAttrReservedMemCurrent, &x) != cudaSuccess) cudaGetLastError();
+        return x;
+    }
     int alloc(const gfd_result* r) {
         void* p = nullptr;
-        if (int rc = pool_alloc(r->mem->pool->p, L.size, st, &p, "violation sort")) return rc;
+        pool = r->mem->pool;
+        if (L.size > SORT_KEEP) reserved = held(pool->p);
+        if (int rc = pool_alloc(pool->p, L.size, st, &p, "violation sort")) return rc;
         base = (uint8_t*)p;
         return GFD_OK;
     }
     ~SortScratch() {
-        if (base) cudaFreeAsync(base, st);
+        if (!base) return;
+        cudaFreeAsync(base, st);
+        if (L.size > SORT_KEEP && held(pool->p) > reserved + SORT_KEEP) {
+            cudaStreamSynchronize(st);
+            cudaMemPoolTrimTo(pool->p, reserved);
+        }
+        cudaGetLastError();
     }
 };
 
