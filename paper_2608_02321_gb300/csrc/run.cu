@@ -297,6 +297,10 @@ namespace {
 // the workspace: no read-back of the counts, no second allocation. Beyond, the
 // counts are read back (one synchronisation) and exactly as much is allocated.
 constexpr size_t IDX_INSIDE = (size_t)1 << 30;
+// A session's requests hold their memory while they run and share a budget, so there
+// the bound may be a sixteenth of the rest of the workspace at most: with more, fewer
+// requests ran at once (their index edges are often a small part of the bound).
+constexpr size_t SESSION_IDX_SHARE = 16;
 
 // Largest units (log2 of vertices) of the adjacency scans, see scan_units.
 constexpr int REFINE_UNIT = 8;
@@ -327,7 +331,7 @@ constexpr uint64_t MIN_CHUNK = 1024;
 // most 32 each)
 constexpr uint64_t MAX_CHUNK = (1ull << 24) - (1ull << 20);
 int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* o, int64_t frontier_per_slot,
-               Group* G, bool strict_budget = false, bool with_big = false) {
+               Group* G, bool strict_budget = false, bool with_big = false, bool session = false) {
     const uint32_t nwords = g->dg.nwords;
     G->n = n;
     G->plans.resize(n);
@@ -526,7 +530,7 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
     G->o_cmp_sums = L.take(4ull * G->cmp_chunks * G->finals.size());
     G->o_cpi_sums = L.take(8ull * std::max<uint32_t>(1, G->cpi_nch));
     G->o_cpi_tot = L.take(4ull * std::max<size_t>(1, G->index.size()));
-    G->idx_inside = G->cpi_bound <= IDX_INSIDE;
+    G->idx_inside = G->cpi_bound <= (session ? std::min(IDX_INSIDE, L.size / SESSION_IDX_SHARE) : IDX_INSIDE);
     if (G->idx_inside)
         for (const IndexSpec& X : G->index) G->o_idx.push_back(L.take(X.entry() * std::max<uint64_t>(1, X.bound)));
     // the region uploaded from the host: keys and job tables
@@ -1221,7 +1225,7 @@ int session_admit(gfd_session* S) {
         Request* R = S->queue.front().get();
         Group trial;
         const gfd_gfd* one[1] = {&R->phi};
-        if (int rc = group_plan(S->g, one, 1, &S->opts, per_slot, &trial)) return rc;
+        if (int rc = group_plan(S->g, one, 1, &S->opts, per_slot, &trial, false, false, true)) return rc;
         const int64_t req_bytes =
             (int64_t)(trial.bytes + (trial.idx_inside ? 0 : trial.cpi_bound)) + (int64_t)(4ull * trial.plans[0].k * S->viol_cap);
         const bool idle = S->used == 0 && take.empty();  // always admit into an idle device
@@ -1239,7 +1243,7 @@ int session_admit(gfd_session* S) {
     // caller may have launched on the session stream
     cudaStream_t sa = S->st_admit;
     auto G = std::make_shared<Group>();
-    if (int rc = group_plan(S->g, phis.data(), n, &S->opts, per_slot, G.get())) return rc;
+    if (int rc = group_plan(S->g, phis.data(), n, &S->opts, per_slot, G.get(), false, false, true)) return rc;
     void* wb = nullptr;
     if (int rc = pool_alloc(S->pool, G->bytes, sa, &wb, "request workspace")) return rc;
     G->base = (uint8_t*)wb;
