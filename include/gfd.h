@@ -267,18 +267,21 @@ int gfd_results_copy_tuples(gfd_result *const *rs, int32_t n, int32_t *out, uint
  * number of launches, when GFD_FLAG_PROFILE was set; else 0. */
 double gfd_result_profile(const gfd_result *r, int32_t which, int64_t *launches);
 /* Statistics of the run: 0 supersteps, 1 work items expanded, 2 partial
- * matches written, 3 edge-lookup probes (whole run), 4 candidate-list entries
+ * matches written, 3 pattern pairs tested (whole run), 4 candidate-list entries
  * (sum over pattern nodes), 5 index entries, 6 number of extra runs made
  * because the violations of the call outgrew max_violations_hint, or because the
- * size of a step was misjudged. With GFD_FLAG_COUNT, 7..29 are the whole call's counters of what its kernels read:
+ * size of a step was misjudged. With GFD_FLAG_COUNT, 7..29 are the whole call's
+ * counters of what its kernels read:
  * 7 work items (entries of the index lists N_u, Section III.B, or of another
  * candidate list), 8 of them at the last level, 9 partial matches expanded,
  * 10 sum over expanded partial matches of the adjacency lengths of their
- * backward non-tree neighbours' images, 11 pair checks, 12 of them settled by
- * a neighbourhood signature or row filter, 13 adjacency binary searches, 14 adjacency
- * entries those searches read, 15 absent-edge checks, 16 sum over absent-edge
- * checks of ceil(log2(d + 1)) (d the shorter adjacency list), 17 signature
- * and row filter loads, 18 attribute loads of literal checks, 19 partial matches written,
+ * backward non-tree neighbours' images, 11 pair checks made (the pairs that a
+ * signature settles, all at once, and those looked up until one fails), 12 of
+ * them settled by a neighbourhood signature or row filter, 13 adjacency binary
+ * searches, 14 adjacency entries those searches read, 15 absent-edge checks (in
+ * order, up to the first edge found), 16 sum over absent-edge checks of
+ * ceil(log2(d + 1)) (d the shorter adjacency list), 17 signature and row filter
+ * loads, 18 attribute loads of literal checks, 19 partial matches written,
  * 20 candidates whose adjacency the refinement and index build scanned, 21
  * adjacency entries they read, 22 warp iterations of the expansion, 23 sum over
  * them of the largest number of search loads one lane made, 24..26 SM cycles

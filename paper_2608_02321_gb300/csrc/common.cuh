@@ -211,13 +211,14 @@ enum : int {
     CNT_PARTIALS,      // partial matches expanded (stored rows, and roots, with fan-out)
     CNT_BACK_DEG,      // sum over expanded partial matches of the degrees (in the edge's
                        // direction) of the images of their backward non-tree neighbours
-    CNT_CHECKS,        // pair checks made (required and absent edges)
-    CNT_SIG_SETTLED,   // of them settled by the neighbourhood signature
+    CNT_CHECKS,        // pair checks made (required and absent edges): the pairs that a signature
+                       // settles, and those looked up until one fails
+    CNT_SIG_SETTLED,   // of them settled by a neighbourhood signature or a row filter
     CNT_SEARCHES,      // binary searches of an adjacency list made
     CNT_SEARCH_LOADS,  // adjacency entries those searches loaded
-    CNT_NEG_CHECKS,    // absent-edge checks made
+    CNT_NEG_CHECKS,    // absent edges checked, up to the first that is there
     CNT_NEG_LOGD,      // sum over absent-edge checks of ceil(log2(d + 1)), d the shorter list
-    CNT_SIG_LOADS,     // neighbourhood-signature loads
+    CNT_SIG_LOADS,     // neighbourhood-signature and row-filter loads
     CNT_ATTR_READS,    // attribute loads of the literal checks
     CNT_ROWS,          // partial matches written
     CNT_SCAN_CANDS,    // refinement and index build: candidates whose adjacency was scanned

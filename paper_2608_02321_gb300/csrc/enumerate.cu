@@ -312,13 +312,15 @@ __device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m
         const uint32_t x = m[(wd & 15u) << 5];
         const uint64_t half = (wd >> 4) & 1u ? sv.x : sv.y;  // edge v -> x, else x -> v
         open |= (uint32_t)((half >> sig_bit(x)) & 1ull) << c;
-        if (COUNT && c != skip) cn.add(CNT_CHECKS, 1);
     }
-    // counting pass: the absent edges, of candidates whose required edges agree
-    bool counted = !COUNT;
-    auto count_absent = [&] {
-        counted = true;
-        for (int c = nreq; c < n; c++) {
+    // All pairs are tested here. Of those the signature leaves open, the counting pass
+    // takes back the ones not looked up any more (doing so in every run, for the
+    // statistic, cost 2 % of the large batch's enumeration).
+    probes += n - (skip >= 0);
+    cn.add(CNT_CHECKS, n - (skip >= 0));
+    // counting pass: absent edges, in order up to the first that is there (check c; n: none)
+    auto count_absent = [&](int c1) {
+        for (int c = nreq; COUNT && c < min(c1 + 1, n); c++) {
             const uint32_t x = m[(cw[c] & 15u) << 5];
             const bool out = (cw[c] >> 4) & 1u;
             const uint32_t dv = out ? g.out_off[v + 1] - g.out_off[v] : g.in_off[v + 1] - g.in_off[v];
@@ -332,13 +334,14 @@ __device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m
         open &= ~(1u << skip);
         required &= ~(1u << skip);
     }
-    probes += n - (skip >= 0);
     if (COUNT) cn.add(CNT_SIG_SETTLED, n - (skip >= 0) - __popc(open));
-    if ((open & required) != required) return false;
+    if ((open & required) != required) {
+        cn.add(CNT_CHECKS, -(uint64_t)__popc(open));
+        return false;
+    }
     #pragma unroll 1
     for (; open; open &= open - 1) {
         const int c = __ffs(open) - 1;
-        if (COUNT && c >= nreq && !counted) count_absent();
         const uint32_t wd = cw[c];
         const uint32_t x = m[(wd & 15u) << 5];
         const bool out = (wd >> 4) & 1u;
@@ -354,9 +357,13 @@ __device__ __forceinline__ bool pairs_agree(const DevGraph& g, const uint32_t* m
         } else {
             cn.add(CNT_SIG_SETTLED, 1);
         }
-        if (!exp_ok(ex, gl)) return false;
+        if (!exp_ok(ex, gl)) {
+            cn.add(CNT_CHECKS, 1 - (uint64_t)__popc(open));
+            count_absent(c);
+            return false;
+        }
     }
-    if (COUNT && !counted) count_absent();
+    count_absent(n);
     return true;
 }
 
@@ -438,7 +445,7 @@ __device__ void expand_warps(const EnumArgs& A) {
     const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const DevGraph& g = A.g;
     const uint32_t total_tiles = *(volatile uint32_t*)&A.sched->total_tiles;
-    uint32_t probes = 0;  // a statistic (saturates per warp)
+    uint32_t probes = 0;  // a statistic
     #pragma unroll 1
     for (uint64_t t = gwarp; t < total_tiles;) {
         cn.mark();
@@ -556,7 +563,13 @@ __device__ void expand_warps(const EnumArgs& A) {
                 const int gen = who >> 5;
                 const bool adjacent = gen != 0 && !(GEN && gen == GEN_LIST);
                 if (adjacent) v = raw >> g.lbits;
-                if (f.bits) ok = f.may_hold(v);
+                if (f.bits) {
+                    ok = f.may_hold(v);
+                    probes += !ok;
+                    cn.add(CNT_SIG_LOADS, 1);
+                    cn.add(CNT_CHECKS, !ok);
+                    cn.add(CNT_SIG_SETTLED, !ok);
+                }
                 if (adjacent && ok)  // from the adjacency of the other end of a required back edge
                     ok = exp_ok(P.chk_exp[P.gen[gen - 1]], (int32_t)(raw & g.lmask)) &&
                          ((__ldg(D->bm[L] + (v >> 5)) >> (v & 31)) & 1u);
