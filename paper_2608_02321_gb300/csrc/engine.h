@@ -201,6 +201,8 @@ int launch_scatter(const DevGraph& g, const ScatterJob* d_jobs, int njobs, const
                    cudaStream_t st);
 int launch_refine(const DevGraph& g, const RefineJob* d_jobs, int njobs, const ScanLaunch& l, ScanCount scan,
                   cudaStream_t st);
+// Zeros in the results of the jobs.
+int launch_clear(const DevGraph& g, const RefineJob* d_jobs, int njobs, cudaStream_t st);
 int launch_compact(const DevGraph& g, const CompactJob* d_jobs, int njobs, cudaStream_t st);
 // Index edges in two steps: counts, offsets and per-job totals first, then the
 // fill (between the two the caller may read the totals back and allocate exactly).

@@ -522,6 +522,12 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, REFINE_BLOCKS) k_refine(D
     scan_flush<COUNT>(scan, sc, se);
 }
 
+__global__ void __launch_bounds__(FILTER_THREADS) k_clear(DevGraph g, const RefineJob* __restrict__ jobs, int njobs) {
+    for (int j = blockIdx.y; j < njobs; j += gridDim.y)
+        for (uint32_t w = blockIdx.x * FILTER_THREADS + threadIdx.x; w < g.nwords; w += gridDim.x * FILTER_THREADS)
+            jobs[j].out[w] = 0;
+}
+
 // Position in the parent's candidate list of the first candidate at or after
 // vertex a.
 __device__ __forceinline__ uint32_t parent_rank(const CpiJob& J, uint32_t a) {
@@ -841,6 +847,13 @@ int launch_filter(const DevGraph& g, const FilterKey* d_keys, int nkeys, uint32_
         if (int rc = check_launch("k_filter")) return rc;
     }
     return GFD_OK;
+}
+
+int launch_clear(const DevGraph& g, const RefineJob* d_jobs, int njobs, cudaStream_t st) {
+    if (njobs <= 0 || g.nwords == 0) return GFD_OK;
+    const uint32_t wide = std::min<uint32_t>((g.nwords + FILTER_THREADS - 1) / FILTER_THREADS, 64);
+    k_clear<<<dim3(wide, (unsigned)std::min(njobs, 1024)), FILTER_THREADS, 0, st>>>(g, d_jobs, njobs);
+    return check_launch("k_clear");
 }
 
 uint32_t compact_chunks(const DevGraph& g) {
