@@ -178,6 +178,9 @@ def make_opts(frontier_budget_bytes=0, chunk_rows=0, kernel_variant=0, max_viola
     return o
 
 
+_PLAIN = (list, tuple, np.ndarray)
+
+
 class _GfdBuf:
     """ctypes image of one GFD (keeps its arrays alive)."""
 
@@ -191,17 +194,23 @@ class _GfdBuf:
         """Plain sequences of whole numbers, as nearly all GFDs hold them: packed
         without numpy or a ctypes object per literal (5 us a GFD against 14, which
         a batch of 64 on a small graph took a quarter of its time for). Anything
-        else raises and is left to _convert."""
-        nl = array("i", gfd.node_label)
+        else raises and is left to _convert: what looks like numbers to array but
+        not to numpy too (bytes, sets, dicts, one-shot iterators)."""
+        def plain(seq):
+            if not isinstance(seq, _PLAIN):
+                raise TypeError
+            return seq
+        nl = array("i", plain(gfd.node_label))
         es, ed, el = array("i"), array("i"), array("i")
-        for a, b, c in gfd.edges:
+        for e in plain(gfd.edges):
+            a, b, c = plain(e)
             es.append(a)
             ed.append(b)
             el.append(c)
 
         def lits(ls):
             flat = array("i")
-            for q in ls:
+            for q in plain(ls):
                 flat.extend((q.kind, q.x, q.a, q.y, q.b, q.c))
             return flat
         X, Y = lits(gfd.X), lits(gfd.Y)
