@@ -292,6 +292,10 @@ struct TmpFree {
     }
 };
 
+// Attribute columns are reordered through scratch of up to this many bytes (one column
+// at least): a second copy of them all would keep graphs with many attributes out.
+constexpr size_t ATTR_SCRATCH = (size_t)256 << 20;
+
 int grid_for(int64_t n, int threads = 256) {
     int64_t b = (n + threads - 1) / threads;
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)device_sms() * 16));
@@ -387,9 +391,10 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
     }
     const size_t cub_bytes = std::max(sort_v, std::max(sort_e, scan_b));
     constexpr size_t LABELS = 65536;
+    const int32_t cols = std::min<int32_t>(d->n_attrs, (int32_t)std::max<size_t>(1, ATTR_SCRATCH / (4 * N + 1)));
     Block S;
     const size_t s_off = S.take(8 * (N + 1)), s_nbr = S.take(4 * M), s_lab = S.take(4 * M), s_vl = S.take(4 * N),
-                 s_at = S.take(4 * NA), s_k0 = S.take(8 * std::max(M, N)), s_k1 = S.take(8 * std::max(M, N)),
+                 s_at = S.take(4 * N * cols), s_k0 = S.take(8 * std::max(M, N)), s_k1 = S.take(8 * std::max(M, N)),
                  s_l0 = S.take(std::max(M, 4 * N)), s_l1 = S.take(std::max(M, 4 * N)), s_rank = S.take(4 * N),
                  s_dout = S.take(4 * (N + 1)), s_din = S.take(4 * (N + 1)), s_zero = S.size,
                  s_odin = S.take(4 * (N + 1)), s_self = S.take(4 * N), s_hist = S.take(8 * 256), s_flag = S.take(sizeof(Flags)),
@@ -448,8 +453,11 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
     if (flag.bad) return bad_rows(" forward CSR:");
     if (m) CK(cudaMemcpyAsync(d_nbr, d->out_dst, sizeof(int32_t) * M, cudaMemcpyHostToDevice, st));
     if (n) CK(cudaMemcpyAsync(d_vl, d->vlabel, sizeof(int32_t) * N, cudaMemcpyHostToDevice, st));
-    if (n && d->n_attrs)
-        CK(cudaMemcpyAsync(S.at<void>(s_at), d->attrs, sizeof(int32_t) * N * d->n_attrs, cudaMemcpyHostToDevice, st));
+    auto copy_attrs = [&](int32_t a) {  // columns [a, a + cols) of those there are
+        return cudaMemcpyAsync(S.at<void>(s_at), d->attrs + (size_t)a * N, sizeof(int32_t) * N * std::min(cols, d->n_attrs - a),
+                               cudaMemcpyHostToDevice, st);
+    };
+    if (n && d->n_attrs) CK(copy_attrs(0));
     cub::DoubleBuffer<uint64_t> kb(S.at<uint64_t>(s_k0), S.at<uint64_t>(s_k1));
     cub::DoubleBuffer<uint32_t> vb(S.at<uint32_t>(s_l0), S.at<uint32_t>(s_l1));
     k_check_rows<<<grid_for((int64_t)n * 32), 256, 0, st>>>(d_off, d_nbr, d_lab, n, lbits, odin, self, d_bad);
@@ -472,7 +480,11 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
     CK(cudaMemsetAsync(din_new + N, 0, 4, st));
     k_renumber<<<grid_for(n), 256, 0, st>>>(orig, kb.Current(), o_vinfo, d_off, odin, n, rank, vinfo, dout_new, din_new,
                                             S.at<Segment>(s_seg), &d_flag->nsegs, d_flag->class_end);
-    if (d->n_attrs) k_gather_attrs<<<grid_for(n), 256, 0, st>>>(S.at<int32_t>(s_at), orig, n, d->n_attrs, attrs);
+    for (int32_t a = 0; n && a < d->n_attrs; a += cols) {
+        if (a) CK(copy_attrs(a));
+        k_gather_attrs<<<grid_for(n), 256, 0, st>>>(S.at<int32_t>(s_at), orig, n, std::min(cols, d->n_attrs - a),
+                                                    attrs + (size_t)a * N);
+    }
     tb = cub_bytes;
     CK(cub::DeviceScan::ExclusiveSum(tstore, tb, dout_new, out_off, n + 1, st));
     tb = cub_bytes;
