@@ -302,8 +302,10 @@ namespace {
 constexpr size_t IDX_INSIDE = (size_t)1 << 30;
 // A session's requests hold their memory while they run and share a budget, so there
 // the bound may be a sixteenth of the rest of the workspace at most: with more, fewer
-// requests ran at once (their index edges are often a small part of the bound).
+// requests ran at once (their index edges are often a small part of the bound). A call
+// whose workspace cannot be had is planned again without such room.
 constexpr size_t SESSION_IDX_SHARE = 16;
+enum class Room { AMPLE, SESSION, LEAN };
 
 // Refinement results and marks up to this many bytes lie apart and are cleared by one
 // call. Beyond, a phase's results take the places of bitmaps that no later phase reads,
@@ -342,7 +344,7 @@ constexpr uint64_t MIN_CHUNK = 1024;
 // most 32 each)
 constexpr uint64_t MAX_CHUNK = (1ull << 24) - (1ull << 20);
 int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* o, int64_t frontier_per_slot,
-               Group* G, bool strict_budget = false, bool with_big = false, bool session = false) {
+               Group* G, bool strict_budget = false, bool with_big = false, Room room = Room::AMPLE) {
     const uint32_t nwords = g->dg.nwords;
     G->n = n;
     G->plans.resize(n);
@@ -446,7 +448,7 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
     }
     // where the refinements' results and marks lie
     const size_t bm_bytes = 4ull * nwords, n_results = G->refines.size();
-    G->reuse = bm_bytes * (n_results + G->n_marks) > BITMAPS_APART;
+    G->reuse = bm_bytes * (n_results + G->n_marks) > (room == Room::LEAN ? 0 : BITMAPS_APART);
     G->place.resize(n_results);
     if (!G->reuse) {
         for (size_t i = 0; i < n_results; i++) G->place[i] = (int)i;
@@ -578,7 +580,8 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
     G->o_cmp_sums = L.take(4ull * G->cmp_chunks * G->finals.size());
     G->o_cpi_sums = L.take(8ull * std::max<uint32_t>(1, G->cpi_nch));
     G->o_cpi_tot = L.take(4ull * std::max<size_t>(1, G->index.size()));
-    G->idx_inside = G->cpi_bound <= (session ? std::min(IDX_INSIDE, L.size / SESSION_IDX_SHARE) : IDX_INSIDE);
+    G->idx_inside = room != Room::LEAN &&
+                    G->cpi_bound <= (room == Room::SESSION ? std::min(IDX_INSIDE, L.size / SESSION_IDX_SHARE) : IDX_INSIDE);
     if (G->idx_inside)
         for (const IndexSpec& X : G->index) G->o_idx.push_back(L.take(X.entry() * std::max<uint64_t>(1, X.bound)));
     // the region uploaded from the host: keys and job tables
@@ -952,7 +955,11 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
         ~Free() { now(); }
     } fr{{T.base}, st};
     void* wb = nullptr;
-    if (int rc = pool_alloc(pool, G.bytes, st, &wb, "device workspace")) return rc;
+    if (pool_alloc(pool, G.bytes, st, &wb, "device workspace")) {
+        G = Group{};
+        if (int rc = group_plan(g, phis, n, o, budget / n, &G, o && o->frontier_budget_bytes > 0, !narrow, Room::LEAN)) return rc;
+        if (int rc = pool_alloc(pool, G.bytes, st, &wb, "device workspace")) return rc;
+    }
     fr.p.push_back(wb);
     G.base = (uint8_t*)wb;
     G.slot.resize(n);
@@ -1283,7 +1290,7 @@ int session_admit(gfd_session* S) {
         Request* R = S->queue.front().get();
         Group trial;
         const gfd_gfd* one[1] = {&R->phi};
-        if (int rc = group_plan(S->g, one, 1, &S->opts, per_slot, &trial, false, false, true)) return rc;
+        if (int rc = group_plan(S->g, one, 1, &S->opts, per_slot, &trial, false, false, Room::SESSION)) return rc;
         const int64_t req_bytes =
             (int64_t)(trial.bytes + (trial.idx_inside ? 0 : trial.cpi_bound)) + (int64_t)(4ull * trial.plans[0].k * S->viol_cap);
         const bool idle = S->used == 0 && take.empty();  // always admit into an idle device
@@ -1301,7 +1308,7 @@ int session_admit(gfd_session* S) {
     // caller may have launched on the session stream
     cudaStream_t sa = S->st_admit;
     auto G = std::make_shared<Group>();
-    if (int rc = group_plan(S->g, phis.data(), n, &S->opts, per_slot, G.get(), false, false, true)) return rc;
+    if (int rc = group_plan(S->g, phis.data(), n, &S->opts, per_slot, G.get(), false, false, Room::SESSION)) return rc;
     void* wb = nullptr;
     if (int rc = pool_alloc(S->pool, G->bytes, sa, &wb, "request workspace")) return rc;
     G->base = (uint8_t*)wb;
