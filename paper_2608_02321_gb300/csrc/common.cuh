@@ -160,11 +160,9 @@ struct SlotDesc {
     uint32_t* rank[MAXK];
     int32_t* cand[MAXK];
     const uint32_t* cand_n[MAXK];  // number of candidates
-    uint32_t cand_cap[MAXK];
     uint32_t* cpi_off[MAXK];  // level i >= 1
     int2* cpi_idx[MAXK];      // (position in C(i), vertex id) per index edge; at the last level,
                               // where no position is needed, the vertex ids alone (u32)
-    uint64_t cpi_cap[MAXK];
     // frontier
     int32_t* rows[MAXK];      // level l >= 1
     uint64_t* wpre[MAXK];     // level l >= 1

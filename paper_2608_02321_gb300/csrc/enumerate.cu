@@ -10,8 +10,8 @@
 // the rows' fan-outs, so hub vertices are split evenly over threads. Each work
 // item yields at most one partial match of level l+1, so a level-l chunk of
 // `cap` items always fits the next buffer (steps that make the second-to-last
-// level take more, since they store few of theirs); when a level is exhausted the
-// slot pops back to the previous level (depth-first), bounding memory.
+// level take more, since they store few of theirs; see control_step); when a level is
+// exhausted the slot pops back to the previous level (depth-first), bounding memory.
 //
 // A candidate v for pattern node u = order[i] extending partial match m passes
 // when: v != m[q] for earlier label-compatible levels q (injectivity), and for
@@ -265,8 +265,8 @@ struct FilterRow {
 };
 
 // Fused expansion: the last-level candidates of one partial match in the warp's
-// sequence. src: where they start in their generator's source - where they start
-// in the sequence; who: lane | generator << 5.
+// sequence, and the row filter they are looked up in. src: where they start in their
+// generator's source - where they start in the sequence.
 struct LastList {
     const uint8_t* base;
     uint32_t bits;
@@ -284,7 +284,6 @@ struct WarpShared {
     int32_t* rows;            // where the tile's new partial matches go
     uint64_t* wpre;
     uint64_t cap;
-    uint64_t unused;
     uint32_t qv[32 + 32 * LAST_WINDOWS];  // last-level candidates waiting for their other checks,
     uint8_t qo[32 + 32 * LAST_WINDOWS];   // and whose they are: lane | generator << 5
     __device__ uint32_t* m(int col) { return reinterpret_cast<uint32_t*>(this + 1) + col; }  // [32 q + col]: the columns

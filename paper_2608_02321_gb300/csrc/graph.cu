@@ -4,11 +4,11 @@
 // The caller's int64/int32 CSR is checked on the device (rows strictly
 // increasing, ids in range, labels in range, reverse CSR equal to the transpose
 // of the forward one) and packed into the layout of common.cuh. Vertices are
-// renumbered inside: by degree class (hubs first), then by label, then by falling degree, then by id. So the scans of a
-// candidate list know where its hubs end without looking at degrees (and give
-// each class its own share of work), candidates of one label have adjacency
-// lists next to each other, and the vertices that edges lead to most often
-// share a few cache lines. Ids leave the library through orig[].
+// renumbered inside: by degree class (hubs first), then by label, then by falling
+// degree, then by id. So the scans of a candidate list know where its hubs end without
+// looking at degrees (and give each class its own share of work), candidates of one
+// label have adjacency lists next to each other, and the vertices that edges lead to
+// most often share a few cache lines. Ids leave the library through orig[].
 #include <cub/cub.cuh>
 
 #include <algorithm>

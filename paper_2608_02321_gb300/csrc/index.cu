@@ -162,9 +162,10 @@ __global__ void __launch_bounds__(COMPACT_THREADS) k_compact_write(DevGraph g, c
 // bitmap word, from L2 or HBM) and by balance. A lane that scans its own list
 // leaves the warp waiting for its longest list with few loads in flight; a warp
 // that happens to get 32 long lists keeps the launch waiting. End to end every
-// lane has FLAT loads in flight whatever the degrees, and by degree classes no
-// warp gets more than 2048 entries at a time (one vertex of up to 2048, 8 of up
-// to 256, 32 of up to 32).
+// lane has FLAT loads in flight whatever the degrees, and by degree classes a warp
+// of a small launch gets no more than 2048 entries at a time (one vertex of up to
+// 2048, 8 of up to 256, 32 of up to 32), one of a large launch no more than 8192 (4,
+// 32 and 32 vertices; see scan_units).
 constexpr int FLAT = 4;
 constexpr int MAX_WORDS = 32;  // most bitmap words per warp item of the last class
 // Resident blocks per SM the scanning kernels are compiled for; at 6 the
@@ -874,7 +875,7 @@ uint32_t cpi_chunks(uint64_t max_parent_candidates) { return (uint32_t)(max_pare
 // A large launch takes larger units, so that its warps' lanes fill up although the
 // bitmaps are sparse and an item's fixed cost (finding its job, its words) is
 // spread; a small one smaller units, so that its few candidates reach all SMs and
-// no warp gets more than 2048 entries. In between, the last class's unit leaves
+// no warp gets more than 2048 entries at a time. In between, the last class's unit leaves
 // every resident warp about four items, up to 2^most vertices: 8 for refinement,
 // whose bitmaps are dense at first (batch of 256 GFDs on 4M vertices: 55 / 48 / 44 /
 // 38 / 38.5 ms at 5 .. 9, with units of 4 to 8 vertices in class 1 and 32 to 64 in

@@ -543,10 +543,6 @@ int group_plan(gfd_graph* g, const gfd_gfd* const* phis, int n, const gfd_opts* 
             }
             big_need = std::max(big_need, B.size);
         }
-        for (int i = 0; i < P.k; i++) {
-            D.cand_cap[i] = (uint32_t)lab_count(P.key[i].label);
-            if (i > 0 && P.lv[i].par >= 0) D.cpi_cap[i] = G->index[G->level_index[s][i]].bound;
-        }
         for (int l = 1; l <= P.k - 2; l++) {
             F.rows[l] = L.take(4ull * row_width(l) * chunk);
             F.wpre[l] = L.take(8ull * chunk);
