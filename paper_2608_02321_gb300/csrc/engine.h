@@ -17,8 +17,6 @@ struct Engine;
 // result that refers to it (a freed graph gives back what is unused).
 struct Pool {
     cudaMemPool_t p = nullptr;
-    std::mutex mu;
-    cudaStream_t own = nullptr;  // the graph's stream, null once that is gone
     ~Pool() {
         if (p) cudaMemPoolDestroy(p);
         cudaGetLastError();
@@ -35,29 +33,19 @@ struct Done {
 };
 
 // Device memory of the pool shared by results (the short lists of one call) or
-// owned by one. The pool must not hand it to another stream, or unmap it, under the
-// kernel that writes it: the free is ordered after that kernel on the graph's stream
-// while there is one (graph_free waits for what is on it), and waits for the kernel
-// when the call was on another stream, which may be gone by then. (A wait for an event
-// in every case took 9 of the 245 us of a small call.)
+// owned by one. Freed without naming a stream, since the call's may be gone by then:
+// such a free waits for nothing, so the kernel that writes the memory is waited for
+// (else the pool could hand it to another stream, or unmap it, under that kernel).
 struct DevBlock {
     void* p = nullptr;
     std::shared_ptr<Pool> pool;
-    bool on_own = false;            // written by a kernel on the graph's stream
-    std::shared_ptr<Done> written;  // by one on another; neither: before the call returned
-    DevBlock(void* q, std::shared_ptr<Pool> from) : p(q), pool(std::move(from)) {}
-    DevBlock(void* q, std::shared_ptr<Pool> from, std::shared_ptr<Done> by)
-        : p(q), pool(std::move(from)), on_own(!by), written(std::move(by)) {}
+    std::shared_ptr<Done> written;  // null: written before the call returned
+    DevBlock(void* q, std::shared_ptr<Pool> from, std::shared_ptr<Done> by = nullptr)
+        : p(q), pool(std::move(from)), written(std::move(by)) {}
     DevBlock(const DevBlock&) = delete;
     ~DevBlock() {
-        std::unique_lock<std::mutex> lock(pool->mu);
-        if (on_own && pool->own) {
-            cudaFreeAsync(p, pool->own);
-        } else {
-            lock.unlock();
-            if (written && written->ev) cudaEventSynchronize(written->ev);
-            cudaFree(p);
-        }
+        if (written && written->ev) cudaEventSynchronize(written->ev);
+        if (p) cudaFree(p);
         cudaGetLastError();  // a failure here must not surface in a later, unrelated call
     }
 };

@@ -41,13 +41,7 @@ struct Engine {
 
 void engine_free(Engine* e) {
     if (!e) return;
-    if (e->pool) {
-        // results may keep the pool itself; what they free from now on is written
-        std::lock_guard<std::mutex> lock(e->pool->mu);
-        if (e->pool->own) cudaStreamSynchronize(e->pool->own);
-        e->pool->own = nullptr;
-        cudaMemPoolTrimTo(e->pool->p, 0);
-    }
+    if (e->pool) cudaMemPoolTrimTo(e->pool->p, 0);  // (results may keep the pool itself)
     cudaGetLastError();
     delete e;
 }
@@ -78,7 +72,6 @@ int get_pool(gfd_graph* g, std::shared_ptr<Pool>* out) {
         GFD_CUDA(cudaMemPoolCreate(&pool->p, &props));
         uint64_t thr = UINT64_MAX;
         GFD_CUDA(cudaMemPoolSetAttribute(pool->p, cudaMemPoolAttrReleaseThreshold, &thr));
-        pool->own = g->stream;
         g->eng->pool = std::move(pool);
     }
     *out = g->eng->pool;
@@ -1040,11 +1033,8 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     // arbitrary; gfd_result_tuples sorts)
     std::vector<int32_t*> vbuf(n, nullptr);
     std::vector<std::shared_ptr<DevBlock>> vmem(n);
-    std::shared_ptr<Done> split;  // on another stream than the graph's
-    if (hs.varena_used && st != g->stream) {
-        split = std::make_shared<Done>();
-        GFD_CUDA(cudaEventCreateWithFlags(&split->ev, cudaEventDisableTiming));
-    }
+    auto split = std::make_shared<Done>();
+    if (hs.varena_used) GFD_CUDA(cudaEventCreateWithFlags(&split->ev, cudaEventDisableTiming));
     size_t small = 0;
     auto list_bytes = [&](int s) { return 4ull * states[s].n_viol * G.plans[s].k; };
     for (int s = 0; s < n; s++)
@@ -1072,7 +1062,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
         GFD_CUDA(cudaMemcpyAsync(T.vptr, vbuf.data(), sizeof(int32_t*) * n, cudaMemcpyHostToDevice, st));
         GFD_CUDA(cudaMemsetAsync(T.vcur, 0, 8ull * n, st));
         if (int rc = launch_split(T.desc, T.varena, hs.varena_used, T.vstride, T.vptr, T.vcur, st)) return rc;
-        if (split) GFD_CUDA(cudaEventRecord(split->ev, st));
+        GFD_CUDA(cudaEventRecord(split->ev, st));
         launches[PROF_ENUM] += 1;  // the split belongs to the enumeration's output
     }
     // the refined candidate lists, kept for inspection when asked for
