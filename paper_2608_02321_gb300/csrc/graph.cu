@@ -618,7 +618,6 @@ int graph_load(const gfd_graph_desc* d, const gfd_opts* o, gfd_graph** out) {
 
 void graph_free(gfd_graph* g) {
     if (!g) return;
-    if (g->stream) cudaStreamSynchronize(g->stream);  // then the pool gives back all that is free
     if (g->eng) engine_free(g->eng);
     for (void* p : g->allocs) cudaFree(p);
     if (g->stream) cudaStreamDestroy(g->stream);

@@ -41,7 +41,15 @@ struct Engine {
 
 void engine_free(Engine* e) {
     if (!e) return;
-    if (e->pool) cudaMemPoolTrimTo(e->pool->p, 0);  // (results may keep the pool itself)
+    if (e->pool) {
+        // results may keep the pool itself; what they free from now on is written
+        std::lock_guard<std::mutex> lock(e->pool->mu);
+        if (e->pool->own) cudaStreamSynchronize(e->pool->own);
+        e->pool->own = nullptr;
+        for (void* q : e->pool->dropped) cudaFree(q);
+        e->pool->dropped.clear();
+        cudaMemPoolTrimTo(e->pool->p, 0);
+    }
     cudaGetLastError();
     delete e;
 }
@@ -72,6 +80,7 @@ int get_pool(gfd_graph* g, std::shared_ptr<Pool>* out) {
         GFD_CUDA(cudaMemPoolCreate(&pool->p, &props));
         uint64_t thr = UINT64_MAX;
         GFD_CUDA(cudaMemPoolSetAttribute(pool->p, cudaMemPoolAttrReleaseThreshold, &thr));
+        pool->own = g->stream;
         g->eng->pool = std::move(pool);
     }
     *out = g->eng->pool;
@@ -929,6 +938,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     cudaStream_t st = (o && o->cuda_stream) ? (cudaStream_t)o->cuda_stream : g->stream;
     const uint64_t vcap = o && o->max_violations_hint > 0 ? (uint64_t)o->max_violations_hint : (1ull << 22);
 
+    if (g->eng && g->eng->pool) g->eng->pool->drain();
     Group G;
     const int64_t budget = (!o || o->frontier_budget_bytes <= 0) && g->tuned_budget > 0 ? g->tuned_budget
                                                                                         : default_budget(g, o);
@@ -1033,8 +1043,11 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
     // arbitrary; gfd_result_tuples sorts)
     std::vector<int32_t*> vbuf(n, nullptr);
     std::vector<std::shared_ptr<DevBlock>> vmem(n);
-    auto split = std::make_shared<Done>();
-    if (hs.varena_used) GFD_CUDA(cudaEventCreateWithFlags(&split->ev, cudaEventDisableTiming));
+    std::shared_ptr<Done> split;  // on another stream than the graph's
+    if (hs.varena_used && st != g->stream) {
+        split = std::make_shared<Done>();
+        GFD_CUDA(cudaEventCreateWithFlags(&split->ev, cudaEventDisableTiming));
+    }
     size_t small = 0;
     auto list_bytes = [&](int s) { return 4ull * states[s].n_viol * G.plans[s].k; };
     for (int s = 0; s < n; s++)
@@ -1062,7 +1075,7 @@ int run_batch(gfd_graph* g, const gfd_gfd* const* phis, int32_t n, const gfd_opt
         GFD_CUDA(cudaMemcpyAsync(T.vptr, vbuf.data(), sizeof(int32_t*) * n, cudaMemcpyHostToDevice, st));
         GFD_CUDA(cudaMemsetAsync(T.vcur, 0, 8ull * n, st));
         if (int rc = launch_split(T.desc, T.varena, hs.varena_used, T.vstride, T.vptr, T.vcur, st)) return rc;
-        GFD_CUDA(cudaEventRecord(split->ev, st));
+        if (split) GFD_CUDA(cudaEventRecord(split->ev, st));
         launches[PROF_ENUM] += 1;  // the split belongs to the enumeration's output
     }
     // the refined candidate lists, kept for inspection when asked for
@@ -1822,7 +1835,9 @@ int result_sort_copy(gfd_result* r, int32_t* dst) {
         k_gather_rows<<<rows_grid(n), 256, 0, st>>>(r->d_viol, k, perm, n, sorted);
     }
     GFD_CUDA(cudaGetLastError());
-    return copy_to_host(dst, sorted, 4 * n * k, st);
+    if (int rc = copy_to_host(dst, sorted, 4 * n * k, st)) return rc;
+    r->mem->written = true;
+    return GFD_OK;
 }
 
 int results_sort_copy(gfd_result* const* rs, int n, int32_t* out, uint64_t capacity) {
@@ -1897,7 +1912,10 @@ int results_sort_copy(gfd_result* const* rs, int n, int32_t* out, uint64_t capac
         k_unpack_multi<<<grid, 256, 0, st>>>(d_src, M, W, perm, total, dout);
     }
     GFD_CUDA(cudaGetLastError());
-    return copy_to_host(out, dout, 4 * ints, st);
+    if (int rc = copy_to_host(out, dout, 4 * ints, st)) return rc;
+    for (int r = 0; r < n; r++)
+        if (rs[r]->mem) rs[r]->mem->written = true;
+    return GFD_OK;
 }
 
 }  // namespace gfd

@@ -38,3 +38,18 @@ def test_unread_results_and_another_stream(batch):
             np.testing.assert_array_equal(got.violations(), pairs)
         last = dg.validate_batch([star] * batch, **opts)
         del dg, got, last   # the graph goes while its last call's lists may still be written
+
+
+def test_unread_results_do_not_pile_up():
+    """What was dropped unread is free for the next call."""
+    star = GFD([-1] * 3, [(0, 1, -1), (0, 2, -1)], [], [], True)   # a list of 27 MB
+    dg = G.Graph(_graph())
+    opts = {"max_violations_hint": LEAVES * LEAVES, "frontier_budget_bytes": 32 << 20}
+    for _ in range(3):
+        dg.validate(star, **opts)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for _ in range(30):
+        assert dg.validate(star, **opts).n_violations == math.perm(LEAVES, 2)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= 64 << 20
