@@ -178,7 +178,7 @@ def make_opts(frontier_budget_bytes=0, chunk_rows=0, kernel_variant=0, max_viola
     return o
 
 
-_PLAIN = (list, tuple, np.ndarray)
+_PLAIN = frozenset((list, tuple, np.ndarray))
 
 
 class _GfdBuf:
@@ -194,26 +194,27 @@ class _GfdBuf:
         """Plain sequences of whole numbers, as nearly all GFDs hold them: packed
         without numpy or a ctypes object per literal (5 us a GFD against 14, which
         a batch of 64 on a small graph took a quarter of its time for). Anything
-        else raises and is left to _convert: what looks like numbers to array but
-        not to numpy too (bytes, sets, dicts, one-shot iterators)."""
-        def plain(seq):
-            if not isinstance(seq, _PLAIN):
-                raise TypeError
-            return seq
-        nl = array("i", plain(gfd.node_label))
+        else raises and is left to _convert, also what array would take for numbers
+        and numpy does not (bytes, sets, dicts, one-shot iterators)."""
+        edges, X, Y = gfd.edges, gfd.X, gfd.Y
+        if not (type(gfd.node_label) in _PLAIN and type(edges) in _PLAIN and type(X) in _PLAIN and type(Y) in _PLAIN):
+            raise TypeError
+        nl = array("i", gfd.node_label)
         es, ed, el = array("i"), array("i"), array("i")
-        for e in plain(gfd.edges):
-            a, b, c = plain(e)
+        for e in edges:
+            if type(e) not in _PLAIN:
+                raise TypeError
+            a, b, c = e
             es.append(a)
             ed.append(b)
             el.append(c)
 
         def lits(ls):
             flat = array("i")
-            for q in plain(ls):
+            for q in ls:
                 flat.extend((q.kind, q.x, q.a, q.y, q.b, q.c))
             return flat
-        X, Y = lits(gfd.X), lits(gfd.Y)
+        X, Y = lits(X), lits(Y)
         self.keep = (nl, es, ed, el, X, Y)
         p = [v.buffer_info()[0] if v else None for v in self.keep]
         self.s = gfd_gfd(len(nl), p[0], len(es), p[1], p[2], p[3], len(X) // 6, p[4], len(Y) // 6, p[5],
